@@ -311,8 +311,14 @@ k_score_f32(const Params P, const RangeArgs R, const ListArgs L) {
 // Warp-per-(candidate, model) predictor for small batches.
 // U1 = ceil(h1 / 32) units per lane in layer 1, U2 = ceil(h2 / 32) (0: no layer 2).
 // Weights come from the transposed copy: W1T[d_in][h1], b1, W2T[h1][h2], b2, W3[2][h], b3.
+// A CTA works for one model (blockIdx.y), its warps for the candidates of its share of the
+// list.  Bound by the latency of the weight reads along the layers: ST stages the model's
+// weights in shared memory with one round of wide loads, where reading each row from L2 as
+// it is needed cost a dependent round trip per input of layer 1 and per batch of layer 2
+// (256 candidates x 6 models of 12->64->64->2: 6.6 us staged, 18.8 from L2; 20->128->128->2
+// x 8: 19 and 104).
 // ---------------------------------------------------------------------------
-template <int U1, int U2>
+template <int U1, int U2, bool ST>
 __global__ void __launch_bounds__(kWideWarps * 32)
 k_wide_f32(const Params P, const uint64_t* __restrict__ idx, const int32_t* __restrict__ genes,
            uint64_t n, float* __restrict__ pred, int allow_empty) {
@@ -320,10 +326,19 @@ k_wide_f32(const Params P, const uint64_t* __restrict__ idx, const int32_t* __re
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   const int N = P.n_models, dl = P.d_local, din = P.d_in, h1 = P.h1, h2 = P.h2;
-  const uint64_t tasks = n * (uint64_t)N;
-  for (uint64_t task = warp; task < tasks; task += nwarps) {
-    const uint64_t cand = task / N;
-    const int m = (int)(task % N);
+  const int m = (int)blockIdx.y;
+  const float* w = P.wT + (size_t)m * P.per_model;
+  extern __shared__ __align__(16) float sw[];
+  if constexpr (ST) {
+    const float4* src = reinterpret_cast<const float4*>(w);
+    float4* dst = reinterpret_cast<float4*>(sw);
+#pragma unroll 8
+    for (int e = threadIdx.x; e < (int)(P.per_model >> 2); e += kWideWarps * 32) dst[e] = __ldg(src + e);
+    __syncthreads();
+    w = sw;
+  }
+  auto ldw = [](const float* p) { return ST ? *p : __ldg(p); };
+  for (uint64_t cand = warp; cand < n; cand += nwarps) {
     // lane j < N resolves model j's option and demand
     int o = 0;
     bool ok = true;
@@ -365,17 +380,17 @@ k_wide_f32(const Params P, const uint64_t* __restrict__ idx, const int32_t* __re
     else if (lane == dl + 2) zown = A2 * P.agg_scale[2];
     else if (lane == dl + 3) zown = (float)N * P.agg_scale[3];
 
-    const float* w = P.wT + (size_t)m * P.per_model;
     const float* W1T = w;
     const float* b1 = W1T + (size_t)din * h1;
     float hv1[U1];
 #pragma unroll
     for (int u = 0; u < U1; ++u) {
       const int j = lane + 32 * u;
-      float s = j < h1 ? __ldg(b1 + j) : 0.f;
+      float s = j < h1 ? ldw(b1 + j) : 0.f;
+#pragma unroll 4
       for (int k = 0; k < din; ++k) {
         const float zk = __shfl_sync(0xffffffffu, zown, k);
-        if (j < h1) s = fmaf(__ldg(W1T + (size_t)k * h1 + j), zk, s);
+        if (j < h1) s = fmaf(ldw(W1T + (size_t)k * h1 + j), zk, s);
       }
       hv1[u] = j < h1 ? relu(s) : 0.f;
     }
@@ -389,7 +404,7 @@ k_wide_f32(const Params P, const uint64_t* __restrict__ idx, const int32_t* __re
 #pragma unroll
       for (int u2 = 0; u2 < U2; ++u2) {
         const int j = lane + 32 * u2;
-        acc2[u2] = j < h2 ? __ldg(b2 + j) : 0.f;
+        acc2[u2] = j < h2 ? ldw(b2 + j) : 0.f;
       }
 #pragma unroll
       for (int u = 0; u < U1; ++u) {
@@ -401,7 +416,7 @@ k_wide_f32(const Params P, const uint64_t* __restrict__ idx, const int32_t* __re
 #pragma unroll
             for (int u2 = 0; u2 < U2; ++u2) {
               const int j = lane + 32 * u2;
-              if (j < h2) acc2[u2] = fmaf(__ldg(W2T + (size_t)k * h2 + j), hk, acc2[u2]);
+              if (j < h2) acc2[u2] = fmaf(ldw(W2T + (size_t)k * h2 + j), hk, acc2[u2]);
             }
           }
         }
@@ -411,8 +426,8 @@ k_wide_f32(const Params P, const uint64_t* __restrict__ idx, const int32_t* __re
         const int j = lane + 32 * u2;
         if (j < h2) {
           const float a = relu(acc2[u2]);
-          t = fmaf(__ldg(W3 + j), a, t);
-          l = fmaf(__ldg(W3 + h2 + j), a, l);
+          t = fmaf(ldw(W3 + j), a, t);
+          l = fmaf(ldw(W3 + h2 + j), a, l);
         }
       }
     } else {
@@ -421,8 +436,8 @@ k_wide_f32(const Params P, const uint64_t* __restrict__ idx, const int32_t* __re
       for (int u = 0; u < U1; ++u) {
         const int j = lane + 32 * u;
         if (j < h1) {
-          t = fmaf(__ldg(W3 + j), hv1[u], t);
-          l = fmaf(__ldg(W3 + h1 + j), hv1[u], l);
+          t = fmaf(ldw(W3 + j), hv1[u], t);
+          l = fmaf(ldw(W3 + h1 + j), hv1[u], l);
         }
       }
     }
@@ -434,8 +449,8 @@ k_wide_f32(const Params P, const uint64_t* __restrict__ idx, const int32_t* __re
     if (lane == 0) {
       const int hl = h2 > 0 ? h2 : h1;
       const float* b3 = w + (size_t)din * h1 + h1 + (h2 > 0 ? (size_t)h1 * h2 + h2 : 0) + 2 * hl;
-      pred[(cand * N + m) * 2 + 0] = out_act(P, t + __ldg(b3));
-      pred[(cand * N + m) * 2 + 1] = out_act(P, l + __ldg(b3 + 1));
+      pred[(cand * N + m) * 2 + 0] = out_act(P, t + ldw(b3));
+      pred[(cand * N + m) * 2 + 1] = out_act(P, l + ldw(b3 + 1));
     }
   }
 }
@@ -444,29 +459,26 @@ k_wide_f32(const Params P, const uint64_t* __restrict__ idx, const int32_t* __re
 __global__ void k_combine(const Params P, const uint64_t* __restrict__ idx,
                           const int32_t* __restrict__ genes, uint64_t n,
                           const float* __restrict__ pred, float* __restrict__ score,
-                          uint8_t* __restrict__ feas, int allow_empty) {
+                          uint8_t* __restrict__ feas) {
   const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
   const int N = P.n_models;
-  bool ok = true;
-  float A1 = 0.f;
-  uint64_t id = genes ? 0 : idx[t];
-  if (!genes && id >= P.total) ok = false;
-  for (int i = 0; i < N && ok; ++i) {
-    const int o = genes ? genes[t * N + i] : digit_of(P, id, i);
-    if (o < 0 || o >= P.K[i]) { ok = false; break; }
-    A1 += __ldg(&P.dem[P.off[i] + o]).y;
-  }
+  const uint64_t id = genes ? 0 : idx[t];
+  bool ok = genes || id < P.total;
+  if (genes)
+    for (int i = 0; i < N; ++i) ok = ok && genes[t * N + i] >= 0 && genes[t * N + i] < P.K[i];
   bool f = false;
   float J = -INFINITY;
   if (ok) {
     Acc acc;
     acc.init();
+    float vram = 0.f;
     for (int i = 0; i < N; ++i) {
-      const int o = genes ? genes[t * N + i] : digit_of(P, id, i);
-      acc.add(P, i, pred[(t * N + i) * 2], pred[(t * N + i) * 2 + 1], P.off[i] + o);
+      const int row = P.off[i] + (genes ? genes[t * N + i] : digit_of(P, id, i));
+      vram += __ldg(&P.dem[row]).y;
+      acc.add(P, i, pred[(t * N + i) * 2], pred[(t * N + i) * 2 + 1], row);
     }
-    f = acc.finish(P, A1);
+    f = acc.finish(P, vram);
     J = acc.J;
   }
   score[t] = J;
@@ -548,44 +560,51 @@ mf_status f32_search_chunk(mf_ctx* c, const RangeArgs& a, cudaStream_t s) {
   return MF_OK;
 }
 
+// A model's weights up to this size are staged in shared memory (two CTAs per SM and more);
+// above it (both hidden layers wider than about 150) they are read from L2.
+constexpr size_t kWideStage = 96 * 1024;
+
 template <int U1, int U2>
-static void launch_wide(const Params& P, const uint64_t* idx, const int32_t* genes, uint64_t n,
-                        float* pred, int grid, cudaStream_t s, int allow_empty) {
-  k_wide_f32<U1, U2><<<grid, kWideWarps * 32, 0, s>>>(P, idx, genes, n, pred, allow_empty);
-}
-
-static mf_status score_wide(mf_ctx* c, const uint64_t* idx, const int32_t* genes, uint64_t n,
-                            float* score, uint8_t* feas, float* pred, cudaStream_t s, int allow_empty) {
+static mf_status launch_wide(mf_ctx* c, const uint64_t* idx, const int32_t* genes, uint64_t n, float* pred,
+                             cudaStream_t s, int allow_empty) {
   const Params& P = c->P;
-  const uint64_t tasks = n * (uint64_t)P.n_models;
-  {  // grid: up to four 8-warp CTAs per SM, warps loop over the tasks
-    const int u1 = (P.h1 + 31) / 32, u2 = (P.h2 + 31) / 32;
-    const uint64_t blocks = (tasks + kWideWarps - 1) / kWideWarps;
-    const int grid = (int)(blocks < 4ull * c->num_sms ? blocks : 4ull * c->num_sms);
-    if (u2 == 0) {
-      if (u1 <= 1) launch_wide<1, 0>(P, idx, genes, n, pred, grid, s, allow_empty);
-      else if (u1 <= 2) launch_wide<2, 0>(P, idx, genes, n, pred, grid, s, allow_empty);
-      else if (u1 <= 4) launch_wide<4, 0>(P, idx, genes, n, pred, grid, s, allow_empty);
-      else launch_wide<8, 0>(P, idx, genes, n, pred, grid, s, allow_empty);
-    } else {
-      const int u = u1 > u2 ? u1 : u2;
-      if (u <= 1) launch_wide<1, 1>(P, idx, genes, n, pred, grid, s, allow_empty);
-      else if (u <= 2) launch_wide<2, 2>(P, idx, genes, n, pred, grid, s, allow_empty);
-      else if (u <= 4) launch_wide<4, 4>(P, idx, genes, n, pred, grid, s, allow_empty);
-      else launch_wide<8, 8>(P, idx, genes, n, pred, grid, s, allow_empty);
-    }
-    MF_CUDA(cudaGetLastError());
-    k_combine<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(P, idx, genes, n, pred, score, feas,
-                                                           allow_empty);
-    MF_CUDA(cudaGetLastError());
-    return MF_OK;
+  const size_t wbytes = (size_t)P.per_model * sizeof(float);
+  const bool st = wbytes <= kWideStage;
+  // up to four 8-warp CTAs per SM (two with large weights), split evenly over the models
+  const uint64_t slots = (uint64_t)c->num_sms * (wbytes <= kWideStage / 2 || !st ? 4 : 2);
+  const uint64_t most = slots / P.n_models > 0 ? slots / P.n_models : 1;
+  const uint64_t blocks = (n + kWideWarps - 1) / kWideWarps;
+  const dim3 grid((unsigned)(blocks < most ? blocks : most), (unsigned)P.n_models);
+  if (st) {
+    MF_CUDA(cudaFuncSetAttribute(k_wide_f32<U1, U2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWideStage));
+    k_wide_f32<U1, U2, true><<<grid, kWideWarps * 32, wbytes, s>>>(P, idx, genes, n, pred, allow_empty);
+  } else {
+    k_wide_f32<U1, U2, false><<<grid, kWideWarps * 32, 0, s>>>(P, idx, genes, n, pred, allow_empty);
   }
+  MF_CUDA(cudaGetLastError());
+  return MF_OK;
 }
 
-mf_status f32_score_list_ex(mf_ctx* c, const uint64_t* idx, uint64_t n, float* score, float* pred,
-                            cudaStream_t s) {
+// Predictions [n][N][2], warp per (candidate, model).
+static mf_status predict_wide(mf_ctx* c, const uint64_t* idx, const int32_t* genes, uint64_t n, float* pred,
+                              cudaStream_t s, int allow_empty) {
+  const int u1 = (c->P.h1 + 31) / 32, u2 = (c->P.h2 + 31) / 32;
+  if (u2 == 0) {
+    if (u1 <= 1) return launch_wide<1, 0>(c, idx, genes, n, pred, s, allow_empty);
+    if (u1 <= 2) return launch_wide<2, 0>(c, idx, genes, n, pred, s, allow_empty);
+    if (u1 <= 4) return launch_wide<4, 0>(c, idx, genes, n, pred, s, allow_empty);
+    return launch_wide<8, 0>(c, idx, genes, n, pred, s, allow_empty);
+  }
+  const int u = u1 > u2 ? u1 : u2;
+  if (u <= 1) return launch_wide<1, 1>(c, idx, genes, n, pred, s, allow_empty);
+  if (u <= 2) return launch_wide<2, 2>(c, idx, genes, n, pred, s, allow_empty);
+  if (u <= 4) return launch_wide<4, 4>(c, idx, genes, n, pred, s, allow_empty);
+  return launch_wide<8, 8>(c, idx, genes, n, pred, s, allow_empty);
+}
+
+mf_status f32_predict_shortlist(mf_ctx* c, const uint64_t* idx, uint64_t n, float* pred, cudaStream_t s) {
   if (n == 0) return MF_OK;
-  return score_wide(c, idx, nullptr, n, score, nullptr, pred, s, 1);
+  return predict_wide(c, idx, nullptr, n, pred, s, 1);
 }
 
 mf_status f32_score_list(mf_ctx* c, const uint64_t* idx, const int32_t* genes, uint64_t n,
@@ -594,7 +613,13 @@ mf_status f32_score_list(mf_ctx* c, const uint64_t* idx, const int32_t* genes, u
   const Params& P = c->P;
   const uint64_t tasks = n * (uint64_t)P.n_models;
   // Small batches: warp per (candidate, model), then a combine pass.
-  if (tasks <= 64ull * 1024 && pred != nullptr) return score_wide(c, idx, genes, n, score, feas, pred, s, 0);
+  if (tasks <= 64ull * 1024 && pred != nullptr) {
+    const mf_status st = predict_wide(c, idx, genes, n, pred, s, 0);
+    if (st != MF_OK) return st;
+    k_combine<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(P, idx, genes, n, pred, score, feas);
+    MF_CUDA(cudaGetLastError());
+    return MF_OK;
+  }
   bool res;
   const size_t smem = f32_smem_bytes(P, 0, res);
   ScoreFn fn = pick_fn(genes ? kModeGenes : kModeList, fixed_shape_id(P), res);

@@ -1,19 +1,107 @@
 // Reductions of the exhaustive search (the argmax of Sec. II extended to a
-// top-k): merging the per-CTA running lists, and selecting the top-k of a
-// re-scored shortlist.  Order: J descending, index ascending.
+// top-k): merging the running lists, and the top-k of a re-scored shortlist.
+// Order: J descending, index ascending.
 #include "mf_internal.cuh"
 
 namespace mf {
 
-// Pairwise merge tree over `nlists` sorted lists of length k, by one CTA.
-// Each element's output position is its position in its own list plus the
-// number of elements of the partner list that precede it (binary search);
-// elements at positions >= k are dropped.  Indices are distinct, so positions
-// never collide.
-__global__ void __launch_bounds__(1024)
-k_merge_lists(const float* __restrict__ in_s, const uint64_t* __restrict__ in_i, int nlists, int k,
-              float* a_s, uint64_t* a_i, float* b_s, uint64_t* b_i,
-              float* __restrict__ out_s, uint64_t* __restrict__ out_i) {
+namespace {
+
+constexpr int kMergeThreads = 1024;
+constexpr int kMergeLane = 20;                       // list entries a lane holds: up to 640 lists
+constexpr int kMergeMaxLists = 32 * kMergeLane;
+constexpr size_t kPair = sizeof(uint64_t) + sizeof(float);
+
+// Unsigned key with the order of the scores (no NaN among them; -0 and +0 compare equal).
+__device__ __forceinline__ uint32_t order_key(float s) {
+  const uint32_t u = __float_as_uint(s + 0.f);
+  return u ^ ((u >> 31) ? 0xFFFFFFFFu : 0x80000000u);
+}
+
+// Sorts n distinct entries (ss, si) of shared memory best first and writes the first k
+// to the output, empty slots after them.  Up to one entry per thread: each warp sorts its
+// 32 in registers (shuffles), then an entry's position is its place in its own row of 32
+// plus, by binary search, the entries of every other row ahead of it.  The sorted entries
+// leave in whole rows: the output may be host memory, where each scattered word costs a
+// transaction.  More entries: a bitonic network over the next power of two.  The arrays
+// hold n rounded up to whole rows of 32, or that power of two (at least 1024).
+__device__ void sort_out(float* ss, uint64_t* si, int n, int k, const ResultOut& out) {
+  const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, row = tid >> 5;
+  const int rows = (n + 31) >> 5;
+  if (n <= nthr) {
+    float s = -INFINITY;
+    uint64_t id = kEmptyIdx;
+    if (tid < n) { s = ss[tid]; id = si[tid]; }
+    if (row < rows) {
+#pragma unroll
+      for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+          const float os = __shfl_xor_sync(0xffffffffu, s, stride);
+          const uint64_t oid = __shfl_xor_sync(0xffffffffu, id, stride);
+          const bool keep_better = ((lane & stride) == 0) == ((lane & size) == 0);
+          if (precedes(s, id, os, oid) != keep_better) { s = os; id = oid; }
+        }
+      ss[tid] = s;
+      si[tid] = id;
+    }
+    __syncthreads();
+    int rank = lane;
+    if (row < rows) {
+#pragma unroll 4
+      for (int r = 0; r < rows; ++r) {
+        const float* rs = ss + 32 * r;
+        int lo = 0;  // entries with a better score: no branch in the search
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1) lo += rs[lo + step - 1] > s ? step : 0;
+        lo += rs[lo] > s ? 1 : 0;
+        if (r == row) continue;
+        for (; lo < 32 && rs[lo] == s && si[32 * r + lo] < id; ++lo) {}  // ties, by index
+        rank += lo;
+      }
+    }
+    __syncthreads();
+    if (row < rows && id != kEmptyIdx) { ss[rank] = s; si[rank] = id; }
+    __syncthreads();
+    for (int j = tid; j < k && j < n; j += nthr) { out.score[j] = ss[j]; out.idx[j] = si[j]; }
+  } else {
+    int n2 = 1024;
+    while (n2 < n) n2 <<= 1;
+    for (int e = n + tid; e < n2; e += nthr) { ss[e] = -INFINITY; si[e] = kEmptyIdx; }
+    __syncthreads();
+    for (int size = 2; size <= n2; size <<= 1)
+      for (int stride = size >> 1; stride > 0; stride >>= 1) {
+        for (int i = tid; i < (n2 >> 1); i += nthr) {
+          const int a = 2 * i - (i & (stride - 1)), b = a + stride;
+          const float sa = ss[a], sb = ss[b];
+          const uint64_t ia = si[a], ib = si[b];
+          const bool best_first = (a & size) == 0;
+          if (best_first ? precedes(sb, ib, sa, ia) : precedes(sa, ia, sb, ib)) {
+            ss[a] = sb; si[a] = ib;
+            ss[b] = sa; si[b] = ia;
+          }
+        }
+        __syncthreads();
+      }
+    for (int e = tid; e < k && e < n; e += nthr) { out.score[e] = ss[e]; out.idx[e] = si[e]; }
+  }
+  for (int e = n + tid; e < k; e += nthr) { out.score[e] = -INFINITY; out.idx[e] = kEmptyIdx; }
+}
+
+// The count and the status word beside the lists (nothing where the caller copies them).
+__device__ __forceinline__ void pass_on(const ResultOut& out) {
+  if (threadIdx.x == 0 && out.count) {
+    *out.count = *out.count_src;
+    *out.status = *out.status_src;
+  }
+}
+
+// Pairwise merge tree over `nlists` sorted lists of length k through the buffers a and b.
+// Each element's output position is its position in its own list plus the number of
+// elements of the partner list that precede it (binary search); elements at positions
+// >= k are dropped.  Indices are distinct, so positions never collide.
+__device__ __noinline__ void merge_tree(const float* in_s, const uint64_t* in_i, int nlists, int k, float* a_s,
+                                        uint64_t* a_i, float* b_s, uint64_t* b_i, const ResultOut& out) {
   const float* src_s = in_s;
   const uint64_t* src_i = in_i;
   float* dst_s = a_s;
@@ -55,71 +143,203 @@ k_merge_lists(const float* __restrict__ in_s, const uint64_t* __restrict__ in_i,
     dst_i = (dst_i == a_i) ? b_i : a_i;
     n = m;
   }
-  for (int e = threadIdx.x; e < k; e += blockDim.x) { out_s[e] = src_s[e]; out_i[e] = src_i[e]; }
+  for (int e = threadIdx.x; e < k; e += blockDim.x) { out.score[e] = src_s[e]; out.idx[e] = src_i[e]; }
 }
 
-// Bitonic sort of up to 8192 (score, index) pairs in shared memory by the total
-// order; the first k go to the output.
-__global__ void __launch_bounds__(1024)
-k_select_topk(const float* __restrict__ in_s, const uint64_t* __restrict__ in_i, int n, int n2, int k,
-              float* __restrict__ out_s, uint64_t* __restrict__ out_i) {
+}  // namespace
+
+// Merge of `nlists` sorted lists of length k into one, by one CTA.
+//
+// Only k of the nlists * k entries survive, so the entries that cannot are dropped before
+// anything is sorted.  If T lists have an entry of score >= x at position p, at least
+// T (p + 1) entries reach x; so for T = ceil(k / (p + 1)) the T-th largest score at
+// position p bounds the k-th best entry from below.  Warp j takes the bound of position
+// p = 4^j - 1 (bisection over the score keys, each lane holding up to kMergeLane lists),
+// and the largest bound is the bar: at most k / 4^j lists then hold more than 4^j - 1
+// entries above it, so one to two k entries remain, and 4 k (log4(k) + 1) at most, ties
+// with the bar aside.  They are gathered into shared memory (`cap` entries) and sorted there.  Where
+// ties leave more than that, and above kMergeMaxLists lists, a merge tree through global
+// memory takes over.
+//
+// Bound by latency (a few dependent L2 reads and block barriers).  608 lists of 256
+// entries: 14 us, where the tree alone took 380-560; 304 lists of 32: 9 (tree: 35).
+__global__ void __launch_bounds__(kMergeThreads)
+k_merge_lists(const float* __restrict__ in_s, const uint64_t* __restrict__ in_i, int nlists, int k, int cap,
+              float* a_s, uint64_t* a_i, float* b_s, uint64_t* b_i, const ResultOut out) {
   extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ uint32_t s_bar[32];
+  __shared__ int s_lists[kMergeMaxLists];
+  __shared__ int s_nlist, s_n;
   uint64_t* si = reinterpret_cast<uint64_t*>(smem);
-  float* ss = reinterpret_cast<float*>(si + n2);
-  for (int e = threadIdx.x; e < n2; e += blockDim.x) {
-    if (e < n) { ss[e] = in_s[e]; si[e] = in_i[e]; }
-    else { ss[e] = -INFINITY; si[e] = kEmptyIdx; }
-    if (ss[e] == -INFINITY) si[e] = kEmptyIdx;  // infeasible entries sort last
-  }
+  float* ss = reinterpret_cast<float*>(si + cap);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid < 32) s_bar[tid] = 0u;
+  if (tid == 0) { s_nlist = 0; s_n = 0; }
   __syncthreads();
-  for (int size = 2; size <= n2; size <<= 1) {
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int i = threadIdx.x; i < n2; i += blockDim.x) {
-        const int j = i ^ stride;
-        if (j > i) {
-          const bool up = (i & size) == 0;
-          const bool sw = up ? precedes(ss[j], si[j], ss[i], si[i]) : precedes(ss[i], si[i], ss[j], si[j]);
-          if (sw) {
-            const float ts = ss[i]; ss[i] = ss[j]; ss[j] = ts;
-            const uint64_t ti = si[i]; si[i] = si[j]; si[j] = ti;
-          }
+  bool few = nlists <= kMergeMaxLists;
+  if (few) {
+    const int p = (1 << (warp < 10 ? 2 * warp : 20)) - 1;
+    const int need = (k + p) / (p + 1);  // T
+    if (p < k && need <= nlists) {
+      uint32_t key[kMergeLane];
+#pragma unroll
+      for (int j = 0; j < kMergeLane; ++j) {
+        const int l = lane + 32 * j;
+        key[j] = l < nlists ? order_key(in_s[(size_t)l * k + p]) : 0u;
+      }
+      uint32_t v = 0u;
+      for (int b = 31; b >= 0; --b) {
+        const uint32_t t = v | (1u << b);
+        int c[4] = {0, 0, 0, 0};  // (short chains of dependent adds)
+#pragma unroll
+        for (int j = 0; j < kMergeLane; ++j) c[j & 3] += key[j] >= t ? 1 : 0;
+        const int reach = __reduce_add_sync(0xffffffffu, (c[0] + c[1]) + (c[2] + c[3]));
+        if (reach >= need) v = t;
+        if (reach == need) break;  // (lower bits would only tighten the bar past ties)
+      }
+      if (lane == 0) s_bar[warp] = v;
+    }
+    __syncthreads();
+    const uint32_t bar = __reduce_max_sync(0xffffffffu, s_bar[lane]);
+    // the lists whose best entry reaches the bar, then their entries that do
+    for (int l = tid; l < nlists; l += kMergeThreads)
+      if (order_key(in_s[(size_t)l * k]) >= bar)
+        s_lists[atomicAdd(&s_nlist, 1)] = l;
+    __syncthreads();
+    const int nl = s_nlist;
+    constexpr int kBatch = 8;  // lists a warp has in flight
+    for (int q0 = warp; q0 < nl; q0 += (kMergeThreads / 32) * kBatch) {
+      float v[kBatch];
+      uint64_t id[kBatch];
+#pragma unroll
+      for (int j = 0; j < kBatch; ++j) {
+        const int q = q0 + j * (kMergeThreads / 32);
+        const bool in = q < nl && lane < k;
+        const size_t at = in ? (size_t)s_lists[q] * k + lane : 0;
+        v[j] = in ? in_s[at] : -INFINITY;
+        id[j] = in ? in_i[at] : kEmptyIdx;
+      }
+      auto place = [&](bool keep, unsigned m, int at, float sc, uint64_t ix) {
+        at += __popc(m & ((1u << lane) - 1u));
+        if (keep && at < cap) { ss[at] = sc; si[at] = ix; }
+      };
+      unsigned m[kBatch];  // the lanes whose entry stays: a prefix (the lists are sorted)
+      int total = 0;
+      unsigned more = 0u;  // the lists whose first 32 entries all stay
+#pragma unroll
+      for (int j = 0; j < kBatch; ++j) {
+        m[j] = __ballot_sync(0xffffffffu, id[j] != kEmptyIdx && order_key(v[j]) >= bar);
+        total += __popc(m[j]);
+        more |= m[j] == 0xffffffffu ? 1u << j : 0u;
+      }
+      int at = 0;
+      if (lane == 0 && total) at = atomicAdd(&s_n, total);
+      at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+      for (int j = 0; j < kBatch; ++j) {
+        place((m[j] >> lane) & 1u, m[j], at, v[j], id[j]);
+        at += __popc(m[j]);
+      }
+      for (; more; more &= more - 1u) {
+        const size_t l = (size_t)s_lists[q0 + (__ffs(more) - 1) * (kMergeThreads / 32)] * k;
+        unsigned whole = 0xffffffffu;
+        for (int pos = lane + 32; whole == 0xffffffffu; pos += 32) {
+          const float sc = pos < k ? in_s[l + pos] : -INFINITY;
+          const uint64_t ix = pos < k ? in_i[l + pos] : kEmptyIdx;
+          const bool keep = ix != kEmptyIdx && order_key(sc) >= bar;
+          whole = __ballot_sync(0xffffffffu, keep);
+          int to = 0;
+          if (lane == 0 && whole) to = atomicAdd(&s_n, __popc(whole));
+          place(keep, whole, __shfl_sync(0xffffffffu, to, 0), sc, ix);
         }
       }
-      __syncthreads();
     }
+    __syncthreads();
+    few = s_n <= cap;
   }
-  for (int e = threadIdx.x; e < k; e += blockDim.x) { out_s[e] = ss[e]; out_i[e] = si[e]; }
+  if (few) sort_out(ss, si, s_n, k, out);
+  else merge_tree(in_s, in_i, nlists, k, a_s, a_i, b_s, b_i, out);
+  pass_on(out);
 }
 
-mf_status merge_lists(mf_ctx* c, const float* ls, const uint64_t* li, int nlists, int k,
-                      float* tmp_s, uint64_t* tmp_i, float* out_s, uint64_t* out_i,
-                      cudaStream_t s) {
+// The end of a bf16 search: objective and constraints of the shortlist's n entries from
+// their fp32 predictions (pred [n][N][2]; an empty entry stays empty), and the best k of
+// them.  One CTA: n is 8 k or 256, and what it costs is latency.  NMAX: a bound on N.
+template <int NMAX>
+__global__ void __launch_bounds__(512)
+k_finish(const Params P, const uint64_t* __restrict__ idx, const float* __restrict__ pred, int n, int n2, int k,
+         const ResultOut out) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ int s_n;
+  uint64_t* si = reinterpret_cast<uint64_t*>(smem);
+  float* ss = reinterpret_cast<float*>(si + n2);
+  if (threadIdx.x == 0) s_n = 0;
+  __syncthreads();
+  for (int e = threadIdx.x; e < n; e += blockDim.x) {
+    const uint64_t id = idx[e];
+    if (id >= P.total) continue;
+    // every operand is read before the first is used: one L2 round trip, not one per model
+    int row[NMAX];
+    float2 pr[NMAX];
+    float vr[NMAX];
+    float4 ut[NMAX];
+#pragma unroll
+    for (int i = 0; i < NMAX; ++i) {
+      if (i < P.n_models) {
+        row[i] = P.off[i] + digit_of(P, id, i);
+        pr[i] = *reinterpret_cast<const float2*>(pred + ((size_t)e * P.n_models + i) * 2);
+        vr[i] = __ldg(&P.dem[row[i]].y);
+        if (P.objective == MF_OBJ_UTILITY) ut[i] = __ldg(&P.util[row[i]]);
+      }
+    }
+    Acc acc;
+    acc.init();
+    float vram = 0.f;
+#pragma unroll
+    for (int i = 0; i < NMAX; ++i) {
+      if (i < P.n_models) {
+        vram += vr[i];
+        acc.add_util(P, i, pr[i].x, pr[i].y, ut[i]);
+      }
+    }
+    acc.finish(P, vram);
+    if (acc.J == -INFINITY) continue;  // infeasible in fp32
+    const int at = atomicAdd(&s_n, 1);
+    ss[at] = acc.J;
+    si[at] = id;
+  }
+  __syncthreads();
+  sort_out(ss, si, s_n, k, out);
+  pass_on(out);
+}
+
+mf_status merge_lists(const float* ls, const uint64_t* li, int nlists, int k, float* tmp_s, uint64_t* tmp_i,
+                      const ResultOut& out, cudaStream_t s) {
   // tmp holds two buffers of ceil(nlists / 2) * k entries each
   const size_t half = (size_t)((nlists + 1) / 2) * k;
-  k_merge_lists<<<1, 1024, 0, s>>>(ls, li, nlists, k, tmp_s, tmp_i, tmp_s + half, tmp_i + half,
-                                   out_s, out_i);
+  // room for 4096 survivors in short lists (k <= 256), else 16384
+  const int cap = k <= 256 ? 4096 : 16384;
+  const size_t smem = (size_t)cap * kPair;
+  MF_CUDA(cudaFuncSetAttribute(k_merge_lists, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k_merge_lists<<<1, kMergeThreads, smem, s>>>(ls, li, nlists, k, cap, tmp_s, tmp_i, tmp_s + half, tmp_i + half,
+                                               out);
   MF_CUDA(cudaGetLastError());
-  (void)c;
   return MF_OK;
 }
 
-mf_status select_topk(mf_ctx* c, const float* in_s, const uint64_t* in_i, int n, int k,
-                      float* out_s, uint64_t* out_i, cudaStream_t s) {
-  int n2 = 1;
+mf_status finish_shortlist(const Params& P, const uint64_t* idx, const float* pred, int n, int k,
+                           const ResultOut& out, cudaStream_t s) {
+  int n2 = 32;
   while (n2 < n) n2 <<= 1;
-  if (n2 < k) n2 = k;
-  int p2 = 1;
-  while (p2 < n2) p2 <<= 1;
-  n2 = p2;
   if (n2 > 8192) {
-    set_error("select_topk: more than 8192 entries");
+    set_error("finish_shortlist: more than 8192 entries");
     return MF_EINVAL;
   }
-  const size_t smem = (size_t)n2 * (sizeof(float) + sizeof(uint64_t));
-  MF_CUDA(cudaFuncSetAttribute(k_select_topk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_select_topk<<<1, 1024, smem, s>>>(in_s, in_i, n, n2, k, out_s, out_i);
+  const size_t smem = (size_t)n2 * kPair;
+  const auto fn = P.n_models <= 8 ? k_finish<8> : k_finish<MF_MAX_MODELS>;
+  MF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  fn<<<1, 512, smem, s>>>(P, idx, pred, n, n2, k, out);
   MF_CUDA(cudaGetLastError());
-  (void)c;
   return MF_OK;
 }
 

@@ -401,10 +401,7 @@ static mf_status search_impl(mf_ctx* ctx, uint64_t lo, uint64_t hi, int32_t k, u
   const size_t o_ti = o; o = align_up(o + sizeof(uint64_t) * 2 * half, 256);
   const size_t o_ms = o; o = align_up(o + sizeof(float) * kcap, 256);
   const size_t o_mi = o; o = align_up(o + sizeof(uint64_t) * kcap, 256);
-  const size_t o_rs = o; o = align_up(o + sizeof(float) * kcap, 256);
   const size_t o_rp = o; o = align_up(o + sizeof(float) * 2 * kcap * ctx->P.n_models, 256);
-  const size_t o_fs = o; o = align_up(o + sizeof(float) * k, 256);
-  const size_t o_fi = o; o = align_up(o + sizeof(uint64_t) * k, 256);
   const size_t o_cnt = o; o = align_up(o + sizeof(unsigned long long), 256);
   mf_status st = ensure_scratch(ctx, o);
   if (st != MF_OK) return st;
@@ -415,11 +412,19 @@ static mf_status search_impl(mf_ctx* ctx, uint64_t lo, uint64_t hi, int32_t k, u
   uint64_t* ti = (uint64_t*)(base + o_ti);
   float* ms = (float*)(base + o_ms);
   uint64_t* mi = (uint64_t*)(base + o_mi);
-  float* rs = (float*)(base + o_rs);
   float* rp = (float*)(base + o_rp);
-  float* fs = (float*)(base + o_fs);
-  uint64_t* fi = (uint64_t*)(base + o_fi);
   unsigned long long* cnt = (unsigned long long*)(base + o_cnt);
+  // the result, in pinned host memory: top-k, count and status word, written by the last
+  // kernel itself (a copy for each cost about 3.7 us apiece on the stream)
+  const size_t h_sc = sizeof(uint64_t) * k, h_cn = align_up(h_sc + sizeof(float) * k, 8);
+  st = ensure_host_stage(ctx, h_cn + sizeof(unsigned long long) + sizeof(uint32_t));
+  if (st != MF_OK) return st;
+  char* h = (char*)ctx->h_stage;
+  const uint64_t* h_i = (uint64_t*)h;
+  const float* h_s = (float*)(h + h_sc);
+  const unsigned long long* h_c = (unsigned long long*)(h + h_cn);
+  const uint32_t* h_status = (uint32_t*)(h_c + 1);
+  const ResultOut result{(uint64_t*)h_i, (float*)h_s, (unsigned long long*)h_c, (uint32_t*)h_status, cnt, ctx->d_status};
   MF_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), s));
 
   int launches = 0, score_launches = 0;
@@ -451,35 +456,21 @@ static mf_status search_impl(mf_ctx* ctx, uint64_t lo, uint64_t hi, int32_t k, u
     score_launches += nl;
   }
   MF_CUDA(cudaEventRecord(ctx->ev[1], s));
-  st = merge_lists(ctx, ls, li, grid, kcap, ts, ti, ms, mi, s);
   ++launches;
-  if (st != MF_OK) return st;
   if (tc) {
     // exact fp32 re-scoring of the tensor-core shortlist, then the final top-k
-    st = f32_score_list_ex(ctx, mi, kcap, rs, rp, s);
-    if (st != MF_OK) return st;
-    st = select_topk(ctx, rs, mi, kcap, k, fs, fi, s);
-    launches += 3;
+    const ResultOut shortlist{mi, ms, nullptr, nullptr, nullptr, nullptr};
+    st = merge_lists(ls, li, grid, kcap, ts, ti, shortlist, s);
+    if (st == MF_OK) st = f32_predict_shortlist(ctx, mi, kcap, rp, s);
+    if (st == MF_OK) st = finish_shortlist(ctx->P, mi, rp, kcap, k, result, s);
+    launches += 2;
   } else {
-    MF_CUDA(cudaMemcpyAsync(fs, ms, sizeof(float) * k, cudaMemcpyDeviceToDevice, s));
-    MF_CUDA(cudaMemcpyAsync(fi, mi, sizeof(uint64_t) * k, cudaMemcpyDeviceToDevice, s));
+    st = merge_lists(ls, li, grid, k, ts, ti, result, s);
   }
   if (st != MF_OK) return st;
-
-  const size_t hbytes = sizeof(uint64_t) * k + sizeof(float) * k + sizeof(unsigned long long) + 16;
-  st = ensure_host_stage(ctx, hbytes);
-  if (st != MF_OK) return st;
-  char* h = (char*)ctx->h_stage;
-  uint64_t* h_i = (uint64_t*)h;
-  float* h_s = (float*)(h + sizeof(uint64_t) * k);
-  unsigned long long* h_c = (unsigned long long*)(h + sizeof(uint64_t) * k + sizeof(float) * k);
-  uint32_t* h_status = (uint32_t*)(h_c + 1);
-  MF_CUDA(cudaMemcpyAsync(h_i, fi, sizeof(uint64_t) * k, cudaMemcpyDeviceToHost, s));
-  MF_CUDA(cudaMemcpyAsync(h_s, fs, sizeof(float) * k, cudaMemcpyDeviceToHost, s));
-  MF_CUDA(cudaMemcpyAsync(h_c, cnt, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
   MF_CUDA(cudaEventRecord(ctx->ev[2], s));
-  st = read_status(ctx, s, h_status, true);
-  if (st != MF_OK) return st;
+  MF_CUDA(cudaStreamSynchronize(s));
+  if (*h_status) MF_CUDA(cudaMemsetAsync(ctx->d_status, 0, sizeof(uint32_t), s));
   ctx->stats.kernel_launches_last = launches;
   ctx->stats.score_launches_last = score_launches;
   ctx->stats.d2h_bytes_last = (sizeof(uint64_t) + sizeof(float)) * k + sizeof(unsigned long long) + sizeof(uint32_t);

@@ -131,9 +131,13 @@ struct Acc {
   __device__ __forceinline__ void init() { J = 0.f; pen = 0.f; sla_ok = true; }
   // thr, lat: predictor outputs after the output activation; row: the option row.
   __device__ __forceinline__ void add(const Params& P, int i, float thr, float lat, int row) {
+    add_util(P, i, thr, lat, P.objective == MF_OBJ_UTILITY ? P.util[row] : make_float4(0.f, 1.f, 0.f, 0.f));
+  }
+  // the same with the option's row of the utility table in `q` (read by that objective only)
+  __device__ __forceinline__ void add_util(const Params& P, int i, float thr, float lat, float4 q) {
     if (P.objective == MF_OBJ_UTILITY) {
       float f;
-      J += util_term(P, i, row, thr, &f);
+      J += util_term_of(P, q, P.u_omega[i], P.u_tau[i], P.u_cost[i], P.u_prev[i], thr, &f);
       sla_ok = sla_ok && (f >= P.u_tau[i]);
       return;
     }
@@ -292,7 +296,7 @@ __device__ void topk_merge_sorted(const CtaTopK& t, int tid, int nthr, Sync sync
   for (int size = 2; size <= n2; size <<= 1) {
     for (int stride = size >> 1; stride > 0; stride >>= 1) {
       for (int i = tid; i < (n2 >> 1); i += nthr) {
-        const int a = 2 * stride * (i / stride) + (i % stride), b = a + stride;
+        const int a = 2 * i - (i & (stride - 1)), b = a + stride;
         const float sa = t.qs[a], sb = t.qs[b];
         const uint64_t ia = t.qi[a], ib = t.qi[b];
         const bool best_first = (a & size) == 0;
@@ -434,18 +438,27 @@ mf_status fc_search_chunk(mf_ctx* c, const RangeArgs& a, cudaStream_t s);
 mf_status f32_search_chunk_params(const Params& P, int grid, const RangeArgs& a, cudaStream_t s);
 mf_status f32_score_list(mf_ctx* c, const uint64_t* idx, const int32_t* genes, uint64_t n,
                          float* score, uint8_t* feas, float* pred, cudaStream_t s);
-// Exact re-scoring of a shortlist that may contain empty slots (index UINT64_MAX),
-// which score -inf without raising the device status.  pred: scratch [n][N][2].
-mf_status f32_score_list_ex(mf_ctx* c, const uint64_t* idx, uint64_t n, float* score, float* pred,
-                            cudaStream_t s);
+// fp32 predictions [n][N][2] of a shortlist that may contain empty slots (index
+// UINT64_MAX, no predictions); an index out of range raises no status here.
+mf_status f32_predict_shortlist(mf_ctx* c, const uint64_t* idx, uint64_t n, float* pred, cudaStream_t s);
 
-// Merge of per-CTA sorted lists into one sorted top-k.
-mf_status merge_lists(mf_ctx* c, const float* ls, const uint64_t* li, int nlists, int k,
-                      float* tmp_s, uint64_t* tmp_i, float* out_s, uint64_t* out_i,
-                      cudaStream_t s);
-// Sort n (score, idx) pairs by the total order and keep the first k (n <= 8192).
-mf_status select_topk(mf_ctx* c, const float* in_s, const uint64_t* in_i, int n, int k,
-                      float* out_s, uint64_t* out_i, cudaStream_t s);
+// Where a reduction leaves the top-k, and with it (where count is given) the feasible
+// count and the status word: device memory, or pinned host memory, which the kernel
+// writes itself instead of three or four copies after it.
+struct ResultOut {
+  uint64_t* idx;                        // [k]
+  float* score;                         // [k]
+  unsigned long long* count;
+  uint32_t* status;
+  const unsigned long long* count_src;  // device
+  const uint32_t* status_src;           // device
+};
+// Merge of per-CTA sorted lists into one sorted top-k (tmp: 2 ceil(nlists / 2) k entries).
+mf_status merge_lists(const float* ls, const uint64_t* li, int nlists, int k, float* tmp_s, uint64_t* tmp_i,
+                      const ResultOut& out, cudaStream_t s);
+// The best k of a shortlist of n <= 8192 entries from their fp32 predictions.
+mf_status finish_shortlist(const Params& P, const uint64_t* idx, const float* pred, int n, int k,
+                           const ResultOut& out, cudaStream_t s);
 
 // Tensor-core scorer (bf16 path).
 bool tc_supported(const Params& P, std::string* why);

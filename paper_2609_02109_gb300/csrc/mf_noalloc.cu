@@ -225,8 +225,10 @@ extern "C" mf_status mf_search_exhaustive_noalloc(const mf_problem* p, int32_t k
     if (r != MF_OK) return r;
     a.first = 0;
   }
-  mf_status r = merge_lists(nullptr, a.lists_s, a.lists_i, grid, k, (float*)(base + o_ts),
-                            (uint64_t*)(base + o_ti), (float*)(base + o_fs), (uint64_t*)(base + o_fi), s);
+  ResultOut merged{};
+  merged.idx = (uint64_t*)(base + o_fi);
+  merged.score = (float*)(base + o_fs);
+  mf_status r = merge_lists(a.lists_s, a.lists_i, grid, k, (float*)(base + o_ts), (uint64_t*)(base + o_ti), merged, s);
   if (r != MF_OK) return r;
 
   // outputs straight into the caller's host memory
