@@ -25,7 +25,11 @@ struct FcLayout {
   float* f;          // [sumK]
   float* u;          // [sumK]
   uint8_t* ok;       // [sumK]
-  // inputs, copied
+};
+
+// The inputs of mf_fc_set, in pinned host memory: every CTA of k_fc_local reads the few
+// values of its option itself, early and used last, so no copy comes before the kernel.
+struct FcInputs {
   float* obs;        // [4]
   int32_t* variant;  // [sumK]
   float* quality;    // [sumK]
@@ -37,7 +41,7 @@ struct FcLayout {
   int32_t* prev;     // [N]
 };
 
-static size_t fc_bytes(int sumK, int N, FcLayout* L, char* base) {
+static size_t fc_bytes(int sumK, FcLayout* L, char* base) {
   size_t o = 0;
   auto take = [&](size_t bytes) {
     const size_t at = o;
@@ -50,6 +54,17 @@ static size_t fc_bytes(int sumK, int N, FcLayout* L, char* base) {
   p = take(sizeof(float) * sumK); if (L) L->f = (float*)p;
   p = take(sizeof(float) * sumK); if (L) L->u = (float*)p;
   p = take(sumK); if (L) L->ok = (uint8_t*)p;
+  return o;
+}
+
+static size_t fc_input_bytes(int sumK, int N, FcInputs* L, char* base) {
+  size_t o = 0;
+  auto take = [&](size_t bytes) {
+    const size_t at = o;
+    o = (o + bytes + 15) / 16 * 16;
+    return base ? base + at : nullptr;
+  };
+  char* p;
   p = take(sizeof(float) * 4); if (L) L->obs = (float*)p;
   p = take(sizeof(int32_t) * sumK); if (L) L->variant = (int32_t*)p;
   p = take(sizeof(float) * sumK); if (L) L->quality = (float*)p;
@@ -70,31 +85,48 @@ struct FcConst {
 // Local predictions: one CTA per option row.  z = [x_i(o) | obs * s_A]; the hidden
 // layers spread their units over the threads; the throughput head reduces over
 // warp 0.  Thread 0 forms f, the floor flag and u.
+//
+// Bound by latency: the model's weights (the transposed copy) come into shared memory with
+// one round of wide loads where they fit kFcStage, since a row read as it was needed cost
+// an L2 round trip per few inputs (12->64->64->2, 144 rows: 7.1 us, staged FC_LOCAL_NOW).
 // ---------------------------------------------------------------------------
+constexpr size_t kFcStage = 96 * 1024;
+
+template <bool ST>
 __global__ void __launch_bounds__(256)
-k_fc_local(const Params P, const FcLayout L, const FcConst C) {
+k_fc_local(const Params P, const FcLayout L, const FcInputs I, const FcConst C) {
+  extern __shared__ __align__(16) float sw[];
   __shared__ float z[MF_MAX_D_LOCAL + 4];
   __shared__ float h1[MF_MAX_HIDDEN], h2[MF_MAX_HIDDEN];
-  __shared__ int s_model;
   const int r = blockIdx.x, tid = threadIdx.x;
   const int N = P.n_models;
-  if (tid == 0) {
-    int m = 0;
-    for (int i = 0; i < N; ++i)
-      if (r >= pick(P.off, i)) m = i;
-    s_model = m;
-  }
+  int m = 0;
+#pragma unroll
+  for (int i = 1; i < MF_MAX_MODELS; ++i) m += i < N && r >= P.off[i] ? 1 : 0;
   const int dl = P.d_local, din = P.d_in, H1 = P.h1, H2 = P.h2;
-  for (int k = tid; k < dl; k += blockDim.x) z[k] = P.x[(size_t)r * dl + k];
-  if (tid < 4) z[dl + tid] = L.obs[tid] * P.agg_scale[tid];
+  const float* w = P.wT + (size_t)m * P.per_model;
+  if (ST) {
+    const float4* src = reinterpret_cast<const float4*>(w);
+    float4* dst = reinterpret_cast<float4*>(sw);
+#pragma unroll 8
+    for (int e = tid; e < (int)(P.per_model >> 2); e += 256) dst[e] = __ldg(src + e);
+    w = sw;
+  }
+  float f_min = 0.f, f_max = 0.f, tau = 0.f, omega = 0.f, cost = 0.f, quality = 0.f, vram = 0.f;
+  int variant = 0, prev = 0;
+  if (tid == 0) {
+    f_min = I.f_min[r]; f_max = I.f_max[r]; quality = I.quality[r]; variant = I.variant[r];
+    tau = I.tau[m]; omega = I.omega[m]; cost = I.cost[m]; prev = I.prev[m];
+    vram = P.dem[r].y;
+  }
+  if (tid < dl) z[tid] = P.x[(size_t)r * dl + tid];
+  if (tid >= 32 && tid < 36) z[dl + tid - 32] = I.obs[tid - 32] * P.agg_scale[tid - 32];
   __syncthreads();
-  const int m = s_model;
-  const float* w = P.w32 + (size_t)m * P.per_model;
-  const float* W1 = w;
-  const float* b1 = W1 + (size_t)H1 * din;
-  for (int j = tid; j < H1; j += blockDim.x) {
+  const float* b1 = w + (size_t)H1 * din;
+  for (int j = tid; j < H1; j += 256) {
     float s = b1[j];
-    for (int k = 0; k < din; ++k) s = fmaf(W1[(size_t)j * din + k], z[k], s);
+#pragma unroll 4
+    for (int k = 0; k < din; ++k) s = fmaf(w[(size_t)k * H1 + j], z[k], s);
     h1[j] = relu(s);
   }
   __syncthreads();
@@ -102,11 +134,11 @@ k_fc_local(const Params P, const FcLayout L, const FcConst C) {
   const float* h = h1;
   int hl = H1;
   if (H2 > 0) {
-    const float* W2 = next;
-    const float* b2 = W2 + (size_t)H2 * H1;
-    for (int j = tid; j < H2; j += blockDim.x) {
+    const float* b2 = next + (size_t)H2 * H1;
+    for (int j = tid; j < H2; j += 256) {
       float s = b2[j];
-      for (int k = 0; k < H1; ++k) s = fmaf(W2[(size_t)j * H1 + k], h1[k], s);
+#pragma unroll 16
+      for (int k = 0; k < H1; ++k) s = fmaf(next[(size_t)k * H2 + j], h1[k], s);
       h2[j] = relu(s);
     }
     __syncthreads();
@@ -122,64 +154,106 @@ k_fc_local(const Params P, const FcLayout L, const FcConst C) {
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (tid == 0) {
       const float fhat = out_act(P, s + W3[2 * hl]);
-      const float f = (fhat - L.f_min[r]) / (L.f_max[r] - L.f_min[r]);
-      const float tau = L.tau[m];
+      const float f = (fhat - f_min) / (f_max - f_min);
       const bool ok = f >= tau;
-      const float eta = (L.prev[m] >= 0 && L.variant[r] != L.prev[m]) ? 1.f : 0.f;
+      const float eta = (prev >= 0 && variant != prev) ? 1.f : 0.f;
       const float margin = tau + C.delta - f;
-      const float u = L.omega[m] * f * L.quality[r] - C.alpha * eta * L.cost[m] -
-                      C.beta * (margin > 0.f ? margin * margin : 0.f);
+      const float u = omega * f * quality - C.alpha * eta * cost - C.beta * (margin > 0.f ? margin * margin : 0.f);
       L.fhat[r] = fhat;
       L.f[r] = f;
       L.u[r] = u;
       L.ok[r] = ok ? 1 : 0;
-      L.tab[r] = make_float2(ok ? u : -INFINITY, P.dem[r].y);
+      L.tab[r] = make_float2(ok ? u : -INFINITY, vram);
     }
   }
 }
 
 // ---------------------------------------------------------------------------
-// Table-lookup scan.  Each thread walks its own contiguous slice of the range, so from
-// one candidate to the next only the last model's option advances: the partial sum over
-// the other models is reused until a carry, and a carry that stops at model N - 2 (all
-// but one in K_{N-2}) costs one lookup.  J is summed in model order either way.
-// Running top-k: a thread queues a candidate only if it beats the list's k-th entry
-// (held in registers), at most kFcBudget between two merge checks (a thread that runs
-// out stops until the merge); a merge check follows every cycle of the last model's
-// options, at least kFcMinRun candidates (kFcMinRunLong in slices long enough that the
-// list settles early).  WL (k <= kFcWarpK): each warp keeps its own list and queue and
-// merges with warp barriers only, the CTA's list taking the warps' lists at the end;
-// otherwise one list per CTA, the merge check a CTA barrier.
+// Table-lookup scan.  Each thread walks its own contiguous slice of the range, so from one
+// candidate to the next only the last model's option advances, and J and the VRAM demand V
+// are summed in model order.  A configuration is not looked at one by one: fp32 addition is
+// monotone (a <= b gives fl(p + a) <= fl(p + b)), so
+//   - for one setting of the leading N - 1 models, the last model's options within the cap
+//     are a prefix of its options in VRAM order: a binary search counts them;
+//   - for one setting of the leading N - 2 models, the sums of the extreme demands tell
+//     whether all or none of the K_{N-2} K_{N-1} configurations fit, and where some do, the
+//     boundary moves one way as model N - 2's demand grows: two pointers count them in
+//     K_{N-2} + K_{N-1} steps;
+//   - the sums with the largest terms bound every J below from above, and where that bound
+//     does not reach the list's k-th entry no candidate is looked at.
+// The counts and the top-k are exactly those of the sums taken one by one.  This needs
+// finite demands and a finite cap (REG); other tables are scanned one candidate at a time.
+//
+// The bar starts high: J is a sum of per-model terms, so the best configurations sit where
+// every model has one of its best options.  Every CTA first scores a corner of the space, the
+// few best options of each model (m_i, at most kFcCorner configurations), by J - lambda V
+// for four weights lambda of the VRAM demand; the k-th best feasible score of the corner
+// with the smallest lambda that has k of them bounds the k-th best of the range from below.
+//
+// Running top-k: a thread queues a candidate only if it beats the bar, at most kFcBudget
+// between two merge checks (a thread that runs out stops until the merge), one check per
+// kFcSteps steps.  WL (k <= kFcWarpK): each warp keeps its own list and queue and merges
+// with warp barriers only, the CTA's list taking the warps' lists at the end; otherwise one
+// list per CTA, the merge check a CTA barrier.
+//
+// Bound by issue and shared-memory latency.  24^6, VRAM binding, k = 32: one launch of
+// FC_SCAN_NOW, where the scan of every candidate took 12 launches of 75-125 us (each of
+// which also filled its lists from nothing); 2^32: FC_SCAN_STRESS.
 // ---------------------------------------------------------------------------
 constexpr int kFcThreads = 512;
 constexpr int kFcBudget = 8;   // the queue: kFcThreads x kFcBudget entries
-constexpr int kFcMinRun = 16, kFcMinRunLong = 64;
+constexpr int kFcSteps = 8;
 constexpr int kFcWarpK = 64, kFcWarps = kFcThreads / 32;
 constexpr int kFcWarpQ = 32 * kFcBudget;              // a warp's queue
 constexpr int kFcEndQ = kFcWarps * kFcWarpK;          // the warps' lists, merged at the end (a power of two)
-constexpr uint64_t kFcLongSlice = 8192;
+constexpr int kFcLambdas = 4, kFcCornerOpts = 64;     // corner sets, options of a model in one
+constexpr int kFcCorner = 4 * kFcThreads;             // configurations of a corner
+constexpr int kFcCornerRows = 1024;                   // option rows up to which the corners are ranked
 
 struct FcScan {
   const float2* tab;
+  int32_t reg;                        // finite demands and cap
+  int32_t corner[MF_MAX_MODELS];      // m_i; all 0: no corner
 };
 
-// Shared-memory bytes of k_fc_scan<.., WL> after the table.
+// Shared-memory bytes of k_fc_scan<.., WL> after the table and the two VRAM orders.
 __host__ __device__ inline size_t fc_scan_list_bytes(int k, bool wl) {
   const size_t e = sizeof(uint64_t) + sizeof(float);
   if (!wl) return e * (2 * (size_t)k + kFcThreads * kFcBudget) + 16;
   return e * (2 * (size_t)k + kFcEndQ) + 16 + kFcWarps * (e * (2 * (size_t)k + kFcWarpQ) + 16);
 }
+__host__ __device__ inline size_t fc_scan_table_bytes(int sumK) {
+  return (((size_t)sumK * sizeof(float2) + 15) & ~(size_t)15) + 2 * 256 * sizeof(float);
+}
 
-template <int NMAX, bool WL>
+// Monotone unsigned key of a float that is not NaN.
+__device__ __forceinline__ uint32_t fc_key(float v) {
+  const uint32_t u = __float_as_uint(v + 0.f);
+  return u ^ ((u >> 31) ? 0xFFFFFFFFu : 0x80000000u);
+}
+__device__ __forceinline__ float fc_unkey(uint32_t k) {
+  return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xFFFFFFFFu));
+}
+
+// The extremes of a model's usable options (finite VRAM in the CTA's table).
+struct FcSpan {
+  float jmax, jmin, vmin, vmax;
+  int n;
+};
+
+template <int NMAX, bool WL, bool REG>
 __global__ void __launch_bounds__(kFcThreads, 1)
 k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
   // NMAX: a bound on N for the unrolled per-model loops
   extern __shared__ __align__(16) unsigned char sm[];
+  __shared__ FcSpan s_span[MF_MAX_MODELS];
   const int N = P.n_models;
   const int sumK = pick(P.off, N - 1) + pick(P.K, N - 1);
   constexpr int QCAP = WL ? kFcEndQ : kFcThreads * kFcBudget;
   float2* tab = reinterpret_cast<float2*>(sm);
-  unsigned char* q = sm + (((size_t)sumK * sizeof(float2) + 15) & ~(size_t)15);
+  float* sv = reinterpret_cast<float*>(sm + (((size_t)sumK * sizeof(float2) + 15) & ~(size_t)15));  // last model, VRAM order
+  float* sa = sv + 256;                                                                             // model N - 2
+  unsigned char* q = reinterpret_cast<unsigned char*>(sa + 256);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // one list + queue block: li, ni [k], qi [qcap], ls, ns [k], qs [qcap], qn
   auto carve = [&](CtaTopK& t, int qcap) {
@@ -215,36 +289,169 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
     tk.li[e] = R.first ? kEmptyIdx : R.lists_i[gl + e];
   }
   if (tid == 0) *tk.qn = 0;
-  // Thread g of the grid scans the contiguous slice [g S, (g + 1) S) of the range.
-  // S = ceil(len / threads); in long scans rounded up to a multiple of the last model's
-  // option count, so all lanes of a warp run the same cycles of the last model's options
-  // (the same table entries, no divergence), while short scans keep slices short (a small
-  // first merge, spread over more CTAs).
-  const uint64_t nthreads = (uint64_t)gridDim.x * blockDim.x;
   const int last = N - 1;
-  const int off_last = pick(P.off, last);
-  const int klast = pick(P.K, last);
-  const uint64_t slice0 = (R.len + nthreads - 1) / nthreads;
-  const uint64_t slice = slice0 >= 4 * (uint64_t)klast ? (slice0 + klast - 1) / klast * klast : slice0;
-  const uint64_t s0 = ((uint64_t)blockIdx.x * blockDim.x + tid) * slice;
-  const uint64_t s1 = s0 + slice < R.len ? s0 + slice : R.len;
+  const int off_last = pick(P.off, last), klast = pick(P.K, last);
+  const int off_prev = last >= 1 ? pick(P.off, last - 1) : 0, kprev = last >= 1 ? pick(P.K, last - 1) : 1;
+  const float cap = P.vram_cap;
+  __syncthreads();
+  // the bar: the CTA's k-th entry, or the corner's k-th best score (entries equal to it enter)
+  float thr0_s = tk.ls[R.k - 1];
+  uint64_t thr0_i = tk.li[R.k - 1];
+  if (REG) {
+    // per model: the extremes of its usable options; models N - 2 and N - 1: their demands in order
+    for (int i = warp; i < N; i += kFcWarps) {
+      const int off = pick(P.off, i), K = pick(P.K, i);
+      FcSpan sp{-INFINITY, INFINITY, INFINITY, -INFINITY, 0};
+      for (int o = lane; o < K; o += 32) {
+        const float2 e = tab[off + o];
+        if (e.y < INFINITY) {
+          sp.jmax = fmaxf(sp.jmax, e.x);
+          sp.jmin = fminf(sp.jmin, e.x);
+          sp.vmin = fminf(sp.vmin, e.y);
+          sp.vmax = fmaxf(sp.vmax, e.y);
+          ++sp.n;
+        }
+      }
+#pragma unroll
+      for (int w = 16; w > 0; w >>= 1) {
+        sp.jmax = fmaxf(sp.jmax, __shfl_xor_sync(0xffffffffu, sp.jmax, w));
+        sp.jmin = fminf(sp.jmin, __shfl_xor_sync(0xffffffffu, sp.jmin, w));
+        sp.vmin = fminf(sp.vmin, __shfl_xor_sync(0xffffffffu, sp.vmin, w));
+        sp.vmax = fmaxf(sp.vmax, __shfl_xor_sync(0xffffffffu, sp.vmax, w));
+        sp.n += __shfl_xor_sync(0xffffffffu, sp.n, w);
+      }
+      if (lane == 0) s_span[i] = sp;
+    }
+    for (int e = tid; e < klast + (last >= 1 ? kprev : 0); e += kFcThreads) {
+      const bool is_last = e < klast;
+      const int off = is_last ? off_last : off_prev, K = is_last ? klast : kprev, o = is_last ? e : e - klast;
+      const float y = tab[off + o].y;
+      int r = 0;
+      for (int u = 0; u < K; ++u) {
+        const float v = tab[off + u].y;
+        r += v < y || (v == y && u < o) ? 1 : 0;
+      }
+      (is_last ? sv : sa)[r] = y;  // (unusable options, at +inf, come last)
+    }
+    __syncthreads();
+    if (S.corner[0] > 0) {
+      // every model's options by J - lambda V, best first (in the queue's memory)
+      uint16_t* order = reinterpret_cast<uint16_t*>(tk.qi);  // [lambda][model][kFcCornerOpts]
+      float sj = 0.f, sy = 0.f;
+      for (int i = 0; i < N; ++i) { sj += s_span[i].jmax - s_span[i].jmin; sy += s_span[i].vmax - s_span[i].vmin; }
+      float lam1 = sj / sy;
+      if (!(lam1 > 0.f && lam1 < 1e30f)) lam1 = 0.f;
+      for (int e = tid; e < kFcLambdas * sumK; e += kFcThreads) {
+        const int g = e / sumK, r = e - g * sumK;
+        const float lam = g == 0 ? 0.f : g == 1 ? 0.3f * lam1 : g == 2 ? lam1 : 3.f * lam1;
+        int i = 0;
+#pragma unroll
+        for (int u = 1; u < NMAX; ++u) i += u < N && r >= P.off[u] ? 1 : 0;
+        const int off = pick(P.off, i), K = pick(P.K, i);
+        const float2 me = tab[r];
+        if (!(me.y < INFINITY)) continue;
+        const float mine = __fsub_rn(me.x, __fmul_rn(lam, me.y));
+        int rank = 0;
+        for (int u = 0; u < K; ++u) {
+          const float2 v = tab[off + u];
+          const float s = __fsub_rn(v.x, __fmul_rn(lam, v.y));
+          rank += v.y < INFINITY && (s > mine || (s == mine && off + u < r)) ? 1 : 0;
+        }
+        if (rank < kFcCornerOpts) order[(g * MF_MAX_MODELS + i) * kFcCornerOpts + rank] = (uint16_t)r;
+      }
+      __syncthreads();
+      int corner = 1;
+#pragma unroll
+      for (int i = 0; i < NMAX; ++i)
+        if (i < N) corner *= min(S.corner[i], s_span[i].n);
+      const bool whole = R.base == 0 && R.len == P.total;
+      constexpr int PER = kFcCorner / kFcThreads;
+      uint32_t key[kFcLambdas][PER];  // 0: not feasible, or not in the range
+#pragma unroll
+      for (int u = 0; u < PER; ++u) {
+        int c = tid + u * kFcThreads;
+        const bool in = c < corner;
+        float2 sum[kFcLambdas];
+        uint64_t idx[kFcLambdas];
+#pragma unroll
+        for (int g = 0; g < kFcLambdas; ++g) { sum[g] = make_float2(0.f, 0.f); idx[g] = 0; }
+#pragma unroll
+        for (int i = 0; i < NMAX; ++i)
+          if (i < N && in) {
+            const int m = min(S.corner[i], s_span[i].n);
+            const int d = c % m;
+            c /= m;
+#pragma unroll
+            for (int g = 0; g < kFcLambdas; ++g) {
+              const int r = order[(g * MF_MAX_MODELS + i) * kFcCornerOpts + d];
+              sum[g] = __fadd2_rn(sum[g], tab[r]);
+              if (!whole) idx[g] += (uint64_t)(r - P.off[i]) * P.stride[i];
+            }
+          }
+#pragma unroll
+        for (int g = 0; g < kFcLambdas; ++g)
+          key[g][u] = in && sum[g].y <= cap && sum[g].x == sum[g].x && (whole || idx[g] - R.base < R.len) ? fc_key(sum[g].x) : 0u;
+      }
+      // the first lambda with k feasible configurations, and their k-th best score
+      uint32_t mine[PER];
+      bool found = false;
+#pragma unroll
+      for (int g = 0; g < kFcLambdas; ++g) {
+        if (found) continue;  // (uniform)
+        int c = 0;
+#pragma unroll
+        for (int u = 0; u < PER; ++u) c += __syncthreads_count(key[g][u] > 0u);
+        found = c >= R.k;
+#pragma unroll
+        for (int u = 0; u < PER; ++u) mine[u] = key[g][u];
+      }
+      if (found) {
+        uint32_t v = 0u;
+        for (int b = 31; b >= 0; --b) {
+          const uint32_t t = v | (1u << b);
+          int c = 0;
+#pragma unroll
+          for (int u = 0; u < PER; ++u) c += mine[u] >= t ? 1 : 0;
+          // (the threads' counts, 0 to PER = 4, summed from three predicates)
+          const int n = __syncthreads_count(c & 1) + 2 * __syncthreads_count(c & 2) + 4 * __syncthreads_count(c & 4);
+          if (n >= R.k) v = t;
+          if (n == R.k) break;
+        }
+        const float b = fc_unkey(v);
+        if (b > thr0_s) { thr0_s = b; thr0_i = kEmptyIdx; }
+      }
+    }
+  }
+  // Thread g of the grid scans `per` units of the range, a unit being the configurations of
+  // one setting of the leading N - 2 models where that leaves four units a thread, else of
+  // the leading N - 1 (so that short scans spread over more threads); units start at whole
+  // multiples of their size, the range's ends cut the first and the last.
+  const uint64_t nthreads = (uint64_t)gridDim.x * blockDim.x;
+  const uint64_t big = (uint64_t)klast * kprev;
+  const uint64_t unit = R.len / big >= 4 * nthreads ? big : (uint64_t)klast;
+  const uint64_t end = R.base + R.len, b0 = R.base / unit * unit;
+  const uint64_t per = ((end - b0 + unit - 1) / unit + nthreads - 1) / nthreads * unit;
+  const uint64_t rel = ((uint64_t)blockIdx.x * blockDim.x + tid) * per;  // (from b0)
+  bool done = rel >= end - b0 || R.len == 0;
+  // this thread's candidates [t, s1), absolute indices
+  uint64_t t = done ? end : b0 + rel > R.base ? b0 + rel : R.base;
+  const uint64_t s1 = done || end - (b0 + rel) <= per ? end : b0 + rel + per;
   int row[NMAX];  // option rows of models 0 .. N - 2
   int o;          // the last model's option
   {
-    const uint64_t idx0 = R.base + (s0 < R.len ? s0 : 0);
+    const uint64_t idx0 = done ? 0 : t;
 #pragma unroll
     for (int i = 0; i < NMAX; ++i)
       if (i < last) row[i] = P.off[i] + (int)((idx0 / P.stride[i]) % (uint64_t)P.K[i]);
-    o = (int)((idx0 / pick(P.stride, last)) % (uint64_t)klast);
+    o = (int)(idx0 % (uint64_t)klast);
   }
-  __syncthreads();
-  float thr_s = tk.ls[R.k - 1];
-  uint64_t thr_i = tk.li[R.k - 1];
-  const float cap = P.vram_cap;
+  float thr_s = thr0_s;
+  uint64_t thr_i = thr0_i;
   // prefix sums in model order: p2 over models 0 .. N - 3, p over 0 .. N - 2; rp is
   // model N - 2's option row (the one a carry usually stops at), endp its end
   float pJ2 = 0.f, pV2 = 0.f, pJ = 0.f, pV = 0.f;
-  int rp = 0, endp = 0;
+  int rp = 0;
+  const int endp = last >= 1 ? off_prev + kprev : 0;
   auto prefix = [&]() {
     pJ2 = 0.f;
     pV2 = 0.f;
@@ -262,57 +469,93 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
       pV += e.y;
     }
   };
-  if (last >= 1) endp = pick(P.off, last - 1) + pick(P.K, last - 1);
   prefix();
-  const float thr0_s = thr_s;  // (WL: the bar until the warp's own list is full)
-  const uint64_t thr0_i = thr_i;
+  // the next setting of models 0 .. N - 3, model N - 2 at its first option
+  auto carry2 = [&]() {
+    bool c = true;
+#pragma unroll
+    for (int i = NMAX - 1; i >= 0; --i) {
+      if (i == last - 1) row[i] = off_prev;
+      if (i < last - 1 && c) {
+        const int off = P.off[i];
+        int d = row[i] + 1 - off;
+        c = d == P.K[i];
+        if (c) d = 0;
+        row[i] = off + d;
+      }
+    }
+    prefix();
+  };
   // the last model's option wrapped: the next option of the models before it
   auto carry = [&]() {
     if (++rp < endp) {
       const float2 e = tab[rp];
       pJ = pJ2 + e.x;
       pV = pV2 + e.y;
-      return;
+    } else {
+      carry2();
     }
-    bool c = true;  // model N - 2 wrapped as well
-#pragma unroll
-    for (int i = NMAX - 1; i >= 0; --i)
-      if (i < last && c) {
-        const int off = P.off[i];
-        int d = (i == last - 1 ? rp : row[i] + 1) - off;
-        c = d == P.K[i];
-        if (c) d = 0;
-        row[i] = off + d;
-      }
-    prefix();
   };
+  const FcSpan sb = REG ? s_span[last] : FcSpan{}, spa = REG && last >= 1 ? s_span[last - 1] : FcSpan{};
   const float2* tl = tab + off_last;
-  const int minrun = slice >= kFcLongSlice ? kFcMinRunLong : kFcMinRun;
-  uint64_t t = s0;  // this thread's next candidate (offset in the range)
-  bool done = t >= s1;
-  unsigned int my_count = 0;
+  unsigned long long my_count = 0;
   for (;;) {
-    int pushed = 0, ran = 0;
-    while (!done && ran < minrun) {
+    int pushed = 0;
+    for (int step = 0; step < kFcSteps && !done; ++step) {
+      if (REG && last >= 1 && o == 0 && rp == off_prev && s1 - t >= big) {
+        // the configurations of one setting of models 0 .. N - 3
+        const bool none = !((pV2 + spa.vmin) + sb.vmin <= cap);
+        const bool all = (pV2 + spa.vmax) + sb.vmax <= cap;
+        const bool hit = !none && (pJ2 + spa.jmax) + sb.jmax >= thr_s;
+        if (!hit) {
+          if (all) {
+            my_count += (unsigned)(spa.n * sb.n);
+          } else if (!none) {
+            int c = sb.n;
+            unsigned n = 0;
+            for (int a = 0; a < spa.n && c > 0; ++a) {
+              const float p = pV2 + sa[a];
+              while (c > 0 && !(p + sv[c - 1] <= cap)) --c;
+              n += (unsigned)c;
+            }
+            my_count += n;
+          }
+          t += big;
+          if (t >= s1) done = true;
+          else carry2();
+          continue;
+        }
+      }
       const int n_here = s1 - t < (uint64_t)(klast - o) ? (int)(s1 - t) : klast - o;
       const float2* e0 = tl + o;
-      // fast pass: the count, and whether any candidate might enter the list
+      // the count, and whether any candidate might enter the list
       bool hit = false;
-      const float2 pjv = make_float2(pJ, pV);
+      unsigned c = 0;
+      if (REG && n_here == klast) {
+        int lo = 0, hi = sb.n;
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (pV + sv[mid] <= cap) lo = mid + 1; else hi = mid;
+        }
+        c = (unsigned)lo;
+        hit = lo > 0 && pJ + sb.jmax >= thr_s;
+      } else {
+        const float2 pjv = make_float2(pJ, pV);
 #pragma unroll 8
-      for (int u = 0; u < n_here; ++u) {
-        const float2 jv = __fadd2_rn(pjv, e0[u]);  // (J, V) = (pJ + x, pV + y), one paired add
-        const bool feas = jv.y <= cap;  // NaN compares false
-        my_count += feas ? 1u : 0u;
-        hit |= feas & (jv.x >= thr_s);
+        for (int u = 0; u < n_here; ++u) {
+          const float2 jv = __fadd2_rn(pjv, e0[u]);  // (J, V) = (pJ + x, pV + y), one paired add
+          const bool feas = jv.y <= cap;  // NaN compares false
+          c += feas ? 1u : 0u;
+          hit |= feas & (jv.x >= thr_s);
+        }
       }
       int u = n_here;
-      if (hit) {  // rare once the list is full: queue what beats its k-th entry
+      if (hit) {  // rare once the bar is high: queue what beats it
         for (u = 0; u < n_here; ++u) {
           const float2 e = e0[u];
           const float J = pJ + e.x, V = pV + e.y;
           if (V <= cap && J >= thr_s) {
-            const uint64_t idx = R.base + t + u;
+            const uint64_t idx = t + u;
             if (precedes(J, idx, thr_s, thr_i)) {
               if (pushed == kFcBudget) break;  // this candidate and the rest wait for the merge
               const int pos = atomicAdd(wt.qn, 1);
@@ -322,11 +565,11 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
             }
           }
         }
-        for (int w = u; w < n_here; ++w) my_count -= (pV + e0[w].y <= cap) ? 1u : 0u;  // counted again later
+        for (int w = u; w < n_here; ++w) c -= (pV + e0[w].y <= cap) ? 1u : 0u;  // counted again later
       }
+      my_count += c;
       t += u;
       o += u;
-      ran += u;
       if (t >= s1) done = true;
       else if (o == klast) { o = 0; carry(); }
       if (u < n_here) break;
@@ -337,9 +580,6 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
         __syncwarp();
         if (*(volatile int*)wt.qn > 32) topk_merge_sorted(wt, lane, 32, [] __device__() { __syncwarp(); });
         else topk_merge(wt, lane, 32, [] __device__() { __syncwarp(); });
-        const bool full = wt.li[R.k - 1] != kEmptyIdx;  // (its entries all beat the CTA's bar)
-        thr_s = full ? wt.ls[R.k - 1] : thr0_s;
-        thr_i = full ? wt.li[R.k - 1] : thr0_i;
       }
       if (!more) break;
     } else {
@@ -348,11 +588,13 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
         // a long queue (the first merges of a search) is sorted first
         if (*(volatile int*)tk.qn > 256) topk_merge_sorted(tk, tid, blockDim.x, [] __device__() { __syncthreads(); });
         else topk_merge(tk, tid, blockDim.x, [] __device__() { __syncthreads(); });
-        thr_s = tk.ls[R.k - 1];
-        thr_i = tk.li[R.k - 1];
       }
       if (!more) break;
     }
+    // the list's k-th entry where it is the better bar (a list not yet full has none)
+    const float ks = wt.ls[R.k - 1];
+    const uint64_t ki = wt.li[R.k - 1];
+    if (ki != kEmptyIdx && precedes(ks, ki, thr_s, thr_i)) { thr_s = ks; thr_i = ki; }
   }
   if (WL) {  // the warps' lists join the CTA's
     __syncthreads();
@@ -372,10 +614,10 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
     R.lists_s[gl + e] = tk.ls[e];
     R.lists_i[gl + e] = tk.li[e];
   }
-  unsigned int c = my_count;
+  unsigned long long c = my_count;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  if ((tid & 31) == 0 && c) atomicAdd(R.count, (unsigned long long)c);
+  for (int w = 16; w > 0; w >>= 1) c += __shfl_xor_sync(0xffffffffu, c, w);
+  if (lane == 0 && c) atomicAdd(R.count, c);
 }
 
 // ---------------------------------------------------------------------------
@@ -679,25 +921,52 @@ k_fc_ga(const Params P, const FcGaArgs A) {
   if (c == 0) *A.out_fit = fc_[e];
 }
 
-int fc_grid(const mf_ctx* c) { return c->num_sms; }
+// One CTA per SM, fewer where the range has fewer settings of the leading N - 1 models
+// than they have threads (a short list of lists to merge).
+int fc_grid(const mf_ctx* c, uint64_t len) {
+  const uint64_t units = len / (uint64_t)c->P.K[c->P.n_models - 1] + 2;
+  const uint64_t ctas = (units + kFcThreads - 1) / kFcThreads;
+  return (int)(ctas < (uint64_t)c->num_sms ? ctas : (uint64_t)c->num_sms);
+}
 
-mf_status fc_search_chunk(mf_ctx* c, const RangeArgs& a, cudaStream_t s) {
+mf_status fc_search_chunk(mf_ctx* c, const RangeArgs& a, int grid, cudaStream_t s) {
   FcLayout L;
-  fc_bytes(c->sumK, c->P.n_models, &L, (char*)c->d_fc);
+  fc_bytes(c->sumK, &L, (char*)c->d_fc);
+  const Params& P = c->P;
   FcScan S{};
   S.tab = L.tab;
+  S.reg = c->finite_vram && std::isfinite(P.vram_cap);
+  if (c->sumK <= kFcCornerRows && a.k <= kFcCorner) {
+    // the corner: one option more of each model in turn while the product stays in bounds
+    int prod = 1;
+    for (int i = 0; i < P.n_models; ++i) S.corner[i] = 1;
+    for (bool grew = true; grew;) {
+      grew = false;
+      for (int i = 0; i < P.n_models; ++i)
+        if (S.corner[i] < P.K[i] && S.corner[i] < kFcCornerOpts && prod / S.corner[i] * (S.corner[i] + 1) <= kFcCorner) {
+          prod = prod / S.corner[i] * (S.corner[i] + 1);
+          ++S.corner[i];
+          grew = true;
+        }
+    }
+  }
   const bool wl = a.k <= kFcWarpK;  // per-warp lists
-  const size_t smem = (((size_t)c->sumK * sizeof(float2) + 15) & ~(size_t)15) + fc_scan_list_bytes(a.k, wl);
-  if (smem > 227 * 1024) {
+  const size_t smem = fc_scan_table_bytes(c->sumK) + fc_scan_list_bytes(a.k, wl);
+  if (smem > 226 * 1024) {
     set_error("fixed-context search: top-k lists do not fit shared memory; use a smaller k");
     return MF_EUNSUPPORTED;
   }
   using ScanFn = void (*)(const Params, const FcScan, const RangeArgs);
-  const bool n8 = c->P.n_models <= 8;
-  const ScanFn fn = wl ? (n8 ? k_fc_scan<8, true> : k_fc_scan<MF_MAX_MODELS, true>)
-                       : (n8 ? k_fc_scan<8, false> : k_fc_scan<MF_MAX_MODELS, false>);
+  const bool n8 = P.n_models <= 8;
+  ScanFn fn;
+  if (S.reg)
+    fn = wl ? (n8 ? k_fc_scan<8, true, true> : k_fc_scan<MF_MAX_MODELS, true, true>)
+            : (n8 ? k_fc_scan<8, false, true> : k_fc_scan<MF_MAX_MODELS, false, true>);
+  else
+    fn = wl ? (n8 ? k_fc_scan<8, true, false> : k_fc_scan<MF_MAX_MODELS, true, false>)
+            : (n8 ? k_fc_scan<8, false, false> : k_fc_scan<MF_MAX_MODELS, false, false>);
   MF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  fn<<<fc_grid(c), kFcThreads, smem, s>>>(c->P, S, a);
+  fn<<<grid, kFcThreads, smem, s>>>(P, S, a);
   MF_CUDA(cudaGetLastError());
   return MF_OK;
 }
@@ -728,28 +997,32 @@ mf_status mf_fc_set(mf_ctx* ctx, const mf_fc_params* p, void* stream) {
     return fc_einval("mf_fc_params: alpha, beta and delta must be finite");
   DeviceGuard guard(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
-  const size_t bytes = fc_bytes(sumK, N, nullptr, nullptr);
+  const size_t bytes = fc_bytes(sumK, nullptr, nullptr);
   if (!ctx->d_fc) MF_CUDA(cudaMalloc(&ctx->d_fc, bytes));
   FcLayout L;
-  fc_bytes(sumK, N, &L, (char*)ctx->d_fc);
-  // inputs to the device (pinned staging, one copy each, then a synchronisation)
-  std::vector<unsigned char> host(bytes);
-  auto put = [&](void* dev, const void* src, size_t n) {
-    std::memcpy(host.data() + ((char*)dev - (char*)ctx->d_fc), src, n);
-  };
-  put(L.obs, p->obs, sizeof(float) * 4);
-  put(L.variant, p->variant, sizeof(int32_t) * sumK);
-  put(L.quality, p->quality, sizeof(float) * sumK);
-  put(L.f_min, p->f_min, sizeof(float) * sumK);
-  put(L.f_max, p->f_max, sizeof(float) * sumK);
-  put(L.omega, p->omega, sizeof(float) * N);
-  put(L.tau, p->tau, sizeof(float) * N);
-  put(L.cost, p->reload_cost, sizeof(float) * N);
-  put(L.prev, p->prev_variant, sizeof(int32_t) * N);
-  const size_t in_lo = (char*)L.obs - (char*)ctx->d_fc;
-  MF_CUDA(cudaMemcpyAsync((char*)ctx->d_fc + in_lo, host.data() + in_lo, bytes - in_lo, cudaMemcpyHostToDevice, s));
+  fc_bytes(sumK, &L, (char*)ctx->d_fc);
+  // (every call of a context that uses the staging buffer waits for its work)
+  mf_status st = ensure_host_stage(ctx, fc_input_bytes(sumK, N, nullptr, nullptr));
+  if (st != MF_OK) return st;
+  FcInputs I;
+  fc_input_bytes(sumK, N, &I, (char*)ctx->h_stage);
+  std::memcpy(I.obs, p->obs, sizeof(float) * 4);
+  std::memcpy(I.variant, p->variant, sizeof(int32_t) * sumK);
+  std::memcpy(I.quality, p->quality, sizeof(float) * sumK);
+  std::memcpy(I.f_min, p->f_min, sizeof(float) * sumK);
+  std::memcpy(I.f_max, p->f_max, sizeof(float) * sumK);
+  std::memcpy(I.omega, p->omega, sizeof(float) * N);
+  std::memcpy(I.tau, p->tau, sizeof(float) * N);
+  std::memcpy(I.cost, p->reload_cost, sizeof(float) * N);
+  std::memcpy(I.prev, p->prev_variant, sizeof(int32_t) * N);
   const FcConst C{p->alpha, p->beta, p->delta};
-  k_fc_local<<<sumK, 256, 0, s>>>(ctx->P, L, C);
+  const size_t wbytes = sizeof(float) * (size_t)ctx->P.per_model;
+  if (wbytes <= kFcStage) {
+    MF_CUDA(cudaFuncSetAttribute(k_fc_local<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFcStage));
+    k_fc_local<true><<<sumK, 256, wbytes, s>>>(ctx->P, L, I, C);
+  } else {
+    k_fc_local<false><<<sumK, 256, 0, s>>>(ctx->P, L, I, C);
+  }
   MF_CUDA(cudaGetLastError());
   MF_CUDA(cudaStreamSynchronize(s));
   ctx->fc_ready = 1;
@@ -763,7 +1036,7 @@ mf_status mf_fc_table(mf_ctx* ctx, float* d_fhat, float* d_f, float* d_u, uint8_
   DeviceGuard guard(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
   FcLayout L;
-  fc_bytes(ctx->sumK, ctx->P.n_models, &L, (char*)ctx->d_fc);
+  fc_bytes(ctx->sumK, &L, (char*)ctx->d_fc);
   const size_t n = (size_t)ctx->sumK;
   if (d_fhat) MF_CUDA(cudaMemcpyAsync(d_fhat, L.fhat, sizeof(float) * n, cudaMemcpyDeviceToDevice, s));
   if (d_f) MF_CUDA(cudaMemcpyAsync(d_f, L.f, sizeof(float) * n, cudaMemcpyDeviceToDevice, s));
@@ -833,7 +1106,7 @@ mf_status mf_fc_ga_run(mf_ctx* ctx, const mf_fc_ga_params* g, uint64_t seed, int
   cudaStream_t s = (cudaStream_t)stream;
   const int N = ctx->P.n_models;
   FcLayout L;
-  fc_bytes(ctx->sumK, N, &L, (char*)ctx->d_fc);
+  fc_bytes(ctx->sumK, &L, (char*)ctx->d_fc);
   // result: genome (16 ints) then the fitness
   mf_status st = ensure_scratch(ctx, sizeof(int32_t) * 17);
   if (st != MF_OK) return st;

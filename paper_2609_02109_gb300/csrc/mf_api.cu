@@ -188,6 +188,8 @@ mf_status mf_create(const mf_problem* p, mf_ctx** out) {
 
   // host-side images
   std::vector<float> dem4((size_t)sumK * 4, 0.f);
+  c->finite_vram = true;
+  for (int r = 0; r < sumK; ++r) c->finite_vram = c->finite_vram && std::isfinite(p->demand[(size_t)r * 3 + 1]);
   for (int r = 0; r < sumK; ++r)
     for (int j = 0; j < 3; ++j) dem4[(size_t)r * 4 + j] = p->demand[(size_t)r * 3 + j];
   std::vector<float> w32((size_t)N * per_pad, 0.f), wT((size_t)N * per_pad, 0.f);
@@ -381,15 +383,18 @@ static mf_status search_impl(mf_ctx* ctx, uint64_t lo, uint64_t hi, int32_t k, u
   if (!ctx || !out) return einval("NULL argument");
   if (k < 1 || k > MF_MAX_TOPK) return einval("k must be in 1..1024");
   if (lo > hi || hi > ctx->P.total) return einval("need lo <= hi <= |Lambda|");
-  if (chunk == 0) chunk = 1ull << 24;
-  if (chunk > (1ull << 31)) chunk = 1ull << 31;
+  // by default one launch takes the range (each launch fills its lists and stages its tables
+  // anew: 12 launches for 24^6 cost the bf16 scorer CHUNK_COST): up to 2^31 candidates, and
+  // 2^36 of the table-lookup scan's, which are cheaper by as much
+  if (chunk == 0) chunk = fc ? 1ull << 36 : 1ull << 31;
+  else if (chunk > (1ull << 31)) chunk = 1ull << 31;
   DeviceGuard guard(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
   const bool tc = !fc && ctx->precision == MF_BF16;
   // the exact (3-term tf32) tensor-core variant, where its lists fit next to the weights
   const bool tx = !fc && !tc && ctx->tc.tf && tc_fits(ctx, k);
   const int kcap = tc ? (k * 8 > 256 ? k * 8 : 256) : k;
-  const int grid = fc ? fc_grid(ctx) : (tc || tx) ? tc_grid(ctx) : f32_grid(ctx);
+  const int grid = fc ? fc_grid(ctx, hi - lo < chunk ? hi - lo : chunk) : (tc || tx) ? tc_grid(ctx) : f32_grid(ctx);
 
   // scratch: per-CTA lists, two merge buffers, merged list, rescored shortlist, count
   const size_t entries = (size_t)grid * kcap;
@@ -440,7 +445,7 @@ static mf_status search_impl(mf_ctx* ctx, uint64_t lo, uint64_t hi, int32_t k, u
     a.base = lo;
     a.len = 0;
     int nl = 1;
-    st = fc ? fc_search_chunk(ctx, a, s) : (tc || tx) ? tc_search_chunk(ctx, a, s, &nl) : f32_search_chunk(ctx, a, s);
+    st = fc ? fc_search_chunk(ctx, a, grid, s) : (tc || tx) ? tc_search_chunk(ctx, a, s, &nl) : f32_search_chunk(ctx, a, s);
     if (st != MF_OK) return st;
     launches += nl;
     score_launches += nl;
@@ -449,7 +454,7 @@ static mf_status search_impl(mf_ctx* ctx, uint64_t lo, uint64_t hi, int32_t k, u
     a.base = b;
     a.len = (hi - b) < chunk ? (hi - b) : chunk;
     int nl = 1;
-    st = fc ? fc_search_chunk(ctx, a, s) : (tc || tx) ? tc_search_chunk(ctx, a, s, &nl) : f32_search_chunk(ctx, a, s);
+    st = fc ? fc_search_chunk(ctx, a, grid, s) : (tc || tx) ? tc_search_chunk(ctx, a, s, &nl) : f32_search_chunk(ctx, a, s);
     if (st != MF_OK) return st;
     a.first = 0;
     launches += nl;

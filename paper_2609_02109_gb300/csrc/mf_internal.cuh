@@ -361,6 +361,7 @@ struct mf_ctx {
   // fixed-context mode: the per-option table of the last mf_fc_set
   void* d_fc = nullptr;           // see mf::FcLayout
   int fc_ready = 0;
+  bool finite_vram = false;       // every option's VRAM demand is finite
   float4* d_util = nullptr;       // [sumK] utility table of mf_set_utility
   int32_t base_objective = 0;     // the problem's own objective
   size_t tc_bytes = 0;
@@ -433,8 +434,8 @@ mf_status f32_prepare(mf_ctx* c);
 mf_status f32_search_chunk(mf_ctx* c, const RangeArgs& a, cudaStream_t s);
 // Fixed-context mode: one range launch of the table-lookup scan over the per-option
 // table of mf_fc_set.
-int fc_grid(const mf_ctx* c);
-mf_status fc_search_chunk(mf_ctx* c, const RangeArgs& a, cudaStream_t s);
+int fc_grid(const mf_ctx* c, uint64_t len);
+mf_status fc_search_chunk(mf_ctx* c, const RangeArgs& a, int grid, cudaStream_t s);
 mf_status f32_search_chunk_params(const Params& P, int grid, const RangeArgs& a, cudaStream_t s);
 mf_status f32_score_list(mf_ctx* c, const uint64_t* idx, const int32_t* genes, uint64_t n,
                          float* score, uint8_t* feas, float* pred, cudaStream_t s);
