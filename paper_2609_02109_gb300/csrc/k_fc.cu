@@ -169,10 +169,9 @@ k_fc_local(const Params P, const FcLayout L, const FcInputs I, const FcConst C) 
 }
 
 // ---------------------------------------------------------------------------
-// Table-lookup scan.  Each thread walks its own contiguous slice of the range, so from one
-// candidate to the next only the last model's option advances, and J and the VRAM demand V
-// are summed in model order.  A configuration is not looked at one by one: fp32 addition is
-// monotone (a <= b gives fl(p + a) <= fl(p + b)), so
+// Table-lookup scan.  J and the VRAM demand V of a configuration are summed in model order,
+// but configurations are not looked at one by one: fp32 addition is monotone (a <= b gives
+// fl(p + a) <= fl(p + b)), so
 //   - for one setting of the leading N - 1 models, the last model's options within the cap
 //     are a prefix of its options in VRAM order: a binary search counts them;
 //   - for one setting of the leading N - 2 models, the sums of the extreme demands tell
@@ -186,40 +185,46 @@ k_fc_local(const Params P, const FcLayout L, const FcInputs I, const FcConst C) 
 //
 // The bar starts high: J is a sum of per-model terms, so the best configurations sit where
 // every model has one of its best options.  Every CTA first scores a corner of the space, the
-// few best options of each model (m_i, at most kFcCorner configurations), by J - lambda V
+// few best options of each model (m_i, 2^kFcCornerBits configurations), by J - lambda V
 // for four weights lambda of the VRAM demand; the k-th best feasible score of the corner
 // with the smallest lambda that has k of them bounds the k-th best of the range from below.
 //
-// Running top-k: a thread queues a candidate only if it beats the bar, at most kFcBudget
-// between two merge checks (a thread that runs out stops until the merge), one check per
-// kFcSteps steps.  WL (k <= kFcWarpK): each warp keeps its own list and queue and merges
-// with warp barriers only, the CTA's list taking the warps' lists at the end; otherwise one
-// list per CTA, the merge check a CTA barrier.
+// The unit of work is one setting of the leading N - 2 models (short ranges: N - 1).  Units
+// go round the threads of the grid, so that neighbours, which hold good scores together,
+// land on different SMs.  A lane settles its unit by the bounds and counts; the units in
+// which a score might beat the bar are then looked at by the whole warp, one after another.
 //
-// Bound by issue and shared-memory latency.  24^6, VRAM binding, k = 32: one launch of
-// FC_SCAN_NOW, where the scan of every candidate took 12 launches of 75-125 us (each of
-// which also filled its lists from nothing); 2^32: FC_SCAN_STRESS.
+// Running top-k: a warp queues the configurations that beat the bar and merges before the
+// queue might overflow.  WL (k <= kFcWarpK): each warp keeps its own list and queue and
+// merges with warp barriers only, the CTA's list taking the warps' lists at the end;
+// otherwise one list and queue per CTA, whose warps meet for a merge when it fills up.
+//
+// Bound by latency (shared-memory chains of the counts; the prologue's ranking and corner).
+// 24^6, VRAM binding, k = 32: FC_SCAN_NOW, where the scan of every candidate took 12
+// launches of 75-125 us, each of which also filled its lists from nothing.
 // ---------------------------------------------------------------------------
 constexpr int kFcThreads = 512;
-constexpr int kFcBudget = 8;   // the queue: kFcThreads x kFcBudget entries
-constexpr int kFcSteps = 8;
 constexpr int kFcWarpK = 64, kFcWarps = kFcThreads / 32;
-constexpr int kFcWarpQ = 32 * kFcBudget;              // a warp's queue
+constexpr int kFcCtaQ = 4096, kFcWarpQ = 256;         // a CTA's and a warp's queue
 constexpr int kFcEndQ = kFcWarps * kFcWarpK;          // the warps' lists, merged at the end (a power of two)
 constexpr int kFcLambdas = 4, kFcCornerOpts = 64;     // corner sets, options of a model in one
-constexpr int kFcCorner = 4 * kFcThreads;             // configurations of a corner
+constexpr int kFcCornerBits = 10;                     // configurations of a corner: 2^10
 constexpr int kFcCornerRows = 1024;                   // option rows up to which the corners are ranked
 
 struct FcScan {
   const float2* tab;
-  int32_t reg;                        // finite demands and cap
-  int32_t corner[MF_MAX_MODELS];      // m_i; all 0: no corner
+  int32_t corner;                     // score the corners first
+  int32_t bits[MF_MAX_MODELS];        // m_i = 2^bits (where the model has as many usable options)
+  // units: one setting of models 0 .. lead - 1 (lead = N - 2 or N - 1); the radix digits of
+  // the grid's thread count in those models
+  int32_t lead;
+  uint32_t step[MF_MAX_MODELS];
 };
 
 // Shared-memory bytes of k_fc_scan<.., WL> after the table and the two VRAM orders.
 __host__ __device__ inline size_t fc_scan_list_bytes(int k, bool wl) {
   const size_t e = sizeof(uint64_t) + sizeof(float);
-  if (!wl) return e * (2 * (size_t)k + kFcThreads * kFcBudget) + 16;
+  if (!wl) return e * (2 * (size_t)k + kFcCtaQ) + 16;
   return e * (2 * (size_t)k + kFcEndQ) + 16 + kFcWarps * (e * (2 * (size_t)k + kFcWarpQ) + 16);
 }
 __host__ __device__ inline size_t fc_scan_table_bytes(int sumK) {
@@ -249,7 +254,7 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
   __shared__ FcSpan s_span[MF_MAX_MODELS];
   const int N = P.n_models;
   const int sumK = pick(P.off, N - 1) + pick(P.K, N - 1);
-  constexpr int QCAP = WL ? kFcEndQ : kFcThreads * kFcBudget;
+  constexpr int QCAP = WL ? kFcEndQ : kFcCtaQ;
   float2* tab = reinterpret_cast<float2*>(sm);
   float* sv = reinterpret_cast<float*>(sm + (((size_t)sumK * sizeof(float2) + 15) & ~(size_t)15));  // last model, VRAM order
   float* sa = sv + 256;                                                                             // model N - 2
@@ -322,78 +327,87 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
       }
       if (lane == 0) s_span[i] = sp;
     }
-    for (int e = tid; e < klast + (last >= 1 ? kprev : 0); e += kFcThreads) {
-      const bool is_last = e < klast;
-      const int off = is_last ? off_last : off_prev, K = is_last ? klast : kprev, o = is_last ? e : e - klast;
-      const float y = tab[off + o].y;
-      int r = 0;
-      for (int u = 0; u < K; ++u) {
-        const float v = tab[off + u].y;
-        r += v < y || (v == y && u < o) ? 1 : 0;
-      }
-      (is_last ? sv : sa)[r] = y;  // (unusable options, at +inf, come last)
-    }
     __syncthreads();
-    if (S.corner[0] > 0) {
-      // every model's options by J - lambda V, best first (in the queue's memory)
-      uint16_t* order = reinterpret_cast<uint16_t*>(tk.qi);  // [lambda][model][kFcCornerOpts]
+    // Rankings, one warp per task, an option per lane (all-to-all by shuffles): tasks 0 and 1
+    // order the demands of models N - 1 and N - 2, the others a model's usable options by
+    // J - lambda V for one lambda, best first (in the queue's memory).
+    uint16_t* order = reinterpret_cast<uint16_t*>(tk.qi);  // [lambda][model][kFcCornerOpts]
+    float lam1 = 0.f;
+    if (S.corner) {
       float sj = 0.f, sy = 0.f;
-      for (int i = 0; i < N; ++i) { sj += s_span[i].jmax - s_span[i].jmin; sy += s_span[i].vmax - s_span[i].vmin; }
-      float lam1 = sj / sy;
-      if (!(lam1 > 0.f && lam1 < 1e30f)) lam1 = 0.f;
-      for (int e = tid; e < kFcLambdas * sumK; e += kFcThreads) {
-        const int g = e / sumK, r = e - g * sumK;
-        const float lam = g == 0 ? 0.f : g == 1 ? 0.3f * lam1 : g == 2 ? lam1 : 3.f * lam1;
-        int i = 0;
-#pragma unroll
-        for (int u = 1; u < NMAX; ++u) i += u < N && r >= P.off[u] ? 1 : 0;
-        const int off = pick(P.off, i), K = pick(P.K, i);
-        const float2 me = tab[r];
-        if (!(me.y < INFINITY)) continue;
-        const float mine = __fsub_rn(me.x, __fmul_rn(lam, me.y));
-        int rank = 0;
-        for (int u = 0; u < K; ++u) {
-          const float2 v = tab[off + u];
-          const float s = __fsub_rn(v.x, __fmul_rn(lam, v.y));
-          rank += v.y < INFINITY && (s > mine || (s == mine && off + u < r)) ? 1 : 0;
-        }
-        if (rank < kFcCornerOpts) order[(g * MF_MAX_MODELS + i) * kFcCornerOpts + rank] = (uint16_t)r;
-      }
-      __syncthreads();
-      int corner = 1;
 #pragma unroll
       for (int i = 0; i < NMAX; ++i)
-        if (i < N) corner *= min(S.corner[i], s_span[i].n);
+        if (i < N) { sj += s_span[i].jmax - s_span[i].jmin; sy += s_span[i].vmax - s_span[i].vmin; }
+      lam1 = sj / sy;
+      if (!(lam1 > 0.f && lam1 < 1e30f)) lam1 = 0.f;
+    }
+    for (int task = warp; task < 2 + (S.corner ? kFcLambdas * N : 0); task += kFcWarps) {
+      const int g = task < 2 ? 0 : (task - 2) / N;
+      const int i = task == 0 ? last : task == 1 ? max(last - 1, 0) : task - 2 - g * N;
+      const float lam = g == 0 ? 0.f : g == 1 ? 0.3f * lam1 : g == 2 ? lam1 : 3.f * lam1;
+      const int off = pick(P.off, i), K = pick(P.K, i);
+      // the value a task ranks by, highest first: -V, or J - lambda V (unusable options last)
+      auto value = [&](int o) {
+        const float2 e = o < K ? tab[off + o] : make_float2(-INFINITY, INFINITY);
+        if (task < 2) return -e.y;
+        return e.y < INFINITY ? __fsub_rn(e.x, __fmul_rn(lam, e.y)) : -INFINITY;
+      };
+      for (int c0 = 0; c0 < K; c0 += 32) {
+        const int o = c0 + lane;
+        const float mine = value(o);
+        int rank = 0;
+        for (int d0 = 0; d0 < K; d0 += 32) {
+          const float other = value(d0 + lane);
+#pragma unroll
+          for (int u = 0; u < 32; ++u) {
+            const float v = __shfl_sync(0xffffffffu, other, u);
+            rank += v > mine || (v == mine && d0 + u < o) ? 1 : 0;
+          }
+        }
+        if (o < K) {
+          const float y = tab[off + o].y;
+          if (task == 0) sv[rank] = y;
+          else if (task == 1) sa[rank] = y;
+          else if (rank < kFcCornerOpts && y < INFINITY)
+            order[(g * MF_MAX_MODELS + i) * kFcCornerOpts + rank] = (uint16_t)(off + o);
+        }
+      }
+    }
+    __syncthreads();
+    if (S.corner) {
       const bool whole = R.base == 0 && R.len == P.total;
-      constexpr int PER = kFcCorner / kFcThreads;
-      uint32_t key[kFcLambdas][PER];  // 0: not feasible, or not in the range
+      constexpr int PER = (1 << kFcCornerBits) / kFcThreads;
+      uint32_t key[kFcLambdas][PER];  // 0: not feasible, not in the range, no such option
 #pragma unroll
       for (int u = 0; u < PER; ++u) {
-        int c = tid + u * kFcThreads;
-        const bool in = c < corner;
+        uint32_t c = tid + u * kFcThreads;
+        bool in = true;
         float2 sum[kFcLambdas];
         uint64_t idx[kFcLambdas];
 #pragma unroll
         for (int g = 0; g < kFcLambdas; ++g) { sum[g] = make_float2(0.f, 0.f); idx[g] = 0; }
 #pragma unroll
         for (int i = 0; i < NMAX; ++i)
-          if (i < N && in) {
-            const int m = min(S.corner[i], s_span[i].n);
-            const int d = c % m;
-            c /= m;
+          if (i < N) {
+            const uint32_t d = c & ((1u << S.bits[i]) - 1u);
+            c >>= S.bits[i];
+            in = in && d < (uint32_t)s_span[i].n;
+            if (in) {
 #pragma unroll
-            for (int g = 0; g < kFcLambdas; ++g) {
-              const int r = order[(g * MF_MAX_MODELS + i) * kFcCornerOpts + d];
-              sum[g] = __fadd2_rn(sum[g], tab[r]);
-              if (!whole) idx[g] += (uint64_t)(r - P.off[i]) * P.stride[i];
+              for (int g = 0; g < kFcLambdas; ++g) {
+                const int r = order[(g * MF_MAX_MODELS + i) * kFcCornerOpts + d];
+                sum[g] = __fadd2_rn(sum[g], tab[r]);
+                if (!whole) idx[g] += (uint64_t)(r - P.off[i]) * P.stride[i];
+              }
             }
           }
+        in = in && c == 0;  // (a corner of fewer configurations: the rest are repeats)
 #pragma unroll
         for (int g = 0; g < kFcLambdas; ++g)
           key[g][u] = in && sum[g].y <= cap && sum[g].x == sum[g].x && (whole || idx[g] - R.base < R.len) ? fc_key(sum[g].x) : 0u;
       }
       // the first lambda with k feasible configurations, and their k-th best score
-      uint32_t mine[PER];
+      uint32_t mine[PER] = {};
       bool found = false;
 #pragma unroll
       for (int g = 0; g < kFcLambdas; ++g) {
@@ -409,192 +423,188 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
         uint32_t v = 0u;
         for (int b = 31; b >= 0; --b) {
           const uint32_t t = v | (1u << b);
-          int c = 0;
+          int n = 0;
 #pragma unroll
-          for (int u = 0; u < PER; ++u) c += mine[u] >= t ? 1 : 0;
-          // (the threads' counts, 0 to PER = 4, summed from three predicates)
-          const int n = __syncthreads_count(c & 1) + 2 * __syncthreads_count(c & 2) + 4 * __syncthreads_count(c & 4);
+          for (int u = 0; u < PER; ++u) n += __syncthreads_count(mine[u] >= t);
           if (n >= R.k) v = t;
-          if (n == R.k) break;
+          if (n >= R.k && n <= R.k + (R.k >> 2)) break;  // (any bar that k scores reach holds)
         }
         const float b = fc_unkey(v);
         if (b > thr0_s) { thr0_s = b; thr0_i = kEmptyIdx; }
       }
     }
   }
-  // Thread g of the grid scans `per` units of the range, a unit being the configurations of
-  // one setting of the leading N - 2 models where that leaves four units a thread, else of
-  // the leading N - 1 (so that short scans spread over more threads); units start at whole
-  // multiples of their size, the range's ends cut the first and the last.
-  const uint64_t nthreads = (uint64_t)gridDim.x * blockDim.x;
-  const uint64_t big = (uint64_t)klast * kprev;
-  const uint64_t unit = R.len / big >= 4 * nthreads ? big : (uint64_t)klast;
-  const uint64_t end = R.base + R.len, b0 = R.base / unit * unit;
-  const uint64_t per = ((end - b0 + unit - 1) / unit + nthreads - 1) / nthreads * unit;
-  const uint64_t rel = ((uint64_t)blockIdx.x * blockDim.x + tid) * per;  // (from b0)
-  bool done = rel >= end - b0 || R.len == 0;
-  // this thread's candidates [t, s1), absolute indices
-  uint64_t t = done ? end : b0 + rel > R.base ? b0 + rel : R.base;
-  const uint64_t s1 = done || end - (b0 + rel) <= per ? end : b0 + rel + per;
-  int row[NMAX];  // option rows of models 0 .. N - 2
-  int o;          // the last model's option
-  {
-    const uint64_t idx0 = done ? 0 : t;
-#pragma unroll
-    for (int i = 0; i < NMAX; ++i)
-      if (i < last) row[i] = P.off[i] + (int)((idx0 / P.stride[i]) % (uint64_t)P.K[i]);
-    o = (int)(idx0 % (uint64_t)klast);
-  }
+  const FcSpan sb = REG ? s_span[last] : FcSpan{}, spa = REG && last >= 1 ? s_span[last - 1] : FcSpan{};
   float thr_s = thr0_s;
   uint64_t thr_i = thr0_i;
-  // prefix sums in model order: p2 over models 0 .. N - 3, p over 0 .. N - 2; rp is
-  // model N - 2's option row (the one a carry usually stops at), endp its end
-  float pJ2 = 0.f, pV2 = 0.f, pJ = 0.f, pV = 0.f;
-  int rp = 0;
-  const int endp = last >= 1 ? off_prev + kprev : 0;
-  auto prefix = [&]() {
-    pJ2 = 0.f;
-    pV2 = 0.f;
+  // Thread g of the grid takes units u0 + g, u0 + g + T, ..; the range's ends cut the first
+  // unit and the last.  BIG (lead = N - 2): the unit's configurations run over models N - 2
+  // and N - 1.
+  const int lead = S.lead;
+  const bool big = lead < last;
+  const int na = big ? kprev : 1;
+  const uint64_t unit = (uint64_t)klast * na;
+  const uint64_t end = R.base + R.len, u0 = R.base / unit;
+  const uint64_t nu = R.len == 0 ? 0 : (end - 1) / unit - u0 + 1;  // units of the range
+  const uint64_t nthreads = (uint64_t)gridDim.x * blockDim.x;
+  uint64_t my = (uint64_t)blockIdx.x * blockDim.x + tid;           // this lane's unit, from u0
+  int row[NMAX];  // option rows of models 0 .. lead - 1
+  {
+    uint64_t v = my < nu ? u0 + my : 0;
 #pragma unroll
-    for (int i = 0; i < NMAX; ++i)
-      if (i < last - 1) { const float2 e = tab[row[i]]; pJ2 += e.x; pV2 += e.y; }
-    pJ = pJ2;
-    pV = pV2;
-    if (last >= 1) {
-#pragma unroll
-      for (int i = 0; i < NMAX; ++i)
-        if (i == last - 1) rp = row[i];
-      const float2 e = tab[rp];
-      pJ += e.x;
-      pV += e.y;
-    }
-  };
-  prefix();
-  // the next setting of models 0 .. N - 3, model N - 2 at its first option
-  auto carry2 = [&]() {
-    bool c = true;
-#pragma unroll
-    for (int i = NMAX - 1; i >= 0; --i) {
-      if (i == last - 1) row[i] = off_prev;
-      if (i < last - 1 && c) {
-        const int off = P.off[i];
-        int d = row[i] + 1 - off;
-        c = d == P.K[i];
-        if (c) d = 0;
-        row[i] = off + d;
+    for (int i = NMAX - 1; i >= 0; --i)
+      if (i < lead) {
+        const uint32_t K = (uint32_t)P.K[i];
+        uint32_t d;
+        if (v <= 0xffffffffull) {
+          const uint32_t q32 = (uint32_t)v / K;
+          d = (uint32_t)v - q32 * K;
+          v = q32;
+        } else {
+          const uint64_t q64 = v / K;
+          d = (uint32_t)(v - q64 * K);
+          v = q64;
+        }
+        row[i] = P.off[i] + (int)d;
       }
-    }
-    prefix();
-  };
-  // the last model's option wrapped: the next option of the models before it
-  auto carry = [&]() {
-    if (++rp < endp) {
-      const float2 e = tab[rp];
-      pJ = pJ2 + e.x;
-      pV = pV2 + e.y;
-    } else {
-      carry2();
-    }
-  };
-  const FcSpan sb = REG ? s_span[last] : FcSpan{}, spa = REG && last >= 1 ? s_span[last - 1] : FcSpan{};
-  const float2* tl = tab + off_last;
+  }
   unsigned long long my_count = 0;
-  for (;;) {
-    int pushed = 0;
-    for (int step = 0; step < kFcSteps && !done; ++step) {
-      if (REG && last >= 1 && o == 0 && rp == off_prev && s1 - t >= big) {
-        // the configurations of one setting of models 0 .. N - 3
-        const bool none = !((pV2 + spa.vmin) + sb.vmin <= cap);
-        const bool all = (pV2 + spa.vmax) + sb.vmax <= cap;
-        const bool hit = !none && (pJ2 + spa.jmax) + sb.jmax >= thr_s;
-        if (!hit) {
-          if (all) {
-            my_count += (unsigned)(spa.n * sb.n);
-          } else if (!none) {
-            int c = sb.n;
-            unsigned n = 0;
-            for (int a = 0; a < spa.n && c > 0; ++a) {
-              const float p = pV2 + sa[a];
-              while (c > 0 && !(p + sv[c - 1] <= cap)) --c;
-              n += (unsigned)c;
-            }
-            my_count += n;
-          }
-          t += big;
-          if (t >= s1) done = true;
-          else carry2();
-          continue;
-        }
-      }
-      const int n_here = s1 - t < (uint64_t)(klast - o) ? (int)(s1 - t) : klast - o;
-      const float2* e0 = tl + o;
-      // the count, and whether any candidate might enter the list
-      bool hit = false;
-      unsigned c = 0;
-      if (REG && n_here == klast) {
-        int lo = 0, hi = sb.n;
-        while (lo < hi) {
-          const int mid = (lo + hi) >> 1;
-          if (pV + sv[mid] <= cap) lo = mid + 1; else hi = mid;
-        }
-        c = (unsigned)lo;
-        hit = lo > 0 && pJ + sb.jmax >= thr_s;
-      } else {
-        const float2 pjv = make_float2(pJ, pV);
-#pragma unroll 8
-        for (int u = 0; u < n_here; ++u) {
-          const float2 jv = __fadd2_rn(pjv, e0[u]);  // (J, V) = (pJ + x, pV + y), one paired add
-          const bool feas = jv.y <= cap;  // NaN compares false
-          c += feas ? 1u : 0u;
-          hit |= feas & (jv.x >= thr_s);
-        }
-      }
-      int u = n_here;
-      if (hit) {  // rare once the bar is high: queue what beats it
-        for (u = 0; u < n_here; ++u) {
-          const float2 e = e0[u];
-          const float J = pJ + e.x, V = pV + e.y;
-          if (V <= cap && J >= thr_s) {
-            const uint64_t idx = t + u;
-            if (precedes(J, idx, thr_s, thr_i)) {
-              if (pushed == kFcBudget) break;  // this candidate and the rest wait for the merge
-              const int pos = atomicAdd(wt.qn, 1);
-              wt.qs[pos] = J;
-              wt.qi[pos] = idx;
-              ++pushed;
-            }
-          }
-        }
-        for (int w = u; w < n_here; ++w) c -= (pV + e0[w].y <= cap) ? 1u : 0u;  // counted again later
-      }
-      my_count += c;
-      t += u;
-      o += u;
-      if (t >= s1) done = true;
-      else if (o == klast) { o = 0; carry(); }
-      if (u < n_here) break;
-    }
-    if (WL) {
-      const bool more = __any_sync(0xffffffffu, !done);
-      if (__any_sync(0xffffffffu, pushed > 0)) {
-        __syncwarp();
-        if (*(volatile int*)wt.qn > 32) topk_merge_sorted(wt, lane, 32, [] __device__() { __syncwarp(); });
-        else topk_merge(wt, lane, 32, [] __device__() { __syncwarp(); });
-      }
-      if (!more) break;
-    } else {
-      const bool more = __syncthreads_or(!done);
-      if (*(volatile int*)tk.qn > 0) {  // (read by every thread after the barrier: uniform)
-        // a long queue (the first merges of a search) is sorted first
-        if (*(volatile int*)tk.qn > 256) topk_merge_sorted(tk, tid, blockDim.x, [] __device__() { __syncthreads(); });
-        else topk_merge(tk, tid, blockDim.x, [] __device__() { __syncthreads(); });
-      }
-      if (!more) break;
-    }
-    // the list's k-th entry where it is the better bar (a list not yet full has none)
+  // look-at state of the warp: the lanes whose units wait, the current unit's next option of
+  // model N - 2 (index within na) and the next row of 32 of the last model's options
+  unsigned waiting = 0u;
+  int at_a = 0, at_b = 0;
+  float pJ2 = 0.f, pV2 = 0.f;  // this lane's unit: sums over models 0 .. lead - 1, in order
+  bool count_there = false;    // it is counted when it is looked at
+  auto merge_warp = [&]() {
+    __syncwarp();
+    if (*(volatile int*)wt.qn > 32) topk_merge_sorted(wt, lane, 32, [] __device__() { __syncwarp(); });
+    else if (*(volatile int*)wt.qn > 0) topk_merge(wt, lane, 32, [] __device__() { __syncwarp(); });
+  };
+  auto raise_bar = [&]() {  // the list's k-th entry where it is the better bar (none while not full)
     const float ks = wt.ls[R.k - 1];
     const uint64_t ki = wt.li[R.k - 1];
     if (ki != kEmptyIdx && precedes(ks, ki, thr_s, thr_i)) { thr_s = ks; thr_i = ki; }
+  };
+  for (;;) {  // rounds; WL needs one only
+    for (;;) {
+      if (!waiting) {
+        // ---- every lane settles its next unit ----
+        if (!__any_sync(0xffffffffu, my < nu)) break;
+        bool look = false;
+        if (my < nu) {
+          pJ2 = 0.f;
+          pV2 = 0.f;
+#pragma unroll
+          for (int i = 0; i < NMAX; ++i)
+            if (i < lead) { const float2 e = tab[row[i]]; pJ2 += e.x; pV2 += e.y; }
+          const uint64_t t0 = (u0 + my) * unit;
+          if (!REG || t0 < R.base || end - t0 < unit) {
+            look = count_there = true;  // looked at one by one
+          } else if (big) {
+            const bool none = !((pV2 + spa.vmin) + sb.vmin <= cap);
+            look = !none && (pJ2 + spa.jmax) + sb.jmax >= thr_s;
+            count_there = false;
+            if ((pV2 + spa.vmax) + sb.vmax <= cap) {
+              my_count += (unsigned)(spa.n * sb.n);
+            } else if (!none) {
+              int c = sb.n;
+              unsigned n = 0;
+              for (int a = 0; a < spa.n && c > 0; ++a) {
+                const float p = pV2 + sa[a];
+                while (c > 0 && !(p + sv[c - 1] <= cap)) --c;
+                n += (unsigned)c;
+              }
+              my_count += n;
+            }
+          } else {
+            int lo = 0, hi = sb.n;
+            while (lo < hi) {
+              const int mid = (lo + hi) >> 1;
+              if (pV2 + sv[mid] <= cap) lo = mid + 1; else hi = mid;
+            }
+            my_count += (unsigned)lo;
+            look = lo > 0 && pJ2 + sb.jmax >= thr_s;
+            count_there = false;
+          }
+        }
+        waiting = __ballot_sync(0xffffffffu, look);
+        at_a = at_b = 0;
+      }
+      // ---- the warp looks at the waiting units, one after another ----
+      bool full = false;
+      while (waiting && !full) {
+        const int src = __ffs(waiting) - 1;
+        const float bJ = __shfl_sync(0xffffffffu, pJ2, src), bV = __shfl_sync(0xffffffffu, pV2, src);
+        const bool cnt = __shfl_sync(0xffffffffu, count_there ? 1 : 0, src) != 0;
+        const uint64_t t0 = (u0 + __shfl_sync(0xffffffffu, my, src)) * unit;
+        for (; at_a < na; ++at_a) {
+          float aJ = bJ, aV = bV;
+          if (big) {
+            const float2 e = tab[off_prev + at_a];
+            aJ += e.x;
+            aV += e.y;
+          }
+          if (REG && !cnt && !(aV + sb.vmin <= cap && aJ + sb.jmax >= thr_s)) continue;  // (uniform)
+          for (; at_b < klast; at_b += 32) {
+            // room for this row of 32 (in a CTA's queue: for a row of every warp)
+            if (WL) {
+              if (*(volatile int*)wt.qn > kFcWarpQ - 32) {
+                merge_warp();
+                raise_bar();
+              }
+            } else {
+              // (one lane reads the queue's length, which other warps move, for all)
+              full = __shfl_sync(0xffffffffu, *(volatile int*)wt.qn, 0) > QCAP - 32 * kFcWarps;
+              if (full) break;
+            }
+            const int o = at_b + lane;
+            const uint64_t idx = t0 + (uint64_t)at_a * klast + o;
+            const bool in = o < klast && idx >= R.base && idx < end;
+            const float2 e = in ? tab[off_last + o] : make_float2(0.f, 0.f);
+            const float J = aJ + e.x;
+            const bool feas = in && aV + e.y <= cap;  // NaN compares false
+            my_count += cnt && feas ? 1u : 0u;
+            const bool push = feas && J >= thr_s && precedes(J, idx, thr_s, thr_i);
+            const unsigned m = __ballot_sync(0xffffffffu, push);
+            if (m) {
+              int pos = 0;
+              if (lane == 0) pos = atomicAdd(wt.qn, __popc(m));
+              pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(m & ((1u << lane) - 1u));
+              if (push) { wt.qs[pos] = J; wt.qi[pos] = idx; }
+              __syncwarp();
+            }
+          }
+          if (full) break;  // (resumed at this row after the merge)
+          at_b = 0;
+        }
+        if (full) break;
+        at_a = 0;
+        waiting &= waiting - 1u;
+      }
+      if (full) break;
+      // ---- the lane's next unit: the thread count added to the leading models' digits ----
+      my += nthreads;
+      uint32_t carry = 0;
+#pragma unroll
+      for (int i = NMAX - 1; i >= 0; --i)
+        if (i < lead) {
+          const int off = P.off[i];
+          uint32_t d = (uint32_t)(row[i] - off) + S.step[i] + carry;
+          carry = d >= (uint32_t)P.K[i];
+          if (carry) d -= (uint32_t)P.K[i];
+          row[i] = off + (int)d;
+        }
+    }
+    if (WL) {
+      merge_warp();
+      break;
+    }
+    const bool more = __syncthreads_or(waiting != 0u);
+    // a long queue (the first merges of a search) is sorted first
+    if (*(volatile int*)tk.qn > 256) topk_merge_sorted(tk, tid, blockDim.x, [] __device__() { __syncthreads(); });
+    else if (*(volatile int*)tk.qn > 0) topk_merge(tk, tid, blockDim.x, [] __device__() { __syncthreads(); });
+    if (!more) break;
+    raise_bar();
   }
   if (WL) {  // the warps' lists join the CTA's
     __syncthreads();
@@ -933,22 +943,32 @@ mf_status fc_search_chunk(mf_ctx* c, const RangeArgs& a, int grid, cudaStream_t 
   FcLayout L;
   fc_bytes(c->sumK, &L, (char*)c->d_fc);
   const Params& P = c->P;
+  const int N = P.n_models;
   FcScan S{};
   S.tab = L.tab;
-  S.reg = c->finite_vram && std::isfinite(P.vram_cap);
-  if (c->sumK <= kFcCornerRows && a.k <= kFcCorner) {
-    // the corner: one option more of each model in turn while the product stays in bounds
-    int prod = 1;
-    for (int i = 0; i < P.n_models; ++i) S.corner[i] = 1;
-    for (bool grew = true; grew;) {
+  const bool reg = c->finite_vram && std::isfinite(P.vram_cap);
+  if (reg && c->sumK <= kFcCornerRows && a.k <= (1 << kFcCornerBits)) {
+    // one bit of the corner for each model in turn, while it has options for it
+    int left = kFcCornerBits;
+    for (bool grew = true; grew && left > 0;) {
       grew = false;
-      for (int i = 0; i < P.n_models; ++i)
-        if (S.corner[i] < P.K[i] && S.corner[i] < kFcCornerOpts && prod / S.corner[i] * (S.corner[i] + 1) <= kFcCorner) {
-          prod = prod / S.corner[i] * (S.corner[i] + 1);
-          ++S.corner[i];
+      for (int i = 0; i < N && left > 0; ++i)
+        if ((1 << S.bits[i]) < P.K[i] && (2 << S.bits[i]) <= kFcCornerOpts) {
+          ++S.bits[i];
+          --left;
           grew = true;
         }
     }
+    S.corner = 1;
+  }
+  // units of N - 2 models' settings where every thread gets one, else of N - 1 models'
+  const uint64_t threads = (uint64_t)grid * kFcThreads;
+  const uint64_t bigunit = (uint64_t)P.K[N - 1] * (N >= 2 ? P.K[N - 2] : 1);
+  S.lead = N >= 2 && a.len / bigunit >= threads ? N - 2 : N - 1;
+  uint64_t v = threads;
+  for (int i = S.lead - 1; i >= 0; --i) {
+    S.step[i] = (uint32_t)(v % (uint64_t)P.K[i]);
+    v /= (uint64_t)P.K[i];
   }
   const bool wl = a.k <= kFcWarpK;  // per-warp lists
   const size_t smem = fc_scan_table_bytes(c->sumK) + fc_scan_list_bytes(a.k, wl);
@@ -959,7 +979,7 @@ mf_status fc_search_chunk(mf_ctx* c, const RangeArgs& a, int grid, cudaStream_t 
   using ScanFn = void (*)(const Params, const FcScan, const RangeArgs);
   const bool n8 = P.n_models <= 8;
   ScanFn fn;
-  if (S.reg)
+  if (reg)
     fn = wl ? (n8 ? k_fc_scan<8, true, true> : k_fc_scan<MF_MAX_MODELS, true, true>)
             : (n8 ? k_fc_scan<8, false, true> : k_fc_scan<MF_MAX_MODELS, false, true>);
   else
