@@ -631,122 +631,173 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
 }
 
 // ---------------------------------------------------------------------------
-// VRAM-feasible space: CTA b scans the contiguous segment [b*seg, (b+1)*seg) of the
-// range, in steps of 512 consecutive candidates.  k_vram_count counts; after an
-// exclusive scan of the counts, k_vram_write writes each CTA's indices in order.
+// VRAM-feasible space as an ascending index list.  A thread takes one setting of the leading
+// N - 1 models, whose demand it sums once for all options of the last model.  k_vram_count
+// counts the feasible configurations of each CTA's contiguous segment of settings;
+// k_vram_write (same segments) starts at the sum of the counts before its own and writes:
+// per step of 512 settings a block-wide scan of the threads' counts gives each warp its
+// place, and the warp then writes its 32 settings' configurations in order, a lane per option
+// (several settings at once where the last model has few options).  Bound by the writes for
+// long lists.  48 M configurations, 15 M indices written: VRAM_NOW; one candidate a thread,
+// N lookups each and two block barriers per 512 candidates took 773 us.
 // ---------------------------------------------------------------------------
 constexpr int kVramThreads = 512;
 
 struct VramArgs {
-  uint64_t lo, len, seg;
-  uint32_t step[MF_MAX_MODELS];   // mixed-radix digits of 512
+  uint64_t lo, hi;                // the range
+  uint64_t first, n, seg;         // settings: the range's first, their number, a CTA's share
+  uint32_t step[MF_MAX_MODELS];   // mixed-radix digits of kVramThreads in models 0 .. N - 2
   unsigned long long* counts;     // [grid]
   uint64_t* out;
   uint64_t cap;
+  unsigned long long* total;      // pinned host memory
 };
 
+// A thread's settings of the leading N - 1 models, from setting p on in steps of kVramThreads.
+struct VramRows {
+  int row[MF_MAX_MODELS];
+  __device__ __forceinline__ void start(const Params& P, uint64_t p) {
+#pragma unroll
+    for (int i = MF_MAX_MODELS - 1; i >= 0; --i)
+      if (i < P.n_models - 1) {
+        const uint32_t K = (uint32_t)P.K[i];
+        uint32_t d;
+        if (p <= 0xffffffffull) {
+          d = (uint32_t)p % K;
+          p = (uint32_t)p / K;
+        } else {
+          d = (uint32_t)(p % K);
+          p /= K;
+        }
+        row[i] = P.off[i] + (int)d;
+      }
+  }
+  __device__ __forceinline__ float sum(const Params& P, const float* vr) const {
+    float V = 0.f;
+#pragma unroll
+    for (int i = 0; i < MF_MAX_MODELS; ++i)
+      if (i < P.n_models - 1) V += vr[row[i]];
+    return V;
+  }
+  __device__ __forceinline__ void advance(const Params& P, const uint32_t (&step)[MF_MAX_MODELS]) {
+    uint32_t carry = 0;
+#pragma unroll
+    for (int i = MF_MAX_MODELS - 1; i >= 0; --i)
+      if (i < P.n_models - 1) {
+        const int off = P.off[i];
+        uint32_t d = (uint32_t)(row[i] - off) + step[i] + carry;
+        carry = d >= (uint32_t)P.K[i];
+        if (carry) d -= (uint32_t)P.K[i];
+        row[i] = off + (int)d;
+      }
+  }
+};
+
+// Feasible options of the last model for a setting whose leading models need V: those of
+// [o0, o1) (the whole row but at the range's ends).
+__device__ __forceinline__ unsigned vram_row_count(const float* vl, float V, float cap, int o0, int o1) {
+  unsigned c = 0;
+#pragma unroll 8
+  for (int o = o0; o < o1; ++o) c += V + vl[o] <= cap ? 1u : 0u;
+  return c;
+}
+
 template <bool WRITE>
-__global__ void __launch_bounds__(kVramThreads)
+__global__ void __launch_bounds__(kVramThreads, 2)
 k_vram(const Params P, const VramArgs A) {
   extern __shared__ __align__(16) float vr[];  // [sumK] VRAM of each option
   __shared__ unsigned int s_warp[kVramThreads / 32];
   __shared__ unsigned long long s_base;
-  const int N = P.n_models;
-  const int sumK = pick(P.off, N - 1) + pick(P.K, N - 1);
+  const int N = P.n_models, K = pick(P.K, N - 1);
+  const int sumK = pick(P.off, N - 1) + K;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int e = tid; e < sumK; e += blockDim.x) vr[e] = P.dem[e].y;
-  const uint64_t s0 = (uint64_t)blockIdx.x * A.seg;
-  const uint64_t s1 = s0 + A.seg < A.len ? s0 + A.seg : A.len;
-  int row[MF_MAX_MODELS];
-  {
-    const uint64_t idx0 = A.lo + (s0 + tid < A.len ? s0 + tid : 0);
-#pragma unroll
-    for (int i = 0; i < MF_MAX_MODELS; ++i)
-      if (i < N) row[i] = P.off[i] + (int)((idx0 / P.stride[i]) % (uint64_t)P.K[i]);
-  }
-  if (tid == 0) s_base = WRITE ? A.counts[blockIdx.x] : 0ull;
+  if (tid == 0) s_base = 0ull;
+  for (int e = tid; e < sumK; e += kVramThreads) vr[e] = P.dem[e].y;
   __syncthreads();
+  if (WRITE) {  // where this CTA's indices start; the last CTA knows the total
+    unsigned long long before = 0;
+    for (int b = tid; b < (int)blockIdx.x; b += kVramThreads) before += A.counts[b];
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) before += __shfl_xor_sync(0xffffffffu, before, w);
+    if (lane == 0 && before) atomicAdd(&s_base, before);
+    __syncthreads();
+    if (blockIdx.x + 1 == gridDim.x && tid == 0) *A.total = s_base + A.counts[blockIdx.x];
+    if (s_base >= A.cap) return;
+    __syncthreads();
+  }
+  const float* vl = vr + (sumK - K);
+  const float cap = P.vram_cap;
+  const uint64_t s0 = (uint64_t)blockIdx.x * A.seg;
+  const uint64_t s1 = s0 + A.seg < A.n ? s0 + A.seg : A.n;
+  VramRows rows;
+  rows.start(P, A.first + (s0 + tid < s1 ? s0 + tid : 0));
+  int kp = 1;  // lanes per setting when the warp writes: K rounded up to a power of two, at most 32
+  while (kp < K && kp < 32) kp <<= 1;
   unsigned long long mine = 0;
   for (uint64_t b = s0; b < s1; b += kVramThreads) {
-    const uint64_t t = b + tid;
-    float V = 0.f;
+    const uint64_t p = b + tid;
+    const bool in = p < s1;
+    const float V = rows.sum(P, vr);
+    const uint64_t i0 = (A.first + p) * (uint64_t)K;  // the setting's first configuration
+    const int o0 = i0 < A.lo ? (int)(A.lo - i0) : 0, o1 = in ? (A.hi - i0 < (uint64_t)K ? (int)(A.hi - i0) : K) : 0;
+    const unsigned c = vram_row_count(vl, V, cap, o0, o1);
+    if (!WRITE) {
+      mine += c;
+    } else {
+      unsigned sum = c;  // the warp's total
 #pragma unroll
-    for (int i = 0; i < MF_MAX_MODELS; ++i)
-      if (i < N) V += vr[row[i]];
-    const bool ok = t < s1 && V <= P.vram_cap;
-    if (WRITE) {
-      // ascending positions: this warp's earlier lanes, then the earlier warps
-      const unsigned int bal = __ballot_sync(0xffffffffu, ok);
-      if (lane == 0) s_warp[warp] = __popc(bal);
+      for (int w = 16; w > 0; w >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, w);
+      if (lane == 0) s_warp[warp] = sum;
       __syncthreads();
-      unsigned int before = __popc(bal & ((1u << lane) - 1u));
-      unsigned int total = 0;
+      unsigned before = 0, total = 0;
+#pragma unroll
       for (int w = 0; w < kVramThreads / 32; ++w) {
-        if (w < warp) before += s_warp[w];
+        before += w < warp ? s_warp[w] : 0u;
         total += s_warp[w];
       }
-      const unsigned long long pos = s_base + before;
-      if (ok && pos < A.cap) A.out[pos] = A.lo + t;
+      uint64_t pos = s_base + before;
+      const uint64_t w0 = (A.first + b + (uint64_t)warp * 32) * (uint64_t)K;  // the warp's first configuration
+      if (sum > 0 && pos < A.cap) {
+        for (int u0 = 0; u0 < 32; u0 += 32 / kp) {  // settings u0 .. of the warp
+          const int u = u0 + lane / kp;
+          const float Vu = __shfl_sync(0xffffffffu, V, u);
+          const int a0 = __shfl_sync(0xffffffffu, o0, u), a1 = __shfl_sync(0xffffffffu, o1, u);
+          for (int c0 = 0; c0 < K; c0 += 32) {
+            const int o = c0 + lane % kp;
+            const bool ok = o >= a0 && o < a1 && Vu + vl[o] <= cap;
+            const unsigned m = __ballot_sync(0xffffffffu, ok);
+            const uint64_t to = pos + __popc(m & ((1u << lane) - 1u));
+            if (ok && to < A.cap) A.out[to] = w0 + (uint64_t)u * K + o;
+            pos += __popc(m);
+          }
+        }
+      }
       __syncthreads();
       if (tid == 0) s_base += total;
-    } else {
-      mine += ok ? 1ull : 0ull;
     }
-    uint32_t carry = 0;
-#pragma unroll
-    for (int i = MF_MAX_MODELS - 1; i >= 0; --i)
-      if (i < N) {
-        const int off = P.off[i];
-        const uint32_t K = (uint32_t)P.K[i];
-        uint32_t d = (uint32_t)(row[i] - off) + A.step[i] + carry;
-        carry = d >= K;
-        if (carry) d -= K;
-        row[i] = off + (int)d;
-      }
+    rows.advance(P, A.step);
   }
   if (!WRITE) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
-    if (lane == 0) atomicAdd(&A.counts[blockIdx.x], mine);
-  }
-}
-
-// Exclusive scan of n counts in place (one CTA; n <= 4096); total to *total.
-__global__ void __launch_bounds__(1024)
-k_scan_counts(unsigned long long* c, int n, unsigned long long* total) {
-  __shared__ unsigned long long s[4096];
-  for (int e = threadIdx.x; e < n; e += blockDim.x) s[e] = c[e];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned long long run = 0;
-    for (int e = 0; e < n; ++e) {
-      const unsigned long long v = s[e];
-      s[e] = run;
-      run += v;
-    }
-    *total = run;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < n; e += blockDim.x) c[e] = s[e];
-}
-
-static void radix_digits(const Params& P, uint64_t v, uint32_t* step) {
-  v %= P.total;
-  for (int i = P.n_models - 1; i >= 0; --i) {
-    step[i] = (uint32_t)(v % (uint64_t)P.K[i]);
-    v /= (uint64_t)P.K[i];
+    for (int w = 16; w > 0; w >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, w);
+    if (lane == 0 && mine) atomicAdd(&s_base, mine);
+    __syncthreads();
+    if (tid == 0) A.counts[blockIdx.x] = s_base;
   }
 }
 
 // ---------------------------------------------------------------------------
-// The paper's GA (Sec. IV-C) on the fixed-context landscape, one CTA: thread c breeds
-// individual c; fitness is the table sum of fc mode.  Operators and draws follow the
-// GA of k_ga.cu with two more: crossover applied with probability crossover_p (draw
-// kGaCrossDo, else the first parent is copied) and repair of an infeasible individual
-// by rejection sampling from the uniform distribution over Lambda (draws kGaRepair,
-// j = a * N + i, at most 256 / N attempts, the first feasible one kept).  The block has
-// 1024 threads whatever the population, and a generation's repairs share all of them
-// (see repair).
+// The paper's GA (Sec. IV-C) on the fixed-context landscape, one CTA; fitness is the table
+// sum of fc mode.  Operators and draws follow the GA of k_ga.cu with two more: crossover
+// applied with probability crossover_p (draw kGaCrossDo, else the first parent is copied)
+// and repair of an infeasible individual by rejection sampling from the uniform
+// distribution over Lambda (draws kGaRepair, j = a * N + i, at most 256 / N attempts, the
+// first feasible one kept).  The block has 1024 threads whatever the population: eight lanes
+// breed an individual (a tournament entry or a gene each), and a generation's repairs share
+// all threads (see repair).  Bound by the latency of a generation's chain: draws, fitness
+// reads, the two tournaments, genes, their terms in model order, one block barrier.
+// Population 100, 30 generations, N = 5: FC_GA_NOW; one thread per individual, its draws
+// one after another, took 180 us.
 // ---------------------------------------------------------------------------
 struct FcGaArgs {
   const float2* tab;
@@ -757,21 +808,17 @@ struct FcGaArgs {
   float* out_fit;
 };
 
-__device__ __forceinline__ float fc_fit(const Params& P, const float2* tab, const uint8_t* g) {
-  float J = 0.f, V = 0.f;
-  for (int i = 0; i < P.n_models; ++i) {
-    const float2 e = tab[pick(P.off, i) + g[i]];
-    J += e.x;
-    V += e.y;
-  }
-  return (V <= P.vram_cap && J > -INFINITY) ? J : -INFINITY;
+// (fitness, slot) as one word that orders by fitness, then by lower slot.
+__device__ __forceinline__ unsigned long long fc_rank(float f, int slot) {
+  return ((unsigned long long)fc_key(f) << 32) | (0xFFFFFFFFu - (uint32_t)slot);
 }
+__device__ __forceinline__ int fc_slot(unsigned long long r) { return (int)(0xFFFFFFFFu - (uint32_t)r); }
 
+// NG: genes a lane of a group of eight holds (N <= 8 NG).
+template <int NG>
 __global__ void __launch_bounds__(1024)
 k_fc_ga(const Params P, const FcGaArgs A) {
   extern __shared__ __align__(16) unsigned char sm[];
-  __shared__ float sval[32];
-  __shared__ int sidx[32];
   __shared__ int s_wcnt[32];
   __shared__ int s_pend[1024];
   const int N = P.n_models, pop = A.pop;
@@ -845,7 +892,7 @@ k_fc_ga(const Params P, const FcGaArgs A) {
       const int a = a0 + lig;
       float Jc = -INFINITY;
       uint8_t cand[MF_MAX_MODELS];
-      if (!done && a < attempts) {  // fc_fit's sums, with the draws kept in registers
+      if (!done && a < attempts) {  // the fitness' sums, with the draws kept in registers
         float Js = 0.f, Vs = 0.f;
 #pragma unroll
         for (int i = 0; i < MF_MAX_MODELS; ++i) {
@@ -871,64 +918,121 @@ k_fc_ga(const Params P, const FcGaArgs A) {
       }
     }
   };
-  bool need = false;
-  if (c < pop) {  // initial population: uniform over Lambda, repaired
-    uint8_t* g = g0 + (size_t)c * N;
-    for (int i = 0; i < N; ++i) g[i] = (uint8_t)ga_unif(ga_rng(sd, 0, (uint32_t)c, kGaInit, (uint32_t)i), (uint32_t)pick(P.K, i));
-    const float J = fc_fit(P, tab, g);
-    fit0[c] = J;
-    need = repairable && J == -INFINITY;
+  // eight lanes per individual: lane gl of a group holds genes gl, gl + 8, ..
+  constexpr int kGroups = 128;
+  const int gl = lane & 7, group = c >> 3, g0l = lane & ~7;  // (g0l: the group's first lane)
+  int off[NG], K[NG];
+#pragma unroll
+  for (int q = 0; q < NG; ++q) {
+    const int i = gl + 8 * q;
+    off[q] = i < N ? pick(P.off, i) : 0;
+    K[q] = i < N ? pick(P.K, i) : 1;
   }
-  repair(0u, need, g0, fit0);
-  __syncthreads();
+  // a group's individual: its genes and its fitness, the terms summed in model order
+  auto place = [&](int child, const int (&gene)[NG], uint8_t* genes, float* fit) {
+    float2 e[NG];
+#pragma unroll
+    for (int q = 0; q < NG; ++q) {
+      e[q] = tab[off[q] + gene[q]];
+      if (gl + 8 * q < N && child < pop) genes[(size_t)child * N + gl + 8 * q] = (uint8_t)gene[q];
+    }
+    float J = 0.f, V = 0.f;
+#pragma unroll
+    for (int q = 0; q < NG; ++q)
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (i + 8 * q < N) {
+          J += __shfl_sync(0xffffffffu, e[q].x, g0l + i);
+          V += __shfl_sync(0xffffffffu, e[q].y, g0l + i);
+        }
+    const bool ok = V <= P.vram_cap && J > -INFINITY;
+    if (gl == 0 && child < pop) fit[child] = ok ? J : -INFINITY;
+    return ok || child >= pop;
+  };
+  // ends a generation (first: the first slot that breeds): a block barrier, and the repairs
+  // where an individual that this thread placed, or another's, is infeasible
+  auto settle = [&](uint32_t G, int first, uint8_t* genes, float* fit, bool bad) {
+    if (!__syncthreads_or(bad && repairable)) return;
+    repair(G, c >= first && c < pop && fit[c] == -INFINITY, genes, fit);
+    __syncthreads();
+  };
+  bool bad = false;
+  for (int c0 = 0; c0 < pop; c0 += kGroups) {  // initial population: uniform over Lambda, repaired
+    const int child = c0 + group;
+    int gene[NG];
+#pragma unroll
+    for (int q = 0; q < NG; ++q)
+      gene[q] = ga_unif(ga_rng(sd, 0, (uint32_t)child, kGaInit, (uint32_t)(gl + 8 * q)), (uint32_t)K[q]);
+    bad = !place(child, gene, g0, fit0) || bad;
+  }
+  settle(0u, 0, g0, fit0, bad);
   uint8_t* gc = g0;
   uint8_t* gn = g1;
   float* fc_ = fit0;
   float* fn = fit1;
+  // fittest individual of the current population (lowest slot among equals), on every lane
+  auto warp_fittest = [&]() {
+    unsigned long long best = 0ull;
+    for (int e = lane; e < pop; e += 32) best = max(best, fc_rank(fc_[e], e));
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, w));
+    return fc_slot(best);
+  };
   for (int gen = 0; gen + 1 < A.gens; ++gen) {
     const uint32_t G = (uint32_t)gen + 1u;
-    int first = 0;
-    if (A.elitism) {  // slot 0 keeps the fittest (lowest slot among equals)
-      const int e = block_argmax(fc_, pop, sval, sidx);
-      if (c < N) gn[c] = gc[(size_t)e * N + c];
-      if (c == 0) fn[0] = fc_[e];
-      first = 1;
-    }
-    need = false;
-    if (c >= first && c < pop) {
-      int win[2];
-      for (int w = 0; w < 2; ++w) {
-        int best = -1;
-        float bf = 0.f;
-        for (int t = 0; t < A.tournament; ++t) {
-          const int s2 = ga_unif(ga_rng(sd, G, (uint32_t)c, w ? kGaTourB : kGaTourA, (uint32_t)t), (uint32_t)pop);
-          const float f = fc_[s2];
-          if (best < 0 || f > bf || (f == bf && s2 < best)) { best = s2; bf = f; }
-        }
-        win[w] = best;
+    bad = false;
+    for (int c0 = 0; c0 < pop; c0 += kGroups) {
+      const int child = c0 + group;
+      const uint32_t cu = (uint32_t)child;
+      // the draws that do not depend on fitness
+      bool take_b[NG], mutate[NG];
+      int mval[NG];
+      const bool cross = (uint32_t)(ga_rng(sd, G, cu, kGaCrossDo, 0u) >> 40) < A.cross_thr;
+#pragma unroll
+      for (int q = 0; q < NG; ++q) {
+        const uint32_t i = (uint32_t)(gl + 8 * q);
+        take_b[q] = cross && (ga_rng(sd, G, cu, kGaCross, i) >> 63);
+        mutate[q] = (uint32_t)(ga_rng(sd, G, cu, kGaMut, i) >> 40) < A.mut_thr;
+        mval[q] = ga_unif(ga_rng(sd, G, cu, kGaMutVal, i), (uint32_t)K[q]);
       }
-      const bool cross = (uint32_t)(ga_rng(sd, G, (uint32_t)c, kGaCrossDo, 0u) >> 40) < A.cross_thr;
-      uint8_t* g = gn + (size_t)c * N;
-      for (int i = 0; i < N; ++i) {
-        const uint64_t rc = ga_rng(sd, G, (uint32_t)c, kGaCross, (uint32_t)i);
-        uint8_t gene = (cross && (rc >> 63)) ? gc[(size_t)win[1] * N + i] : gc[(size_t)win[0] * N + i];
-        const uint64_t rm = ga_rng(sd, G, (uint32_t)c, kGaMut, (uint32_t)i);
-        if ((uint32_t)(rm >> 40) < A.mut_thr)
-          gene = (uint8_t)ga_unif(ga_rng(sd, G, (uint32_t)c, kGaMutVal, (uint32_t)i), (uint32_t)pick(P.K, i));
-        g[i] = gene;
+      // the two tournaments, entries shared out over the group's lanes
+      unsigned long long win[2] = {0ull, 0ull};
+      for (int d = gl; d < 2 * A.tournament; d += 8) {
+        const int w = d < A.tournament ? 0 : 1;
+        const int s2 = ga_unif(ga_rng(sd, G, cu, w ? kGaTourB : kGaTourA, (uint32_t)(d - w * A.tournament)), (uint32_t)pop);
+        const unsigned long long r = fc_rank(fc_[s2], s2);
+        if (w) win[1] = max(win[1], r); else win[0] = max(win[0], r);
       }
-      const float J = fc_fit(P, tab, g);
-      fn[c] = J;
-      need = repairable && J == -INFINITY;
+#pragma unroll
+      for (int w = 4; w > 0; w >>= 1) {
+        win[0] = max(win[0], __shfl_xor_sync(0xffffffffu, win[0], w));
+        win[1] = max(win[1], __shfl_xor_sync(0xffffffffu, win[1], w));
+      }
+      int parent[2] = {fc_slot(win[0]), fc_slot(win[1])};
+      bool elite = false;
+      if (A.elitism && c0 == 0 && warp == 0) {  // slot 0 keeps the fittest
+        const int e = warp_fittest();
+        elite = child == 0;
+        if (elite) parent[0] = parent[1] = e;
+      }
+      int gene[NG];
+#pragma unroll
+      for (int q = 0; q < NG; ++q) {
+        const int i = gl + 8 * q;
+        gene[q] = i < N ? gc[(size_t)(take_b[q] ? parent[1] : parent[0]) * N + i] : 0;
+        if (mutate[q] && !elite && i < N) gene[q] = mval[q];
+      }
+      bad = !place(child, gene, gn, fn) || bad;
     }
-    repair(G, need, gn, fn);
-    __syncthreads();
+    settle(G, A.elitism ? 1 : 0, gn, fn, bad);
     uint8_t* tg = gc; gc = gn; gn = tg;
     float* tf = fc_; fc_ = fn; fn = tf;
   }
-  const int e = block_argmax(fc_, pop, sval, sidx);
-  if (c < N) A.out_genome[c] = gc[(size_t)e * N + c];
-  if (c == 0) *A.out_fit = fc_[e];
+  if (warp == 0) {
+    const int e = warp_fittest();
+    if (c < N) A.out_genome[c] = gc[(size_t)e * N + c];
+    if (c == 0) *A.out_fit = fc_[e];
+  }
 }
 
 // One CTA per SM, fewer where the range has fewer settings of the leading N - 1 models
@@ -1073,40 +1177,42 @@ mf_status mf_vram_feasible(mf_ctx* ctx, uint64_t lo, uint64_t hi, uint64_t* d_ou
   if (cap > 0 && !d_out) return fc_einval("d_out is NULL");
   DeviceGuard guard(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
-  const uint64_t len = hi - lo;
-  // segments of whole steps, at most 4096 CTAs
-  const uint64_t steps = (len + kVramThreads - 1) / kVramThreads;
-  uint64_t grid = 4ull * ctx->num_sms;
-  if (grid > steps) grid = steps > 0 ? steps : 1;
-  const uint64_t seg = ((steps + grid - 1) / grid) * kVramThreads;
-  grid = len > 0 ? (len + seg - 1) / seg : 1;
-  mf_status st = ensure_scratch(ctx, sizeof(unsigned long long) * (grid + 1));
-  if (st != MF_OK) return st;
-  unsigned long long* counts = (unsigned long long*)ctx->d_scratch;
+  if (lo == hi) {
+    *count = 0;
+    return MF_OK;
+  }
+  const int N = ctx->P.n_models;
+  const uint64_t K = (uint64_t)ctx->P.K[N - 1];
   VramArgs A{};
   A.lo = lo;
-  A.len = len;
-  A.seg = seg;
-  radix_digits(ctx->P, kVramThreads, A.step);
-  A.counts = counts;
-  A.out = d_out;
-  A.cap = cap;
-  const size_t smem = sizeof(float) * (size_t)ctx->sumK;
-  MF_CUDA(cudaMemsetAsync(counts, 0, sizeof(unsigned long long) * (grid + 1), s));
-  k_vram<false><<<(unsigned)grid, kVramThreads, smem, s>>>(ctx->P, A);
-  MF_CUDA(cudaGetLastError());
-  k_scan_counts<<<1, 1024, 0, s>>>(counts, (int)grid, counts + grid);
-  MF_CUDA(cudaGetLastError());
-  if (cap > 0) {
-    k_vram<true><<<(unsigned)grid, kVramThreads, smem, s>>>(ctx->P, A);
-    MF_CUDA(cudaGetLastError());
-  }
+  A.hi = hi;
+  A.first = lo / K;
+  A.n = (hi - 1) / K - A.first + 1;
+  // segments of whole steps, two rounds of the two CTAs an SM holds
+  const uint64_t steps = (A.n + kVramThreads - 1) / kVramThreads;
+  const uint64_t most = 4ull * ctx->num_sms;
+  A.seg = (steps + most - 1) / most * kVramThreads;
+  const unsigned grid = (unsigned)((A.n + A.seg - 1) / A.seg);
+  mf_status st = ensure_scratch(ctx, sizeof(unsigned long long) * grid);
+  if (st != MF_OK) return st;
   st = ensure_host_stage(ctx, sizeof(unsigned long long));
   if (st != MF_OK) return st;
-  unsigned long long* h = (unsigned long long*)ctx->h_stage;
-  MF_CUDA(cudaMemcpyAsync(h, counts + grid, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+  uint64_t v = kVramThreads;
+  for (int i = N - 2; i >= 0; --i) {
+    A.step[i] = (uint32_t)(v % (uint64_t)ctx->P.K[i]);
+    v /= (uint64_t)ctx->P.K[i];
+  }
+  A.counts = (unsigned long long*)ctx->d_scratch;
+  A.out = d_out;
+  A.cap = cap;
+  A.total = (unsigned long long*)ctx->h_stage;
+  const size_t smem = sizeof(float) * (size_t)ctx->sumK;
+  k_vram<false><<<grid, kVramThreads, smem, s>>>(ctx->P, A);
+  MF_CUDA(cudaGetLastError());
+  k_vram<true><<<grid, kVramThreads, smem, s>>>(ctx->P, A);
+  MF_CUDA(cudaGetLastError());
   MF_CUDA(cudaStreamSynchronize(s));
-  *count = *h;
+  *count = *A.total;
   return MF_OK;
 }
 
@@ -1127,11 +1233,10 @@ mf_status mf_fc_ga_run(mf_ctx* ctx, const mf_fc_ga_params* g, uint64_t seed, int
   const int N = ctx->P.n_models;
   FcLayout L;
   fc_bytes(ctx->sumK, &L, (char*)ctx->d_fc);
-  // result: genome (16 ints) then the fitness
-  mf_status st = ensure_scratch(ctx, sizeof(int32_t) * 17);
+  // result, written by the kernel itself to pinned host memory: genome (16 ints), fitness
+  mf_status st = ensure_host_stage(ctx, sizeof(int32_t) * 17);
   if (st != MF_OK) return st;
-  st = ensure_host_stage(ctx, sizeof(int32_t) * 17);
-  if (st != MF_OK) return st;
+  int32_t* h = (int32_t*)ctx->h_stage;
   FcGaArgs A{};
   A.tab = L.tab;
   A.pop = g->pop;
@@ -1142,15 +1247,13 @@ mf_status mf_fc_ga_run(mf_ctx* ctx, const mf_fc_ga_params* g, uint64_t seed, int
   A.mut_thr = (uint32_t)std::floor(g->mutation_p * 16777216.0 + 0.5);
   A.cross_thr = (uint32_t)std::floor(g->crossover_p * 16777216.0 + 0.5);
   A.seed = seed;
-  A.out_genome = (int32_t*)ctx->d_scratch;
-  A.out_fit = (float*)((int32_t*)ctx->d_scratch + 16);
+  A.out_genome = h;
+  A.out_fit = (float*)(h + 16);
   const size_t smem = sizeof(float2) * ctx->sumK + sizeof(float) * 2 * g->pop + (size_t)2 * g->pop * N;
-  const int threads = 1024;  // (the repairs use every warp)
-  MF_CUDA(cudaFuncSetAttribute(k_fc_ga, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_fc_ga<<<1, threads, smem, s>>>(ctx->P, A);
+  const auto fn = N <= 8 ? k_fc_ga<1> : k_fc_ga<2>;
+  MF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  fn<<<1, 1024, smem, s>>>(ctx->P, A);
   MF_CUDA(cudaGetLastError());
-  int32_t* h = (int32_t*)ctx->h_stage;
-  MF_CUDA(cudaMemcpyAsync(h, ctx->d_scratch, sizeof(int32_t) * 17, cudaMemcpyDeviceToHost, s));
   MF_CUDA(cudaStreamSynchronize(s));
   std::memcpy(best_genome, h, sizeof(int32_t) * N);
   std::memcpy(best_fitness, h + 16, sizeof(float));
