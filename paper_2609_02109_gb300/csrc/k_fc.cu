@@ -88,7 +88,7 @@ struct FcConst {
 //
 // Bound by latency: the model's weights (the transposed copy) come into shared memory with
 // one round of wide loads where they fit kFcStage, since a row read as it was needed cost
-// an L2 round trip per few inputs (12->64->64->2, 144 rows: 7.1 us, staged FC_LOCAL_NOW).
+// an L2 round trip per few inputs (12->64->64->2, 144 rows: 7.1 us, staged 5).
 // ---------------------------------------------------------------------------
 constexpr size_t kFcStage = 96 * 1024;
 
@@ -200,7 +200,7 @@ k_fc_local(const Params P, const FcLayout L, const FcInputs I, const FcConst C) 
 // otherwise one list and queue per CTA, whose warps meet for a merge when it fills up.
 //
 // Bound by latency (shared-memory chains of the counts; the prologue's ranking and corner).
-// 24^6, VRAM binding, k = 32: FC_SCAN_NOW, where the scan of every candidate took 12
+// 24^6, VRAM binding, k = 32: one launch of 36 us, where the scan of every candidate took 12
 // launches of 75-125 us, each of which also filled its lists from nothing.
 // ---------------------------------------------------------------------------
 constexpr int kFcThreads = 512;
@@ -469,10 +469,12 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
       }
   }
   unsigned long long my_count = 0;
-  // look-at state of the warp: the lanes whose units wait, the current unit's next option of
-  // model N - 2 (index within na) and the next row of 32 of the last model's options
-  unsigned waiting = 0u;
+  // look-at state of the warp: the lanes whose units wait, the current unit's row of 32 of
+  // model N - 2's options, those of the row still to do (when `open`), and the next row of
+  // 32 of the last model's options
+  unsigned waiting = 0u, todo = 0u;
   int at_a = 0, at_b = 0;
+  bool open = false;
   float pJ2 = 0.f, pV2 = 0.f;  // this lane's unit: sums over models 0 .. lead - 1, in order
   bool count_there = false;    // it is counted when it is looked at
   auto merge_warp = [&]() {
@@ -507,12 +509,14 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
             if ((pV2 + spa.vmax) + sb.vmax <= cap) {
               my_count += (unsigned)(spa.n * sb.n);
             } else if (!none) {
-              int c = sb.n;
+              // each step moves one pointer: no lane waits in an inner loop for another
+              int c = sb.n, a = 0;
               unsigned n = 0;
-              for (int a = 0; a < spa.n && c > 0; ++a) {
-                const float p = pV2 + sa[a];
-                while (c > 0 && !(p + sv[c - 1] <= cap)) --c;
-                n += (unsigned)c;
+              while (a < spa.n && c > 0) {
+                const bool fits = (pV2 + sa[a]) + sv[c - 1] <= cap;
+                n += fits ? (unsigned)c : 0u;
+                a += fits ? 1 : 0;
+                c -= fits ? 0 : 1;
               }
               my_count += n;
             }
@@ -528,7 +532,6 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
           }
         }
         waiting = __ballot_sync(0xffffffffu, look);
-        at_a = at_b = 0;
       }
       // ---- the warp looks at the waiting units, one after another ----
       bool full = false;
@@ -537,45 +540,57 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
         const float bJ = __shfl_sync(0xffffffffu, pJ2, src), bV = __shfl_sync(0xffffffffu, pV2, src);
         const bool cnt = __shfl_sync(0xffffffffu, count_there ? 1 : 0, src) != 0;
         const uint64_t t0 = (u0 + __shfl_sync(0xffffffffu, my, src)) * unit;
-        for (; at_a < na; ++at_a) {
+        for (; at_a < na; at_a += 32) {
+          // this lane's option of model N - 2, and the options of the row worth a look
           float aJ = bJ, aV = bV;
-          if (big) {
-            const float2 e = tab[off_prev + at_a];
+          const bool have = at_a + lane < na;
+          if (big && have) {
+            const float2 e = tab[off_prev + at_a + lane];
             aJ += e.x;
             aV += e.y;
           }
-          if (REG && !cnt && !(aV + sb.vmin <= cap && aJ + sb.jmax >= thr_s)) continue;  // (uniform)
-          for (; at_b < klast; at_b += 32) {
-            // room for this row of 32 (in a CTA's queue: for a row of every warp)
-            if (WL) {
-              if (*(volatile int*)wt.qn > kFcWarpQ - 32) {
-                merge_warp();
-                raise_bar();
-              }
-            } else {
-              // (one lane reads the queue's length, which other warps move, for all)
-              full = __shfl_sync(0xffffffffu, *(volatile int*)wt.qn, 0) > QCAP - 32 * kFcWarps;
-              if (full) break;
-            }
-            const int o = at_b + lane;
-            const uint64_t idx = t0 + (uint64_t)at_a * klast + o;
-            const bool in = o < klast && idx >= R.base && idx < end;
-            const float2 e = in ? tab[off_last + o] : make_float2(0.f, 0.f);
-            const float J = aJ + e.x;
-            const bool feas = in && aV + e.y <= cap;  // NaN compares false
-            my_count += cnt && feas ? 1u : 0u;
-            const bool push = feas && J >= thr_s && precedes(J, idx, thr_s, thr_i);
-            const unsigned m = __ballot_sync(0xffffffffu, push);
-            if (m) {
-              int pos = 0;
-              if (lane == 0) pos = atomicAdd(wt.qn, __popc(m));
-              pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(m & ((1u << lane) - 1u));
-              if (push) { wt.qs[pos] = J; wt.qi[pos] = idx; }
-              __syncwarp();
-            }
+          if (!open) {
+            todo = __ballot_sync(0xffffffffu, have && (!REG || cnt || (aV + sb.vmin <= cap && aJ + sb.jmax >= thr_s)));
+            open = true;
           }
-          if (full) break;  // (resumed at this row after the merge)
-          at_b = 0;
+          for (; todo; todo &= todo - 1u) {
+            const int ua = __ffs(todo) - 1;
+            const float uJ = __shfl_sync(0xffffffffu, aJ, ua), uV = __shfl_sync(0xffffffffu, aV, ua);
+            const uint64_t t1 = t0 + (uint64_t)(at_a + ua) * klast;
+            for (; at_b < klast; at_b += 32) {
+              // room for this row of 32 (in a CTA's queue: for a row of every warp)
+              if (WL) {
+                if (*(volatile int*)wt.qn > kFcWarpQ - 32) {
+                  merge_warp();
+                  raise_bar();
+                }
+              } else {
+                // (one lane reads the queue's length, which other warps move, for all)
+                full = __shfl_sync(0xffffffffu, *(volatile int*)wt.qn, 0) > QCAP - 32 * kFcWarps;
+                if (full) break;
+              }
+              const int o = at_b + lane;
+              const uint64_t idx = t1 + o;
+              const bool in = o < klast && idx >= R.base && idx < end;
+              const float2 e = in ? tab[off_last + o] : make_float2(0.f, 0.f);
+              const float J = uJ + e.x;
+              const bool feas = in && uV + e.y <= cap;  // NaN compares false
+              my_count += cnt && feas ? 1u : 0u;
+              const bool push = feas && J >= thr_s && precedes(J, idx, thr_s, thr_i);
+              const unsigned m = __ballot_sync(0xffffffffu, push);
+              if (m) {
+                int pos = 0;
+                if (lane == 0) pos = atomicAdd(wt.qn, __popc(m));
+                pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(m & ((1u << lane) - 1u));
+                if (push) { wt.qs[pos] = J; wt.qi[pos] = idx; }
+                __syncwarp();
+              }
+            }
+            if (full) break;  // (resumed at this row after the merge)
+            at_b = 0;
+          }
+          if (full) break;
+          open = false;
         }
         if (full) break;
         at_a = 0;
@@ -636,9 +651,10 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
 // counts the feasible configurations of each CTA's contiguous segment of settings;
 // k_vram_write (same segments) starts at the sum of the counts before its own and writes:
 // per step of 512 settings a block-wide scan of the threads' counts gives each warp its
-// place, and the warp then writes its 32 settings' configurations in order, a lane per option
-// (several settings at once where the last model has few options).  Bound by the writes for
-// long lists.  48 M configurations, 15 M indices written: VRAM_NOW; one candidate a thread,
+// place.  Where the last model has at most 32 options, each lane lists its setting's
+// configurations in shared memory (16-bit offsets, in order) and the warp streams the list
+// out in whole rows; above that, the warp writes one setting after another, a lane per option.
+// Bound by issue, then by the writes for long lists.  48 M configurations, 15 M indices written: 78 us; one candidate a thread,
 // N lookups each and two block barriers per 512 candidates took 773 us.
 // ---------------------------------------------------------------------------
 constexpr int kVramThreads = 512;
@@ -654,11 +670,13 @@ struct VramArgs {
 };
 
 // A thread's settings of the leading N - 1 models, from setting p on in steps of kVramThreads.
+// NMAX: a bound on N.
+template <int NMAX>
 struct VramRows {
-  int row[MF_MAX_MODELS];
+  int row[NMAX];
   __device__ __forceinline__ void start(const Params& P, uint64_t p) {
 #pragma unroll
-    for (int i = MF_MAX_MODELS - 1; i >= 0; --i)
+    for (int i = NMAX - 1; i >= 0; --i)
       if (i < P.n_models - 1) {
         const uint32_t K = (uint32_t)P.K[i];
         uint32_t d;
@@ -675,14 +693,14 @@ struct VramRows {
   __device__ __forceinline__ float sum(const Params& P, const float* vr) const {
     float V = 0.f;
 #pragma unroll
-    for (int i = 0; i < MF_MAX_MODELS; ++i)
+    for (int i = 0; i < NMAX; ++i)
       if (i < P.n_models - 1) V += vr[row[i]];
     return V;
   }
   __device__ __forceinline__ void advance(const Params& P, const uint32_t (&step)[MF_MAX_MODELS]) {
     uint32_t carry = 0;
 #pragma unroll
-    for (int i = MF_MAX_MODELS - 1; i >= 0; --i)
+    for (int i = NMAX - 1; i >= 0; --i)
       if (i < P.n_models - 1) {
         const int off = P.off[i];
         uint32_t d = (uint32_t)(row[i] - off) + step[i] + carry;
@@ -702,10 +720,70 @@ __device__ __forceinline__ unsigned vram_row_count(const float* vl, float V, flo
   return c;
 }
 
-template <bool WRITE>
+// Counts of the segments: a thread takes one setting of models 0 .. N - 3 at a time (segments
+// are whole such settings) and runs over the options of models N - 2 and N - 1.
+template <int NMAX>
 __global__ void __launch_bounds__(kVramThreads, 2)
-k_vram(const Params P, const VramArgs A) {
+k_vram_count(const Params P, const VramArgs A) {
   extern __shared__ __align__(16) float vr[];  // [sumK] VRAM of each option
+  __shared__ unsigned long long s_sum;
+  const int N = P.n_models, K = pick(P.K, N - 1), KA = N >= 2 ? pick(P.K, N - 2) : 1;
+  const int sumK = pick(P.off, N - 1) + K;
+  const int tid = threadIdx.x;
+  if (tid == 0) s_sum = 0ull;
+  for (int e = tid; e < sumK; e += kVramThreads) vr[e] = P.dem[e].y;
+  __syncthreads();
+  const float* vl = vr + (sumK - K);
+  const float* va = vl - KA;
+  const float cap = P.vram_cap;
+  // units of this segment (in settings of N - 2 models), and its first and last setting
+  const uint64_t s0 = A.first + (uint64_t)blockIdx.x * A.seg;
+  const uint64_t s1 = s0 + A.seg < A.first + A.n ? s0 + A.seg : A.first + A.n;
+  const uint64_t u0 = s0 / KA, u1 = (s1 + KA - 1) / KA;
+  unsigned long long mine = 0;
+  for (uint64_t u = u0 + tid; u < u1; u += kVramThreads) {
+    float V2 = 0.f;
+    {
+      int row[NMAX];
+      uint64_t p = u;
+#pragma unroll
+      for (int i = NMAX - 1; i >= 0; --i)
+        if (i < N - 2) {
+          const uint32_t Ki = (uint32_t)P.K[i];
+          uint32_t d;
+          if (p <= 0xffffffffull) {
+            d = (uint32_t)p % Ki;
+            p = (uint32_t)p / Ki;
+          } else {
+            d = (uint32_t)(p % Ki);
+            p /= Ki;
+          }
+          row[i] = P.off[i] + (int)d;
+        }
+#pragma unroll
+      for (int i = 0; i < NMAX; ++i)
+        if (i < N - 2) V2 += vr[row[i]];
+    }
+    for (int a = 0; a < KA; ++a) {
+      const uint64_t s = u * KA + a;  // the setting of N - 1 models
+      if (s < s0 || s >= s1) continue;
+      const uint64_t i0 = s * (uint64_t)K;
+      const int o0 = i0 < A.lo ? (int)(A.lo - i0) : 0, o1 = A.hi - i0 < (uint64_t)K ? (int)(A.hi - i0) : K;
+      mine += vram_row_count(vl, N >= 2 ? V2 + va[a] : V2, cap, o0, o1);
+    }
+  }
+#pragma unroll
+  for (int w = 16; w > 0; w >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, w);
+  if ((tid & 31) == 0 && mine) atomicAdd(&s_sum, mine);
+  __syncthreads();
+  if (tid == 0) A.counts[blockIdx.x] = s_sum;
+}
+
+template <int NMAX>
+__global__ void __launch_bounds__(kVramThreads, 2)
+k_vram_write(const Params P, const VramArgs A) {
+  extern __shared__ __align__(16) float vr[];  // [sumK] VRAM of each option
+  __shared__ uint16_t s_list[kVramThreads / 32][32 * 32];
   __shared__ unsigned int s_warp[kVramThreads / 32];
   __shared__ unsigned long long s_base;
   const int N = P.n_models, K = pick(P.K, N - 1);
@@ -714,26 +792,22 @@ k_vram(const Params P, const VramArgs A) {
   if (tid == 0) s_base = 0ull;
   for (int e = tid; e < sumK; e += kVramThreads) vr[e] = P.dem[e].y;
   __syncthreads();
-  if (WRITE) {  // where this CTA's indices start; the last CTA knows the total
-    unsigned long long before = 0;
-    for (int b = tid; b < (int)blockIdx.x; b += kVramThreads) before += A.counts[b];
+  // where this CTA's indices start; the last CTA knows the total
+  unsigned long long before_me = 0;
+  for (int b = tid; b < (int)blockIdx.x; b += kVramThreads) before_me += A.counts[b];
 #pragma unroll
-    for (int w = 16; w > 0; w >>= 1) before += __shfl_xor_sync(0xffffffffu, before, w);
-    if (lane == 0 && before) atomicAdd(&s_base, before);
-    __syncthreads();
-    if (blockIdx.x + 1 == gridDim.x && tid == 0) *A.total = s_base + A.counts[blockIdx.x];
-    if (s_base >= A.cap) return;
-    __syncthreads();
-  }
+  for (int w = 16; w > 0; w >>= 1) before_me += __shfl_xor_sync(0xffffffffu, before_me, w);
+  if (lane == 0 && before_me) atomicAdd(&s_base, before_me);
+  __syncthreads();
+  if (blockIdx.x + 1 == gridDim.x && tid == 0) *A.total = s_base + A.counts[blockIdx.x];
+  if (s_base >= A.cap) return;
+  __syncthreads();
   const float* vl = vr + (sumK - K);
   const float cap = P.vram_cap;
   const uint64_t s0 = (uint64_t)blockIdx.x * A.seg;
   const uint64_t s1 = s0 + A.seg < A.n ? s0 + A.seg : A.n;
-  VramRows rows;
+  VramRows<NMAX> rows;
   rows.start(P, A.first + (s0 + tid < s1 ? s0 + tid : 0));
-  int kp = 1;  // lanes per setting when the warp writes: K rounded up to a power of two, at most 32
-  while (kp < K && kp < 32) kp <<= 1;
-  unsigned long long mine = 0;
   for (uint64_t b = s0; b < s1; b += kVramThreads) {
     const uint64_t p = b + tid;
     const bool in = p < s1;
@@ -741,29 +815,45 @@ k_vram(const Params P, const VramArgs A) {
     const uint64_t i0 = (A.first + p) * (uint64_t)K;  // the setting's first configuration
     const int o0 = i0 < A.lo ? (int)(A.lo - i0) : 0, o1 = in ? (A.hi - i0 < (uint64_t)K ? (int)(A.hi - i0) : K) : 0;
     const unsigned c = vram_row_count(vl, V, cap, o0, o1);
-    if (!WRITE) {
-      mine += c;
-    } else {
-      unsigned sum = c;  // the warp's total
+    unsigned sum = c;  // the warp's total
 #pragma unroll
-      for (int w = 16; w > 0; w >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, w);
-      if (lane == 0) s_warp[warp] = sum;
-      __syncthreads();
-      unsigned before = 0, total = 0;
+    for (int w = 16; w > 0; w >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, w);
+    if (lane == 0) s_warp[warp] = sum;
+    __syncthreads();
+    unsigned before = 0, total = 0;
 #pragma unroll
-      for (int w = 0; w < kVramThreads / 32; ++w) {
-        before += w < warp ? s_warp[w] : 0u;
-        total += s_warp[w];
-      }
-      uint64_t pos = s_base + before;
-      const uint64_t w0 = (A.first + b + (uint64_t)warp * 32) * (uint64_t)K;  // the warp's first configuration
-      if (sum > 0 && pos < A.cap) {
-        for (int u0 = 0; u0 < 32; u0 += 32 / kp) {  // settings u0 .. of the warp
-          const int u = u0 + lane / kp;
+    for (int w = 0; w < kVramThreads / 32; ++w) {
+      const unsigned v = s_warp[w];
+      before += w < warp ? v : 0u;
+      total += v;
+    }
+    uint64_t pos = s_base + before;
+    const uint64_t w0 = (A.first + b + (uint64_t)warp * 32) * (uint64_t)K;  // the warp's first configuration
+    if (sum > 0 && pos < A.cap) {
+      if (K <= 32) {
+        unsigned at = c;  // this lane's place in the warp's list: an exclusive scan
+#pragma unroll
+        for (int w = 1; w < 32; w <<= 1) {
+          const unsigned left = __shfl_up_sync(0xffffffffu, at, w);
+          at += lane >= w ? left : 0u;
+        }
+        at -= c;
+        uint16_t* list = s_list[warp];
+#pragma unroll 8
+        for (int o = o0; o < o1; ++o)
+          if (V + vl[o] <= cap) list[at++] = (uint16_t)(lane * K + o);
+        __syncwarp();
+        const unsigned room = A.cap - pos < sum ? (unsigned)(A.cap - pos) : sum;
+        uint64_t* out = A.out + pos;
+#pragma unroll 4
+        for (unsigned e = lane; e < room; e += 32) out[e] = w0 + list[e];
+        __syncwarp();
+      } else {
+        for (int u = 0; u < 32; ++u) {
           const float Vu = __shfl_sync(0xffffffffu, V, u);
           const int a0 = __shfl_sync(0xffffffffu, o0, u), a1 = __shfl_sync(0xffffffffu, o1, u);
           for (int c0 = 0; c0 < K; c0 += 32) {
-            const int o = c0 + lane % kp;
+            const int o = c0 + lane;
             const bool ok = o >= a0 && o < a1 && Vu + vl[o] <= cap;
             const unsigned m = __ballot_sync(0xffffffffu, ok);
             const uint64_t to = pos + __popc(m & ((1u << lane) - 1u));
@@ -772,17 +862,10 @@ k_vram(const Params P, const VramArgs A) {
           }
         }
       }
-      __syncthreads();
-      if (tid == 0) s_base += total;
     }
-    rows.advance(P, A.step);
-  }
-  if (!WRITE) {
-#pragma unroll
-    for (int w = 16; w > 0; w >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, w);
-    if (lane == 0 && mine) atomicAdd(&s_base, mine);
     __syncthreads();
-    if (tid == 0) A.counts[blockIdx.x] = s_base;
+    if (tid == 0) s_base += total;
+    rows.advance(P, A.step);
   }
 }
 
@@ -793,10 +876,10 @@ k_vram(const Params P, const VramArgs A) {
 // and repair of an infeasible individual by rejection sampling from the uniform
 // distribution over Lambda (draws kGaRepair, j = a * N + i, at most 256 / N attempts, the
 // first feasible one kept).  The block has 1024 threads whatever the population: eight lanes
-// breed an individual (a tournament entry or a gene each), and a generation's repairs share
-// all threads (see repair).  Bound by the latency of a generation's chain: draws, fitness
+// breed an individual (a tournament entry or a gene each), and a warp's lanes share the
+// repairs of its individuals.  Bound by the latency of a generation's chain: draws, fitness
 // reads, the two tournaments, genes, their terms in model order, one block barrier.
-// Population 100, 30 generations, N = 5: FC_GA_NOW; one thread per individual, its draws
+// Population 100, 30 generations, N = 5, some repairs: 93 us; one thread per individual, its draws
 // one after another, took 180 us.
 // ---------------------------------------------------------------------------
 struct FcGaArgs {
@@ -819,8 +902,7 @@ template <int NG>
 __global__ void __launch_bounds__(1024)
 k_fc_ga(const Params P, const FcGaArgs A) {
   extern __shared__ __align__(16) unsigned char sm[];
-  __shared__ int s_wcnt[32];
-  __shared__ int s_pend[1024];
+  __shared__ unsigned long long s_best[3];  // the fittest of generation g in s_best[g % 3]
   const int N = P.n_models, pop = A.pop;
   const int sumK = pick(P.off, N - 1) + pick(P.K, N - 1);
   float2* tab = reinterpret_cast<float2*>(sm);
@@ -830,6 +912,7 @@ k_fc_ga(const Params P, const FcGaArgs A) {
   uint8_t* g1 = g0 + (size_t)pop * N;
   const int c = threadIdx.x;
   for (int e = c; e < sumK; e += blockDim.x) tab[e] = A.tab[e];
+  if (c < 3) s_best[c] = 0ull;
   __syncthreads();
   // Does any configuration meet the floors and the VRAM bound?  Exactly when every model
   // has an option with a finite term and the smallest such VRAM demands, summed in model
@@ -858,66 +941,7 @@ k_fc_ga(const Params P, const FcGaArgs A) {
   const bool repairable = A.repair && s_any_feasible;
   const uint64_t sd = A.seed;
   const int attempts = 256 / N;
-  // Repair of the generation's infeasible children (need): the cnt of them, in ascending
-  // order, each get a group of gs lanes of one warp (gs a power of two, as many lanes as
-  // the block has for cnt rounded up to a power of two, at most 32), which tries the
-  // child's attempts gs at a time; the lowest feasible attempt of a group's first
-  // successful round is the sequential search's result.  The winning lane writes the
-  // child's genes and fitness over the unrepaired ones already in shared memory.
-  const int lane = c & 31, warp = c >> 5, nwarps = (int)(blockDim.x >> 5);
-  auto repair = [&](uint32_t G, bool need, uint8_t* genes, float* fit) {
-    const unsigned bal = __ballot_sync(0xffffffffu, need);
-    if (lane == 0) s_wcnt[warp] = __popc(bal);
-    __syncthreads();
-    int before = 0, cnt = 0;
-    for (int w = 0; w < (pop + 31) / 32; ++w) {  // (only the population's warps breed)
-      const int v = s_wcnt[w];
-      before += w < warp ? v : 0;
-      cnt += v;
-    }
-    if (need) s_pend[before + __popc(bal & ((1u << lane) - 1u))] = c;
-    __syncthreads();
-    if (cnt == 0) return;  // (uniform)
-    int m = 1;
-    while (m < cnt) m <<= 1;
-    int gs = nwarps * 32 / m;
-    gs = gs > 32 ? 32 : (gs < 1 ? 1 : gs);
-    const int grp = lane / gs, lig = lane % gs;
-    const int gid = warp * (32 / gs) + grp;
-    const int child = gid < cnt ? s_pend[gid] : -1;
-    const unsigned gmask = gs == 32 ? 0xffffffffu : ((1u << gs) - 1u) << (grp * gs);
-    bool done = child < 0;
-    for (int a0 = 0; a0 < attempts; a0 += gs) {
-      if (!__any_sync(0xffffffffu, !done)) break;
-      const int a = a0 + lig;
-      float Jc = -INFINITY;
-      uint8_t cand[MF_MAX_MODELS];
-      if (!done && a < attempts) {  // the fitness' sums, with the draws kept in registers
-        float Js = 0.f, Vs = 0.f;
-#pragma unroll
-        for (int i = 0; i < MF_MAX_MODELS; ++i) {
-          if (i < N) {
-            cand[i] = (uint8_t)ga_unif(ga_rng(sd, G, (uint32_t)child, kGaRepair, (uint32_t)(a * N + i)),
-                                       (uint32_t)pick(P.K, i));
-            const float2 e = tab[pick(P.off, i) + cand[i]];
-            Js += e.x;
-            Vs += e.y;
-          }
-        }
-        Jc = (Vs <= P.vram_cap && Js > -INFINITY) ? Js : -INFINITY;
-      }
-      const unsigned ok = __ballot_sync(0xffffffffu, Jc != -INFINITY) & gmask;
-      if (!done && ok) {
-        if (lane == __ffs(ok) - 1) {
-#pragma unroll
-          for (int i = 0; i < MF_MAX_MODELS; ++i)
-            if (i < N) genes[(size_t)child * N + i] = cand[i];
-          fit[child] = Jc;
-        }
-        done = true;
-      }
-    }
-  };
+  const int lane = c & 31;
   // eight lanes per individual: lane gl of a group holds genes gl, gl + 8, ..
   constexpr int kGroups = 128;
   const int gl = lane & 7, group = c >> 3, g0l = lane & ~7;  // (g0l: the group's first lane)
@@ -947,40 +971,80 @@ k_fc_ga(const Params P, const FcGaArgs A) {
         }
     const bool ok = V <= P.vram_cap && J > -INFINITY;
     if (gl == 0 && child < pop) fit[child] = ok ? J : -INFINITY;
-    return ok || child >= pop;
+    return ok ? J : -INFINITY;
   };
-  // ends a generation (first: the first slot that breeds): a block barrier, and the repairs
-  // where an individual that this thread placed, or another's, is infeasible
-  auto settle = [&](uint32_t G, int first, uint8_t* genes, float* fit, bool bad) {
-    if (!__syncthreads_or(bad && repairable)) return;
-    repair(G, c >= first && c < pop && fit[c] == -INFINITY, genes, fit);
-    __syncthreads();
+  // Repair of the warp's infeasible children (`bad`: this lane's group has one, child `child`):
+  // the warp's lanes are shared out over them (32, 16 or 8 lanes each), which try the child's
+  // attempts in order, so many at a time; the lowest feasible attempt of the first successful
+  // round is the sequential search's result.  The winning lane writes the child's genes and
+  // fitness over the unrepaired ones.
+  auto repair = [&](uint32_t G, bool bad, int child, uint8_t* genes, float* fit) {
+    const unsigned bal = __ballot_sync(0xffffffffu, bad && gl == 0);
+    if (!bal) return;
+    __syncwarp();
+    const int cnt = __popc(bal);
+    const int gs = cnt == 1 ? 32 : cnt == 2 ? 16 : 8;
+    const int mine = lane / gs;  // this lane works for the mine-th of them
+    unsigned rest = bal;
+    for (int j = 0; j < mine; ++j) rest &= rest - 1u;
+    const int who = __shfl_sync(0xffffffffu, child, rest ? __ffs(rest) - 1 : 0);
+    const unsigned gmask = gs == 32 ? 0xffffffffu : ((1u << gs) - 1u) << (mine * gs);
+    bool done = rest == 0u;
+    for (int a0 = 0; a0 < attempts && __any_sync(0xffffffffu, !done); a0 += gs) {
+      const int a = a0 + lane % gs;
+      float Jc = -INFINITY;
+      uint64_t cand[NG] = {};
+      if (!done && a < attempts) {  // the fitness' sums, with the draws kept in registers
+        float Js = 0.f, Vs = 0.f;
+#pragma unroll
+        for (int i = 0; i < 8 * NG; ++i)
+          if (i < N) {
+            const int o = ga_unif(ga_rng(sd, G, (uint32_t)who, kGaRepair, (uint32_t)(a * N + i)), (uint32_t)P.K[i]);
+            cand[i >> 3] |= (uint64_t)o << (8 * (i & 7));
+            const float2 e = tab[P.off[i] + o];
+            Js += e.x;
+            Vs += e.y;
+          }
+        Jc = (Vs <= P.vram_cap && Js > -INFINITY) ? Js : -INFINITY;
+      }
+      const unsigned ok = __ballot_sync(0xffffffffu, Jc != -INFINITY) & gmask;
+      if (!done && ok) {
+        if (lane == __ffs(ok) - 1) {
+          for (int i = 0; i < N; ++i) genes[(size_t)who * N + i] = (uint8_t)(cand[i >> 3] >> (8 * (i & 7)));
+          fit[who] = Jc;
+        }
+        done = true;
+      }
+    }
+    __syncwarp();
   };
-  bool bad = false;
+  // the fittest of the warp's individuals joins the population's (gl: one lane of a group)
+  auto rank_in = [&](int child, const float* fit, unsigned long long* best) {
+    unsigned long long r = gl == 0 && child < pop ? fc_rank(fit[child], child) : 0ull;
+    r = max(r, __shfl_xor_sync(0xffffffffu, r, 8));
+    r = max(r, __shfl_xor_sync(0xffffffffu, r, 16));
+    if (lane == 0 && r) atomicMax(best, r);
+  };
   for (int c0 = 0; c0 < pop; c0 += kGroups) {  // initial population: uniform over Lambda, repaired
     const int child = c0 + group;
     int gene[NG];
 #pragma unroll
     for (int q = 0; q < NG; ++q)
       gene[q] = ga_unif(ga_rng(sd, 0, (uint32_t)child, kGaInit, (uint32_t)(gl + 8 * q)), (uint32_t)K[q]);
-    bad = !place(child, gene, g0, fit0) || bad;
+    const float J = place(child, gene, g0, fit0);
+    repair(0u, repairable && child < pop && J == -INFINITY, child, g0, fit0);
+    rank_in(child, fit0, &s_best[0]);
   }
-  settle(0u, 0, g0, fit0, bad);
+  __syncthreads();
   uint8_t* gc = g0;
   uint8_t* gn = g1;
   float* fc_ = fit0;
   float* fn = fit1;
-  // fittest individual of the current population (lowest slot among equals), on every lane
-  auto warp_fittest = [&]() {
-    unsigned long long best = 0ull;
-    for (int e = lane; e < pop; e += 32) best = max(best, fc_rank(fc_[e], e));
-#pragma unroll
-    for (int w = 16; w > 0; w >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, w));
-    return fc_slot(best);
-  };
   for (int gen = 0; gen + 1 < A.gens; ++gen) {
     const uint32_t G = (uint32_t)gen + 1u;
-    bad = false;
+    // (three words in turn: the one for the generation after this is cleared now, which no
+    // warp reads or writes before the barrier)
+    if (c == 0) s_best[(gen + 2) % 3] = 0ull;
     for (int c0 = 0; c0 < pop; c0 += kGroups) {
       const int child = c0 + group;
       const uint32_t cu = (uint32_t)child;
@@ -1009,12 +1073,8 @@ k_fc_ga(const Params P, const FcGaArgs A) {
         win[1] = max(win[1], __shfl_xor_sync(0xffffffffu, win[1], w));
       }
       int parent[2] = {fc_slot(win[0]), fc_slot(win[1])};
-      bool elite = false;
-      if (A.elitism && c0 == 0 && warp == 0) {  // slot 0 keeps the fittest
-        const int e = warp_fittest();
-        elite = child == 0;
-        if (elite) parent[0] = parent[1] = e;
-      }
+      const bool elite = A.elitism && child == 0;  // slot 0 keeps the fittest (lowest slot among equals)
+      if (elite) parent[0] = parent[1] = fc_slot(s_best[gen % 3]);
       int gene[NG];
 #pragma unroll
       for (int q = 0; q < NG; ++q) {
@@ -1022,14 +1082,16 @@ k_fc_ga(const Params P, const FcGaArgs A) {
         gene[q] = i < N ? gc[(size_t)(take_b[q] ? parent[1] : parent[0]) * N + i] : 0;
         if (mutate[q] && !elite && i < N) gene[q] = mval[q];
       }
-      bad = !place(child, gene, gn, fn) || bad;
+      const float J = place(child, gene, gn, fn);
+      repair(G, repairable && child < pop && !elite && J == -INFINITY, child, gn, fn);
+      rank_in(child, fn, &s_best[(gen + 1) % 3]);
     }
-    settle(G, A.elitism ? 1 : 0, gn, fn, bad);
+    __syncthreads();
     uint8_t* tg = gc; gc = gn; gn = tg;
     float* tf = fc_; fc_ = fn; fn = tf;
   }
-  if (warp == 0) {
-    const int e = warp_fittest();
+  {
+    const int e = fc_slot(s_best[(A.gens - 1) % 3]);
     if (c < N) A.out_genome[c] = gc[(size_t)e * N + c];
     if (c == 0) *A.out_fit = fc_[e];
   }
@@ -1207,9 +1269,9 @@ mf_status mf_vram_feasible(mf_ctx* ctx, uint64_t lo, uint64_t hi, uint64_t* d_ou
   A.cap = cap;
   A.total = (unsigned long long*)ctx->h_stage;
   const size_t smem = sizeof(float) * (size_t)ctx->sumK;
-  k_vram<false><<<grid, kVramThreads, smem, s>>>(ctx->P, A);
+  (N <= 8 ? k_vram_count<8> : k_vram_count<MF_MAX_MODELS>)<<<grid, kVramThreads, smem, s>>>(ctx->P, A);
   MF_CUDA(cudaGetLastError());
-  k_vram<true><<<grid, kVramThreads, smem, s>>>(ctx->P, A);
+  (N <= 8 ? k_vram_write<8> : k_vram_write<MF_MAX_MODELS>)<<<grid, kVramThreads, smem, s>>>(ctx->P, A);
   MF_CUDA(cudaGetLastError());
   MF_CUDA(cudaStreamSynchronize(s));
   *count = *A.total;

