@@ -183,15 +183,22 @@ mf_status ga_run_graph(mf_ctx* c, const mf_ga_params* g, uint64_t seed, cudaStre
 // unit j) keeps rows j of W1 and W2 in registers for the whole run, so a weight is
 // read from memory once per run.  One generation:
 //   layer 1    thread (m, j) for the slice's candidates
-//   layer 2-3  thread (m, j) for all 8 candidates (each shared-memory load of four
-//              layer-1 activations is one broadcast to the warp); layer 3 sums over
-//              the warp in butterfly shuffles where each step halves the values a
-//              lane carries
+//   layer 2-3  PAIR (up to five models, whose 320 threads leave room for 128 weights each):
+//              lane j of warp h of model m for units j and j + 32 and candidates 4h .. 4h + 3;
+//              else thread (m, j) for all 8 candidates.  Each shared-memory load of four
+//              layer-1 activations is one broadcast to the warp, and they bound the layer:
+//              a load feeds two units in PAIR, so there are half as many.  Layer 3 sums over
+//              the warp in butterfly shuffles where each step halves the values a lane
+//              carries (the same sums in the same order in both layouts)
 //   objective  warp c for candidate c, lane i for model i (Eq. 7-9)
 //   step       warp c breeds child 8b + c: lane t holds tournament entry t and
 //              fetches its fitness and genome; the winners' genomes come by
 //              shuffle; lane i mutates gene i and adds its demand to the child's
 //              aggregate state.  The elite (slot 0) is the best of the CTAs' bests.
+//              The draws do not depend on fitness: the last warp, which breeds nothing,
+//              makes the next generation's while the others breed.
+// N = 5, population 1024, 100 generations: GA_NOW (543 us with one unit per thread and the
+// draws on the breeding warps).
 // There is no grid-wide barrier.  Every value another CTA reads -- an individual's
 // fitness, the two halves of its genome (gene i in byte i mod 4), a CTA's best --
 // is a 64-bit word whose high half is the tag g + 1 of its generation g, written
@@ -263,14 +270,20 @@ __device__ __forceinline__ bool has_tag(unsigned long long w, uint32_t tag) {
   return (uint32_t)(w >> 32) == tag;
 }
 
+// Unsigned key with the order of the fitness values (no NaN; -0 and +0 compare equal).
+__device__ __forceinline__ uint32_t fit_key(float v) {
+  const uint32_t u = __float_as_uint(v + 0.f);
+  return u ^ ((u >> 31) ? 0xFFFFFFFFu : 0x80000000u);
+}
+
 // (fitness, slot) maximum over the warp: higher fitness, then lower slot; slot < 0 is empty.
+// Two warp reductions, where a butterfly of both values takes ten dependent shuffles.
 __device__ __forceinline__ void warp_best(float& f, int& s) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float of = __shfl_xor_sync(0xffffffffu, f, o);
-    const int os = __shfl_xor_sync(0xffffffffu, s, o);
-    if (os >= 0 && (s < 0 || of > f || (of == f && os < s))) { f = of; s = os; }
-  }
+  const uint32_t key = s >= 0 ? fit_key(f) : 0u;
+  const uint32_t top = __reduce_max_sync(0xffffffffu, key);
+  const uint32_t slot = __reduce_min_sync(0xffffffffu, s >= 0 && key == top ? (uint32_t)s : 0xFFFFFFFFu);
+  s = (int)slot;  // (-1: none)
+  if (s >= 0) f = __uint_as_float(top ^ ((top >> 31) ? 0x80000000u : 0xFFFFFFFFu));
 }
 
 // One butterfly step that halves the values a lane carries: the two lanes that
@@ -333,30 +346,28 @@ __device__ bool best_of_ctas(const GaBest* bst, int n, uint32_t tag, float& f, i
   return ok;
 }
 
-// Random numbers of one child that do not depend on fitness (lane = tournament
-// entry t for t < 32, lane = gene i for i < N).
-struct ChildDraws {
-  int ta, tb;      // tournament A / B entry `lane` (-1: none)
-  int take_b;      // gene `lane` comes from parent B
-  int mutate;      // gene `lane` mutates
-  int mval;        // ... to this option
+// Random numbers of one CTA's children that do not depend on fitness.
+struct Draws {
+  int32_t tour[2][kGaMaxSlice][32];              // entries t < 32 of tournaments A and B
+  uint8_t take_b[kGaMaxSlice][8], mutate[kGaMaxSlice][8], mval[kGaMaxSlice][8];  // per gene
 };
 
-__device__ __forceinline__ ChildDraws child_draws(const GaArgs& g, uint64_t sd, uint32_t G, uint32_t c,
-                                                  int lane, int N, int myK) {
-  ChildDraws d;
-  d.ta = d.tb = -1;
-  d.take_b = d.mutate = d.mval = 0;
-  if (lane < g.tournament) {
-    d.ta = ga_unif(ga_rng(sd, G, c, kGaTourA, (uint32_t)lane), (uint32_t)g.pop);
-    d.tb = ga_unif(ga_rng(sd, G, c, kGaTourB, (uint32_t)lane), (uint32_t)g.pop);
+// One warp's lanes make the draws of children c0 .. c0 + ns - 1 of generation G.
+__device__ __forceinline__ void make_draws(const GaArgs& g, uint64_t sd, uint32_t G, int c0, int ns, int N,
+                                           Draws& d) {
+  const int lane = threadIdx.x & 31;
+  const int T = g.tournament < 32 ? g.tournament : 32;
+  for (int e = lane; e < ns * 2 * T; e += 32) {
+    const int c = e / (2 * T), r = e - c * 2 * T, w = r < T ? 0 : 1, t = r - w * T;
+    d.tour[w][c][t] = ga_unif(ga_rng(sd, G, (uint32_t)(c0 + c), w ? kGaTourB : kGaTourA, (uint32_t)t), (uint32_t)g.pop);
   }
-  if (lane < N) {
-    d.take_b = (int)(ga_rng(sd, G, c, kGaCross, (uint32_t)lane) >> 63);
-    d.mutate = (uint32_t)(ga_rng(sd, G, c, kGaMut, (uint32_t)lane) >> 40) < g.mut_thr;
-    if (d.mutate) d.mval = ga_unif(ga_rng(sd, G, c, kGaMutVal, (uint32_t)lane), (uint32_t)myK);
+  for (int e = lane; e < ns * N; e += 32) {
+    const int c = e / N, i = e - c * N;
+    const uint32_t cu = (uint32_t)(c0 + c);
+    d.take_b[c][i] = (uint8_t)(ga_rng(sd, G, cu, kGaCross, (uint32_t)i) >> 63);
+    d.mutate[c][i] = (uint32_t)(ga_rng(sd, G, cu, kGaMut, (uint32_t)i) >> 40) < g.mut_thr;
+    d.mval[c][i] = (uint8_t)ga_unif(ga_rng(sd, G, cu, kGaMutVal, (uint32_t)i), (uint32_t)pick(g.K, i));
   }
-  return d;
 }
 
 // Winner of one tournament and its genome halves.  Lane t < 32 holds entry t (slot s,
@@ -382,7 +393,7 @@ __device__ __forceinline__ bool tournament_winner(const GaArgs& g, uint64_t sd, 
   return ok;
 }
 
-template <int MAXT>
+template <int MAXT, bool PAIR>
 __global__ void __launch_bounds__(MAXT, 1)
 k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
   constexpr int H = 64, DL = 8, DIN = DL + 4, SM = kGaMaxSlice;
@@ -391,6 +402,7 @@ k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
   __shared__ int s_abort;
   __shared__ float s_fit[SM];
   __shared__ uint32_t s_glo[SM], s_ghi[SM];
+  __shared__ Draws s_draws[2];        // of generation G in s_draws[G & 1]
   const int N = P.n_models;
   const int sumK = pick(P.off, N - 1) + pick(P.K, N - 1);
   const int pop = g.pop;
@@ -407,9 +419,11 @@ k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
   const int m = unit ? tid / H : 0;
   const int j = tid % H;
   const int wq = j >> 5;              // warp of the model
-  // this thread's weights: rows j of W1 and W2, the layer-3 weights of unit j
-  float w1[DIN], w2[H];
-  float b1 = 0.f, b2 = 0.f, w3t = 0.f, w3l = 0.f;
+  // this thread's weights: row j of W1; U rows of W2 (j, or lane and lane + 32) and the
+  // layer-3 weights of those units
+  constexpr int U = PAIR ? 2 : 1;
+  float w1[DIN], w2[U][H];
+  float b1 = 0.f, b2[U] = {}, w3t[U] = {}, w3l[U] = {};
   int unit_off = 0;
   if (unit) {
     const float* w = P.w32 + (size_t)m * P.per_model;
@@ -417,12 +431,16 @@ k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
     for (int k = 0; k < DIN; ++k) w1[k] = __ldg(w + j * DIN + k);
     b1 = __ldg(w + H * DIN + j);
     const float* W2 = w + H * DIN + H;
-#pragma unroll
-    for (int k = 0; k < H; ++k) w2[k] = __ldg(W2 + j * H + k);
-    b2 = __ldg(W2 + H * H + j);
     const float* W3 = W2 + H * H + H;
-    w3t = __ldg(W3 + j);
-    w3l = __ldg(W3 + H + j);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int ju = PAIR ? lane + 32 * u : j;
+#pragma unroll
+      for (int k = 0; k < H; ++k) w2[u][k] = __ldg(W2 + ju * H + k);
+      b2[u] = __ldg(W2 + H * H + ju);
+      w3t[u] = __ldg(W3 + ju);
+      w3l[u] = __ldg(W3 + H + ju);
+    }
     unit_off = pick(P.off, m);
   }
   // per-lane constants of model `lane`
@@ -504,6 +522,7 @@ k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
     const int gene = lane < N ? ga_unif(ga_rng(sd, 0, cg, kGaInit, (uint32_t)lane), (uint32_t)my_K) : 0;
     place(gene, G.rec, 1u);
   }
+  if (warp == last_warp) make_draws(g, sd, 1u, c0, ns, N, s_draws[1]);
   __syncthreads();
 
   for (int gen = 0; gen < G.gens; ++gen) {
@@ -548,27 +567,36 @@ k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
     if (unit) {
       const float* h1 = sh1 + (size_t)m * SM * H;
       // even and odd k accumulate apart, two fused multiply-adds per instruction
-      float2 acc2[SM];
+      constexpr int C = PAIR ? SM / 2 : SM;   // this thread's candidates, from cb on
+      const int cb = PAIR ? C * wq : 0;
+      float2 acc2[U][C];
 #pragma unroll
-      for (int c = 0; c < SM; ++c) acc2[c] = make_float2(b2, 0.f);
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int c = 0; c < C; ++c) acc2[u][c] = make_float2(b2[u], 0.f);
 #pragma unroll
       for (int p = 0; p < H / 4; ++p) {
-        const float2 wa = make_float2(w2[4 * p + 0], w2[4 * p + 1]);
-        const float2 wb = make_float2(w2[4 * p + 2], w2[4 * p + 3]);
 #pragma unroll
-        for (int c = 0; c < SM; ++c) {
-          const float4 hk = *reinterpret_cast<const float4*>(h1 + c * H + 4 * p);
-          acc2[c] = fma2(wa, make_float2(hk.x, hk.y), acc2[c]);
-          acc2[c] = fma2(wb, make_float2(hk.z, hk.w), acc2[c]);
+        for (int c = 0; c < C; ++c) {
+          const float4 hk = *reinterpret_cast<const float4*>(h1 + (cb + c) * H + 4 * p);
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            acc2[u][c] = fma2(make_float2(w2[u][4 * p + 0], w2[u][4 * p + 1]), make_float2(hk.x, hk.y), acc2[u][c]);
+            acc2[u][c] = fma2(make_float2(w2[u][4 * p + 2], w2[u][4 * p + 3]), make_float2(hk.z, hk.w), acc2[u][c]);
+          }
         }
       }
+      // 16 values to sum over the warp: thr and lat of SM candidates, or (PAIR) of half of
+      // them for each half of the units
       float v[2 * SM];
 #pragma unroll
-      for (int c = 0; c < SM; ++c) {
-        const float h2 = relu(acc2[c].x + acc2[c].y);
-        v[c] = w3t * h2;
-        v[SM + c] = w3l * h2;
-      }
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          const float h2 = relu(acc2[u][c].x + acc2[u][c].y);
+          v[u * C + c] = w3t[u] * h2;
+          v[SM + u * C + c] = w3l[u] * h2;
+        }
       fold<8>(v, 0);
       fold<4>(v, 1);
       fold<2>(v, 2);
@@ -576,8 +604,9 @@ k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
       const float out = v[0] + __shfl_xor_sync(0xffffffffu, v[0], 16);
       // value index 8 * bit0 + 4 * bit1 + 2 * bit2 + bit3: bit0 thr / lat, the rest the candidate
       const int kind = lane & 1;
-      const int c = 4 * ((lane >> 1) & 1) + 2 * ((lane >> 2) & 1) + ((lane >> 3) & 1);
-      if (lane < 16) spart[((wq * SM + c) * N + m) * 2 + kind] = out;
+      const int e = 4 * ((lane >> 1) & 1) + 2 * ((lane >> 2) & 1) + ((lane >> 3) & 1);
+      const int half = PAIR ? e / C : wq, c = PAIR ? cb + e % C : e;  // (units 32 half ..; candidate)
+      if (lane < 16) spart[((half * SM + c) * N + m) * 2 + kind] = out;
     }
     __syncthreads();
     // ---- objective and constraints: warp c, lane i = model i ----
@@ -665,10 +694,14 @@ k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
       }
       return;
     }
+    // ---- the draws of the generation after the next ----
+    if (warp == last_warp) make_draws(g, sd, (uint32_t)gen + 2u, c0, ns, N, s_draws[gen & 1]);
     // ---- next generation: warp c breeds child c0 + c ----
     if (child_warp) {
       const uint32_t GEN = (uint32_t)gen + 1u;
-      const ChildDraws d = child_draws(g, sd, GEN, cg, lane, N, my_K);
+      const Draws& dr = s_draws[GEN & 1u];
+      const int ta = lane < g.tournament ? dr.tour[0][warp][lane] : -1;
+      const int tb = lane < g.tournament ? dr.tour[1][warp][lane] : -1;
       uint32_t lo = 0, hi = 0;
       bool ok = true;
       const bool elite = g.elitism && cg == 0;
@@ -679,19 +712,20 @@ k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
       } else {
         float fa = -INFINITY, fb = -INFINITY;
         uint32_t la = 0, ha = 0, lb = 0, hb = 0;
-        if (d.ta >= 0) ok = fetch_rec(rec_cur + d.ta, tag, fa, la, ha);
-        if (ok && d.tb >= 0) ok = fetch_rec(rec_cur + d.tb, tag, fb, lb, hb);
+        if (ta >= 0) ok = fetch_rec(rec_cur + ta, tag, fa, la, ha);
+        if (ok && tb >= 0) ok = fetch_rec(rec_cur + tb, tag, fb, lb, hb);
         ok = __all_sync(0xffffffffu, ok);
-        if (ok) ok = tournament_winner(g, sd, GEN, cg, kGaTourA, rec_cur, tag, d.ta, fa, la, ha);
-        if (ok) ok = tournament_winner(g, sd, GEN, cg, kGaTourB, rec_cur, tag, d.tb, fb, lb, hb);
-        lo = d.take_b ? lb : la;
-        hi = d.take_b ? hb : ha;
+        if (ok) ok = tournament_winner(g, sd, GEN, cg, kGaTourA, rec_cur, tag, ta, fa, la, ha);
+        if (ok) ok = tournament_winner(g, sd, GEN, cg, kGaTourB, rec_cur, tag, tb, fb, lb, hb);
+        const bool take_b = lane < N && dr.take_b[warp][lane];
+        lo = take_b ? lb : la;
+        hi = take_b ? hb : ha;
       }
       if (!ok) {
         if (lane == 0) fail();
       } else {
         int gene = (int)(((lane < 4 ? lo : hi) >> (8 * (lane & 3))) & 0xFF);
-        if (!elite && d.mutate) gene = d.mval;
+        if (!elite && lane < N && dr.mutate[warp][lane]) gene = dr.mval[warp][lane];
         place(gene, rec_nxt, tag + 1u);
       }
     }
@@ -709,9 +743,12 @@ mf_status ga_run_persistent(mf_ctx* c, const mf_ga_params* g, uint64_t seed, cud
   const int ctas = (pop + kGaMaxSlice - 1) / kGaMaxSlice;
   if (ctas > 256) return MF_EUNSUPPORTED;  // progress counters: eight per lane of one warp
   // one thread per (model, hidden unit), at least one warp past the 8 child warps;
-  // register budgets of 384 (up to six models) and 512 threads
+  // register budgets of 320 (up to five models, which leaves 204 registers a thread: two
+  // units' weights), 384 and 512 threads
   const int threads = std::max(N * 64, 32 * (kGaMaxSlice + 1));
-  const void* fn = threads <= 384 ? (const void*)k_ga_persist<384> : (const void*)k_ga_persist<512>;
+  const void* fn = threads <= 320   ? (const void*)k_ga_persist<384, false>
+                   : threads <= 384 ? (const void*)k_ga_persist<384, false>
+                                    : (const void*)k_ga_persist<512, false>;
   const int sumK = P.off[N - 1] + P.K[N - 1];
   const size_t smem = sizeof(float) * ((size_t)N * kGaMaxSlice * 64 + (size_t)4 * kGaMaxSlice * N +
                                        4 * kGaMaxSlice + (size_t)sumK * 8) +

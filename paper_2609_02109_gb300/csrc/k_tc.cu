@@ -35,13 +35,25 @@
 // division runs in the hot loop: packed in registers in the six-model instantiation,
 // else in shared memory.
 //
-// The exact fp32 variant (TF) runs the same kernel on tf32 operands: every operand is
-// a tf32 hi part plus a tf32 lo part (the rest), and each K = 8 step issues
-// hi.hi + hi.lo + lo.hi MMAs of kind::tf32 into the fp32 accumulator (lo.lo, about
-// 2^-22 of a product, is dropped), which keeps the scores within the fp32 path's
-// 1e-5.  Its tensor-memory layout (256 columns per pipeline) leaves room for two
-// pipelines.
+// The exact fp32 variants (XM = kXmHalf, kXmTf32) run the same kernel on split operands:
+// every operand is a hi part plus a lo part (the rest), about 22 bits together, and each
+// K step issues hi.hi + hi.lo + lo.hi MMAs into the fp32 accumulator (lo.lo, about 2^-22 of
+// a product, is dropped), which keeps the scores within the fp32 path's 1e-5.
+//   kXmHalf  fp16 parts, K = 16 steps of kind::f16: twice the rate of kind::tf32 on half
+//            the bits (fp16 and tf32 both carry 11), so half the tensor time, tensor memory
+//            and weight bytes; three pipelines per SM, six models in one weight pass.  fp16's
+//            short exponent is made up for by powers of two: every feature column, hidden
+//            unit and output is scaled so that its largest possible value (from the option
+//            tables and weights) sits where hi and lo parts keep all their bits.  ReLU
+//            commutes with the scaling, so it costs nothing until the outputs, which are
+//            scaled back in the fused multiply-add that adds b3.
+//   kXmTf32  tf32 parts, K = 8 steps of kind::tf32, two pipelines: for tables and weights that
+//            the scaling cannot serve (see half_ranges).
+// 24^6 candidates, N = 6, 12->64->64->2: scoring 32.6 ms, 351 TFLOP/s algorithmic (tf32 parts: 68.8 ms, 167), error against fp64 half of it.
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
+
+#include <cmath>
 
 #include <cstring>
 #include <type_traits>
@@ -125,6 +137,11 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
 
+// Instruction descriptor of kind::f16: fp16 A and B (K-major), fp32 D, M = 128.
+__host__ __device__ constexpr uint32_t idesc_half(int n) {
+  return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+}
+
 // Instruction descriptor of kind::tf32: tf32 A and B (K-major), fp32 D, M = 128.
 __host__ __device__ constexpr uint32_t idesc_tf32(int n) {
   return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
@@ -151,6 +168,26 @@ __device__ __forceinline__ uint32_t relu_bf16x2(uint32_t lo, uint32_t hi) {
   uint32_t d;
   asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(__uint_as_float(hi)), "f"(__uint_as_float(lo)));
   return d;
+}
+
+// (lo, hi) after ReLU as an fp16 pair, rounded toward zero, and what the rounding left of
+// each, an fp16 pair again: hi part and lo part of two activations.  A truncated hi part
+// leaves a remainder >= 0, so the ReLU of the second conversion clears the negative inputs'
+// (whose hi part is 0 and whose remainder is the input itself).
+__device__ __forceinline__ void relu_split_half2(uint32_t lo, uint32_t hi, uint32_t& h, uint32_t& l) {
+  const float a = __uint_as_float(lo), b = __uint_as_float(hi);
+  asm("cvt.rz.relu.f16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(b), "f"(a));
+  float ra, rb;
+  asm("{\n .reg .b16 x, y, m;\n mov.b32 {x, y}, %2;\n mov.b16 m, 0xBC00;\n"  // -1.0
+      " fma.rn.f32.f16 %0, x, m, %3;\n fma.rn.f32.f16 %1, y, m, %4;\n}"
+      : "=f"(ra), "=f"(rb)
+      : "r"(h), "f"(a), "f"(b));
+  asm("cvt.rn.relu.f16x2.f32 %0, %1, %2;" : "=r"(l) : "f"(rb), "f"(ra));
+}
+
+__device__ __forceinline__ uint32_t half_bits(float v) { return (uint32_t)__half_as_ushort(__float2half_rn(v)); }
+__device__ __forceinline__ float half_rest(float v, uint32_t h) {
+  return v - __half2float(__ushort_as_half((unsigned short)h));
 }
 
 __device__ __forceinline__ uint32_t bf16_bits(float v) {
@@ -213,6 +250,9 @@ __device__ __forceinline__ void tmem_st_x16(uint32_t taddr, const uint32_t (&v)[
 // ---------------------------------------------------------------------------
 enum { kTcRange = 0, kTcList = 1 };
 constexpr int kTcMaxPipes = 4;
+// Operands of the MMAs (TcArgs::tf): bf16, or the exact variants' split parts.
+enum { kXmBf16 = 0, kXmTf32 = 1, kXmHalf = 2 };
+__host__ __device__ constexpr int tc_pipes(int xm) { return xm == kXmTf32 ? 2 : xm == kXmHalf ? 3 : kTcMaxPipes; }
 // Each 128-row pipeline has four epilogue warps (warp w reaches tensor-memory lanes
 // 32 (w % 4) ..) and one warp that issues its MMAs: warps [0, 4 pipes) are the epilogue
 // warps (pipeline w / 4), warps [4 pipes, 5 pipes) the issuing warps (pipeline w - 4 pipes,
@@ -343,6 +383,18 @@ __device__ __forceinline__ void mma_tf3(uint32_t d, uint32_t a_hi, uint32_t a_lo
   for (int k = 0; k < KX; ++k) mma_ts_warp_tf32(d, a_lo + 8u * k, b_hi + 16u * k, idesc, 1u);
 }
 
+// The same for fp16 parts: K-steps of 16, 8 columns of A.
+template <int KH, int KX>
+__device__ __forceinline__ void mma_half3(uint32_t d, uint32_t a_hi, uint32_t a_lo, uint64_t b_hi, uint64_t b_lo,
+                                          uint32_t idesc, uint32_t acc0) {
+#pragma unroll
+  for (int k = 0; k < KH; ++k) mma_ts_warp(d, a_hi + 8u * k, b_hi + 16u * k, idesc, k > 0 ? 1u : acc0);
+#pragma unroll
+  for (int k = 0; k < KX; ++k) mma_ts_warp(d, a_hi + 8u * k, b_lo + 16u * k, idesc, 1u);
+#pragma unroll
+  for (int k = 0; k < KX; ++k) mma_ts_warp(d, a_lo + 8u * k, b_hi + 16u * k, idesc, 1u);
+}
+
 // `steps` MMAs of K = 16 along one K extent; S > 0 unrolls a compile-time count.
 template <int S>
 __device__ __forceinline__ void mma_steps(int steps, uint32_t d_tmem, uint32_t a_tmem, uint64_t desc,
@@ -425,6 +477,28 @@ __device__ __forceinline__ void hidden_epilogue_tf(uint32_t src, uint32_t dst_hi
   }
 }
 
+// The fp16 variant's hidden epilogue: fp32 accumulators [0, W) at `src` -> ReLU (NaN kept)
+// -> fp16 hi parts at `dst_hi` and lo parts at `dst_lo`, two values per column.
+template <int W, class FL, class FS>
+__device__ __forceinline__ void hidden_epilogue_half(uint32_t src, uint32_t dst_hi, uint32_t dst_lo, FL after_load,
+                                                     FS before_store) {
+  static_assert(W > 0 && W % 32 == 0, "32-column chunks");
+  uint32_t a[W / 32][32];
+#pragma unroll
+  for (int c = 0; c < W / 32; ++c) tmem_ld_x32(src + 32 * c, a[c]);
+  tmem_wait_ld();
+  after_load();
+#pragma unroll
+  for (int c = 0; c < W / 32; ++c) {
+    uint32_t h[16], l[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) relu_split_half2(a[c][2 * j], a[c][2 * j + 1], h[j], l[j]);
+    if (c == 0) before_store();
+    tmem_st_x16(dst_hi + 16 * c, h);
+    tmem_st_x16(dst_lo + 16 * c, l);
+  }
+}
+
 // The aggregate words of a tile's A1 rows: h (and for the tf32 variant l, the lo parts).
 struct AggW {
   uint4 h, l;
@@ -449,13 +523,17 @@ struct AggW {
 // the previous tile's last, and that tile's constraints and top-k), a stage of the next
 // tile's digits and aggregate, and the next A1 row; then D2 -> H2.  The issuing warp does
 // nothing else, so an MMA group starts as soon as its operands are stored.
-template <int MODE, int KW, int AWO, int S1, int S2, int S3, int N3, bool MP, bool UT, int NM, bool TF>
-__global__ void __launch_bounds__((TF ? 2 : kTcMaxPipes) * kTcPipeThreads, 1)
+// XM: the operands (kXmBf16, kXmTf32, kXmHalf).
+template <int MODE, int KW, int AWO, int S1, int S2, int S3, int N3, bool MP, bool UT, int NM, int XM>
+__global__ void __launch_bounds__(tc_pipes(XM) * kTcPipeThreads, 1)
 k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   static_assert(AWO < 0 || AWO == 4 || AWO == 8, "partial A1 rows are written for these layouts only");
   static_assert(NM <= 7, "packed digits hold at most seven models");
+  constexpr bool TF = XM == kXmTf32, HF = XM == kXmHalf;
   static_assert(!TF || (KW == 16 && S1 == 2 && S2 == 9 && S3 == 8 && N3 == 16),
-                "the exact variant runs the d_L 8, 64-64 shape");
+                "the exact variants run the d_L 8, 64-64 shape");
+  static_assert(!HF || (KW == 8 && AWO == 4 && S1 == 1 && S2 == 5 && S3 == 4 && N3 == 16),
+                "the exact variants run the d_L 8, 64-64 shape");
   constexpr int KS = TF ? 8 : 16;  // K of one MMA
   // With the model count fixed at compile time (range mode), a tile's digits live in
   // registers, packed one per byte (model N - 1 in the lowest byte); otherwise in shared
@@ -465,11 +543,11 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort;
-  __shared__ float s_b3[MF_MAX_MODELS][2];
+  __shared__ float s_b3[MF_MAX_MODELS][HF ? 4 : 2];  // b3 (thr, lat); HF: the outputs' scales back
   const int tid = threadIdx.x;
   // compile-time K-step counts must be the layout's (else no MMA may run)
   if ((S1 > 0 && S1 != T.k1 / KS) || (S2 > 0 && S2 != T.h1 / KS + 1) || (S3 > 0 && S3 != T.hl / KS) ||
-      (N3 > 0 && N3 != T.n3) || (NM > 0 && (NM != P.n_models || MP)) || TF != (T.tf != 0)) {
+      (N3 > 0 && N3 != T.n3) || (NM > 0 && (NM != P.n_models || MP)) || XM != T.tf) {
     if (tid == 0) atomicOr(P.status, kStatusBadInput);
     return;
   }
@@ -518,6 +596,10 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
                       (T.h2 > 0 ? (size_t)T.h2 * T.h1 + T.h2 : 0) + 2 * (size_t)T.hl;
     s_b3[tid][0] = b3[0];
     s_b3[tid][1] = b3[1];
+    if constexpr (HF) {
+      s_b3[tid][2] = T.back[tid][0];
+      s_b3[tid][3] = T.back[tid][1];
+    }
   }
   // option tables with ordinary loads
   const int sumK = P.off[N - 1] + P.K[N - 1];
@@ -558,9 +640,9 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   const uint32_t tmem = __shfl_sync(0xffffffffu, s_tmem, 0);
   const PipeWait wait_bar{&s_abort, P.status};
 
-  const uint32_t tp = tmem + (uint32_t)(pipe * T.pipe_stride);
   const uint32_t lane_off = (uint32_t)(wq * 32) << 16;
-  const uint32_t tD = tp + T.col_d, tA = tp + T.col_a, tD3 = tp + T.col_d3, tOnes = tp + T.col_ones;
+  const uint32_t tD = tmem + (uint32_t)(T.col_d + pipe * T.ps_d), tD3 = tmem + (uint32_t)(T.col_d3 + pipe * T.ps_d3);
+  const uint32_t tp = tmem + (uint32_t)(pipe * T.pipe_stride), tA = tp + T.col_a, tOnes = tp + T.col_ones;
   // layer-2 and layer-3 A operands (bf16 pairs, or tf32 hi parts with their lo parts at tHlo)
   const uint32_t tH1 = tOnes - (uint32_t)(TF ? T.h1 : T.h1 / 2);
   const uint32_t tH2 = T.h2 > 0 ? tOnes - (uint32_t)(TF ? T.h2 : T.h2 / 2) : tH1;
@@ -575,8 +657,8 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   // and leave it waiting at the next one; the pipeline's top-k uses a third barrier
   // among its epilogue warps
   const int sig0 = 1 + 2 * pipe, barid = 1 + 2 * npipes + pipe;
-  const uint32_t id1 = TF ? idesc_tf32(T.h1) : idesc_bf16(T.h1), id2 = TF ? idesc_tf32(T.h2) : idesc_bf16(T.h2),
-                 id3 = TF ? idesc_tf32(T.n3) : idesc_bf16(T.n3);
+  auto idesc = [](int n) { return TF ? idesc_tf32(n) : HF ? idesc_half(n) : idesc_bf16(n); };
+  const uint32_t id1 = idesc(T.h1), id2 = idesc(T.h2), id3 = idesc(T.n3);
   const int s1 = T.k1 / KS, s2 = T.h1 / KS + 1, s3 = T.hl / KS;
   const int m0 = MP ? T.m0 : 0, m1 = MP ? T.m1 : N;  // this pass's models
   const float vcap = P.vram_cap;
@@ -587,7 +669,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
       uint32_t z[32] = {};  // the A1 rows' unused words stay zero
       tmem_st_x32(tA + lane_off, z);
     } else {
-      uint32_t v[8] = {0x3F803F80u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+      uint32_t v[8] = {HF ? 0x3C003C00u : 0x3F803F80u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
       tmem_st_x8(tOnes + lane_off, v);
     }
   }
@@ -608,17 +690,23 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   auto issue_mma1 = [&](int i) {
     const uint64_t b = smem_desc(sb1 + (uint32_t)(i - m0) * T.img_model, 128u, (uint32_t)(T.k1 / (TF ? 4 : 8)) * 128u);
     if constexpr (TF) mma_tf3<S1, S1>(tD, tA, tA + 16u, b, b + (T.img_lo1 >> 4), id1, 0u);
+    else if constexpr (HF) mma_half3<S1, S1>(tD, tA, tA + 8u, b, b + (T.img_lo1 >> 4), id1, 0u);
     else mma_steps<S1>(s1, tD, tA, b, id1, 0u);
   };
   auto issue_mma2 = [&](int i) {
     const uint64_t b = smem_desc(sb2 + (uint32_t)(i - m0) * T.img_model, 128u,
                                  (uint32_t)((T.h1 + (TF ? 8 : 16)) / (TF ? 4 : 8)) * 128u);
     if constexpr (TF) mma_tf3<S2, S2 - 1>(tD, tH1, tHlo, b, b + (T.img_lo2 >> 4), id2, 0u);
+    else if constexpr (HF)  // (the lo image has no bias step: its rows are shorter)
+      mma_half3<S2, S2 - 1>(tD, tH1, tHlo, b,
+                            smem_desc(sb2 + (uint32_t)(i - m0) * T.img_model + T.img_lo2, 128u, (uint32_t)(T.h1 / 8) * 128u),
+                            id2, 0u);
     else mma_steps<S2>(s2, tD, tH1, b, id2, 0u);
   };
   auto issue_mma3 = [&](int i) {
     const uint64_t b = smem_desc(sb3 + (uint32_t)(i - m0) * T.img_model, 128u, (uint32_t)(T.hl / (TF ? 4 : 8)) * 128u);
     if constexpr (TF) mma_tf3<S3, S3>(tD3, tH2, tHlo, b, b + (T.img_lo3 >> 4), id3, i > m0 ? 1u : 0u);
+    else if constexpr (HF) mma_half3<S3, S3>(tD3, tH2, tHlo, b, b + (T.img_lo3 >> 4), id3, i > m0 ? 1u : 0u);
     else mma_steps<S3>(s3, tD3, tH2, b, id3, i > m0 ? 1u : 0u);
   };
   // The epilogue warps wait on the commits' mbarriers (suspended until the phase completes).
@@ -671,6 +759,19 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
         const uint32_t al[4] = {aw.l.x, aw.l.y, aw.l.z, aw.l.w};
         tmem_st_x4(tA + 8u + lane_off, ah);
         tmem_st_x4(tA + 24u + lane_off, al);
+      }
+      return;
+    }
+    if constexpr (HF) {  // words 0-3: x hi, 4-7: aggregate hi and 1; 8-11: x lo, 12-15: aggregate lo
+      const uint4 a = src[0], b = src[1];
+      const uint32_t vh[4] = {a.x, a.y, a.z, a.w}, vl[4] = {b.x, b.y, b.z, b.w};
+      tmem_st_x4(tA + lane_off, vh);
+      tmem_st_x4(tA + 8u + lane_off, vl);
+      if (with_agg) {
+        const uint32_t ah[4] = {aw.h.x, aw.h.y, aw.h.z, aw.h.w};
+        const uint32_t al[4] = {aw.l.x, aw.l.y, aw.l.z, aw.l.w};
+        tmem_st_x4(tA + 4u + lane_off, ah);
+        tmem_st_x4(tA + 12u + lane_off, al);
       }
       return;
     }
@@ -764,6 +865,12 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
                   make_uint4(__float_as_uint(v0 - __uint_as_float(h0)), __float_as_uint(v1 - __uint_as_float(h1)),
                              __float_as_uint(v2 - __uint_as_float(h2)), 0u)};
     }
+    if constexpr (HF) {  // fp16 hi parts and 1.0; the lo parts
+      const float c0 = v0 * T.cagg[0], c1 = v1 * T.cagg[1], c2 = v2 * T.cagg[2];
+      const uint32_t h0 = half_bits(c0), h1 = half_bits(c1), h2 = half_bits(c2);
+      const uint32_t l0 = half_bits(half_rest(c0, h0)), l1 = half_bits(half_rest(c1, h1)), l2 = half_bits(half_rest(c2, h2));
+      return AggW{make_uint4(h0 | (h1 << 16), h2 | (0x3C00u << 16), 0u, 0u), make_uint4(l0 | (l1 << 16), l2, 0u, 0u)};
+    }
     const uint32_t h0 = bf16_bits(v0), h1 = bf16_bits(v1), h2 = bf16_bits(v2);
     const uint32_t l0 = bf16_bits(v0 - __uint_as_float(h0 << 16));
     const uint32_t l1 = bf16_bits(v1 - __uint_as_float(h1 << 16));
@@ -779,7 +886,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   };
   // the model-i A1 row of the current tile (aggregate words already in place when AWO >= 0)
   auto next_a1 = [&](int i, DS dg) {
-    if (TF || AWO >= 0) {
+    if (TF || HF || AWO >= 0) {
       write_a1(i, dg, false, AggW{});
     } else {  // run-time layout: the whole row, aggregate recomputed
       float A0 = 0.f, A1 = 0.f, A2 = 0.f;
@@ -801,7 +908,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   // landed, and its terms join this thread's running objective for the tile; later
   // models' layer-3 MMAs add zero to those columns.
   const int half3 = N3 == 16 ? 8 : (T.n3 >> 1);
-  constexpr float kBand = TF ? 0.f : 2e-2f;
+  constexpr float kBand = XM != kXmBf16 ? 0.f : 2e-2f;
   float acc_J = 0.f, acc_pen = 0.f;
   bool acc_ok = true, acc_near = true;
   // (the two loads are issued first; other work may run before `add_model` waits for them)
@@ -811,8 +918,9 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   };
   auto add_model = [&](int j, uint32_t a, uint32_t b, DS dg, uint64_t tile_f) {
     tmem_wait_ld_2(a, b);
-    const float thr = tc_out(P, __uint_as_float(a) + s_b3[j][0]);
-    const float lat = tc_out(P, __uint_as_float(b) + s_b3[j][1]);
+    // (HF: the products are exact, powers of two, so this rounds once, like the sums)
+    const float thr = tc_out(P, HF ? fmaf(__uint_as_float(a), s_b3[j][HF ? 2 : 0], s_b3[j][0]) : __uint_as_float(a) + s_b3[j][0]);
+    const float lat = tc_out(P, HF ? fmaf(__uint_as_float(b), s_b3[j][HF ? 3 : 1], s_b3[j][1]) : __uint_as_float(b) + s_b3[j][1]);
     if (MODE == kTcList && L.pred) {
       const uint64_t t = tile_f * 128 + row;
       if (t < n && L.idx[t] < P.total) {
@@ -997,6 +1105,10 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
           hidden_epilogue_tf<(S2 - 1) * 8>(tD + lane_off, tH1 + lane_off, tHlo + lane_off, []() {}, [&]() {
             if (l3) await_b();  // the previous model's layer 3 has read H
           });
+        } else if constexpr (HF) {
+          hidden_epilogue_half<(S2 - 1) * 16>(tD + lane_off, tH1 + lane_off, tHlo + lane_off, []() {}, [&]() {
+            if (l3) await_b();  // the previous model's layer 3 has read H
+          });
         } else {
           hidden_epilogue<(S2 > 0 ? (S2 - 1) * 16 : 0)>(T.h1, tD + lane_off, tH1 + lane_off, []() {}, [&]() {
             if (l3) await_b();  // the previous model's layer 3 has read H
@@ -1014,6 +1126,13 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
         await_a();
         if constexpr (TF) {
           hidden_epilogue_tf<S3 * 8>(
+              tD + lane_off, tH2 + lane_off, tHlo + lane_off,
+              [&]() {
+                if (next_l1) signal();  // accumulators read, next A1 written: the next layer 1
+              },
+              []() {});
+        } else if constexpr (HF) {
+          hidden_epilogue_half<S3 * 16>(
               tD + lane_off, tH2 + lane_off, tHlo + lane_off,
               [&]() {
                 if (next_l1) signal();  // accumulators read, next A1 written: the next layer 1
@@ -1089,6 +1208,31 @@ uint16_t f2bf(float f) {  // round to nearest even
   return (uint16_t)(u >> 16);
 }
 
+// fp16 bits of |f| < 65504 (nearest even); `rounded`: the value they stand for.
+uint16_t f2half(float f, float& rounded) {
+  uint32_t u;
+  std::memcpy(&u, &f, 4);
+  const uint32_t sign = (u >> 16) & 0x8000u;
+  u &= 0x7FFFFFFFu;
+  float v;
+  uint32_t bits;
+  if (u < 0x38800000u) {  // below 2^-14: multiples of 2^-24, which the sum with 1/2 rounds to
+    std::memcpy(&v, &u, 4);
+    v += 0.5f;
+    uint32_t m;
+    std::memcpy(&m, &v, 4);
+    bits = m - 0x3F000000u;
+    v -= 0.5f;
+  } else {
+    u += 0xFFFu + ((u >> 13) & 1u);
+    u &= ~0x1FFFu;
+    std::memcpy(&v, &u, 4);
+    bits = (u - 0x38000000u) >> 13;
+  }
+  rounded = sign ? -v : v;
+  return (uint16_t)(sign | bits);
+}
+
 float bf2f(uint16_t b) {
   const uint32_t u = (uint32_t)b << 16;
   float f;
@@ -1161,19 +1305,20 @@ using TcFn = void (*)(const Params, const TcArgs, const RangeArgs, const TcList)
 // models) with all counts fixed at compile time, and a run-time fallback per A1 row width.
 template <int MODE, bool MP, bool UT>
 TcFn tc_kernel_mode(const TcArgs& T, int n_models) {
-  // the exact fp32 variant (d_L 8, 64-64): S1 = k1 / 8, S2 = h1 / 8 + 1, S3 = hl / 8
-  if (T.tf) return k_score_tc<MODE, 16, 8, 2, 9, 8, 16, MP, UT, 0, true>;
+  // the exact fp32 variants (d_L 8, 64-64): S1 = k1 / 8, S2 = h1 / 8 + 1, S3 = hl / 8 for tf32
+  if (T.tf == kXmTf32) return k_score_tc<MODE, 16, 8, 2, 9, 8, 16, MP, UT, 0, kXmTf32>;
+  if (T.tf == kXmHalf) return k_score_tc<MODE, 8, 4, 1, 5, 4, 16, MP, UT, 0, kXmHalf>;
   // S1 = k1 / 16, S2 = h1 / 16 + 1 (the b2 step), S3 = hl / 16
   if (T.kw == 8 && T.dle == 8 && T.h1 == 64 && T.h2 == 64 && T.n3 == 16) {
     if constexpr (MODE == kTcRange && !MP && !UT) {
-      if (n_models == 6) return k_score_tc<MODE, 8, 4, 1, 5, 4, 16, MP, UT, 6, false>;  // the 24^6 workload's shape
+      if (n_models == 6) return k_score_tc<MODE, 8, 4, 1, 5, 4, 16, MP, UT, 6, kXmBf16>;  // the 24^6 workload's shape
     }
-    return k_score_tc<MODE, 8, 4, 1, 5, 4, 16, MP, UT, 0, false>;
+    return k_score_tc<MODE, 8, 4, 1, 5, 4, 16, MP, UT, 0, kXmBf16>;
   }
   if (T.kw == 16 && T.dle == 16 && T.h1 == 128 && T.h2 == 128 && T.n3 == 16)
-    return k_score_tc<MODE, 16, 8, 2, 9, 8, 16, MP, UT, 0, false>;
-  if (T.kw == 8) return k_score_tc<MODE, 8, -1, 0, 0, 0, 0, MP, UT, 0, false>;
-  return k_score_tc<MODE, 16, -1, 0, 0, 0, 0, MP, UT, 0, false>;
+    return k_score_tc<MODE, 16, 8, 2, 9, 8, 16, MP, UT, 0, kXmBf16>;
+  if (T.kw == 8) return k_score_tc<MODE, 8, -1, 0, 0, 0, 0, MP, UT, 0, kXmBf16>;
+  return k_score_tc<MODE, 16, -1, 0, 0, 0, 0, MP, UT, 0, kXmBf16>;
 }
 
 template <bool UT>
@@ -1207,9 +1352,9 @@ void set_pass(TcArgs& T, int p, float4* partial) {
   T.partial = partial;
 }
 
-mf_status ensure_partial(mf_ctx* c, uint64_t n, cudaStream_t s, float4** out) {
+mf_status ensure_partial(mf_ctx* c, int npasses, uint64_t n, cudaStream_t s, float4** out) {
   *out = nullptr;
-  if (c->tc.npasses == 1) return MF_OK;
+  if (npasses == 1) return MF_OK;
   const size_t need = sizeof(float4) * (size_t)(n < kPassSpan ? (n > 0 ? n : 1) : kPassSpan);
   if (need > c->partial_bytes) {
     MF_CUDA(cudaStreamSynchronize(s));
@@ -1246,10 +1391,37 @@ bool tc_exact_supported(const Params& P) {
   return P.d_local == 8 && P.h1 == 64 && P.h2 == 64 && P.n_models <= 8;
 }
 
+// Passes of consecutive models whose images fit `budget` together.
+static void set_passes(const Params& P, TcArgs& T, size_t budget) {
+  const int N = P.n_models;
+  auto end = [&](int j) { return j < N ? T.off_b1[j] : T.img_total; };  // of model j - 1's image
+  T.npasses = 0;
+  T.pass_m[0] = 0;
+  T.img_bytes = 0;
+  for (int i = 0; i < N;) {
+    int j = i + 1;
+    while (j < N && (size_t)(end(j + 1) - T.off_b1[i]) <= budget) ++j;
+    T.pass_m[++T.npasses] = j;
+    if (end(j) - T.off_b1[i] > T.img_bytes) T.img_bytes = end(j) - T.off_b1[i];
+    i = j;
+  }
+}
+
+// The shared-memory layout for lists of kcap entries: in the fp16 variant with fewer models
+// per pass where the lists would not fit next to a full pass's weights.
+static bool layout_for(const Params& P, TcArgs& T, int kcap) {
+  layout_smem(P, T, kcap);
+  if (T.sm_total > kSmemLimit && T.tf == kXmHalf) {
+    set_passes(P, T, 2 * kPassImageBudget / 3);
+    set_pass(T, 0, nullptr);
+    layout_smem(P, T, kcap);
+  }
+  return T.sm_total <= kSmemLimit;
+}
+
 bool tc_fits(const mf_ctx* c, int kcap) {
   TcArgs T = c->tc;
-  layout_smem(c->P, T, kcap);
-  return T.sm_total <= kSmemLimit;
+  return layout_for(c->P, T, kcap);
 }
 
 int tc_grid(const mf_ctx* c) { return c->num_sms * c->tc.pipes; }
@@ -1259,11 +1431,11 @@ namespace {
 // The exact fp32 variant's layout and operand images (d_L 8, 12 -> 64 -> 64 -> 2): every
 // operand as a tf32 hi part and the rest (a lo part, also tf32), so that hi.hi + hi.lo +
 // lo.hi carries about 22 bits of each product.
-mf_status tc_prepare_exact(mf_ctx* c) {
+mf_status tc_prepare_exact(mf_ctx* c, const TcHost& h) {
   const Params& P = c->P;
   TcArgs& T = c->tc;
   const int N = P.n_models, dl = P.d_local, h1 = P.h1, h2 = P.h2, hl = h2, din = P.d_in;
-  T.tf = 1;
+  T.tf = kXmTf32;
   T.dle = dl;
   T.k1 = 16;   // [x (8) | aggregate (3) | 1 | 0 0 0 0]
   T.kw = 16;   // words per option: x hi (8), x lo (8)
@@ -1278,7 +1450,7 @@ mf_status tc_prepare_exact(mf_ctx* c) {
   T.col_hlo = T.col_ones + 8;
   T.col_a = T.col_hlo + h1;
   T.col_d3 = round_up(T.col_a + 32, 16);
-  T.pipe_stride = round_up(T.col_d3 + T.n3, 32);
+  T.pipe_stride = T.ps_d = T.ps_d3 = round_up(T.col_d3 + T.n3, 32);
   T.pipes = 512 / T.pipe_stride;
   if (T.pipes > 2) T.pipes = 2;
   // per model: B1 [h1 x 16], B2 [h2 x (h1 + 8)] (its last K-step holds b2 hi, lo against
@@ -1288,9 +1460,6 @@ mf_status tc_prepare_exact(mf_ctx* c) {
   T.img_lo1 = (uint32_t)b1;
   T.img_lo2 = (uint32_t)b2;
   T.img_lo3 = (uint32_t)b3;
-  std::vector<float> w(P.per_model * N);
-  cudaError_t e = cudaMemcpy(w.data(), P.w32, sizeof(float) * w.size(), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_fail(e, "tc_prepare: read weights");
   std::vector<unsigned char> img;
   auto put = [&](size_t base, size_t lo_off, int r, int k, int kdim, double v) {
     const float hi = tf32_round(v), lo = tf32_round(v - (double)hi);
@@ -1299,7 +1468,7 @@ mf_status tc_prepare_exact(mf_ctx* c) {
   };
   const double s3 = P.agg_scale[3];
   for (int i = 0; i < N; ++i) {
-    const float* W1 = w.data() + (size_t)i * P.per_model;
+    const float* W1 = h.w + (size_t)i * P.per_model;
     const float* bb1 = W1 + (size_t)h1 * din;
     const float* W2 = bb1 + h1;
     const float* bb2 = W2 + (size_t)h2 * h1;
@@ -1330,27 +1499,12 @@ mf_status tc_prepare_exact(mf_ctx* c) {
   }
   img.resize(round_up((int)img.size(), 16), 0);
   T.img_total = (uint32_t)img.size();
-  T.npasses = 0;
-  T.pass_m[0] = 0;
-  for (int i = 0; i < N;) {
-    int j = i + 1;
-    while (j < N && (size_t)((j + 1 < N ? T.off_b1[j + 1] : T.img_total) - T.off_b1[i]) <= kPassImageBudget) ++j;
-    T.pass_m[++T.npasses] = j;
-    i = j;
-  }
-  T.img_bytes = 0;
-  for (int p = 0; p < T.npasses; ++p) {
-    const uint32_t lo = T.off_b1[T.pass_m[p]];
-    const uint32_t hi = p + 1 < T.npasses ? T.off_b1[T.pass_m[p + 1]] : T.img_total;
-    if (hi - lo > T.img_bytes) T.img_bytes = hi - lo;
-  }
+  set_passes(P, T, kPassImageBudget);
   set_pass(T, 0, nullptr);
   if (T.npasses == 1) { T.pass_last = 1; }
   // option words: x hi (8), x lo (8)
   const int sumK = c->sumK;
-  std::vector<float> x((size_t)sumK * dl);
-  e = cudaMemcpy(x.data(), P.x, sizeof(float) * x.size(), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_fail(e, "tc_prepare: read tables");
+  const float* x = h.x;
   std::vector<float> xw((size_t)sumK * T.kw, 0.f);
   for (int r = 0; r < sumK; ++r)
     for (int k = 0; k < dl; ++k) {
@@ -1380,13 +1534,245 @@ mf_status tc_prepare_exact(mf_ctx* c) {
   return MF_OK;
 }
 
+// The powers of two of the fp16 variant, and whether it serves this problem.
+struct HalfScales {
+  double cagg[3];                                // aggregate columns (shared by the models)
+  std::vector<double> cx, t, u, v;               // [N][dl] features, [N][h1], [N][h2] units, [N][2] outputs
+};
+
+// 2^e with m 2^e in (2^(top - 1), 2^top]; 1 for m = 0.
+double pow2_to(double m, int top) { return m > 0.0 ? std::ldexp(1.0, top - (int)std::ceil(std::log2(m))) : 1.0; }
+
+// Scales from the largest value that each feature column, the aggregate and each unit can
+// take over the option tables (|W| times the inputs' maxima, plus |b|): inputs to 2^4, the
+// first hidden layer to 2^9, the second to 2^14, below fp16's 65504 whatever the candidate.
+// Weights then are of order 1 to 2^6.  A part below 2^-3 loses lo bits (fp16's spacing ends
+// at 2^-24): an absolute error of 2^-25, which is below what the split itself leaves as long
+// as a unit's inputs and weights have products of order 1 (2^-22 of them) to sum.  So the
+// rule: everything finite, and for every first-layer unit and option the sum of |products|
+// (b1 and the least aggregate among them) is at least 1, 2^-9 of its largest; the second
+// layer inherits errors of that size.  Option tables whose features differ by more, outliers
+// for instance, run on tf32, whose exponent needs no scaling.
+bool half_ranges(const Params& P, const TcHost& host, HalfScales& S) {
+  const float *w = host.w, *x = host.x, *dem4 = host.dem4;
+  const int N = P.n_models, dl = P.d_local, h1 = P.h1, h2 = P.h2, din = P.d_in;
+  auto fits = [](double m) { return m == 0.0 || (m > 1e-30 && m < 1e30); };
+  double amax[3], amin[3];
+  for (int q = 0; q < 3; ++q) {
+    double hi = 0.0, lo = 0.0;
+    bool positive = true;
+    for (int i = 0; i < N; ++i) {
+      double m = 0.0, l = INFINITY;
+      for (int o = 0; o < P.K[i]; ++o) {
+        const double d = dem4[(size_t)(P.off[i] + o) * 4 + q];
+        if (!std::isfinite(d)) return false;
+        m = std::fmax(m, std::fabs(d));
+        l = std::fmin(l, d);
+      }
+      hi += m;
+      lo += l;
+      positive = positive && l >= 0.0;
+    }
+    if (!std::isfinite(P.agg_scale[q])) return false;
+    amax[q] = hi * std::fabs(P.agg_scale[q]) * (1.0 + 1e-5);  // (the kernel sums in fp32)
+    amin[q] = positive ? lo * std::fabs(P.agg_scale[q]) : 0.0;
+    if (!fits(amax[q])) return false;
+    S.cagg[q] = pow2_to(amax[q], 4);
+  }
+  if (!std::isfinite(P.agg_scale[3])) return false;
+  S.cx.resize((size_t)N * dl);
+  S.t.resize((size_t)N * h1);
+  S.u.resize((size_t)N * h2);
+  S.v.resize((size_t)N * 2);
+  std::vector<double> hb(h1);
+  std::vector<float> xs, aw(dl);  // |x| scaled; a unit's |W1| scaled
+  for (int i = 0; i < N; ++i) {
+    const float* W1 = w + (size_t)i * P.per_model;
+    const float* b1 = W1 + (size_t)h1 * din;
+    const float* W2 = b1 + h1;
+    const float* b2 = W2 + (size_t)h2 * h1;
+    const float* W3 = b2 + h2;
+    for (int64_t e = 0; e < P.per_model; ++e)
+      if (!std::isfinite(W1[e])) return false;
+    const float* xi = x + (size_t)P.off[i] * dl;
+    double xmax[MF_MAX_D_LOCAL];
+    for (int k = 0; k < dl; ++k) {
+      xmax[k] = 0.0;
+      for (int o = 0; o < P.K[i]; ++o) {
+        if (!std::isfinite(xi[(size_t)o * dl + k])) return false;
+        xmax[k] = std::fmax(xmax[k], std::fabs((double)xi[(size_t)o * dl + k]));
+      }
+      if (!fits(xmax[k])) return false;
+      S.cx[(size_t)i * dl + k] = pow2_to(xmax[k], 4);
+    }
+    xs.resize((size_t)P.K[i] * dl);
+    for (size_t e = 0; e < xs.size(); ++e) xs[e] = (float)(std::fabs((double)xi[e]) * S.cx[(size_t)i * dl + e % dl]);
+    for (int j = 0; j < h1; ++j) {
+      const double bb = std::fabs((double)b1[j] + (double)W1[(size_t)j * din + dl + 3] * P.agg_scale[3] * N);
+      double m = bb, least = bb;
+      for (int k = 0; k < dl; ++k) m += std::fabs((double)W1[(size_t)j * din + k]) * xmax[k];
+      for (int q = 0; q < 3; ++q) {
+        m += std::fabs((double)W1[(size_t)j * din + dl + q]) * amax[q];
+        least += std::fabs((double)W1[(size_t)j * din + dl + q]) * amin[q];
+      }
+      if (!fits(m)) return false;
+      hb[j] = m;
+      const double t = S.t[(size_t)i * h1 + j] = pow2_to(m, 9);
+      if (m == 0.0 || least * t >= 1.0) continue;
+      for (int k = 0; k < dl; ++k) aw[k] = (float)(std::fabs((double)W1[(size_t)j * din + k]) * t / S.cx[(size_t)i * dl + k]);
+      for (int o = 0; o < P.K[i]; ++o) {
+        float sum = (float)(least * t);
+        for (int k = 0; k < dl; ++k) sum += aw[k] * xs[(size_t)o * dl + k];
+        if (sum < 1.f) return false;
+      }
+    }
+    double top[2] = {0.0, 0.0};
+    for (int j = 0; j < h2; ++j) {
+      double m = std::fabs((double)b2[j]);
+      for (int k = 0; k < h1; ++k) m += std::fabs((double)W2[(size_t)j * h1 + k]) * hb[k];
+      if (!fits(m)) return false;
+      const double u = S.u[(size_t)i * h2 + j] = pow2_to(m, 14);
+      for (int r = 0; r < 2; ++r) top[r] = std::fmax(top[r], std::fabs((double)W3[(size_t)r * h2 + j]) / u);
+    }
+    for (int r = 0; r < 2; ++r) {
+      if (!fits(top[r])) return false;
+      S.v[(size_t)i * 2 + r] = pow2_to(top[r], 6);
+    }
+  }
+  return true;
+}
+
+// The fp16 variant's layout and operand images; MF_EUNSUPPORTED (nothing changed) where
+// half_ranges rules it out.
+mf_status tc_prepare_half(mf_ctx* c, const TcHost& h) {
+  const Params& P = c->P;
+  TcArgs& T = c->tc;
+  const int N = P.n_models, dl = P.d_local, h1 = P.h1, h2 = P.h2, hl = h2, din = P.d_in, sumK = c->sumK;
+  const float *w = h.w, *x = h.x;
+  HalfScales S;
+  if (!half_ranges(P, h, S)) return MF_EUNSUPPORTED;
+  T.tf = kXmHalf;
+  T.dle = dl;
+  T.k1 = 16;  // [x (8) | aggregate (3) | 1 | 0 0 0 0]
+  T.kw = 8;   // words per option: x hi pairs (4), x lo pairs (4)
+  T.h1 = h1;
+  T.h2 = h2;
+  T.hl = hl;
+  T.n3 = 16;
+  // TMEM columns: the pipelines' D (64 each), their D3 (16 each), then per pipeline
+  // H hi (32) | ones (8) | H lo (32) | A1 hi (8), A1 lo (8): 504 of 512 for three pipelines
+  T.pipes = tc_pipes(kXmHalf);
+  T.ps_d = h1;
+  T.ps_d3 = T.n3;
+  T.col_d = 0;
+  T.col_d3 = T.pipes * h1;
+  T.col_h = T.col_d3 + T.pipes * T.n3;
+  T.col_ones = T.col_h + h1 / 2;
+  T.col_hlo = T.col_ones + 8;
+  T.col_a = T.col_hlo + h1 / 2;
+  T.pipe_stride = T.col_a + 16 - T.col_h;
+  for (int q = 0; q < 3; ++q) T.cagg[q] = (float)S.cagg[q];
+  // per model: B1 [h1 x 16] hi, lo; B2 [h2 x (h1 + 16)] hi (its last K-step holds b2 hi, lo
+  // against the ones block), [h2 x h1] lo; B3 [16 x hl] hi, lo
+  const int k2 = h1 + 16;
+  const size_t b1 = (size_t)h1 * T.k1 * 2, b2 = (size_t)h2 * k2 * 2, b2lo = (size_t)h2 * h1 * 2, b3 = (size_t)T.n3 * hl * 2;
+  T.img_lo1 = (uint32_t)b1;
+  T.img_lo2 = (uint32_t)b2;
+  T.img_lo3 = (uint32_t)b3;
+  T.img_model = (uint32_t)(2 * b1 + b2 + b2lo + 2 * b3);
+  std::vector<unsigned char> img(round_up((int)(T.img_model * N), 16), 0);
+  auto split = [](float v, uint16_t& hi, uint16_t& lo) {
+    float rounded, rest;
+    hi = f2half(v, rounded);
+    lo = f2half(v - rounded, rest);
+  };
+  // (scaling by powers of two is exact in fp32)
+  auto put = [&](size_t at, size_t at_lo, float v) {
+    uint16_t hi, lo;
+    split(v, hi, lo);
+    std::memcpy(img.data() + at, &hi, 2);
+    std::memcpy(img.data() + at_lo, &lo, 2);
+  };
+  const double s3 = P.agg_scale[3];
+  for (int i = 0; i < N; ++i) {
+    const float* W1 = w + (size_t)i * P.per_model;
+    const float* bb1 = W1 + (size_t)h1 * din;
+    const float* W2 = bb1 + h1;
+    const float* bb2 = W2 + (size_t)h2 * h1;
+    const float* W3 = bb2 + h2;
+    float it[MF_MAX_HIDDEN], iu[MF_MAX_HIDDEN];  // 1 / t, 1 / u
+    for (int k = 0; k < h1; ++k) it[k] = (float)(1.0 / S.t[(size_t)i * h1 + k]);
+    for (int k = 0; k < h2; ++k) iu[k] = (float)(1.0 / S.u[(size_t)i * h2 + k]);
+    const double *cx = &S.cx[(size_t)i * dl], *t = &S.t[(size_t)i * h1], *u = &S.u[(size_t)i * h2], *v = &S.v[(size_t)i * 2];
+    T.off_b1[i] = T.img_model * i;
+    T.off_b2[i] = T.off_b1[i] + (uint32_t)(2 * b1);
+    T.off_b3[i] = T.off_b2[i] + (uint32_t)(b2 + b2lo);
+    for (int j = 0; j < h1; ++j) {
+      auto put1 = [&](int k, double val) {  // (the constant column rounds to fp32 first)
+        const size_t at = T.off_b1[i] + umma_off(j, k, T.k1);
+        put(at, at + b1, (float)val);
+      };
+      for (int k = 0; k < dl; ++k) put1(k, W1[(size_t)j * din + k] * t[j] / cx[k]);
+      for (int q = 0; q < 3; ++q) put1(dl + q, W1[(size_t)j * din + dl + q] * t[j] / S.cagg[q]);
+      // the constant-1 column: b1 plus the weight of the constant feature N * s_3
+      put1(dl + 3, ((double)bb1[j] + (double)W1[(size_t)j * din + dl + 3] * s3 * N) * t[j]);
+    }
+    for (int j = 0; j < h2; ++j) {
+      for (int k = 0; k < h1; ++k)
+        put(T.off_b2[i] + umma_off(j, k, k2), T.off_b2[i] + b2 + umma_off(j, k, h1), W2[(size_t)j * h1 + k] * (float)u[j] * it[k]);
+      put(T.off_b2[i] + umma_off(j, h1, k2), T.off_b2[i] + umma_off(j, h1 + 1, k2), bb2[j] * (float)u[j]);
+    }
+    for (int r = 0; r < 2; ++r) {
+      T.back[i][r] = (float)(1.0 / v[r]);
+      for (int k = 0; k < hl; ++k) {
+        const size_t at = T.off_b3[i] + umma_off(r * (T.n3 / 2) + i, k, hl);
+        put(at, at + b3, W3[(size_t)r * hl + k] * (float)v[r] * iu[k]);
+      }
+    }
+  }
+  T.img_total = (uint32_t)img.size();
+  set_passes(P, T, kPassImageBudget);
+  set_pass(T, 0, nullptr);
+  std::vector<uint32_t> xw((size_t)sumK * T.kw, 0u);
+  for (int i = 0; i < N; ++i)
+    for (int r = P.off[i]; r < P.off[i] + P.K[i]; ++r)
+      for (int k = 0; k < dl; ++k) {
+        uint16_t hi, lo;
+        split(x[(size_t)r * dl + k] * (float)S.cx[(size_t)i * dl + k], hi, lo);
+        xw[(size_t)r * T.kw + k / 2] |= (uint32_t)hi << (16 * (k & 1));
+        xw[(size_t)r * T.kw + 4 + k / 2] |= (uint32_t)lo << (16 * (k & 1));
+      }
+  layout_smem(P, T, 0);
+  if (T.sm_total > kSmemLimit) return MF_EUNSUPPORTED;
+  const size_t o_xw = round_up((int)img.size(), 256);
+  const size_t total = o_xw + round_up((int)(xw.size() * 4), 256);
+  MF_CUDA(cudaMalloc(&c->d_tc, total));
+  c->tc_bytes = total;
+  unsigned char* base = static_cast<unsigned char*>(c->d_tc);
+  MF_CUDA(cudaMemcpy(base, img.data(), img.size(), cudaMemcpyHostToDevice));
+  MF_CUDA(cudaMemcpy(base + o_xw, xw.data(), xw.size() * 4, cudaMemcpyHostToDevice));
+  c->stats.h2d_bytes_create += img.size() + xw.size() * 4;
+  T.img = base;
+  T.xw = reinterpret_cast<const uint32_t*>(base + o_xw);
+  for (int u = 0; u < 2; ++u) {
+    MF_CUDA(cudaFuncSetAttribute(tc_kernel(kTcRange, T, u, N), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit));
+    MF_CUDA(cudaFuncSetAttribute(tc_kernel(kTcList, T, u, N), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit));
+  }
+  return MF_OK;
+}
+
 }  // namespace
 
-mf_status tc_prepare(mf_ctx* c, bool exact) {
+mf_status tc_prepare(mf_ctx* c, bool exact, const TcHost& h) {
   const Params& P = c->P;
   TcArgs& T = c->tc;
   std::memset(&T, 0, sizeof(T));
-  if (exact) return tc_prepare_exact(c);
+  if (exact) {
+    const mf_status st = tc_prepare_half(c, h);
+    if (st != MF_EUNSUPPORTED) return st;
+    std::memset(&T, 0, sizeof(T));
+    return tc_prepare_exact(c, h);
+  }
   const int N = P.n_models, dl = P.d_local, h1 = P.h1, h2 = P.h2, hl = h2 > 0 ? h2 : h1;
   const int din = P.d_in;
   T.dle = dl + (dl & 1);
@@ -1402,7 +1788,7 @@ mf_status tc_prepare(mf_ctx* c, bool exact) {
   T.col_ones = hmax + hmax / 2;
   T.col_a = T.col_ones + 8;
   T.col_d3 = round_up(T.col_a + T.kw, 16);
-  T.pipe_stride = round_up(T.col_d3 + T.n3, 32);
+  T.pipe_stride = T.ps_d = T.ps_d3 = round_up(T.col_d3 + T.n3, 32);
   T.pipes = 512 / T.pipe_stride;
   if (T.pipes > kTcMaxPipes) T.pipes = kTcMaxPipes;
 
@@ -1411,9 +1797,6 @@ mf_status tc_prepare(mf_ctx* c, bool exact) {
   const size_t b1_bytes = (size_t)h1 * T.k1 * 2, b2_bytes = (size_t)h2 * k2 * 2, b3_bytes = (size_t)T.n3 * k3 * 2;
   std::vector<unsigned char> img;
   const double s3 = P.agg_scale[3];
-  std::vector<float> w(P.per_model * N);
-  cudaError_t e = cudaMemcpy(w.data(), P.w32, sizeof(float) * w.size(), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_fail(e, "tc_prepare: read weights");
   auto put = [&](uint32_t base, int r, int k, int kdim, double v) {
     const uint16_t b = f2bf((float)v);
     std::memcpy(img.data() + base + umma_off(r, k, kdim), &b, 2);
@@ -1425,7 +1808,7 @@ mf_status tc_prepare(mf_ctx* c, bool exact) {
     put(base, r, k + 1, kdim, (double)v - (double)bf2f(hi));
   };
   for (int i = 0; i < N; ++i) {
-    const float* src = w.data() + (size_t)i * P.per_model;
+    const float* src = h.w + (size_t)i * P.per_model;
     const float* W1 = src;
     const float* b1 = W1 + (size_t)h1 * din;
     const float* W2 = b1 + h1;
@@ -1459,29 +1842,13 @@ mf_status tc_prepare(mf_ctx* c, bool exact) {
   }
   img.resize(round_up((int)img.size(), 16), 0);
   T.img_total = (uint32_t)img.size();
-  // passes: consecutive models whose images fit the budget together
-  T.npasses = 0;
-  T.pass_m[0] = 0;
-  for (int i = 0; i < N;) {
-    int j = i + 1;
-    while (j < N && (size_t)((j + 1 < N ? T.off_b1[j + 1] : T.img_total) - T.off_b1[i]) <= kPassImageBudget) ++j;
-    T.pass_m[++T.npasses] = j;
-    i = j;
-  }
-  T.img_bytes = 0;
-  for (int p = 0; p < T.npasses; ++p) {
-    const uint32_t lo = T.off_b1[T.pass_m[p]];
-    const uint32_t hi = p + 1 < T.npasses ? T.off_b1[T.pass_m[p + 1]] : T.img_total;
-    if (hi - lo > T.img_bytes) T.img_bytes = hi - lo;
-  }
+  set_passes(P, T, kPassImageBudget);
   set_pass(T, 0, nullptr);  // single-pass defaults (a pass-0 image of all models)
   if (T.npasses == 1) { T.pass_last = 1; }
 
   // local-feature words
   const int sumK = c->sumK;
-  std::vector<float> x((size_t)sumK * dl);
-  e = cudaMemcpy(x.data(), P.x, sizeof(float) * x.size(), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_fail(e, "tc_prepare: read tables");
+  const float* x = h.x;
   std::vector<uint32_t> xw((size_t)sumK * T.kw, 0u);
   for (int r = 0; r < sumK; ++r)
     for (int k = 0; k < dl; ++k)
@@ -1511,11 +1878,13 @@ mf_status tc_prepare(mf_ctx* c, bool exact) {
 
 mf_status tc_search_chunk(mf_ctx* c, const RangeArgs& a, cudaStream_t s, int* nlaunch) {
   TcArgs T = c->tc;
-  layout_smem(c->P, T, a.k);
-  if (T.sm_total > kSmemLimit) {
+  if (!layout_for(c->P, T, a.k)) {
     set_error("tensor-core path: top-k lists do not fit shared memory; use a smaller k");
     return MF_EUNSUPPORTED;
   }
+  if (T.npasses != c->tc.npasses)  // (another kernel than the one prepared)
+    MF_CUDA(cudaFuncSetAttribute(tc_kernel(kTcRange, T, c->P.objective == MF_OBJ_UTILITY, c->P.n_models),
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit));
   // digits of the per-tile index stride (grid x pipes x 128), modulo |Lambda|
   const uint64_t stride = ((uint64_t)c->num_sms * T.pipes * 128) % c->P.total;
   uint64_t v = stride;
@@ -1533,7 +1902,7 @@ mf_status tc_search_chunk(mf_ctx* c, const RangeArgs& a, cudaStream_t s, int* nl
   const uint32_t smem = T.sm_total > kSmemFloor ? T.sm_total : kSmemFloor;
   TcList L{};
   float4* partial = nullptr;
-  mf_status st = ensure_partial(c, a.len, s, &partial);
+  mf_status st = ensure_partial(c, T.npasses, a.len, s, &partial);
   if (st != MF_OK) return st;
   // one launch per pass and span of candidates; the lists and the count belong to the
   // last pass only
@@ -1562,7 +1931,7 @@ mf_status tc_score_list(mf_ctx* c, const uint64_t* idx, uint64_t n, float* score
   layout_smem(c->P, T, 0);
   const uint32_t smem = T.sm_total > kSmemFloor ? T.sm_total : kSmemFloor;
   float4* partial = nullptr;
-  mf_status st = ensure_partial(c, n, s, &partial);
+  mf_status st = ensure_partial(c, T.npasses, n, s, &partial);
   if (st != MF_OK) return st;
   const uint64_t span = T.npasses == 1 ? n : kPassSpan;
   const int N = c->P.n_models;

@@ -240,17 +240,18 @@ mf_status mf_create(const mf_problem* p, mf_ctx** out) {
   P.status = c->d_status;
 
   mf_status st3 = f32_prepare(c);
+  const TcHost host{w32.data(), p->local_feats, dem4.data()};
   if (st3 == MF_OK && c->precision == MF_BF16) {
     std::string why;
     if (!tc_supported(P, &why)) {
       g_last_error = "bf16 tensor-core path: " + why;
       st3 = MF_EUNSUPPORTED;
     } else {
-      st3 = tc_prepare(c);
+      st3 = tc_prepare(c, false, host);
     }
   } else if (st3 == MF_OK && c->precision == MF_FP32 && tc_exact_supported(P)) {
     // the exact tensor-core variant where its operands fit; else the CUDA-core path
-    if (tc_prepare(c, true) != MF_OK) {
+    if (tc_prepare(c, true, host) != MF_OK) {
       cudaFree(c->d_tc);
       c->d_tc = nullptr;
       std::memset(&c->tc, 0, sizeof(c->tc));

@@ -51,12 +51,15 @@ struct TcArgs {
   const uint32_t* xw;                 // [sumK][kw] local features: bf16 pairs, or tf32 hi then lo words
   int32_t k1, kw, h1, h2, hl, n3, dle;
   uint32_t off_b1[MF_MAX_MODELS], off_b2[MF_MAX_MODELS], off_b3[MF_MAX_MODELS];  // bytes in img
-  int32_t pipes, col_d, col_h, col_ones, col_a, col_d3, pipe_stride;  // TMEM columns
-  // the exact fp32 variant (3-term tf32 split): operands as tf32 hi and lo parts; col_hlo
-  // holds the hidden layer's lo parts, img_lo1..3 are the byte offsets of each B image's
-  // lo part after its hi part
+  // TMEM columns; from pipeline to pipeline D moves by ps_d, D3 by ps_d3, the rest by pipe_stride
+  int32_t pipes, col_d, col_h, col_ones, col_a, col_d3, pipe_stride, ps_d, ps_d3;
+  // the exact fp32 variants (tf: 1 tf32 parts, 2 fp16 parts; 0 bf16): operands as hi and lo
+  // parts; col_hlo holds the hidden layer's lo parts, img_lo1..3 are the byte offsets of
+  // each B image's lo part after its hi part
   int32_t tf, col_hlo;
   uint32_t img_lo1, img_lo2, img_lo3;
+  // fp16 parts: the aggregate's scales, and the factors that scale the outputs back
+  float cagg[3], back[MF_MAX_MODELS][2];
   uint32_t sm_xw, sm_dem, sm_rows, sm_topk, sm_bar, sm_total;  // shared-memory byte offsets
   uint32_t img_model;                 // bytes of one model's B1 + B2 + B3 images
   int32_t kcap;                       // per-pipeline list length the layout was sized for
@@ -465,7 +468,12 @@ mf_status finish_shortlist(const Params& P, const uint64_t* idx, const float* pr
 bool tc_supported(const Params& P, std::string* why);
 bool tc_exact_supported(const Params& P);  // the exact fp32 (3-term tf32) variant's shapes
 bool tc_fits(const mf_ctx* c, int kcap);    // the context's tensor-core layout with lists of kcap
-mf_status tc_prepare(mf_ctx* c, bool exact = false);
+// The host arrays that tc_prepare lays out: packed weights (as P.w32), features, demands
+// (as P.dem).
+struct TcHost {
+  const float *w, *x, *dem4;
+};
+mf_status tc_prepare(mf_ctx* c, bool exact, const TcHost& h);
 int tc_grid(const mf_ctx* c);
 mf_status tc_search_chunk(mf_ctx* c, const RangeArgs& a, cudaStream_t s, int* nlaunch);
 mf_status tc_score_list(mf_ctx* c, const uint64_t* idx, uint64_t n, float* score,
