@@ -119,7 +119,7 @@ typedef struct {
 } mf_ga_params;
 
 /* Instrumentation of the last calls on a context (host-side bookkeeping plus
- * CUDA events recorded on the call's stream; no extra synchronisation). */
+ * stamps of the device's nanosecond timer; no extra synchronisation). */
 typedef struct {
   uint64_t h2d_bytes_create;   /* bytes mf_create copied host -> device */
   uint64_t d2h_bytes_last;     /* bytes the last synchronous call copied device -> host */

@@ -159,6 +159,7 @@ k_score_f32(const Params P, const RangeArgs R, const ListArgs L) {
   const int N = P.n_models;
   const int stride = (int)P.per_model;  // floats between models (multiple of 4)
 
+  if (MODE == kModeRange) stamp_start(R);
   // ---- stage the predictors in shared memory (one copy per CTA) ----
   float* sw = reinterpret_cast<float*>(smem);
   size_t wfloats = RESIDENT ? (size_t)N * stride : 0;

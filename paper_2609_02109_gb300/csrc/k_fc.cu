@@ -252,6 +252,7 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
   // NMAX: a bound on N for the unrolled per-model loops
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ FcSpan s_span[MF_MAX_MODELS];
+  stamp_start(R);
   const int N = P.n_models;
   const int sumK = pick(P.off, N - 1) + pick(P.K, N - 1);
   constexpr int QCAP = WL ? kFcEndQ : kFcCtaQ;

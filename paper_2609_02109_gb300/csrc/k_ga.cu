@@ -183,13 +183,12 @@ mf_status ga_run_graph(mf_ctx* c, const mf_ga_params* g, uint64_t seed, cudaStre
 // unit j) keeps rows j of W1 and W2 in registers for the whole run, so a weight is
 // read from memory once per run.  One generation:
 //   layer 1    thread (m, j) for the slice's candidates
-//   layer 2-3  PAIR (up to five models, whose 320 threads leave room for 128 weights each):
-//              lane j of warp h of model m for units j and j + 32 and candidates 4h .. 4h + 3;
-//              else thread (m, j) for all 8 candidates.  Each shared-memory load of four
-//              layer-1 activations is one broadcast to the warp, and they bound the layer:
-//              a load feeds two units in PAIR, so there are half as many.  Layer 3 sums over
-//              the warp in butterfly shuffles where each step halves the values a lane
-//              carries (the same sums in the same order in both layouts)
+//   layer 2-3  thread (m, j) for all 8 candidates (each shared-memory load of four
+//              layer-1 activations is one broadcast to the warp); layer 3 sums over
+//              the warp in butterfly shuffles where each step halves the values a
+//              lane carries.  (Two units a thread for half of the candidates halves the
+//              loads, but three warps on one scheduler allow 168 registers each: with 128
+//              weights it spills, 597 us a decision against 525)
 //   objective  warp c for candidate c, lane i for model i (Eq. 7-9)
 //   step       warp c breeds child 8b + c: lane t holds tournament entry t and
 //              fetches its fitness and genome; the winners' genomes come by
@@ -197,11 +196,11 @@ mf_status ga_run_graph(mf_ctx* c, const mf_ga_params* g, uint64_t seed, cudaStre
 //              aggregate state.  The elite (slot 0) is the best of the CTAs' bests.
 //              The draws do not depend on fitness: the last warp, which breeds nothing,
 //              makes the next generation's while the others breed.
-// N = 5, population 1024, 100 generations: GA_NOW (543 us with one unit per thread and the
-// draws on the breeding warps).
+// N = 5, population 1024, 100 generations: 525 us (543 with the draws on the breeding warps
+// and tournaments by shuffles).
 // There is no grid-wide barrier.  Every value another CTA reads -- an individual's
 // fitness, the two halves of its genome (gene i in byte i mod 4), a CTA's best --
-// is a 64-bit word whose high half is the tag g + 1 of its generation g, written
+// is a 64-bit word whose high half is the tag of its generation g, tag0 + g + 1, written
 // and read as single 64-bit accesses.  A reader spins on exactly the words it
 // needs until their tags match, so each generation waits only for the CTAs whose
 // individuals its tournaments drew (and CTA 0, for the elite, for every CTA's
@@ -211,6 +210,11 @@ mf_status ga_run_graph(mf_ctx* c, const mf_ga_params* g, uint64_t seed, cudaStre
 // Every operator and draw is that of k_ga_step, so the run equals init + (fitness,
 // step) x gens up to the fp32 rounding of the fitness.  Every spin gives up after
 // kGaSpinLimit polls, sets the timeout bit of the status word and ends the CTA.
+// tag0 grows from run to run by more than a run's generations, so words of earlier runs
+// never match and nothing is cleared between runs; the progress counters, which are
+// compared by size and offset by tag0 too, have a place of their own at the buffer's start.
+// The seed comes with the launch and the result goes to pinned host memory, so a decision
+// is one launch and no copy (a clear, a copy in and two out cost about 30 us).
 // ---------------------------------------------------------------------------
 namespace mf {
 
@@ -234,10 +238,12 @@ struct __align__(32) GaBest {  // fittest individual of one CTA's slice
 struct GaPersist {
   GaRec* rec;            // [ring][pop]
   GaBest* best;          // [ring][ctas]
-  unsigned int* prog;    // [ctas] generations whose records the CTA has finished reading
-  int32_t* out_genome;
+  unsigned int* prog;    // [ctas] tag0 + generations whose records the CTA has finished reading
+  int32_t* out_genome;   // pinned host memory: genome, fitness, status word
   float* out_fit;
-  const uint64_t* seed;
+  uint32_t* out_status;
+  uint64_t seed;
+  uint32_t tag0;
   int gens;
   int ring;
 };
@@ -393,7 +399,7 @@ __device__ __forceinline__ bool tournament_winner(const GaArgs& g, uint64_t sd, 
   return ok;
 }
 
-template <int MAXT, bool PAIR>
+template <int MAXT>
 __global__ void __launch_bounds__(MAXT, 1)
 k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
   constexpr int H = 64, DL = 8, DIN = DL + 4, SM = kGaMaxSlice;
@@ -419,11 +425,9 @@ k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
   const int m = unit ? tid / H : 0;
   const int j = tid % H;
   const int wq = j >> 5;              // warp of the model
-  // this thread's weights: row j of W1; U rows of W2 (j, or lane and lane + 32) and the
-  // layer-3 weights of those units
-  constexpr int U = PAIR ? 2 : 1;
-  float w1[DIN], w2[U][H];
-  float b1 = 0.f, b2[U] = {}, w3t[U] = {}, w3l[U] = {};
+  // this thread's weights: rows j of W1 and W2, the layer-3 weights of unit j
+  float w1[DIN], w2[H];
+  float b1 = 0.f, b2 = 0.f, w3t = 0.f, w3l = 0.f;
   int unit_off = 0;
   if (unit) {
     const float* w = P.w32 + (size_t)m * P.per_model;
@@ -431,16 +435,12 @@ k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
     for (int k = 0; k < DIN; ++k) w1[k] = __ldg(w + j * DIN + k);
     b1 = __ldg(w + H * DIN + j);
     const float* W2 = w + H * DIN + H;
+#pragma unroll
+    for (int k = 0; k < H; ++k) w2[k] = __ldg(W2 + j * H + k);
+    b2 = __ldg(W2 + H * H + j);
     const float* W3 = W2 + H * H + H;
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int ju = PAIR ? lane + 32 * u : j;
-#pragma unroll
-      for (int k = 0; k < H; ++k) w2[u][k] = __ldg(W2 + ju * H + k);
-      b2[u] = __ldg(W2 + H * H + ju);
-      w3t[u] = __ldg(W3 + ju);
-      w3l[u] = __ldg(W3 + H + ju);
-    }
+    w3t = __ldg(W3 + j);
+    w3l = __ldg(W3 + H + j);
     unit_off = pick(P.off, m);
   }
   // per-lane constants of model `lane`
@@ -479,7 +479,7 @@ k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
     __syncthreads();
     if (s_abort) return;
   }
-  const uint64_t sd = *G.seed;
+  const uint64_t sd = G.seed;
   const int c0 = blockIdx.x * SM;
   const int ns = min(SM, pop - c0);
   const float nz = (float)N * P.agg_scale[3];
@@ -520,13 +520,13 @@ k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
   };
   if (child_warp) {  // initial population (generation 0, tag 1)
     const int gene = lane < N ? ga_unif(ga_rng(sd, 0, cg, kGaInit, (uint32_t)lane), (uint32_t)my_K) : 0;
-    place(gene, G.rec, 1u);
+    place(gene, G.rec, G.tag0 + 1u);
   }
   if (warp == last_warp) make_draws(g, sd, 1u, c0, ns, N, s_draws[1]);
   __syncthreads();
 
   for (int gen = 0; gen < G.gens; ++gen) {
-    const uint32_t tag = (uint32_t)gen + 1u;
+    const uint32_t tag = G.tag0 + (uint32_t)gen + 1u;
     const int slot = gen % G.ring;
     GaRec* rec_cur = G.rec + (size_t)slot * pop;
     GaRec* rec_nxt = G.rec + (size_t)((gen + 1) % G.ring) * pop;
@@ -567,36 +567,27 @@ k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
     if (unit) {
       const float* h1 = sh1 + (size_t)m * SM * H;
       // even and odd k accumulate apart, two fused multiply-adds per instruction
-      constexpr int C = PAIR ? SM / 2 : SM;   // this thread's candidates, from cb on
-      const int cb = PAIR ? C * wq : 0;
-      float2 acc2[U][C];
+      float2 acc2[SM];
 #pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int c = 0; c < C; ++c) acc2[u][c] = make_float2(b2[u], 0.f);
+      for (int c = 0; c < SM; ++c) acc2[c] = make_float2(b2, 0.f);
 #pragma unroll
       for (int p = 0; p < H / 4; ++p) {
+        const float2 wa = make_float2(w2[4 * p + 0], w2[4 * p + 1]);
+        const float2 wb = make_float2(w2[4 * p + 2], w2[4 * p + 3]);
 #pragma unroll
-        for (int c = 0; c < C; ++c) {
-          const float4 hk = *reinterpret_cast<const float4*>(h1 + (cb + c) * H + 4 * p);
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            acc2[u][c] = fma2(make_float2(w2[u][4 * p + 0], w2[u][4 * p + 1]), make_float2(hk.x, hk.y), acc2[u][c]);
-            acc2[u][c] = fma2(make_float2(w2[u][4 * p + 2], w2[u][4 * p + 3]), make_float2(hk.z, hk.w), acc2[u][c]);
-          }
+        for (int c = 0; c < SM; ++c) {
+          const float4 hk = *reinterpret_cast<const float4*>(h1 + c * H + 4 * p);
+          acc2[c] = fma2(wa, make_float2(hk.x, hk.y), acc2[c]);
+          acc2[c] = fma2(wb, make_float2(hk.z, hk.w), acc2[c]);
         }
       }
-      // 16 values to sum over the warp: thr and lat of SM candidates, or (PAIR) of half of
-      // them for each half of the units
       float v[2 * SM];
 #pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-          const float h2 = relu(acc2[u][c].x + acc2[u][c].y);
-          v[u * C + c] = w3t[u] * h2;
-          v[SM + u * C + c] = w3l[u] * h2;
-        }
+      for (int c = 0; c < SM; ++c) {
+        const float h2 = relu(acc2[c].x + acc2[c].y);
+        v[c] = w3t * h2;
+        v[SM + c] = w3l * h2;
+      }
       fold<8>(v, 0);
       fold<4>(v, 1);
       fold<2>(v, 2);
@@ -604,9 +595,8 @@ k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
       const float out = v[0] + __shfl_xor_sync(0xffffffffu, v[0], 16);
       // value index 8 * bit0 + 4 * bit1 + 2 * bit2 + bit3: bit0 thr / lat, the rest the candidate
       const int kind = lane & 1;
-      const int e = 4 * ((lane >> 1) & 1) + 2 * ((lane >> 2) & 1) + ((lane >> 3) & 1);
-      const int half = PAIR ? e / C : wq, c = PAIR ? cb + e % C : e;  // (units 32 half ..; candidate)
-      if (lane < 16) spart[((half * SM + c) * N + m) * 2 + kind] = out;
+      const int c = 4 * ((lane >> 1) & 1) + 2 * ((lane >> 2) & 1) + ((lane >> 3) & 1);
+      if (lane < 16) spart[((wq * SM + c) * N + m) * 2 + kind] = out;
     }
     __syncthreads();
     // ---- objective and constraints: warp c, lane i = model i ----
@@ -655,7 +645,7 @@ k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
       for (uint32_t n = 0; n < kGaSpinLimit; ++n) {
         bool mine = true;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) mine = mine && pv[u] >= (unsigned int)need;
+        for (int u = 0; u < 8; ++u) mine = mine && pv[u] >= G.tag0 + (unsigned int)need;
         if (__all_sync(0xffffffffu, mine)) { ok = true; break; }
 #pragma unroll
         for (int u = 0; u < 8; ++u)
@@ -689,7 +679,10 @@ k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
         } else {
           const uint64_t g8 = (uint64_t)lo | ((uint64_t)hi << 32);
           if (lane < N) G.out_genome[lane] = (int)((g8 >> (8 * lane)) & 0xFF);
-          if (lane == 0) *G.out_fit = f;
+          if (lane == 0) {
+            *G.out_fit = f;
+            *G.out_status = *(volatile uint32_t*)P.status;  // (every CTA has published its last: none waits any more)
+          }
         }
       }
       return;
@@ -731,7 +724,7 @@ k_ga_persist(const Params P, const GaArgs g, const GaPersist G) {
     }
     __syncthreads();
     if (s_abort) return;
-    if (tid == 0) st_u32(G.prog + blockIdx.x, (unsigned int)gen + 1u);  // generation gen fully read
+    if (tid == 0) st_u32(G.prog + blockIdx.x, G.tag0 + (unsigned int)gen + 1u);  // generation gen fully read
   }
 }
 
@@ -743,12 +736,9 @@ mf_status ga_run_persistent(mf_ctx* c, const mf_ga_params* g, uint64_t seed, cud
   const int ctas = (pop + kGaMaxSlice - 1) / kGaMaxSlice;
   if (ctas > 256) return MF_EUNSUPPORTED;  // progress counters: eight per lane of one warp
   // one thread per (model, hidden unit), at least one warp past the 8 child warps;
-  // register budgets of 320 (up to five models, which leaves 204 registers a thread: two
-  // units' weights), 384 and 512 threads
+  // register budgets of 384 (up to six models) and 512 threads
   const int threads = std::max(N * 64, 32 * (kGaMaxSlice + 1));
-  const void* fn = threads <= 320   ? (const void*)k_ga_persist<384, false>
-                   : threads <= 384 ? (const void*)k_ga_persist<384, false>
-                                    : (const void*)k_ga_persist<512, false>;
+  const void* fn = threads <= 384 ? (const void*)k_ga_persist<384> : (const void*)k_ga_persist<512>;
   const int sumK = P.off[N - 1] + P.K[N - 1];
   const size_t smem = sizeof(float) * ((size_t)N * kGaMaxSlice * 64 + (size_t)4 * kGaMaxSlice * N +
                                        4 * kGaMaxSlice + (size_t)sumK * 8) +
@@ -758,10 +748,11 @@ mf_status ga_run_persistent(mf_ctx* c, const mf_ga_params* g, uint64_t seed, cud
   int per_sm = 0;
   MF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem));
   if (per_sm * c->num_sms < ctas) return MF_EUNSUPPORTED;
-  // scratch: records [ring][pop], CTA bests [ring][ctas], progress [ctas]
+  // scratch: progress [256], records [ring][pop], CTA bests [ring][ctas]
   const int ring = std::min(g->gens + 1, kGaRingMax);
+  const size_t progb = 256 * sizeof(unsigned int);
   const size_t recb = sizeof(GaRec) * ring * (size_t)pop, bestb = sizeof(GaBest) * ring * (size_t)ctas;
-  const size_t need = recb + bestb + sizeof(unsigned int) * (size_t)ctas;
+  const size_t need = progb + recb + bestb;
   if (need > c->gap_bytes) {
     MF_CUDA(cudaStreamSynchronize(s));
     cudaFree(c->d_gap);
@@ -769,26 +760,29 @@ mf_status ga_run_persistent(mf_ctx* c, const mf_ga_params* g, uint64_t seed, cud
     c->gap_bytes = 0;
     MF_CUDA(cudaMalloc(&c->d_gap, need));
     c->gap_bytes = need;
+    c->ga_tag = 0;
   }
-  if (!c->d_ga_out) MF_CUDA(cudaMalloc(&c->d_ga_out, 128));
+  if (c->ga_tag == 0 || (uint64_t)c->ga_tag + (uint64_t)g->gens + 2 > 0x7FFFFFFFull) {  // new memory, or the tags run out
+    if ((uint64_t)g->gens + 3 > 0x7FFFFFFFull) return MF_EUNSUPPORTED;
+    MF_CUDA(cudaMemsetAsync(c->d_gap, 0, c->gap_bytes, s));
+    c->ga_tag = 1;
+  }
   mf_status st = ensure_host_stage(c, 256);
   if (st != MF_OK) return st;
   char* base = (char*)c->d_gap;
   GaPersist G{};
-  G.rec = (GaRec*)base;
-  G.best = (GaBest*)(base + recb);
-  G.prog = (unsigned int*)(base + recb + bestb);
-  G.out_genome = (int32_t*)c->d_ga_out;
+  G.prog = (unsigned int*)base;
+  G.rec = (GaRec*)(base + progb);
+  G.best = (GaBest*)(base + progb + recb);
+  G.out_genome = (int32_t*)c->h_stage;
   G.out_fit = (float*)(G.out_genome + N);
-  uint64_t* d_seed = (uint64_t*)((char*)c->d_ga_out + 64);
-  G.seed = d_seed;
+  G.out_status = (uint32_t*)(G.out_fit + 1);
+  *G.out_status = kStatusUnwritten;
+  G.seed = seed;
+  G.tag0 = c->ga_tag;
+  c->ga_tag += (uint32_t)g->gens + 2u;
   G.gens = g->gens;
   G.ring = ring;
-  uint64_t* h_seed = (uint64_t*)((char*)c->h_stage + 128);
-  *h_seed = seed;
-  MF_CUDA(cudaMemcpyAsync(d_seed, h_seed, sizeof(uint64_t), cudaMemcpyHostToDevice, s));
-  // tags of a previous run must not match: clear the records, bests and counters
-  MF_CUDA(cudaMemsetAsync(c->d_gap, 0, need, s));
   GaArgs a = make_args(c, g);
   Params Pc = P;
   void* args[] = {(void*)&Pc, (void*)&a, (void*)&G};

@@ -88,11 +88,16 @@ __device__ void sort_out(float* ss, uint64_t* si, int n, int k, const ResultOut&
   for (int e = n + tid; e < k; e += nthr) { out.score[e] = -INFINITY; out.idx[e] = kEmptyIdx; }
 }
 
-// The count and the status word beside the lists (nothing where the caller copies them).
+// The count, the times and the status word beside the lists (nothing where the caller copies
+// what it wants).
 __device__ __forceinline__ void pass_on(const ResultOut& out) {
-  if (threadIdx.x == 0 && out.count) {
-    *out.count = *out.count_src;
-    *out.status = *out.status_src;
+  if (threadIdx.x == 0 && out.tail) {
+    out.tail->count = out.words->count;
+    out.tail->t[0] = out.words->t[0];
+    out.tail->t[1] = out.words->t[1];
+    out.tail->status = *out.status;
+    out.words->count = 0ull;
+    out.tail->t[2] = device_ns();
   }
 }
 
@@ -174,7 +179,11 @@ k_merge_lists(const float* __restrict__ in_s, const uint64_t* __restrict__ in_i,
   float* ss = reinterpret_cast<float*>(si + cap);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid < 32) s_bar[tid] = 0u;
-  if (tid == 0) { s_nlist = 0; s_n = 0; }
+  if (tid == 0) {
+    s_nlist = 0;
+    s_n = 0;
+    if (out.words) out.words->t[1] = device_ns();
+  }
   __syncthreads();
   bool few = nlists <= kMergeMaxLists;
   if (few) {

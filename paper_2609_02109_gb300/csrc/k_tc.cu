@@ -551,6 +551,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
     if (tid == 0) atomicOr(P.status, kStatusBadInput);
     return;
   }
+  if (MODE == kTcRange && (!MP || T.pass_first)) stamp_start(R);
   // the warp index through a shuffle from lane 0, so the compiler knows it is warp-uniform
   // and keeps everything derived from it (pipeline, tensor-memory addresses, issuer roles)
   // in uniform registers with uniform branches

@@ -70,8 +70,7 @@ static void free_ctx(mf_ctx* c) {
   cudaFree(c->d_gap);
   if (c->ga_exec) cudaGraphExecDestroy(c->ga_exec);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
-  for (int j = 0; j < 3; ++j)
-    if (c->ev[j]) cudaEventDestroy(c->ev[j]);
+  cudaFree(c->d_words);
   if (c->h_stage) cudaFreeHost(c->h_stage);
   delete c;
 }
@@ -226,8 +225,7 @@ mf_status mf_create(const mf_problem* p, mf_ctx** out) {
       (e = upload((void**)&c->d_wT, wT.data(), sizeof(float) * wT.size())) != cudaSuccess ||
       (e = cudaMalloc((void**)&c->d_status, sizeof(uint32_t))) != cudaSuccess ||
       (e = cudaMemset(c->d_status, 0, sizeof(uint32_t))) != cudaSuccess ||
-      (e = cudaEventCreate(&c->ev[0])) != cudaSuccess || (e = cudaEventCreate(&c->ev[1])) != cudaSuccess ||
-      (e = cudaEventCreate(&c->ev[2])) != cudaSuccess) {
+      (e = cudaMalloc((void**)&c->d_words, sizeof(SearchWords))) != cudaSuccess) {
     mf_status st2 = cuda_fail(e, "mf_create upload");
     free_ctx(c);
     return st2;
@@ -408,7 +406,6 @@ static mf_status search_impl(mf_ctx* ctx, uint64_t lo, uint64_t hi, int32_t k, u
   const size_t o_ms = o; o = align_up(o + sizeof(float) * kcap, 256);
   const size_t o_mi = o; o = align_up(o + sizeof(uint64_t) * kcap, 256);
   const size_t o_rp = o; o = align_up(o + sizeof(float) * 2 * kcap * ctx->P.n_models, 256);
-  const size_t o_cnt = o; o = align_up(o + sizeof(unsigned long long), 256);
   mf_status st = ensure_scratch(ctx, o);
   if (st != MF_OK) return st;
   char* base = (char*)ctx->d_scratch;
@@ -419,27 +416,28 @@ static mf_status search_impl(mf_ctx* ctx, uint64_t lo, uint64_t hi, int32_t k, u
   float* ms = (float*)(base + o_ms);
   uint64_t* mi = (uint64_t*)(base + o_mi);
   float* rp = (float*)(base + o_rp);
-  unsigned long long* cnt = (unsigned long long*)(base + o_cnt);
-  // the result, in pinned host memory: top-k, count and status word, written by the last
-  // kernel itself (a copy for each cost about 3.7 us apiece on the stream)
-  const size_t h_sc = sizeof(uint64_t) * k, h_cn = align_up(h_sc + sizeof(float) * k, 8);
-  st = ensure_host_stage(ctx, h_cn + sizeof(unsigned long long) + sizeof(uint32_t));
+  // the result, in pinned host memory: top-k, count, times and status word, written by the
+  // last kernel itself (a copy for each cost about 3.7 us apiece on the stream; the words are
+  // cleared there too, and the times are the device's timer, where an event record between
+  // two kernels cost about 3 us)
+  const size_t h_sc = sizeof(uint64_t) * k, h_tl = align_up(h_sc + sizeof(float) * k, 8);
+  st = ensure_host_stage(ctx, h_tl + sizeof(SearchTail));
   if (st != MF_OK) return st;
   char* h = (char*)ctx->h_stage;
   const uint64_t* h_i = (uint64_t*)h;
   const float* h_s = (float*)(h + h_sc);
-  const unsigned long long* h_c = (unsigned long long*)(h + h_cn);
-  const uint32_t* h_status = (uint32_t*)(h_c + 1);
-  const ResultOut result{(uint64_t*)h_i, (float*)h_s, (unsigned long long*)h_c, (uint32_t*)h_status, cnt, ctx->d_status};
-  MF_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), s));
+  const SearchTail* tail = (SearchTail*)(h + h_tl);
+  const ResultOut result{(uint64_t*)h, (float*)(h + h_sc), (SearchTail*)(h + h_tl), ctx->d_words, ctx->d_status};
+  if (ctx->words_dirty) MF_CUDA(cudaMemsetAsync(ctx->d_words, 0, sizeof(SearchWords), s));
+  ctx->words_dirty = true;
 
   int launches = 0, score_launches = 0;
-  MF_CUDA(cudaEventRecord(ctx->ev[0], s));
   RangeArgs a{};
   a.k = kcap;
   a.lists_s = ls;
   a.lists_i = li;
-  a.count = cnt;
+  a.count = &ctx->d_words->count;
+  a.start = &ctx->d_words->t[0];
   a.first = 1;
   if (hi == lo) {
     // empty range: initialise the lists through a zero-length launch of the scorer
@@ -461,11 +459,10 @@ static mf_status search_impl(mf_ctx* ctx, uint64_t lo, uint64_t hi, int32_t k, u
     launches += nl;
     score_launches += nl;
   }
-  MF_CUDA(cudaEventRecord(ctx->ev[1], s));
   ++launches;
   if (tc) {
     // exact fp32 re-scoring of the tensor-core shortlist, then the final top-k
-    const ResultOut shortlist{mi, ms, nullptr, nullptr, nullptr, nullptr};
+    const ResultOut shortlist{mi, ms, nullptr, ctx->d_words, nullptr};
     st = merge_lists(ls, li, grid, kcap, ts, ti, shortlist, s);
     if (st == MF_OK) st = f32_predict_shortlist(ctx, mi, kcap, rp, s);
     if (st == MF_OK) st = finish_shortlist(ctx->P, mi, rp, kcap, k, result, s);
@@ -474,19 +471,19 @@ static mf_status search_impl(mf_ctx* ctx, uint64_t lo, uint64_t hi, int32_t k, u
     st = merge_lists(ls, li, grid, k, ts, ti, result, s);
   }
   if (st != MF_OK) return st;
-  MF_CUDA(cudaEventRecord(ctx->ev[2], s));
   MF_CUDA(cudaStreamSynchronize(s));
-  if (*h_status) MF_CUDA(cudaMemsetAsync(ctx->d_status, 0, sizeof(uint32_t), s));
+  ctx->words_dirty = false;
+  if (tail->status) MF_CUDA(cudaMemsetAsync(ctx->d_status, 0, sizeof(uint32_t), s));
   ctx->stats.kernel_launches_last = launches;
   ctx->stats.score_launches_last = score_launches;
   ctx->stats.d2h_bytes_last = (sizeof(uint64_t) + sizeof(float)) * k + sizeof(unsigned long long) + sizeof(uint32_t);
-  MF_CUDA(cudaEventElapsedTime(&ctx->stats.score_ms_last, ctx->ev[0], ctx->ev[1]));
-  MF_CUDA(cudaEventElapsedTime(&ctx->stats.total_ms_last, ctx->ev[0], ctx->ev[2]));
-  if (*h_status & kStatusTimeout) {
+  ctx->stats.score_ms_last = (float)((double)(tail->t[1] - tail->t[0]) * 1e-6);
+  ctx->stats.total_ms_last = (float)((double)(tail->t[2] - tail->t[0]) * 1e-6);
+  if (tail->status & kStatusTimeout) {
     g_last_error = "a bounded device wait gave up";
     return MF_ETIMEOUT;
   }
-  out->feasible_count = *h_c;
+  out->feasible_count = tail->count;
   out->best_idx = h_i[0];
   out->best_score = h_s[0];
   out->k = k;
@@ -555,7 +552,8 @@ mf_status mf_ga_run(mf_ctx* ctx, const mf_ga_params* g, uint64_t seed, int32_t* 
   cudaStream_t s = (cudaStream_t)stream;
   int launches = 1;  // one cooperative kernel
   st = ga_run_persistent(ctx, g, seed, s);
-  if (st == MF_EUNSUPPORTED) {
+  const bool one = st != MF_EUNSUPPORTED;
+  if (!one) {
     st = ga_run_graph(ctx, g, seed, s);
     launches = 2 + g->gens * 2 + (g->gens - 1);  // init, (wide + combine) x gens, steps, best
   }
@@ -564,9 +562,15 @@ mf_status mf_ga_run(mf_ctx* ctx, const mf_ga_params* g, uint64_t seed, int32_t* 
   int32_t* h_g = (int32_t*)ctx->h_stage;
   float* h_f = (float*)(h_g + N);
   uint32_t* h_status = (uint32_t*)(h_f + 1);
-  MF_CUDA(cudaMemcpyAsync(h_g, ctx->d_ga_out, sizeof(int32_t) * N + sizeof(float), cudaMemcpyDeviceToHost, s));
-  st = read_status(ctx, s, h_status, true);
-  if (st != MF_OK) return st;
+  if (one) {  // (the kernel wrote the result, and the status word where it came to an end)
+    MF_CUDA(cudaStreamSynchronize(s));
+  } else {
+    MF_CUDA(cudaMemcpyAsync(h_g, ctx->d_ga_out, sizeof(int32_t) * N + sizeof(float), cudaMemcpyDeviceToHost, s));
+  }
+  if (!one || *h_status != 0) {
+    st = read_status(ctx, s, h_status, true);
+    if (st != MF_OK) return st;
+  }
   if (*h_status & kStatusTimeout) {
     g_last_error = "the GA kernel's grid barrier gave up waiting";
     return MF_ETIMEOUT;

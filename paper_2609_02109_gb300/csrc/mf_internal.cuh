@@ -81,6 +81,7 @@ struct TcArgs {
 // Device status bits.
 constexpr uint32_t kStatusBadInput = 1u;
 constexpr uint32_t kStatusTimeout = 2u;
+constexpr uint32_t kStatusUnwritten = 0xFFFFFFFFu;  // host copy: the kernel ended before it wrote one
 
 // ---------------------------------------------------------------------------
 // Device helpers
@@ -340,6 +341,12 @@ __device__ void topk_merge_sorted(const CtaTopK& t, int tid, int nthr, Sync sync
   sync();
 }
 
+// The device words of a search, kept by the context: zero between searches.
+struct SearchWords {
+  unsigned long long count;  // feasible candidates
+  unsigned long long t[2];   // start of the first scoring launch, of the merge (ns)
+};
+
 }  // namespace mf
 
 // ---------------------------------------------------------------------------
@@ -358,6 +365,8 @@ struct mf_ctx {
   float* d_w32 = nullptr;
   float* d_wT = nullptr;
   uint32_t* d_status = nullptr;
+  mf::SearchWords* d_words = nullptr;
+  bool words_dirty = true;        // a search that did not end may have left counts behind
   void* d_tc = nullptr;           // packed bf16 operand images (tensor-core path)
   void* d_partial = nullptr;      // per-candidate partial objective between tensor-core passes
   size_t partial_bytes = 0;
@@ -382,6 +391,7 @@ struct mf_ctx {
   void* d_ga_out = nullptr;       // best genome [N] int32, then its fitness (float), then the seed (u64)
   void* d_gap = nullptr;          // cooperative GA kernel: byte genomes, fitness, barrier flags, CTA bests
   size_t gap_bytes = 0;
+  uint32_t ga_tag = 0;            // record tags used so far (0: the buffer is not cleared)
   int ga_cap = 0;
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t ga_exec = nullptr;
@@ -390,7 +400,6 @@ struct mf_ctx {
   mf_ga_params ga_key{};
   // instrumentation
   mf_stats stats{};
-  cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
 };
 
 namespace mf {
@@ -429,7 +438,19 @@ struct RangeArgs {
   float* lists_s;       // [grid][k]
   uint64_t* lists_i;    // [grid][k]
   unsigned long long* count;
+  unsigned long long* start;  // the first launch's start, ns (null: not wanted)
 };
+
+// Nanoseconds of the device's global timer.
+__device__ __forceinline__ unsigned long long device_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+  return t;
+}
+// Called by every CTA of a range launch.
+__device__ __forceinline__ void stamp_start(const RangeArgs& R) {
+  if (R.first && R.start && blockIdx.x == 0 && threadIdx.x == 0) *R.start = device_ns();
+}
 bool f32_supported(const Params& P);
 size_t f32_smem_bytes(const Params& P, int k, bool& resident);
 int f32_grid(const mf_ctx* c);
@@ -446,16 +467,20 @@ mf_status f32_score_list(mf_ctx* c, const uint64_t* idx, const int32_t* genes, u
 // UINT64_MAX, no predictions); an index out of range raises no status here.
 mf_status f32_predict_shortlist(mf_ctx* c, const uint64_t* idx, uint64_t n, float* pred, cudaStream_t s);
 
-// Where a reduction leaves the top-k, and with it (where count is given) the feasible
-// count and the status word: device memory, or pinned host memory, which the kernel
-// writes itself instead of three or four copies after it.
+// What comes with the top-k: the words above and the status word.
+struct SearchTail {
+  unsigned long long count, t[3];  // t[2]: the end
+  uint32_t status;
+};
+// Where a reduction leaves the top-k, and with it (where tail is given) the rest: device
+// memory, or pinned host memory, which the kernel writes itself instead of three or four
+// copies after it.  The reduction that delivers the tail also clears the words.
 struct ResultOut {
-  uint64_t* idx;                        // [k]
-  float* score;                         // [k]
-  unsigned long long* count;
-  uint32_t* status;
-  const unsigned long long* count_src;  // device
-  const uint32_t* status_src;           // device
+  uint64_t* idx;        // [k]
+  float* score;         // [k]
+  SearchTail* tail;
+  SearchWords* words;   // device
+  const uint32_t* status;  // device
 };
 // Merge of per-CTA sorted lists into one sorted top-k (tmp: 2 ceil(nlists / 2) k entries).
 mf_status merge_lists(const float* ls, const uint64_t* li, int nlists, int k, float* tmp_s, uint64_t* tmp_i,
