@@ -803,10 +803,16 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
     if constexpr (KW == 8) tmem_st_x8(tA + lane_off, v);
     else tmem_st_x16(tA + lane_off, v);
   };
+  // List mode: this thread's index of a tile, kEmptyIdx past the list's end.  It is read a
+  // whole tile before its digits are wanted, so the read's latency is off the chain.
+  auto list_index = [&](uint64_t tile) -> uint64_t {
+    const uint64_t t = tile * 128 + row;
+    return MODE == kTcList && t < n ? __ldg(L.idx + t) : kEmptyIdx;
+  };
   // Digits of tile `tile` (in shared memory: written to buffer `into`).  Range mode:
   // from the index at the first tile, else `from` (the previous tile's digits) stepped
-  // by the tile stride.
-  auto tile_digits = [&](uint64_t tile, uint8_t* into, DS from, bool first) -> DS {
+  // by the tile stride.  List mode: of the index `at`.
+  auto tile_digits = [&](uint64_t tile, uint8_t* into, DS from, bool first, uint64_t at) -> DS {
     const uint64_t t = tile * 128 + row;
     if constexpr (RD) {
       if (first) {
@@ -840,12 +846,23 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
       }
       return into;
     } else {
-      uint64_t idx = t < n ? L.idx[t] : 0;
-      if (t < n && idx >= P.total) {
-        atomicOr(P.status, kStatusBadInput);
+      uint64_t idx = at;
+      if (idx >= P.total) {
+        if (t < n) atomicOr(P.status, kStatusBadInput);
         idx = 0;  // compute on candidate 0, discard at the end
       }
-      for (int i = 0; i < N; ++i) into[i * 128 + row] = (uint8_t)digit_of(P, idx, i);
+      // last model first, one division each (the quotient goes on to the next model)
+      if (P.total <= 0x100000000ull) {
+        uint32_t q = (uint32_t)idx;
+#pragma unroll (NM > 0 ? NM : 1)
+        for (int i = N - 1; i >= 0; --i) {
+          const uint32_t K = (uint32_t)P.K[i], qn = q / K;
+          into[i * 128 + row] = (uint8_t)(q - qn * K);
+          q = qn;
+        }
+      } else {
+        for (int i = 0; i < N; ++i) into[i * 128 + row] = (uint8_t)digit_of(P, idx, i);
+      }
       return into;
     }
   };
@@ -880,8 +897,8 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
                 make_uint4(0u, 0u, 0u, 0u)};
   };
   // Digits of a pipeline's first tile and its first A1 row (model m0) with the aggregate words.
-  auto load_tile = [&](uint64_t tile, uint8_t* into, float& vram) -> DS {
-    const DS d = tile_digits(tile, into, DS{}, true);
+  auto load_tile = [&](uint64_t tile, uint8_t* into, float& vram, uint64_t at) -> DS {
+    const DS d = tile_digits(tile, into, DS{}, true, at);
     write_a1(m0, d, true, tile_agg(d, vram));
     return d;
   };
@@ -917,16 +934,23 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
     a = tmem_ld_x1(tD3 + lane_off + (uint32_t)j);
     b = tmem_ld_x1(tD3 + lane_off + (uint32_t)(half3 + j));
   };
-  auto add_model = [&](int j, uint32_t a, uint32_t b, DS dg, uint64_t tile_f) {
+  // (list mode: `at` is the row's index)
+  auto add_model = [&](int j, uint32_t a, uint32_t b, DS dg, uint64_t tile_f, uint64_t at) {
     tmem_wait_ld_2(a, b);
     // (HF: the products are exact, powers of two, so this rounds once, like the sums)
     const float thr = tc_out(P, HF ? fmaf(__uint_as_float(a), s_b3[j][HF ? 2 : 0], s_b3[j][0]) : __uint_as_float(a) + s_b3[j][0]);
     const float lat = tc_out(P, HF ? fmaf(__uint_as_float(b), s_b3[j][HF ? 3 : 1], s_b3[j][1]) : __uint_as_float(b) + s_b3[j][1]);
     if (MODE == kTcList && L.pred) {
-      const uint64_t t = tile_f * 128 + row;
-      if (t < n && L.idx[t] < P.total) {
-        L.pred[(t * N + j) * 2 + 0] = thr;
-        L.pred[(t * N + j) * 2 + 1] = lat;
+      // (one 8-byte store where the caller's array allows it: always, but for a bare
+      // pointer that is not 8-byte aligned)
+      float* to = L.pred + ((tile_f * 128 + row) * N + j) * 2;
+      if (at < P.total) {
+        if ((reinterpret_cast<uintptr_t>(L.pred) & 7u) == 0) {
+          *reinterpret_cast<float2*>(to) = make_float2(thr, lat);
+        } else {
+          to[0] = thr;
+          to[1] = lat;
+        }
       }
     }
     if (UT) {  // Eq. 3 utility, floors f >= tau
@@ -958,14 +982,14 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
       bar_i = tk.li[kcap - 1];
     }
   };
-  auto finish_tile = [&](uint64_t tile_f, float vram) {
+  auto finish_tile = [&](uint64_t tile_f, float vram, uint64_t at) {
     const uint64_t t = tile_f * 128 + row;
     bool valid = t < n;
     uint64_t idx;
     if (MODE == kTcRange) {
       idx = R.base + t;
     } else {
-      idx = valid ? L.idx[t] : 0;
+      idx = at;
       valid = valid && idx < P.total;
     }
     float J = acc_J, pen = acc_pen;
@@ -1054,8 +1078,10 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
     int buf = 0;
     float vram_cur = 0.f, vram_prev = 0.f, vram_nx = 0.f;  // VRAM demand of this thread's rows
     DS dcur{}, dprev{}, dnx{};
+    // list mode: the row's index in the previous, this and the next two tiles
+    uint64_t x_prev = kEmptyIdx, x_cur = list_index(tile), x_nx = list_index(tile + gstride), x_nx2 = kEmptyIdx;
     if (tile * 128 < n) {
-      dcur = load_tile(tile, digits, vram_cur);
+      dcur = load_tile(tile, digits, vram_cur, x_cur);
       signal();  // ones block and the first A1 row
     }
     // the previous tile is finished once its last layer 3 (issued at the end of that
@@ -1070,7 +1096,8 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
       uint8_t* buf_nx = digits + (buf ^ 1) * (MF_MAX_MODELS * 128);  // (shared-memory digits)
       const bool has_next = (tile + gstride) * 128 < n;
       auto stage = [&](int i) {
-        if (has_next && i == st_dig) dnx = tile_digits(tile + gstride, buf_nx, dcur, false);
+        if (has_next && i == st_dig) dnx = tile_digits(tile + gstride, buf_nx, dcur, false, x_nx);
+        if (i == st_dig) x_nx2 = list_index(tile + 2 * gstride);
         if (has_next && i == st_agg) aw_nx = tile_agg(dnx, vram_nx);
       };
       // Work off the critical path, while layer 2 of model i runs (or, with one hidden
@@ -1084,13 +1111,13 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
           load_model(i - 1, oa, ob);
           stage(i);
           if (i + 1 < m1) next_a1(i + 1, dcur);
-          add_model(i - 1, oa, ob, dcur, tile);
+          add_model(i - 1, oa, ob, dcur, tile, x_cur);
         } else {
           if (pending) load_model(m1 - 1, oa, ob);
           if (i + 1 < m1) next_a1(i + 1, dcur);
           if (pending) {  // (before the stage: with one model it overwrites these digits)
-            add_model(m1 - 1, oa, ob, dprev, tile - gstride);
-            finish_tile(tile - gstride, vram_prev);
+            add_model(m1 - 1, oa, ob, dprev, tile - gstride, x_prev);
+            finish_tile(tile - gstride, vram_prev, x_prev);
           }
           stage(i);
         }
@@ -1152,6 +1179,9 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
       pending = true;
       dprev = dcur;
       dcur = dnx;
+      x_prev = x_cur;
+      x_cur = x_nx;
+      x_nx = x_nx2;
       vram_prev = vram_cur;
       vram_cur = vram_nx;
       buf ^= 1;
@@ -1160,8 +1190,8 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
       await_b();
       uint32_t oa, ob;
       load_model(m1 - 1, oa, ob);
-      add_model(m1 - 1, oa, ob, dprev, tile - gstride);
-      finish_tile(tile - gstride, vram_prev);
+      add_model(m1 - 1, oa, ob, dprev, tile - gstride, x_prev);
+      finish_tile(tile - gstride, vram_prev, x_prev);
     }
   }
   if (MODE == kTcRange && (!MP || T.pass_last) && !issuer) {  // what is still queued joins the list
@@ -1209,29 +1239,35 @@ uint16_t f2bf(float f) {  // round to nearest even
   return (uint16_t)(u >> 16);
 }
 
-// fp16 bits of |f| < 65504 (nearest even); `rounded`: the value they stand for.
-uint16_t f2half(float f, float& rounded) {
-  uint32_t u;
+// fp16 bits of |f| < 65504 (nearest even); `rounded`: the value they stand for.  Without a
+// branch, so that loops over it vectorise.
+inline uint16_t f2half(float f, float& rounded) {
+  uint32_t u, m, r;
   std::memcpy(&u, &f, 4);
-  const uint32_t sign = (u >> 16) & 0x8000u;
-  u &= 0x7FFFFFFFu;
-  float v;
-  uint32_t bits;
-  if (u < 0x38800000u) {  // below 2^-14: multiples of 2^-24, which the sum with 1/2 rounds to
-    std::memcpy(&v, &u, 4);
-    v += 0.5f;
-    uint32_t m;
-    std::memcpy(&m, &v, 4);
-    bits = m - 0x3F000000u;
-    v -= 0.5f;
-  } else {
-    u += 0xFFFu + ((u >> 13) & 1u);
-    u &= ~0x1FFFu;
-    std::memcpy(&v, &u, 4);
-    bits = (u - 0x38000000u) >> 13;
+  const uint32_t sign = u & 0x80000000u;
+  u ^= sign;
+  // from 2^-14 on: the mantissa rounded to 10 bits
+  const uint32_t un = (u + 0xFFFu + ((u >> 13) & 1u)) & ~0x1FFFu;
+  // below: multiples of 2^-24, which the sum with 1/2 rounds to
+  float a;
+  std::memcpy(&a, &u, 4);
+  const float v = a + 0.5f, vs = v - 0.5f;
+  std::memcpy(&m, &v, 4);
+  std::memcpy(&r, &vs, 4);
+  const uint32_t small = u < 0x38800000u ? 0xFFFFFFFFu : 0u;
+  const uint32_t bits = (small & (m - 0x3F000000u)) | (~small & ((un - 0x38000000u) >> 13));
+  const uint32_t val = ((small & r) | (~small & un)) | sign;
+  std::memcpy(&rounded, &val, 4);
+  return (uint16_t)((sign >> 16) | bits);
+}
+
+// Hi and lo parts of n <= 8 values.
+inline void split_half(const float* v, int n, uint16_t* hi, uint16_t* lo) {
+  for (int k = 0; k < n; ++k) {
+    float r, rest;
+    hi[k] = f2half(v[k], r);
+    lo[k] = f2half(v[k] - r, rest);
   }
-  rounded = sign ? -v : v;
-  return (uint16_t)(sign | bits);
 }
 
 float bf2f(uint16_t b) {
@@ -1308,6 +1344,8 @@ template <int MODE, bool MP, bool UT>
 TcFn tc_kernel_mode(const TcArgs& T, int n_models) {
   // the exact fp32 variants (d_L 8, 64-64): S1 = k1 / 8, S2 = h1 / 8 + 1, S3 = hl / 8 for tf32
   if (T.tf == kXmTf32) return k_score_tc<MODE, 16, 8, 2, 9, 8, 16, MP, UT, 0, kXmTf32>;
+  // (a compile-time model count with register digits, which serves bf16, is slower here:
+  // 24^6 32.9 ms against 31.4 with the run-time loop)
   if (T.tf == kXmHalf) return k_score_tc<MODE, 8, 4, 1, 5, 4, 16, MP, UT, 0, kXmHalf>;
   // S1 = k1 / 16, S2 = h1 / 16 + 1 (the b2 step), S3 = hl / 16
   if (T.kw == 8 && T.dle == 8 && T.h1 == 64 && T.h2 == 64 && T.n3 == 16) {
@@ -1535,14 +1573,29 @@ mf_status tc_prepare_exact(mf_ctx* c, const TcHost& h) {
   return MF_OK;
 }
 
-// The powers of two of the fp16 variant, and whether it serves this problem.
+// The powers of two of the fp16 variant (all exact in fp32).
 struct HalfScales {
-  double cagg[3];                                // aggregate columns (shared by the models)
-  std::vector<double> cx, t, u, v;               // [N][dl] features, [N][h1], [N][h2] units, [N][2] outputs
+  float cagg[3];                    // aggregate columns (shared by the models)
+  std::vector<float> cx, t, u, v;   // [N][dl] features, [N][h1], [N][h2] units, [N][2] outputs
 };
 
 // 2^e with m 2^e in (2^(top - 1), 2^top]; 1 for m = 0.
-double pow2_to(double m, int top) { return m > 0.0 ? std::ldexp(1.0, top - (int)std::ceil(std::log2(m))) : 1.0; }
+float pow2_to(float m, int top) {
+  if (m == 0.f) return 1.f;
+  int e;
+  const float f = std::frexp(m, &e);
+  return std::ldexp(1.f, top - (f == 0.5f ? e - 1 : e));
+}
+
+// sum of |w_k| x_k, in eight partial sums (so that it vectorises)
+float abs_dot(const float* w, const float* x, int n) {
+  float s[8] = {};
+  int k = 0;
+  for (; k + 8 <= n; k += 8)
+    for (int j = 0; j < 8; ++j) s[j] += std::fabs(w[k + j]) * x[k + j];
+  for (; k < n; ++k) s[0] += std::fabs(w[k]) * x[k];
+  return ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+}
 
 // Scales from the largest value that each feature column, the aggregate and each unit can
 // take over the option tables (|W| times the inputs' maxima, plus |b|): inputs to 2^4, the
@@ -1557,86 +1610,87 @@ double pow2_to(double m, int top) { return m > 0.0 ? std::ldexp(1.0, top - (int)
 bool half_ranges(const Params& P, const TcHost& host, HalfScales& S) {
   const float *w = host.w, *x = host.x, *dem4 = host.dem4;
   const int N = P.n_models, dl = P.d_local, h1 = P.h1, h2 = P.h2, din = P.d_in;
-  auto fits = [](double m) { return m == 0.0 || (m > 1e-30 && m < 1e30); };
-  double amax[3], amin[3];
+  // (NaN fails every comparison; the bounds carry a margin for their own rounding)
+  auto fits = [](float m) { return m == 0.f || (m > 1e-15f && m < 1e15f); };
+  constexpr float kMargin = 1.0001f;
+  float amax[3], amin[3];
   for (int q = 0; q < 3; ++q) {
-    double hi = 0.0, lo = 0.0;
+    float hi = 0.f, lo = 0.f;
     bool positive = true;
     for (int i = 0; i < N; ++i) {
-      double m = 0.0, l = INFINITY;
+      float m = 0.f, l = INFINITY;
       for (int o = 0; o < P.K[i]; ++o) {
-        const double d = dem4[(size_t)(P.off[i] + o) * 4 + q];
+        const float d = dem4[(size_t)(P.off[i] + o) * 4 + q];
         if (!std::isfinite(d)) return false;
         m = std::fmax(m, std::fabs(d));
         l = std::fmin(l, d);
       }
       hi += m;
       lo += l;
-      positive = positive && l >= 0.0;
+      positive = positive && l >= 0.f;
     }
-    if (!std::isfinite(P.agg_scale[q])) return false;
-    amax[q] = hi * std::fabs(P.agg_scale[q]) * (1.0 + 1e-5);  // (the kernel sums in fp32)
-    amin[q] = positive ? lo * std::fabs(P.agg_scale[q]) : 0.0;
+    amax[q] = hi * std::fabs(P.agg_scale[q]) * kMargin;
+    amin[q] = positive ? lo * std::fabs(P.agg_scale[q]) : 0.f;
     if (!fits(amax[q])) return false;
     S.cagg[q] = pow2_to(amax[q], 4);
   }
-  if (!std::isfinite(P.agg_scale[3])) return false;
   S.cx.resize((size_t)N * dl);
   S.t.resize((size_t)N * h1);
   S.u.resize((size_t)N * h2);
   S.v.resize((size_t)N * 2);
-  std::vector<double> hb(h1);
-  std::vector<float> xs, aw(dl);  // |x| scaled; a unit's |W1| scaled
+  float hb[MF_MAX_HIDDEN], in[MF_MAX_D_LOCAL + 4];
+  std::vector<float> xs;  // |x| scaled
   for (int i = 0; i < N; ++i) {
     const float* W1 = w + (size_t)i * P.per_model;
     const float* b1 = W1 + (size_t)h1 * din;
     const float* W2 = b1 + h1;
     const float* b2 = W2 + (size_t)h2 * h1;
     const float* W3 = b2 + h2;
-    for (int64_t e = 0; e < P.per_model; ++e)
-      if (!std::isfinite(W1[e])) return false;
     const float* xi = x + (size_t)P.off[i] * dl;
-    double xmax[MF_MAX_D_LOCAL];
     for (int k = 0; k < dl; ++k) {
-      xmax[k] = 0.0;
+      in[k] = 0.f;
       for (int o = 0; o < P.K[i]; ++o) {
-        if (!std::isfinite(xi[(size_t)o * dl + k])) return false;
-        xmax[k] = std::fmax(xmax[k], std::fabs((double)xi[(size_t)o * dl + k]));
+        const float v = std::fabs(xi[(size_t)o * dl + k]);
+        if (!std::isfinite(v)) return false;
+        in[k] = std::fmax(in[k], v);
       }
-      if (!fits(xmax[k])) return false;
-      S.cx[(size_t)i * dl + k] = pow2_to(xmax[k], 4);
+      if (!fits(in[k])) return false;
+      S.cx[(size_t)i * dl + k] = pow2_to(in[k], 4);
     }
-    xs.resize((size_t)P.K[i] * dl);
-    for (size_t e = 0; e < xs.size(); ++e) xs[e] = (float)(std::fabs((double)xi[e]) * S.cx[(size_t)i * dl + e % dl]);
+    for (int q = 0; q < 3; ++q) in[dl + q] = amax[q];
+    xs.clear();
     for (int j = 0; j < h1; ++j) {
-      const double bb = std::fabs((double)b1[j] + (double)W1[(size_t)j * din + dl + 3] * P.agg_scale[3] * N);
-      double m = bb, least = bb;
-      for (int k = 0; k < dl; ++k) m += std::fabs((double)W1[(size_t)j * din + k]) * xmax[k];
-      for (int q = 0; q < 3; ++q) {
-        m += std::fabs((double)W1[(size_t)j * din + dl + q]) * amax[q];
-        least += std::fabs((double)W1[(size_t)j * din + dl + q]) * amin[q];
-      }
+      const float* wj = W1 + (size_t)j * din;
+      const float bb = std::fabs(b1[j]) + std::fabs(wj[dl + 3] * P.agg_scale[3] * (float)N);
+      const float m = (abs_dot(wj, in, dl + 3) + bb) * kMargin;
       if (!fits(m)) return false;
       hb[j] = m;
-      const double t = S.t[(size_t)i * h1 + j] = pow2_to(m, 9);
-      if (m == 0.0 || least * t >= 1.0) continue;
-      for (int k = 0; k < dl; ++k) aw[k] = (float)(std::fabs((double)W1[(size_t)j * din + k]) * t / S.cx[(size_t)i * dl + k]);
-      for (int o = 0; o < P.K[i]; ++o) {
-        float sum = (float)(least * t);
-        for (int k = 0; k < dl; ++k) sum += aw[k] * xs[(size_t)o * dl + k];
-        if (sum < 1.f) return false;
+      const float t = S.t[(size_t)i * h1 + j] = pow2_to(m, 9);
+      const float cst = std::fabs(b1[j] + wj[dl + 3] * P.agg_scale[3] * (float)N);
+      const float least = (cst + abs_dot(wj + dl, amin, 3)) * t;
+      if (m == 0.f || least >= 1.f) continue;
+      if (xs.empty()) {
+        xs.resize((size_t)P.K[i] * dl);
+        for (size_t e = 0; e < xs.size(); ++e) xs[e] = std::fabs(xi[e]) * S.cx[(size_t)i * dl + e % dl];
+      }
+      float aw[MF_MAX_D_LOCAL];
+      for (int k = 0; k < dl; ++k) aw[k] = wj[k] * t / S.cx[(size_t)i * dl + k];
+      for (int o = 0; o < P.K[i]; ++o)
+        if (!(least + abs_dot(aw, xs.data() + (size_t)o * dl, dl) >= 1.f)) return false;
+    }
+    float top[2] = {0.f, 0.f};
+    for (int j = 0; j < h2; ++j) {
+      const float m = (abs_dot(W2 + (size_t)j * h1, hb, h1) + std::fabs(b2[j])) * kMargin;
+      if (!fits(m)) return false;
+      const float u = S.u[(size_t)i * h2 + j] = pow2_to(m, 14);
+      for (int r = 0; r < 2; ++r) {
+        const float v = std::fabs(W3[(size_t)r * h2 + j]) / u;
+        if (!std::isfinite(v)) return false;
+        top[r] = std::fmax(top[r], v);
       }
     }
-    double top[2] = {0.0, 0.0};
-    for (int j = 0; j < h2; ++j) {
-      double m = std::fabs((double)b2[j]);
-      for (int k = 0; k < h1; ++k) m += std::fabs((double)W2[(size_t)j * h1 + k]) * hb[k];
-      if (!fits(m)) return false;
-      const double u = S.u[(size_t)i * h2 + j] = pow2_to(m, 14);
-      for (int r = 0; r < 2; ++r) top[r] = std::fmax(top[r], std::fabs((double)W3[(size_t)r * h2 + j]) / u);
-    }
     for (int r = 0; r < 2; ++r) {
-      if (!fits(top[r])) return false;
+      if (!fits(top[r]) || !std::isfinite(W3[2 * h2 + r])) return false;
       S.v[(size_t)i * 2 + r] = pow2_to(top[r], 6);
     }
   }
@@ -1672,7 +1726,7 @@ mf_status tc_prepare_half(mf_ctx* c, const TcHost& h) {
   T.col_hlo = T.col_ones + 8;
   T.col_a = T.col_hlo + h1 / 2;
   T.pipe_stride = T.col_a + 16 - T.col_h;
-  for (int q = 0; q < 3; ++q) T.cagg[q] = (float)S.cagg[q];
+  for (int q = 0; q < 3; ++q) T.cagg[q] = S.cagg[q];
   // per model: B1 [h1 x 16] hi, lo; B2 [h2 x (h1 + 16)] hi (its last K-step holds b2 hi, lo
   // against the ones block), [h2 x h1] lo; B3 [16 x hl] hi, lo
   const int k2 = h1 + 16;
@@ -1682,53 +1736,53 @@ mf_status tc_prepare_half(mf_ctx* c, const TcHost& h) {
   T.img_lo3 = (uint32_t)b3;
   T.img_model = (uint32_t)(2 * b1 + b2 + b2lo + 2 * b3);
   std::vector<unsigned char> img(round_up((int)(T.img_model * N), 16), 0);
-  auto split = [](float v, uint16_t& hi, uint16_t& lo) {
-    float rounded, rest;
-    hi = f2half(v, rounded);
-    lo = f2half(v - rounded, rest);
-  };
-  // (scaling by powers of two is exact in fp32)
-  auto put = [&](size_t at, size_t at_lo, float v) {
-    uint16_t hi, lo;
-    split(v, hi, lo);
-    std::memcpy(img.data() + at, &hi, 2);
-    std::memcpy(img.data() + at_lo, &lo, 2);
+  // n columns (a multiple of 8) of row r of an image with kdim columns, hi and lo image apart
+  auto put_row = [&](size_t at, int kdim, size_t at_lo, int kdim_lo, int r, const float* v, int n) {
+    unsigned char* ph = img.data() + at + umma_off(r, 0, kdim);
+    unsigned char* pl = img.data() + at_lo + umma_off(r, 0, kdim_lo);
+    for (int k = 0; k < n; k += 8, ph += 128, pl += 128) {
+      uint16_t hi[8], lo[8];
+      split_half(v + k, 8, hi, lo);
+      std::memcpy(ph, hi, 16);
+      std::memcpy(pl, lo, 16);
+    }
   };
   const double s3 = P.agg_scale[3];
+  float row[MF_MAX_HIDDEN], it[MF_MAX_HIDDEN], iu[MF_MAX_HIDDEN];  // a row; 1 / t, 1 / u
   for (int i = 0; i < N; ++i) {
     const float* W1 = w + (size_t)i * P.per_model;
     const float* bb1 = W1 + (size_t)h1 * din;
     const float* W2 = bb1 + h1;
     const float* bb2 = W2 + (size_t)h2 * h1;
     const float* W3 = bb2 + h2;
-    float it[MF_MAX_HIDDEN], iu[MF_MAX_HIDDEN];  // 1 / t, 1 / u
-    for (int k = 0; k < h1; ++k) it[k] = (float)(1.0 / S.t[(size_t)i * h1 + k]);
-    for (int k = 0; k < h2; ++k) iu[k] = (float)(1.0 / S.u[(size_t)i * h2 + k]);
-    const double *cx = &S.cx[(size_t)i * dl], *t = &S.t[(size_t)i * h1], *u = &S.u[(size_t)i * h2], *v = &S.v[(size_t)i * 2];
+    const float *cx = &S.cx[(size_t)i * dl], *t = &S.t[(size_t)i * h1], *u = &S.u[(size_t)i * h2], *v = &S.v[(size_t)i * 2];
+    for (int k = 0; k < h1; ++k) it[k] = 1.f / t[k];
+    for (int k = 0; k < h2; ++k) iu[k] = 1.f / u[k];
     T.off_b1[i] = T.img_model * i;
     T.off_b2[i] = T.off_b1[i] + (uint32_t)(2 * b1);
     T.off_b3[i] = T.off_b2[i] + (uint32_t)(b2 + b2lo);
     for (int j = 0; j < h1; ++j) {
-      auto put1 = [&](int k, double val) {  // (the constant column rounds to fp32 first)
-        const size_t at = T.off_b1[i] + umma_off(j, k, T.k1);
-        put(at, at + b1, (float)val);
-      };
-      for (int k = 0; k < dl; ++k) put1(k, W1[(size_t)j * din + k] * t[j] / cx[k]);
-      for (int q = 0; q < 3; ++q) put1(dl + q, W1[(size_t)j * din + dl + q] * t[j] / S.cagg[q]);
+      const float* wj = W1 + (size_t)j * din;
+      std::memset(row, 0, sizeof(float) * 16);
+      for (int k = 0; k < dl; ++k) row[k] = wj[k] * t[j] / cx[k];
+      for (int q = 0; q < 3; ++q) row[dl + q] = wj[dl + q] * t[j] / S.cagg[q];
       // the constant-1 column: b1 plus the weight of the constant feature N * s_3
-      put1(dl + 3, ((double)bb1[j] + (double)W1[(size_t)j * din + dl + 3] * s3 * N) * t[j]);
+      row[dl + 3] = (float)(((double)bb1[j] + (double)wj[dl + 3] * s3 * N) * t[j]);
+      put_row(T.off_b1[i], T.k1, T.off_b1[i] + b1, T.k1, j, row, 16);
     }
     for (int j = 0; j < h2; ++j) {
-      for (int k = 0; k < h1; ++k)
-        put(T.off_b2[i] + umma_off(j, k, k2), T.off_b2[i] + b2 + umma_off(j, k, h1), W2[(size_t)j * h1 + k] * (float)u[j] * it[k]);
-      put(T.off_b2[i] + umma_off(j, h1, k2), T.off_b2[i] + umma_off(j, h1 + 1, k2), bb2[j] * (float)u[j]);
+      for (int k = 0; k < h1; ++k) row[k] = W2[(size_t)j * h1 + k] * u[j] * it[k];
+      put_row(T.off_b2[i], k2, T.off_b2[i] + b2, h1, j, row, h1);
+      uint16_t hi, lo;
+      row[0] = bb2[j] * u[j];
+      split_half(row, 1, &hi, &lo);
+      std::memcpy(img.data() + T.off_b2[i] + umma_off(j, h1, k2), &hi, 2);
+      std::memcpy(img.data() + T.off_b2[i] + umma_off(j, h1 + 1, k2), &lo, 2);
     }
     for (int r = 0; r < 2; ++r) {
-      T.back[i][r] = (float)(1.0 / v[r]);
-      for (int k = 0; k < hl; ++k) {
-        const size_t at = T.off_b3[i] + umma_off(r * (T.n3 / 2) + i, k, hl);
-        put(at, at + b3, W3[(size_t)r * hl + k] * (float)v[r] * iu[k]);
-      }
+      T.back[i][r] = 1.f / v[r];
+      for (int k = 0; k < hl; ++k) row[k] = W3[(size_t)r * hl + k] * v[r] * iu[k];
+      put_row(T.off_b3[i], hl, T.off_b3[i] + b3, hl, r * (T.n3 / 2) + i, row, hl);
     }
   }
   T.img_total = (uint32_t)img.size();
@@ -1736,13 +1790,13 @@ mf_status tc_prepare_half(mf_ctx* c, const TcHost& h) {
   set_pass(T, 0, nullptr);
   std::vector<uint32_t> xw((size_t)sumK * T.kw, 0u);
   for (int i = 0; i < N; ++i)
-    for (int r = P.off[i]; r < P.off[i] + P.K[i]; ++r)
-      for (int k = 0; k < dl; ++k) {
-        uint16_t hi, lo;
-        split(x[(size_t)r * dl + k] * (float)S.cx[(size_t)i * dl + k], hi, lo);
-        xw[(size_t)r * T.kw + k / 2] |= (uint32_t)hi << (16 * (k & 1));
-        xw[(size_t)r * T.kw + 4 + k / 2] |= (uint32_t)lo << (16 * (k & 1));
-      }
+    for (int r = P.off[i]; r < P.off[i] + P.K[i]; ++r) {
+      uint16_t hi[8], lo[8];  // (d_L 8)
+      for (int k = 0; k < dl; ++k) row[k] = x[(size_t)r * dl + k] * S.cx[(size_t)i * dl + k];
+      split_half(row, dl, hi, lo);
+      std::memcpy(&xw[(size_t)r * T.kw], hi, 16);
+      std::memcpy(&xw[(size_t)r * T.kw + 4], lo, 16);
+    }
   layout_smem(P, T, 0);
   if (T.sm_total > kSmemLimit) return MF_EUNSUPPORTED;
   const size_t o_xw = round_up((int)img.size(), 256);

@@ -121,8 +121,28 @@ def _check(status: int, where: str):
         raise MFError(status, where, _lib.mf_last_error().decode())
 
 
-def _stream(device) -> C.c_void_p:
-    return C.c_void_p(torch.cuda.current_stream(device).cuda_stream)
+def _stream(device) -> int:
+    """torch's current stream on a device (an ordinal, or a tensor's device), as an address."""
+    return torch._C._cuda_getCurrentRawStream(device if isinstance(device, int) else device.index)
+
+
+def _ptr(a) -> int:
+    """Address of a numpy array (``a.ctypes`` builds an object for it on every use)."""
+    return a.__array_interface__["data"][0]
+
+
+def _search_result(k: int):
+    """Result arrays of a search and the struct that points to them."""
+    ti = np.empty(k, dtype=np.uint64)
+    ts = np.empty(k, dtype=np.float32)
+    return _Result(0, 0.0, 0, k, _ptr(ti), _ptr(ts)), ti, ts
+
+
+def _as(a, dtype) -> np.ndarray:
+    """`a` as a contiguous array of the type (itself where it is one)."""
+    if type(a) is np.ndarray and a.dtype == dtype and a.flags.c_contiguous:
+        return a
+    return np.ascontiguousarray(a, dtype=dtype)
 
 
 def _ga(params: dict) -> _GAParams:
@@ -161,9 +181,7 @@ def search_exhaustive_noalloc(prob: dict, k: int, chunk: int = 0, device: int | 
     Context.search."""
     device = torch.cuda.current_device() if device is None else int(device)
     p, _keep = _problem_struct(prob, device, "fp32")
-    ti = np.empty(k, dtype=np.uint64)
-    ts = np.empty(k, dtype=np.float32)
-    r = _Result(0, 0.0, 0, k, ti.ctypes.data, ts.ctypes.data)
+    r, ti, ts = _search_result(k)
     _check(_lib.mf_search_exhaustive_noalloc(C.byref(p), int(k), int(chunk), C.byref(r),
                                               _stream(device)), "mf_search_exhaustive_noalloc")
     return dict(best_idx=int(r.best_idx), best_score=float(r.best_score),
@@ -183,6 +201,9 @@ class Context:
             _check(_lib.mf_create(C.byref(p), C.byref(h)), "mf_create")
         self._h = h
         self.precision = prec
+        v = C.c_uint64()  # (fixed for the context's life)
+        _check(_lib.mf_space_size(self._h, C.byref(v)), "mf_space_size")
+        self._space = int(v.value)
 
     # -- lifetime -----------------------------------------------------------------
     def close(self):
@@ -205,9 +226,7 @@ class Context:
     # -- calls ----------------------------------------------------------------------
     @property
     def space_size(self) -> int:
-        v = C.c_uint64()
-        _check(_lib.mf_space_size(self._h, C.byref(v)), "mf_space_size")
-        return int(v.value)
+        return self._space
 
     def set_objective(self, sla=None, obj_w=None):
         s = None if sla is None else _f32(sla)
@@ -232,9 +251,7 @@ class Context:
 
     def search(self, k: int, lo: int = 0, hi: int | None = None, chunk: int = 0) -> dict:
         hi = self.space_size if hi is None else int(hi)
-        ti = np.empty(k, dtype=np.uint64)
-        ts = np.empty(k, dtype=np.float32)
-        r = _Result(0, 0.0, 0, k, ti.ctypes.data, ts.ctypes.data)
+        r, ti, ts = _search_result(k)
         _check(_lib.mf_search_range(self._h, int(lo), hi, int(k), int(chunk), C.byref(r),
                                     _stream(self.device)), "mf_search_range")
         return dict(best_idx=int(r.best_idx), best_score=float(r.best_score),
@@ -267,27 +284,17 @@ class Context:
         g = _ga(params)
         genome = np.zeros(self.n_models, dtype=np.int32)
         fit = C.c_float()
-        _check(_lib.mf_ga_run(self._h, C.byref(g), int(seed), genome.ctypes.data, C.byref(fit),
+        _check(_lib.mf_ga_run(self._h, C.byref(g), int(seed), _ptr(genome), C.byref(fit),
                               _stream(self.device)), "mf_ga_run")
         return float(fit.value), genome
 
     # -- fixed-context mode ---------------------------------------------------
     @staticmethod
     def _fc_params(fc: dict):
-        keep = {
-            "obs": np.ascontiguousarray(fc["obs"], dtype=np.float32),
-            "variant": np.ascontiguousarray(fc["variant"], dtype=np.int32),
-            "quality": np.ascontiguousarray(fc["quality"], dtype=np.float32),
-            "f_min": np.ascontiguousarray(fc["f_min"], dtype=np.float32),
-            "f_max": np.ascontiguousarray(fc["f_max"], dtype=np.float32),
-            "omega": np.ascontiguousarray(fc["omega"], dtype=np.float32),
-            "tau": np.ascontiguousarray(fc["tau"], dtype=np.float32),
-            "reload_cost": np.ascontiguousarray(fc["reload_cost"], dtype=np.float32),
-            "prev_variant": np.ascontiguousarray(fc["prev_variant"], dtype=np.int32),
-        }
-        p = _FcParams(*(keep[k].ctypes.data for k in ("obs", "variant", "quality", "f_min", "f_max", "omega",
-                                                       "tau", "reload_cost", "prev_variant")),
-                      float(fc["alpha"]), float(fc["beta"]), float(fc["delta"]))
+        f, i = np.dtype(np.float32), np.dtype(np.int32)
+        keep = [_as(fc[k], t) for k, t in (("obs", f), ("variant", i), ("quality", f), ("f_min", f), ("f_max", f),
+                                           ("omega", f), ("tau", f), ("reload_cost", f), ("prev_variant", i))]
+        p = _FcParams(*map(_ptr, keep), float(fc["alpha"]), float(fc["beta"]), float(fc["delta"]))
         return p, keep
 
     def fc_set(self, fc: dict) -> None:
@@ -316,9 +323,7 @@ class Context:
 
     def fc_search(self, k: int, lo: int = 0, hi: int | None = None, chunk: int = 0) -> dict:
         hi = self.space_size if hi is None else int(hi)
-        ti = np.empty(k, dtype=np.uint64)
-        ts = np.empty(k, dtype=np.float32)
-        r = _Result(0, 0.0, 0, k, ti.ctypes.data, ts.ctypes.data)
+        r, ti, ts = _search_result(k)
         _check(_lib.mf_fc_search(self._h, int(lo), hi, int(k), int(chunk), C.byref(r), _stream(self.device)),
                "mf_fc_search")
         return dict(best_idx=int(r.best_idx), best_score=float(r.best_score), count=int(r.feasible_count),
@@ -331,7 +336,7 @@ class Context:
                         int(params["repair"]))
         genome = np.zeros(self.n_models, dtype=np.int32)
         fit = C.c_float()
-        _check(_lib.mf_fc_ga_run(self._h, C.byref(g), int(seed), genome.ctypes.data, C.byref(fit),
+        _check(_lib.mf_fc_ga_run(self._h, C.byref(g), int(seed), _ptr(genome), C.byref(fit),
                                  _stream(self.device)), "mf_fc_ga_run")
         return float(fit.value), genome
 
