@@ -231,15 +231,6 @@ __host__ __device__ inline size_t fc_scan_table_bytes(int sumK) {
   return (((size_t)sumK * sizeof(float2) + 15) & ~(size_t)15) + 2 * 256 * sizeof(float);
 }
 
-// Monotone unsigned key of a float that is not NaN.
-__device__ __forceinline__ uint32_t fc_key(float v) {
-  const uint32_t u = __float_as_uint(v + 0.f);
-  return u ^ ((u >> 31) ? 0xFFFFFFFFu : 0x80000000u);
-}
-__device__ __forceinline__ float fc_unkey(uint32_t k) {
-  return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xFFFFFFFFu));
-}
-
 // The extremes of a model's usable options (finite VRAM in the CTA's table).
 struct FcSpan {
   float jmax, jmin, vmin, vmax;
@@ -405,7 +396,7 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
         in = in && c == 0;  // (a corner of fewer configurations: the rest are repeats)
 #pragma unroll
         for (int g = 0; g < kFcLambdas; ++g)
-          key[g][u] = in && sum[g].y <= cap && sum[g].x == sum[g].x && (whole || idx[g] - R.base < R.len) ? fc_key(sum[g].x) : 0u;
+          key[g][u] = in && sum[g].y <= cap && sum[g].x == sum[g].x && (whole || idx[g] - R.base < R.len) ? order_key(sum[g].x) : 0u;
       }
       // the first lambda with k feasible configurations, and their k-th best score
       uint32_t mine[PER] = {};
@@ -430,7 +421,7 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
           if (n >= R.k) v = t;
           if (n >= R.k && n <= R.k + (R.k >> 2)) break;  // (any bar that k scores reach holds)
         }
-        const float b = fc_unkey(v);
+        const float b = from_key(v);
         if (b > thr0_s) { thr0_s = b; thr0_i = kEmptyIdx; }
       }
     }
@@ -894,7 +885,7 @@ struct FcGaArgs {
 
 // (fitness, slot) as one word that orders by fitness, then by lower slot.
 __device__ __forceinline__ unsigned long long fc_rank(float f, int slot) {
-  return ((unsigned long long)fc_key(f) << 32) | (0xFFFFFFFFu - (uint32_t)slot);
+  return ((unsigned long long)order_key(f) << 32) | (0xFFFFFFFFu - (uint32_t)slot);
 }
 __device__ __forceinline__ int fc_slot(unsigned long long r) { return (int)(0xFFFFFFFFu - (uint32_t)r); }
 

@@ -276,20 +276,14 @@ __device__ __forceinline__ bool has_tag(unsigned long long w, uint32_t tag) {
   return (uint32_t)(w >> 32) == tag;
 }
 
-// Unsigned key with the order of the fitness values (no NaN; -0 and +0 compare equal).
-__device__ __forceinline__ uint32_t fit_key(float v) {
-  const uint32_t u = __float_as_uint(v + 0.f);
-  return u ^ ((u >> 31) ? 0xFFFFFFFFu : 0x80000000u);
-}
-
 // (fitness, slot) maximum over the warp: higher fitness, then lower slot; slot < 0 is empty.
 // Two warp reductions, where a butterfly of both values takes ten dependent shuffles.
 __device__ __forceinline__ void warp_best(float& f, int& s) {
-  const uint32_t key = s >= 0 ? fit_key(f) : 0u;
+  const uint32_t key = s >= 0 ? order_key(f) : 0u;
   const uint32_t top = __reduce_max_sync(0xffffffffu, key);
   const uint32_t slot = __reduce_min_sync(0xffffffffu, s >= 0 && key == top ? (uint32_t)s : 0xFFFFFFFFu);
   s = (int)slot;  // (-1: none)
-  if (s >= 0) f = __uint_as_float(top ^ ((top >> 31) ? 0x80000000u : 0xFFFFFFFFu));
+  if (s >= 0) f = from_key(top);
 }
 
 // One butterfly step that halves the values a lane carries: the two lanes that

@@ -10,13 +10,8 @@ namespace {
 constexpr int kMergeThreads = 1024;
 constexpr int kMergeLane = 20;                       // list entries a lane holds: up to 640 lists
 constexpr int kMergeMaxLists = 32 * kMergeLane;
+static_assert(kMergeMaxLists == kMaxTops, "one bound for both");
 constexpr size_t kPair = sizeof(uint64_t) + sizeof(float);
-
-// Unsigned key with the order of the scores (no NaN among them; -0 and +0 compare equal).
-__device__ __forceinline__ uint32_t order_key(float s) {
-  const uint32_t u = __float_as_uint(s + 0.f);
-  return u ^ ((u >> 31) ? 0xFFFFFFFFu : 0x80000000u);
-}
 
 // Sorts n distinct entries (ss, si) of shared memory best first and writes the first k
 // to the output, empty slots after them.  Up to one entry per thread: each warp sorts its
@@ -184,6 +179,7 @@ k_merge_lists(const float* __restrict__ in_s, const uint64_t* __restrict__ in_i,
     s_n = 0;
     if (out.words) out.words->t[1] = device_ns();
   }
+  if (out.words && tid < kMaxTops) out.words->tops[tid] = 0u;  // (for the next search)
   __syncthreads();
   bool few = nlists <= kMergeMaxLists;
   if (few) {

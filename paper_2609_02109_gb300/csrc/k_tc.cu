@@ -130,7 +130,7 @@ TcFn tc_kernel_mode(const TcArgs& T, int n_models) {
     // digits fit seven bytes (one or two models have nothing to unroll): 435 cycles a model
     // and tile against 577 with the run-time loop (N = 6 and 7, 24^6 and 13^7), lists of 8 M candidates 541 against 681.
     if constexpr (!MP && !UT) {
-      if (n_models >= 3 && n_models <= 7) return MODE == kTcRange ? tc_kernel_nm_range(n_models) : tc_kernel_nm_list(n_models);
+      if (n_models >= 3 && n_models <= 7) return MODE == kTcRange ? tc_kernel_nm_range(n_models, T.sb != 0) : tc_kernel_nm_list(n_models);
     }
     return k_score_tc<MODE, 8, 4, 1, 5, 4, 16, MP, UT, 0, kXmBf16>;
   }
@@ -713,11 +713,12 @@ mf_status tc_prepare(mf_ctx* c, bool exact, const TcHost& h) {
 
 mf_status tc_search_chunk(mf_ctx* c, const RangeArgs& a, cudaStream_t s, int* nlaunch) {
   TcArgs T = c->tc;
+  T.sb = a.tops != nullptr;
   if (!layout_for(c->P, T, a.k)) {
     set_error("tensor-core path: top-k lists do not fit shared memory; use a smaller k");
     return MF_EUNSUPPORTED;
   }
-  if (T.npasses != c->tc.npasses)  // (another kernel than the one prepared)
+  if (T.npasses != c->tc.npasses || T.sb)  // (another kernel than the one prepared)
     MF_CUDA(cudaFuncSetAttribute(tc_kernel(kTcRange, T, c->P.objective == MF_OBJ_UTILITY, c->P.n_models),
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit));
   // digits of the per-tile index stride (grid x pipes x 128), modulo |Lambda|

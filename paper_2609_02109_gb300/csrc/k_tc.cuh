@@ -278,6 +278,37 @@ static __device__ __noinline__ void tc_topk_merge(const CtaTopK& tk, int row, in
   else topk_merge_sorted(tk, row, 128, NamedSync128{barid});
 }
 
+// The bar that all lists of a search share: the k-th largest of the lists' best scores, which
+// k candidates reach (-inf while fewer than k lists have one).  A pipeline's epilogue warps
+// publish their list's best score (`mine`: a thread's, as a key) and take the bar, which
+// its first warp works out; out of line, since it runs after tiles 1, 2, 4, 8, .. only.
+// Without it each list fills and tightens on its own candidates: 24^5 candidates at bf16
+// (lists of 256) took 0.68 ms, with it 0.56.
+static __device__ __noinline__ float tc_shared_bar(uint32_t* tops, int ntops, int k, uint32_t own, uint32_t mine,
+                                                   bool first_warp, volatile float* out, int barid) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t top = __reduce_max_sync(0xffffffffu, mine);
+  if (lane == 0) atomicMax(tops + own, top);
+  if (first_warp) {
+    uint32_t key[kMaxTops / 32];
+#pragma unroll
+    for (int j = 0; j < kMaxTops / 32; ++j) key[j] = lane + 32 * j < ntops ? __ldcg(tops + lane + 32 * j) : 0u;
+    uint32_t v = 0u;
+    for (int b = 31; b >= 8; --b) {  // (a bar a little low holds as well)
+      const uint32_t t = v | (1u << b);
+      int c[4] = {0, 0, 0, 0};
+#pragma unroll
+      for (int j = 0; j < kMaxTops / 32; ++j) c[j & 3] += key[j] >= t ? 1 : 0;
+      const int reach = __reduce_add_sync(0xffffffffu, (c[0] + c[1]) + (c[2] + c[3]));
+      if (reach >= k) v = t;
+      if (reach == k) break;
+    }
+    if (lane == 0) *out = v > kKeyMinusInf ? from_key(v) : -INFINITY;
+  }
+  named_bar(barid, 128);
+  return *out;
+}
+
 // The rest of a bounded wait, out of line: on giving up it flags the status word and
 // every later wait returns at once, so the kernel still runs to its end.
 static __device__ __noinline__ void mbar_wait_slow(uint64_t* bar, uint32_t parity, volatile int* abort, uint32_t* status) {
@@ -521,8 +552,8 @@ struct AggW {
 // the previous tile's last, and that tile's constraints and top-k), a stage of the next
 // tile's digits and aggregate, and the next A1 row; then D2 -> H2.  The issuing warp does
 // nothing else, so an MMA group starts as soon as its operands are stored.
-// XM: the operands (kXmBf16, kXmTf32, kXmHalf).
-template <int MODE, int KW, int AWO, int S1, int S2, int S3, int N3, bool MP, bool UT, int NM, int XM>
+// XM: the operands (kXmBf16, kXmTf32, kXmHalf).  SB: the lists share a bar (tc_shared_bar).
+template <int MODE, int KW, int AWO, int S1, int S2, int S3, int N3, bool MP, bool UT, int NM, int XM, bool SB = false>
 __global__ void __launch_bounds__(tc_pipes(XM) * kTcPipeThreads, 1)
 k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   static_assert(AWO < 0 || AWO == 4 || AWO == 8, "partial A1 rows are written for these layouts only");
@@ -540,6 +571,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   using DS = typename std::conditional<RD, uint64_t, uint8_t*>::type;
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ uint32_t s_tmem;
+  __shared__ float s_shared_bar[kTcMaxPipes];
   __shared__ int s_abort;
   __shared__ float s_b3[MF_MAX_MODELS][HF ? 4 : 2];  // b3 (thr, lat); HF: the outputs' scales back
   const int tid = threadIdx.x;
@@ -999,13 +1031,20 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   // passes' record, feasibility, the count and the top-k queue; then a fresh objective.
   // The list's k-th entry (the bar a candidate must pass to be queued) changes only in a
   // merge; each thread keeps a copy.
-  float bar_s = -INFINITY;
+  // The lists' shared bar, where it is the higher one, admits scores equal to it.
+  float bar_s = -INFINITY, shared_bar = -INFINITY;
   uint64_t bar_i = kEmptyIdx;
+  uint32_t my_top = 0u;    // the best score this thread has queued, as a key
+  uint32_t tiles_done = 0u;
   auto reload_bar = [&]() {
     if (MODE == kTcRange) {
       const CtaTopK tk = topk();
       bar_s = tk.ls[kcap - 1];
       bar_i = tk.li[kcap - 1];
+      if (SB && shared_bar > bar_s) {
+        bar_s = shared_bar;
+        bar_i = kEmptyIdx;
+      }
     }
   };
   auto finish_tile = [&](uint64_t tile_f, float vram, uint64_t at) {
@@ -1058,10 +1097,22 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
         const int pos = atomicAdd(tk.qn, 1);
         tk.qs[pos] = J;
         tk.qi[pos] = idx;
+        if (SB) my_top = max(my_top, order_key(J));
       }
       // Candidates wait in the queue (against the list's k-th entry of the last merge)
       // until another tile's 128 might not fit; then one merge takes them all.
       named_bar(barid, 128);
+      if constexpr (SB) {
+        ++tiles_done;
+        if ((tiles_done & (tiles_done - 1u)) == 0u) {
+          shared_bar = fmaxf(shared_bar, tc_shared_bar(R.tops, R.ntops, kcap, (uint32_t)gpipe, my_top, wq == 0,
+                                                       &s_shared_bar[pipe], barid));
+          if (shared_bar > bar_s) {
+            bar_s = shared_bar;
+            bar_i = kEmptyIdx;
+          }
+        }
+      }
       if (*(volatile int*)tk.qn > T.qcap - 128) {
         tc_topk_merge(tk, row, barid);
         reload_bar();
@@ -1082,20 +1133,22 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
 #pragma unroll (NM > 0 ? NM : 1)
       for (int i = m0; i < m1; ++i) {
         const bool next_l1 = i + 1 < m1 || has_next;
-        // (the descriptors are made ahead of the hand-offs, off the chain)
-        const uint64_t d1 = desc1(i + 1 < m1 ? i + 1 : m0), d2 = desc2(i), d3 = desc3(i);
+        // (the descriptors are made ahead of the hand-offs, off the chain; not in HF, whose
+        // many MMAs a hand-off hide that: 13^7 14.0 ms, ahead 14.5)
+        const int i1 = i + 1 < m1 ? i + 1 : m0;
+        const uint64_t d1 = HF ? 0 : desc1(i1), d2 = HF ? 0 : desc2(i), d3 = HF ? 0 : desc3(i);
         if (T.h2 > 0) {
           take();  // H1 of model i stored
-          issue_mma2(d2);
+          issue_mma2(HF ? desc2(i) : d2);
           mma_commit_warp(barA);
         }
         if (next_l1) {
           take();  // accumulators read, the next A1 row written
-          issue_mma1(d1);
+          issue_mma1(HF ? desc1(i1) : d1);
           mma_commit_warp(barA);
         }
         take();  // the last hidden layer of model i stored
-        issue_mma3(d3, i > m0 ? 1u : 0u);
+        issue_mma3(HF ? desc3(i) : d3, i > m0 ? 1u : 0u);
         mma_commit_warp(barB);
       }
     }
@@ -1259,7 +1312,7 @@ using TcFn = void (*)(const Params, const TcArgs, const RangeArgs, const TcList)
 // Instantiations in translation units of their own (they compile side by side): the exact
 // variants, and the bf16 kernel of the d_L 8, 64-64 shape for 3 to 7 models.
 TcFn tc_kernel_exact(int xm, int mode, bool mp, bool util);
-TcFn tc_kernel_nm_range(int n_models);
+TcFn tc_kernel_nm_range(int n_models, bool shared_bar);
 TcFn tc_kernel_nm_list(int n_models);
 
 }  // namespace mf

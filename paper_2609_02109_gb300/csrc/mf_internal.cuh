@@ -12,6 +12,7 @@
 namespace mf {
 
 constexpr uint64_t kEmptyIdx = ~0ull;
+constexpr int kMaxTops = 640;        // lists whose best scores a search shares
 constexpr int kScoreThreads = 512;   // CTA size of the CUDA-core scorer
 constexpr int kWideWarps = 8;        // warps per CTA of the warp-per-(candidate, model) scorer
 
@@ -62,6 +63,7 @@ struct TcArgs {
   float cagg[3], back[MF_MAX_MODELS][2];
   uint32_t sm_xw, sm_dem, sm_rows, sm_topk, sm_bar, sm_total;  // shared-memory byte offsets
   uint32_t img_model;                 // bytes of one model's B1 + B2 + B3 images
+  int32_t sb;                         // the lists share a bar (RangeArgs::tops)
   int32_t kcap;                       // per-pipeline list length the layout was sized for
   int32_t qcap;                       // per-pipeline candidate queue (128 or 512, a power of two)
   uint32_t step[MF_MAX_MODELS];       // mixed-radix digits of the per-tile index stride (range mode)
@@ -91,6 +93,16 @@ constexpr uint32_t kStatusUnwritten = 0xFFFFFFFFu;  // host copy: the kernel end
 __device__ __forceinline__ bool precedes(float ja, uint64_t ia, float jb, uint64_t ib) {
   return ja > jb || (ja == jb && ia < ib);
 }
+
+// Unsigned key with the order of floats that are not NaN (-0 and +0 alike), and back.
+__device__ __forceinline__ uint32_t order_key(float v) {
+  const uint32_t u = __float_as_uint(v + 0.f);
+  return u ^ ((u >> 31) ? 0xFFFFFFFFu : 0x80000000u);
+}
+__device__ __forceinline__ float from_key(uint32_t k) {
+  return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xFFFFFFFFu));
+}
+constexpr uint32_t kKeyMinusInf = 0x007FFFFFu;
 
 // ReLU that keeps NaN (so a NaN weight reaches the outputs and marks the
 // candidate infeasible).
@@ -345,6 +357,7 @@ __device__ void topk_merge_sorted(const CtaTopK& t, int tid, int nthr, Sync sync
 struct SearchWords {
   unsigned long long count;  // feasible candidates
   unsigned long long t[2];   // start of the first scoring launch, of the merge (ns)
+  uint32_t tops[kMaxTops];   // see RangeArgs::tops
 };
 
 }  // namespace mf
@@ -439,6 +452,8 @@ struct RangeArgs {
   uint64_t* lists_i;    // [grid][k]
   unsigned long long* count;
   unsigned long long* start;  // the first launch's start, ns (null: not wanted)
+  uint32_t* tops;             // [ntops] best score of each list's owner so far, as a key (null: not kept)
+  int ntops;
 };
 
 // Nanoseconds of the device's global timer.
