@@ -608,7 +608,7 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
     }
     const bool more = __syncthreads_or(waiting != 0u);
     // a long queue (the first merges of a search) is sorted first
-    if (*(volatile int*)tk.qn > 256) topk_merge_sorted(tk, tid, blockDim.x, [] __device__() { __syncthreads(); });
+    if (*(volatile int*)tk.qn > 64) topk_merge_sorted(tk, tid, blockDim.x, [] __device__() { __syncthreads(); });
     else if (*(volatile int*)tk.qn > 0) topk_merge(tk, tid, blockDim.x, [] __device__() { __syncthreads(); });
     if (!more) break;
     raise_bar();
@@ -623,7 +623,7 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
       }
     __syncthreads();
     if (*(volatile int*)tk.qn > 0) {
-      if (*(volatile int*)tk.qn > 256) topk_merge_sorted(tk, tid, blockDim.x, [] __device__() { __syncthreads(); });
+      if (*(volatile int*)tk.qn > 64) topk_merge_sorted(tk, tid, blockDim.x, [] __device__() { __syncthreads(); });
       else topk_merge(tk, tid, blockDim.x, [] __device__() { __syncthreads(); });
     }
   }

@@ -104,7 +104,7 @@ void layout_smem(const Params& P, TcArgs& T, int kcap) {
   uint32_t o = round_up((int)T.img_bytes, 1024);
   T.sm_xw = o; o += round_up(sumK * T.kw * 4, 16);
   T.sm_dem = o; o += sumK * 16;
-  T.sm_rows = o; o += T.pipes * 2 * MF_MAX_MODELS * 128;  // byte digits of two tiles per pipeline
+  T.sm_rows = o; o += T.pipes * tc_row_bytes(T.ew);
   // the candidate queue: 512 entries (a merge every few tiles) where shared memory allows,
   // else one tile's 128 (a merge after every tile that queued a candidate)
   const uint32_t rest = o + 16 + 8 * (3 + 2 * kTcMaxPipes);
@@ -118,6 +118,9 @@ void layout_smem(const Params& P, TcArgs& T, int kcap) {
 }
 
 constexpr size_t kPassImageBudget = 160 * 1024;      // weights staged per pass
+
+// The 20 -> 128 -> 128 -> 2 shape (up to 8 models), with an instantiation of its own.
+bool tc_wide(const TcArgs& T) { return T.kw == 16 && T.dle == 16 && T.h1 == 128 && T.h2 == 128 && T.n3 == 16; }
 
 // Instantiations: the two benchmark shapes (d_L 8, 64-64 and d_L 16, 128-128, up to 8
 // models) with all counts fixed at compile time, and a run-time fallback per A1 row width.
@@ -134,7 +137,7 @@ TcFn tc_kernel_mode(const TcArgs& T, int n_models) {
     }
     return k_score_tc<MODE, 8, 4, 1, 5, 4, 16, MP, UT, 0, kXmBf16>;
   }
-  if (T.kw == 16 && T.dle == 16 && T.h1 == 128 && T.h2 == 128 && T.n3 == 16)
+  if (tc_wide(T))
     return k_score_tc<MODE, 16, 8, 2, 9, 8, 16, MP, UT, 0, kXmBf16>;
   if (T.kw == 8) return k_score_tc<MODE, 8, -1, 0, 0, 0, 0, MP, UT, 0, kXmBf16>;
   return k_score_tc<MODE, 16, -1, 0, 0, 0, 0, MP, UT, 0, kXmBf16>;
@@ -226,11 +229,12 @@ static void set_passes(const Params& P, TcArgs& T, size_t budget) {
   }
 }
 
-// The shared-memory layout for lists of kcap entries: in the fp16 variant with fewer models
-// per pass where the lists would not fit next to a full pass's weights.
+// The shared-memory layout for lists of kcap entries: in the fp16 variant (three pipelines'
+// lists), and where two epilogue warps share a lane quarter (their rows take more), with
+// fewer models per pass if the lists would not fit next to a full pass's weights.
 static bool layout_for(const Params& P, TcArgs& T, int kcap) {
   layout_smem(P, T, kcap);
-  if (T.sm_total > kSmemLimit && T.tf == kXmHalf) {
+  if (T.sm_total > kSmemLimit && (T.tf == kXmHalf || T.ew == 2)) {
     set_passes(P, T, 2 * kPassImageBudget / 3);
     set_pass(T, 0, nullptr);
     layout_smem(P, T, kcap);
@@ -255,6 +259,7 @@ mf_status tc_prepare_exact(mf_ctx* c, const TcHost& h) {
   TcArgs& T = c->tc;
   const int N = P.n_models, dl = P.d_local, h1 = P.h1, h2 = P.h2, hl = h2, din = P.d_in;
   T.tf = kXmTf32;
+  T.ew = 1;
   T.dle = dl;
   T.k1 = 16;   // [x (8) | aggregate (3) | 1 | 0 0 0 0]
   T.kw = 16;   // words per option: x hi (8), x lo (8)
@@ -497,6 +502,7 @@ mf_status tc_prepare_half(mf_ctx* c, const TcHost& h) {
   // TMEM columns: the pipelines' D (64 each), their D3 (16 each), then per pipeline
   // H hi (32) | ones (8) | H lo (32) | A1 hi (8), A1 lo (8): 504 of 512 for three pipelines
   T.pipes = tc_pipes(kXmHalf);
+  T.ew = 1;
   T.ps_d = h1;
   T.ps_d3 = T.n3;
   T.col_d = 0;
@@ -626,6 +632,7 @@ mf_status tc_prepare(mf_ctx* c, bool exact, const TcHost& h) {
   T.pipe_stride = T.ps_d = T.ps_d3 = round_up(T.col_d3 + T.n3, 32);
   T.pipes = 512 / T.pipe_stride;
   if (T.pipes > kTcMaxPipes) T.pipes = kTcMaxPipes;
+  T.ew = tc_wide(T) ? 2 : 1;
 
   // B operand images (K-major): B1 [h1 x k1], B2 [h2 x (h1 + 16)], B3 [n3 x hl]
   const int k2 = h1 + 16, k3 = hl;
@@ -751,7 +758,7 @@ mf_status tc_search_chunk(mf_ctx* c, const RangeArgs& a, cudaStream_t s, int* nl
     r.first = a.first && b == 0;
     for (int p = 0; p < T.npasses; ++p) {
       set_pass(T, p, partial);
-      tc_kernel(kTcRange, T, c->P.objective == MF_OBJ_UTILITY, c->P.n_models)<<<c->num_sms, T.pipes * kTcPipeThreads, smem, s>>>(c->P, T, r, L);
+      tc_kernel(kTcRange, T, c->P.objective == MF_OBJ_UTILITY, c->P.n_models)<<<c->num_sms, T.pipes * tc_pipe_threads(T.ew), smem, s>>>(c->P, T, r, L);
       MF_CUDA(cudaGetLastError());
       ++launches;
     }
@@ -781,7 +788,7 @@ mf_status tc_score_list(mf_ctx* c, const uint64_t* idx, uint64_t n, float* score
     TcList L{idx + b, m, score + b, feas ? feas + b : nullptr, pred ? pred + b * N * 2 : nullptr};
     for (int p = 0; p < T.npasses; ++p) {
       set_pass(T, p, partial);
-      tc_kernel(kTcList, T, c->P.objective == MF_OBJ_UTILITY, c->P.n_models)<<<(unsigned)grid, T.pipes * kTcPipeThreads, smem, s>>>(c->P, T, R, L);
+      tc_kernel(kTcList, T, c->P.objective == MF_OBJ_UTILITY, c->P.n_models)<<<(unsigned)grid, T.pipes * tc_pipe_threads(T.ew), smem, s>>>(c->P, T, R, L);
       MF_CUDA(cudaGetLastError());
     }
   }

@@ -255,8 +255,20 @@ __host__ __device__ constexpr int tc_pipes(int xm) { return xm == kXmTf32 ? 2 : 
 // 32 (w % 4) ..) and one warp that issues its MMAs: warps [0, 4 pipes) are the epilogue
 // warps (pipeline w / 4), warps [4 pipes, 5 pipes) the issuing warps (pipeline w - 4 pipes,
 // so the issuers sit on different schedulers).
-constexpr int kTcPipeThreads = 160;
+// Where a hidden layer's conversion is long and only two pipelines fit (128-wide layers) a
+// pipeline has two epilogue warps per lane quarter (TcArgs::ew): each converts half of the
+// columns, and the work beside is split too: the first half's warps prepare inputs (digits,
+// aggregate, A1 rows), the second half's take outputs (objective, constraints, top-k).
+// 50 M candidates of eight 20->128->128->2 predictors: 15.3 ms against 16.7.  (The fp16 split
+// converts as long, but its three pipelines then leave 72 registers a thread: 22 M candidates
+// 4.08 ms against 3.84.  Four pipelines would need 1152 threads.)
+__host__ __device__ constexpr int tc_pipe_threads(int ew) { return 32 * (4 * ew + 1); }
 constexpr uint32_t kWaitLimit = 4096;  // suspended retries (~1 ms each at most)
+
+// Shared memory of a pipeline's rows: byte digits of two tiles, or of three and VRAM demands.
+__host__ __device__ constexpr int tc_row_bytes(int ew) {
+  return ew == 2 ? 3 * (MF_MAX_MODELS * 128 + 128 * 4) : 2 * MF_MAX_MODELS * 128;
+}
 
 struct TcList {
   const uint64_t* idx;
@@ -271,10 +283,11 @@ struct NamedSync128 {
   __device__ void operator()() const { named_bar(id, 128); }
 };
 
+// (a queue of 128 into a list of 256: 3 k cycles sorted, 15 k by counting)
 // The pipeline's top-k merge, out of line: it runs rarely and its registers stay off
 // the hot loop.
 static __device__ __noinline__ void tc_topk_merge(const CtaTopK& tk, int row, int barid) {
-  if (*tk.qn <= 128) topk_merge(tk, row, 128, NamedSync128{barid});
+  if (*tk.qn <= 24) topk_merge(tk, row, 128, NamedSync128{barid});
   else topk_merge_sorted(tk, row, 128, NamedSync128{barid});
 }
 
@@ -553,8 +566,11 @@ struct AggW {
 // tile's digits and aggregate, and the next A1 row; then D2 -> H2.  The issuing warp does
 // nothing else, so an MMA group starts as soon as its operands are stored.
 // XM: the operands (kXmBf16, kXmTf32, kXmHalf).  SB: the lists share a bar (tc_shared_bar).
+// EW: epilogue warps per lane quarter.
+__host__ __device__ constexpr int tc_ew(int xm, int s2) { return xm == kXmBf16 && s2 == 9 ? 2 : 1; }
+
 template <int MODE, int KW, int AWO, int S1, int S2, int S3, int N3, bool MP, bool UT, int NM, int XM, bool SB = false>
-__global__ void __launch_bounds__(tc_pipes(XM) * kTcPipeThreads, 1)
+__global__ void __launch_bounds__((XM == kXmBf16 && S2 == 9 ? 2 : tc_pipes(XM)) * tc_pipe_threads(tc_ew(XM, S2)), 1)
 k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   static_assert(AWO < 0 || AWO == 4 || AWO == 8, "partial A1 rows are written for these layouts only");
   static_assert(NM <= 7, "packed digits hold at most seven models");
@@ -564,6 +580,8 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   static_assert(!HF || (KW == 8 && AWO == 4 && S1 == 1 && S2 == 5 && S3 == 4 && N3 == 16),
                 "the exact variants run the d_L 8, 64-64 shape");
   constexpr int KS = TF ? 8 : 16;  // K of one MMA
+  constexpr int EW = tc_ew(XM, S2);
+  static_assert(EW == 1 || NM == 0, "two epilogue warps share digits through shared memory");
   // With the model count fixed at compile time, a tile's digits live in registers, packed
   // one per byte (model N - 1 in the lowest byte); otherwise in shared memory, one byte per
   // model and row, two tiles.
@@ -577,7 +595,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   const int tid = threadIdx.x;
   // compile-time K-step counts must be the layout's (else no MMA may run)
   if ((S1 > 0 && S1 != T.k1 / KS) || (S2 > 0 && S2 != T.h1 / KS + 1) || (S3 > 0 && S3 != T.hl / KS) ||
-      (N3 > 0 && N3 != T.n3) || (NM > 0 && (NM != P.n_models || MP)) || XM != T.tf) {
+      (N3 > 0 && N3 != T.n3) || (NM > 0 && (NM != P.n_models || MP)) || XM != T.tf || EW != T.ew) {
     if (tid == 0) atomicOr(P.status, kStatusBadInput);
     return;
   }
@@ -588,16 +606,20 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int N = NM > 0 ? NM : P.n_models;
   const int npipes = T.pipes;
-  const bool issuer = warp >= 4 * npipes;  // the pipeline's MMA-issuing warp
-  const int pipe = issuer ? warp - 4 * npipes : warp >> 2, wq = warp & 3;
+  const bool issuer = warp >= 4 * EW * npipes;  // the pipeline's MMA-issuing warp
+  const int pipe = issuer ? warp - 4 * EW * npipes : warp / (4 * EW), wq = warp & 3;
   const int row = wq * 32 + lane;
+  const int half = EW == 2 ? (warp >> 2) & 1 : 0;  // the half of the columns this warp converts
+  const bool in_side = EW == 1 || half == 0, out_side = !issuer && (EW == 1 || half == 1);
+  constexpr int kBufs = EW == 2 ? 3 : 2;           // tiles whose digits are kept
 
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + T.sm_bar);
   const uint4* xw_s = reinterpret_cast<const uint4*>(smem + T.sm_xw);
   float4* dem_s = reinterpret_cast<float4*>(smem + T.sm_dem);
-  // this thread's digits (option index within the model) of every model, two tiles:
-  // digits[b * MF_MAX_MODELS * 128 + i * 128 + row]
-  uint8_t* digits = reinterpret_cast<uint8_t*>(smem + T.sm_rows) + (size_t)pipe * 2 * MF_MAX_MODELS * 128;
+  // this row's digits (option index within the model) of every model, kBufs tiles:
+  // digits[b * MF_MAX_MODELS * 128 + i * 128 + row]; EW 2: then its VRAM demand, as many tiles
+  uint8_t* digits = reinterpret_cast<uint8_t*>(smem + T.sm_rows) + (size_t)pipe * tc_row_bytes(EW);
+  float* vrams = reinterpret_cast<float*>(digits + kBufs * MF_MAX_MODELS * 128);
 
   if (tid == 0) {
     s_abort = 0;
@@ -656,7 +678,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
     tk.k = kcap;
     return tk;
   };
-  if (MODE == kTcRange && !issuer) {
+  if (MODE == kTcRange && out_side) {
     const CtaTopK tk = topk();
     const size_t gl = ((size_t)blockIdx.x * npipes + pipe) * kcap;
     for (int e = row; e < kcap; e += 128) {
@@ -682,7 +704,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   uint64_t* barB = &bars[2 + 2 * pipe];  // layer 3 completed
   uint32_t phA = 0, phB = 0;
   // epilogue -> issuer hand-offs alternate between two named barriers per pipeline, each
-  // a full rendezvous of the 160 threads: the epilogue warps cannot run ahead of the
+  // a full rendezvous of the pipeline's threads: the epilogue warps cannot run ahead of the
   // issuing warp even where their mbarrier waits return early (after a wait gave up),
   // which with arrive-only hand-offs could complete a barrier without the issuing warp
   // and leave it waiting at the next one; the pipeline's top-k uses a third barrier
@@ -693,7 +715,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   const int s1 = T.k1 / KS, s2 = T.h1 / KS + 1, s3 = T.hl / KS;
   const int m0 = MP ? T.m0 : 0, m1 = MP ? T.m1 : N;  // this pass's models
   const float vcap = P.vram_cap;
-  if (!issuer) {  // constant ones block: (1, 1) feeds the bias hi/lo rows of B2
+  if (!issuer && in_side) {  // constant ones block: (1, 1) feeds the bias hi/lo rows of B2
     if constexpr (TF) {
       uint32_t v[8] = {0x3F800000u, 0x3F800000u, 0u, 0u, 0u, 0u, 0u, 0u};
       tmem_st_x8(tOnes + lane_off, v);
@@ -762,12 +784,12 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   auto signal = [&]() {
     tmem_wait_st();
     tc_fence_before();
-    named_bar(sig0 + (int)(ksig & 1u), 160);
+    named_bar(sig0 + (int)(ksig & 1u), tc_pipe_threads(EW));
     ++ksig;
   };
   // issuing warp: the epilogue warps' next hand-off
   auto take = [&]() {
-    named_bar(sig0 + (int)(ksig & 1u), 160);
+    named_bar(sig0 + (int)(ksig & 1u), tc_pipe_threads(EW));
     ++ksig;
     tc_fence_after();
   };
@@ -1154,17 +1176,24 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
     }
   } else {
     // ---- the epilogue warps ----
-    reload_bar();
+    if (out_side) reload_bar();
     uint64_t tile = gpipe;
     int buf = 0;
+    auto buffer = [&](int b) { return digits + b * (MF_MAX_MODELS * 128); };
     float vram_cur = 0.f, vram_prev = 0.f, vram_nx = 0.f;  // VRAM demand of this thread's rows
     DS dcur{}, dprev{}, dnx{};
     // list mode: the row's index in the previous, this and the next two tiles
     uint64_t x_prev = kEmptyIdx, x_cur = list_index(tile), x_nx = list_index(tile + gstride), x_nx2 = kEmptyIdx;
     if (tile * 128 < n) {
-      dcur = load_tile(tile, digits, vram_cur, x_cur);
+      if (in_side) {
+        dcur = load_tile(tile, digits, vram_cur, x_cur);
+        if (EW == 2) vrams[row] = vram_cur;
+      } else if constexpr (!RD) {
+        dcur = digits;
+      }
       signal();  // ones block and the first A1 row
     }
+    constexpr uint32_t kColsD = EW == 2 ? S3 * 8 : 0;  // columns a warp converts, where two share them
     // the previous tile is finished once its last layer 3 (issued at the end of that
     // tile) has landed, during this tile's first model
     bool pending = false;
@@ -1174,7 +1203,8 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
     const int st_agg = m0 + 2 < m1 ? m0 + 2 : m1 - 1;
     AggW aw_nx{};
     for (; tile * 128 < n; tile += gstride) {
-      uint8_t* buf_nx = digits + (buf ^ 1) * (MF_MAX_MODELS * 128);  // (shared-memory digits)
+      const int b_nx = buf + 1 == kBufs ? 0 : buf + 1;
+      uint8_t* buf_nx = buffer(b_nx);  // (shared-memory digits)
       const bool has_next = (tile + gstride) * 128 < n;
       auto stage = [&](int i) {
         if (has_next && i == st_dig) dnx = tile_digits(tile + gstride, buf_nx, dcur, false, x_nx);
@@ -1187,6 +1217,26 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
       // a stage of the next tile, the next A1 row.  The layer-3 outputs are loaded first
       // and used last.
       auto side_work = [&](int i) {
+        if constexpr (EW == 2) {  // inputs by the first half's warps, outputs by the second's
+          if (in_side) {
+            if (i + 1 < m1) next_a1(i + 1, dcur);
+            stage(i);
+            if (i == st_agg && has_next) vrams[b_nx * 128 + row] = vram_nx;
+            if (i + 1 >= m1 && has_next) write_a1(m0, dnx, true, aw_nx);
+          } else {
+            uint32_t oa, ob;
+            if (i > m0) {
+              load_model(i - 1, oa, ob);
+              add_model(i - 1, oa, ob, dcur, tile, x_cur);
+            } else if (pending) {
+              load_model(m1 - 1, oa, ob);
+              add_model(m1 - 1, oa, ob, dprev, tile - gstride, x_prev);
+              finish_tile(tile - gstride, vrams[(buf == 0 ? kBufs - 1 : buf - 1) * 128 + row], x_prev);
+            }
+            if (i == st_dig) x_nx2 = list_index(tile + 2 * gstride);
+          }
+          return;
+        }
         uint32_t oa = 0u, ob = 0u;
         if (i > m0) {
           load_model(i - 1, oa, ob);
@@ -1219,7 +1269,8 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
             if (l3) await_b();  // the previous model's layer 3 has read H
           });
         } else {
-          hidden_epilogue<(S2 > 0 ? (S2 - 1) * 16 : 0)>(T.h1, tD + lane_off, tH1 + lane_off, []() {}, [&]() {
+          hidden_epilogue<(S2 > 0 ? (S2 - 1) * 16 / EW : 0)>(T.h1, tD + kColsD * half + lane_off,
+                                                             tH1 + kColsD / 2 * half + lane_off, []() {}, [&]() {
             if (l3) await_b();  // the previous model's layer 3 has read H
           });
         }
@@ -1248,8 +1299,8 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
               },
               []() {});
         } else {
-          hidden_epilogue<(S3 > 0 ? S3 * 16 : 0)>(
-              T.h2, tD + lane_off, tH2 + lane_off,
+          hidden_epilogue<(S3 > 0 ? S3 * 16 / EW : 0)>(
+              T.h2, tD + kColsD * half + lane_off, tH2 + kColsD / 2 * half + lane_off,
               [&]() {
                 if (next_l1) signal();  // accumulators read, next A1 written: the next layer 1
               },
@@ -1259,29 +1310,30 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
       }
       pending = true;
       dprev = dcur;
+      if constexpr (EW == 2) dnx = buf_nx;
       dcur = dnx;
       x_prev = x_cur;
       x_cur = x_nx;
       x_nx = x_nx2;
       vram_prev = vram_cur;
       vram_cur = vram_nx;
-      buf ^= 1;
+      buf = b_nx;
     }
-    if (pending) {  // the last tile's last layer 3
+    if (pending && out_side) {  // the last tile's last layer 3
       await_b();
       uint32_t oa, ob;
       load_model(m1 - 1, oa, ob);
       add_model(m1 - 1, oa, ob, dprev, tile - gstride, x_prev);
-      finish_tile(tile - gstride, vram_prev, x_prev);
+      finish_tile(tile - gstride, EW == 2 ? vrams[(buf == 0 ? kBufs - 1 : buf - 1) * 128 + row] : vram_prev, x_prev);
     }
   }
-  if (MODE == kTcRange && (!MP || T.pass_last) && !issuer) {  // what is still queued joins the list
+  if (MODE == kTcRange && (!MP || T.pass_last) && out_side) {  // what is still queued joins the list
     const CtaTopK tk = topk();
     named_bar(barid, 128);
     if (*(volatile int*)tk.qn > 0) tc_topk_merge(tk, row, barid);
   }
 
-  if (MODE == kTcRange && (!MP || T.pass_last) && !issuer) {
+  if (MODE == kTcRange && (!MP || T.pass_last) && out_side) {
     const CtaTopK tk = topk();
     const size_t gl = ((size_t)blockIdx.x * npipes + pipe) * kcap;
     for (int e = row; e < kcap; e += 128) {

@@ -63,6 +63,7 @@ struct TcArgs {
   float cagg[3], back[MF_MAX_MODELS][2];
   uint32_t sm_xw, sm_dem, sm_rows, sm_topk, sm_bar, sm_total;  // shared-memory byte offsets
   uint32_t img_model;                 // bytes of one model's B1 + B2 + B3 images
+  int32_t ew;                         // epilogue warps per tensor-memory lane quarter (1 or 2)
   int32_t sb;                         // the lists share a bar (RangeArgs::tops)
   int32_t kcap;                       // per-pipeline list length the layout was sized for
   int32_t qcap;                       // per-pipeline candidate queue (128 or 512, a power of two)
