@@ -539,7 +539,11 @@ size_t f32_smem_bytes(const Params& P, int k, bool& resident) {
   return (resident ? wbytes : 0) + tk;
 }
 
-int f32_grid(const mf_ctx* c) { return c->num_sms; }
+// One CTA per SM, no more than the range has tiles (fewer lists to merge).
+int f32_grid(const mf_ctx* c, uint64_t len) {
+  const uint64_t tiles = len > 0 ? (len + kScoreThreads - 1) / kScoreThreads : 1;
+  return (int)(tiles < (uint64_t)c->num_sms ? tiles : (uint64_t)c->num_sms);
+}
 
 mf_status f32_prepare(mf_ctx* c) {
   const int shape = fixed_shape_id(c->P);
@@ -551,12 +555,12 @@ mf_status f32_prepare(mf_ctx* c) {
   return MF_OK;
 }
 
-mf_status f32_search_chunk(mf_ctx* c, const RangeArgs& a, cudaStream_t s) {
+mf_status f32_search_chunk(mf_ctx* c, const RangeArgs& a, int grid, cudaStream_t s) {
   bool res;
   const size_t smem = f32_smem_bytes(c->P, a.k, res);
   ScoreFn fn = pick_fn(kModeRange, fixed_shape_id(c->P), res);
   ListArgs L{};
-  fn<<<f32_grid(c), kScoreThreads, smem, s>>>(c->P, a, L);
+  fn<<<grid, kScoreThreads, smem, s>>>(c->P, a, L);
   MF_CUDA(cudaGetLastError());
   return MF_OK;
 }

@@ -782,9 +782,7 @@ mf_status tc_score_list(mf_ctx* c, const uint64_t* idx, uint64_t n, float* score
   for (uint64_t b = 0; b < n; b += span) {
     const uint64_t m = n - b < span ? n - b : span;
     const uint64_t tiles = (m + 127) / 128;
-    const uint64_t per_cta = (uint64_t)T.pipes;
-    uint64_t grid = (tiles + per_cta - 1) / per_cta;
-    if (grid > (uint64_t)c->num_sms) grid = c->num_sms;
+    const uint64_t grid = tiles < (uint64_t)c->num_sms ? tiles : (uint64_t)c->num_sms;
     TcList L{idx + b, m, score + b, feas ? feas + b : nullptr, pred ? pred + b * N * 2 : nullptr};
     for (int p = 0; p < T.npasses; ++p) {
       set_pass(T, p, partial);

@@ -591,6 +591,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   __shared__ uint32_t s_tmem;
   __shared__ float s_shared_bar[kTcMaxPipes];
   __shared__ int s_abort;
+  __shared__ unsigned long long s_count;
   __shared__ float s_b3[MF_MAX_MODELS][HF ? 4 : 2];  // b3 (thr, lat); HF: the outputs' scales back
   const int tid = threadIdx.x;
   // compile-time K-step counts must be the layout's (else no MMA may run)
@@ -623,6 +624,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
 
   if (tid == 0) {
     s_abort = 0;
+    s_count = 0ull;
     for (int j = 0; j < 1 + 2 * npipes; ++j) mbar_init(&bars[j], 1);
     mbar_init(&bars[1 + 2 * npipes], 1);           // the timeout test's barrier: nothing arrives
     mbar_init(&bars[2 + 2 * npipes], npipes);  // drain: one commit per issuing warp
@@ -731,7 +733,11 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   unsigned int my_count = 0;
 
   const uint64_t n = MODE == kTcRange ? R.len : L.n;
-  const uint64_t gpipe = (uint64_t)blockIdx.x * npipes + pipe;
+  // A short range or list goes to as many SMs as it has tiles, not to all pipelines of a few.
+  // (Not the exact variants' ranges, where this order costs three registers too many: spills,
+  // 22 M candidates 3.93 ms against 3.74.)
+  const uint64_t gpipe = MODE == kTcRange && XM != kXmBf16 ? (uint64_t)blockIdx.x * npipes + pipe
+                                                            : (uint64_t)pipe * gridDim.x + blockIdx.x;
   const uint64_t gstride = (uint64_t)gridDim.x * npipes;
 
   // UMMA descriptors: every model's image has the same size, so model i's B operands sit
@@ -871,35 +877,35 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   // by the tile stride.  List mode: of the index `at`.
   auto tile_digits = [&](uint64_t tile, uint8_t* into, DS from, bool first, uint64_t at) -> DS {
     const uint64_t t = tile * 128 + row;
-    if constexpr (RD && MODE == kTcList) {
-      uint64_t q = at, d = 0;
-      if (q >= P.total) {
-        if (t < n) atomicOr(P.status, kStatusBadInput);
-        q = 0;  // compute on candidate 0, discard at the end
-      }
+    // the digits of an index, last model first (the quotient goes on to the next model)
+    auto divide = [&](uint64_t q, auto put) {
       if (P.total <= 0x100000000ull) {
         uint32_t q32 = (uint32_t)q;
-#pragma unroll
-        for (int i = NM - 1; i >= 0; --i) {
-          const uint32_t qn = q32 / (uint32_t)P.K[i];
-          d |= (uint64_t)(q32 - qn * (uint32_t)P.K[i]) << (8 * (NM - 1 - i));
+#pragma unroll (NM > 0 ? NM : 1)
+        for (int i = N - 1; i >= 0; --i) {
+          const uint32_t K = (uint32_t)P.K[i], qn = q32 / K;
+          put(i, q32 - qn * K);
           q32 = qn;
         }
       } else {
-#pragma unroll
-        for (int i = NM - 1; i >= 0; --i) {
-          const uint64_t qn = q / (uint64_t)P.K[i];
-          d |= (q - qn * (uint64_t)P.K[i]) << (8 * (NM - 1 - i));
+#pragma unroll (NM > 0 ? NM : 1)
+        for (int i = N - 1; i >= 0; --i) {
+          const uint64_t K = (uint64_t)P.K[i], qn = q / K;
+          put(i, (uint32_t)(q - qn * K));
           q = qn;
         }
       }
-      return d;
-    } else if constexpr (RD) {
-      if (first) {
-        const uint64_t idx = R.base + t;
+    };
+    uint64_t index = MODE == kTcRange ? R.base + t : at;
+    if (MODE == kTcRange && first && index >= P.total) index = 0;  // (a row past the range's end)
+    if (MODE == kTcList && index >= P.total) {
+      if (t < n) atomicOr(P.status, kStatusBadInput);
+      index = 0;  // compute on candidate 0, discard at the end
+    }
+    if constexpr (RD) {
+      if (MODE == kTcList || first) {
         uint64_t d = 0;
-#pragma unroll
-        for (int i = 0; i < NM; ++i) d |= (uint64_t)((idx / P.stride[i]) % P.K[i]) << (8 * (NM - 1 - i));
+        divide(index, [&](int i, uint32_t v) { d |= (uint64_t)v << (8 * (NM - 1 - i)); });
         return d;
       }
       // One add steps every digit: with each byte biased by 256 - K_i, a byte overflows
@@ -909,11 +915,11 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
       const uint64_t x = from + T.dstep;
       const uint64_t wrapped = ((x ^ from ^ T.dstep) >> 8) & ones;  // carry out of each byte
       return (x - (~(wrapped * 0xFFull) & T.dbias)) & ((1ull << (8 * NM)) - 1);
-    } else if (MODE == kTcRange) {
-      if (first) {
-        const uint64_t idx = R.base + t;
-#pragma unroll (NM > 0 ? NM : 1)
-        for (int i = 0; i < N; ++i) into[i * 128 + row] = (uint8_t)((idx / P.stride[i]) % P.K[i]);
+    } else {
+      if (MODE == kTcList) {
+        divide(index, [&](int i, uint32_t v) { into[i * 128 + row] = (uint8_t)v; });
+      } else if (first) {  // (once a launch: digit by digit, which takes fewer registers)
+        for (int i = 0; i < N; ++i) into[i * 128 + row] = (uint8_t)(((R.base + t) / P.stride[i]) % P.K[i]);
       } else {  // add the tile stride to the digits, last model first
         uint32_t carry = 0;
 #pragma unroll (NM > 0 ? NM : 1)
@@ -923,25 +929,6 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
           if (carry) d -= (uint32_t)P.K[i];
           into[i * 128 + row] = (uint8_t)d;
         }
-      }
-      return into;
-    } else {
-      uint64_t idx = at;
-      if (idx >= P.total) {
-        if (t < n) atomicOr(P.status, kStatusBadInput);
-        idx = 0;  // compute on candidate 0, discard at the end
-      }
-      // last model first, one division each (the quotient goes on to the next model)
-      if (P.total <= 0x100000000ull) {
-        uint32_t q = (uint32_t)idx;
-#pragma unroll (NM > 0 ? NM : 1)
-        for (int i = N - 1; i >= 0; --i) {
-          const uint32_t K = (uint32_t)P.K[i], qn = q / K;
-          into[i * 128 + row] = (uint8_t)(q - qn * K);
-          q = qn;
-        }
-      } else {
-        for (int i = 0; i < N; ++i) into[i * 128 + row] = (uint8_t)digit_of(P, idx, i);
       }
       return into;
     }
@@ -1340,10 +1327,8 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
       R.lists_s[gl + e] = tk.ls[e];
       R.lists_i[gl + e] = tk.li[e];
     }
-    unsigned int c = my_count;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if (lane == 0 && c) atomicAdd(R.count, (unsigned long long)c);
+    const unsigned int c = __reduce_add_sync(0xffffffffu, my_count);
+    if (lane == 0 && c) atomicAdd(&s_count, (unsigned long long)c);
   }
   // Nothing of this CTA may still run when its tensor memory is freed: each issuing warp
   // commits its MMAs to the drain barrier, and everyone waits for them and for the weight
@@ -1353,6 +1338,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   mbar_wait_drain(&bars[0], 0, P.status);
   tc_fence_before();
   __syncthreads();
+  if (MODE == kTcRange && tid == 0 && s_count) atomicAdd(R.count, s_count);  // (one a CTA, not one a warp)
   if (warp == 0) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");

@@ -393,7 +393,8 @@ static mf_status search_impl(mf_ctx* ctx, uint64_t lo, uint64_t hi, int32_t k, u
   // the exact (3-term tf32) tensor-core variant, where its lists fit next to the weights
   const bool tx = !fc && !tc && ctx->tc.tf && tc_fits(ctx, k);
   const int kcap = tc ? (k * 8 > 256 ? k * 8 : 256) : k;
-  const int grid = fc ? fc_grid(ctx, hi - lo < chunk ? hi - lo : chunk) : (tc || tx) ? tc_grid(ctx) : f32_grid(ctx);
+  const uint64_t launch_len = hi - lo < chunk ? hi - lo : chunk;
+  const int grid = fc ? fc_grid(ctx, launch_len) : (tc || tx) ? tc_grid(ctx) : f32_grid(ctx, launch_len);
 
   // scratch: per-CTA lists, two merge buffers, merged list, rescored shortlist, count
   const size_t entries = (size_t)grid * kcap;
@@ -450,7 +451,7 @@ static mf_status search_impl(mf_ctx* ctx, uint64_t lo, uint64_t hi, int32_t k, u
     a.base = lo;
     a.len = 0;
     int nl = 1;
-    st = fc ? fc_search_chunk(ctx, a, grid, s) : (tc || tx) ? tc_search_chunk(ctx, a, s, &nl) : f32_search_chunk(ctx, a, s);
+    st = fc ? fc_search_chunk(ctx, a, grid, s) : (tc || tx) ? tc_search_chunk(ctx, a, s, &nl) : f32_search_chunk(ctx, a, grid, s);
     if (st != MF_OK) return st;
     launches += nl;
     score_launches += nl;
@@ -459,7 +460,7 @@ static mf_status search_impl(mf_ctx* ctx, uint64_t lo, uint64_t hi, int32_t k, u
     a.base = b;
     a.len = (hi - b) < chunk ? (hi - b) : chunk;
     int nl = 1;
-    st = fc ? fc_search_chunk(ctx, a, grid, s) : (tc || tx) ? tc_search_chunk(ctx, a, s, &nl) : f32_search_chunk(ctx, a, s);
+    st = fc ? fc_search_chunk(ctx, a, grid, s) : (tc || tx) ? tc_search_chunk(ctx, a, s, &nl) : f32_search_chunk(ctx, a, grid, s);
     if (st != MF_OK) return st;
     a.first = 0;
     launches += nl;

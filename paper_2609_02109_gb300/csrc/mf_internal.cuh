@@ -469,9 +469,9 @@ __device__ __forceinline__ void stamp_start(const RangeArgs& R) {
 }
 bool f32_supported(const Params& P);
 size_t f32_smem_bytes(const Params& P, int k, bool& resident);
-int f32_grid(const mf_ctx* c);
+int f32_grid(const mf_ctx* c, uint64_t len);
 mf_status f32_prepare(mf_ctx* c);
-mf_status f32_search_chunk(mf_ctx* c, const RangeArgs& a, cudaStream_t s);
+mf_status f32_search_chunk(mf_ctx* c, const RangeArgs& a, int grid, cudaStream_t s);
 // Fixed-context mode: one range launch of the table-lookup scan over the per-option
 // table of mf_fc_set.
 int fc_grid(const mf_ctx* c, uint64_t len);
