@@ -1,4 +1,6 @@
-// Tensor-core (tcgen05: bf16 x bf16 -> fp32, or 3-term tf32 -> fp32) scorer for sm_103a.
+// Tensor-core (tcgen05: bf16 x bf16 -> fp32, or 3-term fp16 / tf32 splits -> fp32) scorer
+// for sm_103a.  Included by the translation units that instantiate it; the host side is in
+// k_tc.cu.
 //
 // Same computation as the exact fp32 path (arXiv 2609.02109: Eq. 1 decode, the
 // aggregate GPU state, the per-model MeanField MLP of Eq. 6, the constraints of
@@ -12,8 +14,8 @@
 //                                                    (b3 is added in the final epilogue).
 //
 // One persistent CTA per SM runs up to four independent 128-row pipelines.  Each has
-// four epilogue warps (warp q of a pipeline owns TMEM lanes 32q..32q+31) and one warp
-// that only issues the pipeline's MMAs: every MMA group starts on a named-barrier
+// four epilogue warps (warp q of a pipeline owns TMEM lanes 32q..32q+31), or eight (see
+// tc_ew), and one warp that only issues the pipeline's MMAs: every MMA group starts on a named-barrier
 // rendezvous with the epilogue warps once its operands are stored, and is committed to
 // an mbarrier the epilogue warps wait on (bounded; a wait that gives up raises the
 // status word and the kernel runs to completion without further waits).  Every A
@@ -32,8 +34,8 @@
 //
 // Each thread keeps its candidate's digits (option index per model) and steps them
 // from tile to tile by adding the digits of the tile stride with carries, so no
-// division runs in the hot loop: packed in registers in the six-model instantiation,
-// else in shared memory.
+// division runs in the hot loop: packed in registers in the unrolled instantiations (three
+// to seven models), else in shared memory.
 //
 // The exact fp32 variants (XM = kXmHalf, kXmTf32) run the same kernel on split operands:
 // every operand is a hi part plus a lo part (the rest), about 22 bits together, and each
@@ -49,7 +51,8 @@
 //            scaled back in the fused multiply-add that adds b3.
 //   kXmTf32  tf32 parts, K = 8 steps of kind::tf32, two pipelines: for tables and weights that
 //            the scaling cannot serve (see half_ranges).
-// 24^6 candidates, N = 6, 12->64->64->2: scoring 32.6 ms, 351 TFLOP/s algorithmic (tf32 parts: 68.8 ms, 167), error against fp64 half of it.
+// 24^6 candidates, N = 6, 12->64->64->2: 31.2 ms, 367 TFLOP/s algorithmic (tf32 parts: 68.8
+// ms, 167), the error against fp64 half of theirs.  Tensor pipe 62 % busy, issue 57 %.
 #pragma once
 
 #include <cuda_bf16.h>
