@@ -867,9 +867,12 @@ k_vram_write(const Params P, const VramArgs A) {
 // applied with probability crossover_p (draw kGaCrossDo, else the first parent is copied)
 // and repair of an infeasible individual by rejection sampling from the uniform
 // distribution over Lambda (draws kGaRepair, j = a * N + i, at most 256 / N attempts, the
-// first feasible one kept).  The block has 1024 threads whatever the population: eight lanes
-// breed an individual (a tournament entry or a gene each), and a warp's lanes share the
-// repairs of its individuals.  Bound by the latency of a generation's chain: draws, fitness
+// first feasible one kept).  The block has 1024 threads whatever the population: LPC lanes
+// breed an individual (tournament entries and genes shared out over them), and a warp's lanes
+// share the repairs of its individuals.  LPC is the most that holds the population in one
+// round (8 up to 128 individuals, 4 up to 256, 2 up to 512, else 1): the lanes cut a generation's chain,
+// but rounds of them one after another cost more than a thread per individual (population
+// 908, 11 generations, with its table: 137 us with one thread each, 224 with eight).  Bound by the latency of a generation's chain: draws, fitness
 // reads, the two tournaments, genes, their terms in model order, one block barrier.
 // Population 100, 30 generations, N = 5, some repairs: 93 us; one thread per individual, its draws
 // one after another, took 180 us.
@@ -889,8 +892,8 @@ __device__ __forceinline__ unsigned long long fc_rank(float f, int slot) {
 }
 __device__ __forceinline__ int fc_slot(unsigned long long r) { return (int)(0xFFFFFFFFu - (uint32_t)r); }
 
-// NG: genes a lane of a group of eight holds (N <= 8 NG).
-template <int NG>
+// LPC: lanes per individual (a power of two); NG: genes a lane holds (N <= NG LPC).
+template <int NG, int LPC>
 __global__ void __launch_bounds__(1024)
 k_fc_ga(const Params P, const FcGaArgs A) {
   extern __shared__ __align__(16) unsigned char sm[];
@@ -934,13 +937,13 @@ k_fc_ga(const Params P, const FcGaArgs A) {
   const uint64_t sd = A.seed;
   const int attempts = 256 / N;
   const int lane = c & 31;
-  // eight lanes per individual: lane gl of a group holds genes gl, gl + 8, ..
-  constexpr int kGroups = 128;
-  const int gl = lane & 7, group = c >> 3, g0l = lane & ~7;  // (g0l: the group's first lane)
+  // LPC lanes per individual: lane gl of a group holds genes gl, gl + LPC, ..
+  constexpr int kGroups = 1024 / LPC;
+  const int gl = lane % LPC, group = c / LPC, g0l = lane - gl;  // (g0l: the group's first lane)
   int off[NG], K[NG];
 #pragma unroll
   for (int q = 0; q < NG; ++q) {
-    const int i = gl + 8 * q;
+    const int i = gl + LPC * q;
     off[q] = i < N ? pick(P.off, i) : 0;
     K[q] = i < N ? pick(P.K, i) : 1;
   }
@@ -950,23 +953,23 @@ k_fc_ga(const Params P, const FcGaArgs A) {
 #pragma unroll
     for (int q = 0; q < NG; ++q) {
       e[q] = tab[off[q] + gene[q]];
-      if (gl + 8 * q < N && child < pop) genes[(size_t)child * N + gl + 8 * q] = (uint8_t)gene[q];
+      if (gl + LPC * q < N && child < pop) genes[(size_t)child * N + gl + LPC * q] = (uint8_t)gene[q];
     }
     float J = 0.f, V = 0.f;
 #pragma unroll
     for (int q = 0; q < NG; ++q)
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
-        if (i + 8 * q < N) {
-          J += __shfl_sync(0xffffffffu, e[q].x, g0l + i);
-          V += __shfl_sync(0xffffffffu, e[q].y, g0l + i);
+      for (int i = 0; i < LPC; ++i)
+        if (i + LPC * q < N) {
+          J += LPC == 1 ? e[q].x : __shfl_sync(0xffffffffu, e[q].x, g0l + i);
+          V += LPC == 1 ? e[q].y : __shfl_sync(0xffffffffu, e[q].y, g0l + i);
         }
     const bool ok = V <= P.vram_cap && J > -INFINITY;
     if (gl == 0 && child < pop) fit[child] = ok ? J : -INFINITY;
     return ok ? J : -INFINITY;
   };
   // Repair of the warp's infeasible children (`bad`: this lane's group has one, child `child`):
-  // the warp's lanes are shared out over them (32, 16 or 8 lanes each), which try the child's
+  // the warp's lanes are shared out over them (32, 16, 8, .. lanes each), which try the child's
   // attempts in order, so many at a time; the lowest feasible attempt of the first successful
   // round is the sequential search's result.  The winning lane writes the child's genes and
   // fitness over the unrepaired ones.
@@ -975,7 +978,8 @@ k_fc_ga(const Params P, const FcGaArgs A) {
     if (!bal) return;
     __syncwarp();
     const int cnt = __popc(bal);
-    const int gs = cnt == 1 ? 32 : cnt == 2 ? 16 : 8;
+    int gs = 32;
+    while (gs * cnt > 32) gs >>= 1;
     const int mine = lane / gs;  // this lane works for the mine-th of them
     unsigned rest = bal;
     for (int j = 0; j < mine; ++j) rest &= rest - 1u;
@@ -985,11 +989,11 @@ k_fc_ga(const Params P, const FcGaArgs A) {
     for (int a0 = 0; a0 < attempts && __any_sync(0xffffffffu, !done); a0 += gs) {
       const int a = a0 + lane % gs;
       float Jc = -INFINITY;
-      uint64_t cand[NG] = {};
+      uint64_t cand[(NG * LPC + 7) / 8] = {};
       if (!done && a < attempts) {  // the fitness' sums, with the draws kept in registers
         float Js = 0.f, Vs = 0.f;
 #pragma unroll
-        for (int i = 0; i < 8 * NG; ++i)
+        for (int i = 0; i < LPC * NG; ++i)
           if (i < N) {
             const int o = ga_unif(ga_rng(sd, G, (uint32_t)who, kGaRepair, (uint32_t)(a * N + i)), (uint32_t)P.K[i]);
             cand[i >> 3] |= (uint64_t)o << (8 * (i & 7));
@@ -1013,8 +1017,8 @@ k_fc_ga(const Params P, const FcGaArgs A) {
   // the fittest of the warp's individuals joins the population's (gl: one lane of a group)
   auto rank_in = [&](int child, const float* fit, unsigned long long* best) {
     unsigned long long r = gl == 0 && child < pop ? fc_rank(fit[child], child) : 0ull;
-    r = max(r, __shfl_xor_sync(0xffffffffu, r, 8));
-    r = max(r, __shfl_xor_sync(0xffffffffu, r, 16));
+#pragma unroll
+    for (int w = LPC; w < 32; w <<= 1) r = max(r, __shfl_xor_sync(0xffffffffu, r, w));
     if (lane == 0 && r) atomicMax(best, r);
   };
   for (int c0 = 0; c0 < pop; c0 += kGroups) {  // initial population: uniform over Lambda, repaired
@@ -1022,7 +1026,7 @@ k_fc_ga(const Params P, const FcGaArgs A) {
     int gene[NG];
 #pragma unroll
     for (int q = 0; q < NG; ++q)
-      gene[q] = ga_unif(ga_rng(sd, 0, (uint32_t)child, kGaInit, (uint32_t)(gl + 8 * q)), (uint32_t)K[q]);
+      gene[q] = ga_unif(ga_rng(sd, 0, (uint32_t)child, kGaInit, (uint32_t)(gl + LPC * q)), (uint32_t)K[q]);
     const float J = place(child, gene, g0, fit0);
     repair(0u, repairable && child < pop && J == -INFINITY, child, g0, fit0);
     rank_in(child, fit0, &s_best[0]);
@@ -1046,21 +1050,21 @@ k_fc_ga(const Params P, const FcGaArgs A) {
       const bool cross = (uint32_t)(ga_rng(sd, G, cu, kGaCrossDo, 0u) >> 40) < A.cross_thr;
 #pragma unroll
       for (int q = 0; q < NG; ++q) {
-        const uint32_t i = (uint32_t)(gl + 8 * q);
+        const uint32_t i = (uint32_t)(gl + LPC * q);
         take_b[q] = cross && (ga_rng(sd, G, cu, kGaCross, i) >> 63);
         mutate[q] = (uint32_t)(ga_rng(sd, G, cu, kGaMut, i) >> 40) < A.mut_thr;
         mval[q] = ga_unif(ga_rng(sd, G, cu, kGaMutVal, i), (uint32_t)K[q]);
       }
       // the two tournaments, entries shared out over the group's lanes
       unsigned long long win[2] = {0ull, 0ull};
-      for (int d = gl; d < 2 * A.tournament; d += 8) {
+      for (int d = gl; d < 2 * A.tournament; d += LPC) {
         const int w = d < A.tournament ? 0 : 1;
         const int s2 = ga_unif(ga_rng(sd, G, cu, w ? kGaTourB : kGaTourA, (uint32_t)(d - w * A.tournament)), (uint32_t)pop);
         const unsigned long long r = fc_rank(fc_[s2], s2);
         if (w) win[1] = max(win[1], r); else win[0] = max(win[0], r);
       }
 #pragma unroll
-      for (int w = 4; w > 0; w >>= 1) {
+      for (int w = LPC / 2; w > 0; w >>= 1) {
         win[0] = max(win[0], __shfl_xor_sync(0xffffffffu, win[0], w));
         win[1] = max(win[1], __shfl_xor_sync(0xffffffffu, win[1], w));
       }
@@ -1070,7 +1074,7 @@ k_fc_ga(const Params P, const FcGaArgs A) {
       int gene[NG];
 #pragma unroll
       for (int q = 0; q < NG; ++q) {
-        const int i = gl + 8 * q;
+        const int i = gl + LPC * q;
         gene[q] = i < N ? gc[(size_t)(take_b[q] ? parent[1] : parent[0]) * N + i] : 0;
         if (mutate[q] && !elite && i < N) gene[q] = mval[q];
       }
@@ -1304,7 +1308,11 @@ mf_status mf_fc_ga_run(mf_ctx* ctx, const mf_fc_ga_params* g, uint64_t seed, int
   A.out_genome = h;
   A.out_fit = (float*)(h + 16);
   const size_t smem = sizeof(float2) * ctx->sumK + sizeof(float) * 2 * g->pop + (size_t)2 * g->pop * N;
-  const auto fn = N <= 8 ? k_fc_ga<1> : k_fc_ga<2>;
+  const bool n8 = N <= 8;
+  const auto fn = g->pop <= 128   ? (n8 ? k_fc_ga<1, 8> : k_fc_ga<2, 8>)
+                  : g->pop <= 256 ? (n8 ? k_fc_ga<2, 4> : k_fc_ga<4, 4>)
+                  : g->pop <= 512 ? (n8 ? k_fc_ga<4, 2> : k_fc_ga<8, 2>)
+                                  : (n8 ? k_fc_ga<8, 1> : k_fc_ga<16, 1>);
   MF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   fn<<<1, 1024, smem, s>>>(ctx->P, A);
   MF_CUDA(cudaGetLastError());
