@@ -179,6 +179,7 @@ def search_exhaustive_noalloc(prob: dict, k: int, chunk: int = 0, device: int | 
     """mf_search_exhaustive_noalloc: the exact fp32 search with no device allocation
     (all device memory in the library's fixed array); same result fields as
     Context.search."""
+    torch.cuda.init()  # (a no-op once done; the stream is asked for without it)
     device = torch.cuda.current_device() if device is None else int(device)
     p, _keep = _problem_struct(prob, device, "fp32")
     r, ti, ts = _search_result(k)
