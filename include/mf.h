@@ -55,9 +55,8 @@ typedef enum {
 
 /* MF_FP32: fp32 results (scores within 1e-5 of the fp64 definition).  For the
  * d_L 8, 12 -> 64 -> 64 -> 2 predictor shape (up to 8 models) the scoring runs on the
- * tensor cores with every operand split into two parts of 11 bits (hi.hi + hi.lo + lo.hi,
- * about 22 bits per product, fp32 accumulation; fp16 parts scaled by powers of two, or
- * tf32 parts where the values' ranges do not allow that); other shapes run on the CUDA cores.
+ * tensor cores with every operand split into two tf32 parts (hi.hi + hi.lo + lo.hi,
+ * about 22 bits per product, fp32 accumulation); other shapes run on the CUDA cores.
  * MF_FP32_SIMT: the same results on the CUDA cores for every shape.
  * MF_BF16: bf16 tensor-core scoring, search results re-scored in fp32. */
 typedef enum { MF_FP32 = 0, MF_BF16 = 1, MF_FP32_SIMT = 2 } mf_precision;

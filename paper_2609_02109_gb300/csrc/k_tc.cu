@@ -22,37 +22,6 @@ uint16_t f2bf(float f) {  // round to nearest even
   return (uint16_t)(u >> 16);
 }
 
-// fp16 bits of |f| < 65504 (nearest even); `rounded`: the value they stand for.  Without a
-// branch, so that loops over it vectorise.
-inline uint16_t f2half(float f, float& rounded) {
-  uint32_t u, m, r;
-  std::memcpy(&u, &f, 4);
-  const uint32_t sign = u & 0x80000000u;
-  u ^= sign;
-  // from 2^-14 on: the mantissa rounded to 10 bits
-  const uint32_t un = (u + 0xFFFu + ((u >> 13) & 1u)) & ~0x1FFFu;
-  // below: multiples of 2^-24, which the sum with 1/2 rounds to
-  float a;
-  std::memcpy(&a, &u, 4);
-  const float v = a + 0.5f, vs = v - 0.5f;
-  std::memcpy(&m, &v, 4);
-  std::memcpy(&r, &vs, 4);
-  const uint32_t small = u < 0x38800000u ? 0xFFFFFFFFu : 0u;
-  const uint32_t bits = (small & (m - 0x3F000000u)) | (~small & ((un - 0x38000000u) >> 13));
-  const uint32_t val = ((small & r) | (~small & un)) | sign;
-  std::memcpy(&rounded, &val, 4);
-  return (uint16_t)((sign >> 16) | bits);
-}
-
-// Hi and lo parts of n <= 8 values.
-inline void split_half(const float* v, int n, uint16_t* hi, uint16_t* lo) {
-  for (int k = 0; k < n; ++k) {
-    float r, rest;
-    hi[k] = f2half(v[k], r);
-    lo[k] = f2half(v[k] - r, rest);
-  }
-}
-
 float bf2f(uint16_t b) {
   const uint32_t u = (uint32_t)b << 16;
   float f;
@@ -126,7 +95,7 @@ bool tc_wide(const TcArgs& T) { return T.kw == 16 && T.dle == 16 && T.h1 == 128 
 // models) with all counts fixed at compile time, and a run-time fallback per A1 row width.
 template <int MODE, bool MP, bool UT>
 TcFn tc_kernel_mode(const TcArgs& T, int n_models) {
-  if (T.tf != kXmBf16) return tc_kernel_exact(T.tf, MODE, MP, UT);
+  if (T.tf != kXmBf16) return tc_kernel_exact(MODE, MP, UT);
   // S1 = k1 / 16, S2 = h1 / 16 + 1 (the b2 step), S3 = hl / 16
   if (T.kw == 8 && T.dle == 8 && T.h1 == 64 && T.h2 == 64 && T.n3 == 16) {
     // The model loop unrolled with register digits, where a pass holds all models and their
@@ -229,12 +198,12 @@ static void set_passes(const Params& P, TcArgs& T, size_t budget) {
   }
 }
 
-// The shared-memory layout for lists of kcap entries: in the fp16 variant (three pipelines'
-// lists), and where two epilogue warps share a lane quarter (their rows take more), with
-// fewer models per pass if the lists would not fit next to a full pass's weights.
+// The shared-memory layout for lists of kcap entries: where two epilogue warps share a lane
+// quarter (their rows take more), with fewer models per pass if the lists would not fit next
+// to a full pass's weights.
 static bool layout_for(const Params& P, TcArgs& T, int kcap) {
   layout_smem(P, T, kcap);
-  if (T.sm_total > kSmemLimit && (T.tf == kXmHalf || T.ew == 2)) {
+  if (T.sm_total > kSmemLimit && T.ew == 2) {
     set_passes(P, T, 2 * kPassImageBudget / 3);
     set_pass(T, 0, nullptr);
     layout_smem(P, T, kcap);
@@ -358,262 +327,13 @@ mf_status tc_prepare_exact(mf_ctx* c, const TcHost& h) {
   return MF_OK;
 }
 
-// The powers of two of the fp16 variant (all exact in fp32).
-struct HalfScales {
-  float cagg[3];                    // aggregate columns (shared by the models)
-  std::vector<float> cx, t, u, v;   // [N][dl] features, [N][h1], [N][h2] units, [N][2] outputs
-};
-
-// 2^e with m 2^e in (2^(top - 1), 2^top]; 1 for m = 0.
-float pow2_to(float m, int top) {
-  if (m == 0.f) return 1.f;
-  int e;
-  const float f = std::frexp(m, &e);
-  return std::ldexp(1.f, top - (f == 0.5f ? e - 1 : e));
-}
-
-// sum of |w_k| x_k, in eight partial sums (so that it vectorises)
-float abs_dot(const float* w, const float* x, int n) {
-  float s[8] = {};
-  int k = 0;
-  for (; k + 8 <= n; k += 8)
-    for (int j = 0; j < 8; ++j) s[j] += std::fabs(w[k + j]) * x[k + j];
-  for (; k < n; ++k) s[0] += std::fabs(w[k]) * x[k];
-  return ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
-}
-
-// Scales from the largest value that each feature column, the aggregate and each unit can
-// take over the option tables (|W| times the inputs' maxima, plus |b|): inputs to 2^4, the
-// first hidden layer to 2^9, the second to 2^14, below fp16's 65504 whatever the candidate.
-// Weights then are of order 1 to 2^6.  A part below 2^-3 loses lo bits (fp16's spacing ends
-// at 2^-24): an absolute error of 2^-25, which is below what the split itself leaves as long
-// as a unit's inputs and weights have products of order 1 (2^-22 of them) to sum.  So the
-// rule: everything finite, and for every first-layer unit and option the sum of |products|
-// (b1 and the least aggregate among them) is at least 1, 2^-9 of its largest; the second
-// layer inherits errors of that size.  Option tables whose features differ by more, outliers
-// for instance, run on tf32, whose exponent needs no scaling.
-bool half_ranges(const Params& P, const TcHost& host, HalfScales& S) {
-  const float *w = host.w, *x = host.x, *dem4 = host.dem4;
-  const int N = P.n_models, dl = P.d_local, h1 = P.h1, h2 = P.h2, din = P.d_in;
-  // (NaN fails every comparison; the bounds carry a margin for their own rounding)
-  auto fits = [](float m) { return m == 0.f || (m > 1e-15f && m < 1e15f); };
-  constexpr float kMargin = 1.0001f;
-  float amax[3], amin[3];
-  for (int q = 0; q < 3; ++q) {
-    float hi = 0.f, lo = 0.f;
-    bool positive = true;
-    for (int i = 0; i < N; ++i) {
-      float m = 0.f, l = INFINITY;
-      for (int o = 0; o < P.K[i]; ++o) {
-        const float d = dem4[(size_t)(P.off[i] + o) * 4 + q];
-        if (!std::isfinite(d)) return false;
-        m = std::fmax(m, std::fabs(d));
-        l = std::fmin(l, d);
-      }
-      hi += m;
-      lo += l;
-      positive = positive && l >= 0.f;
-    }
-    amax[q] = hi * std::fabs(P.agg_scale[q]) * kMargin;
-    amin[q] = positive ? lo * std::fabs(P.agg_scale[q]) : 0.f;
-    if (!fits(amax[q])) return false;
-    S.cagg[q] = pow2_to(amax[q], 4);
-  }
-  S.cx.resize((size_t)N * dl);
-  S.t.resize((size_t)N * h1);
-  S.u.resize((size_t)N * h2);
-  S.v.resize((size_t)N * 2);
-  float hb[MF_MAX_HIDDEN], in[MF_MAX_D_LOCAL + 4];
-  std::vector<float> xs;  // |x| scaled
-  for (int i = 0; i < N; ++i) {
-    const float* W1 = w + (size_t)i * P.per_model;
-    const float* b1 = W1 + (size_t)h1 * din;
-    const float* W2 = b1 + h1;
-    const float* b2 = W2 + (size_t)h2 * h1;
-    const float* W3 = b2 + h2;
-    const float* xi = x + (size_t)P.off[i] * dl;
-    for (int k = 0; k < dl; ++k) {
-      in[k] = 0.f;
-      for (int o = 0; o < P.K[i]; ++o) {
-        const float v = std::fabs(xi[(size_t)o * dl + k]);
-        if (!std::isfinite(v)) return false;
-        in[k] = std::fmax(in[k], v);
-      }
-      if (!fits(in[k])) return false;
-      S.cx[(size_t)i * dl + k] = pow2_to(in[k], 4);
-    }
-    for (int q = 0; q < 3; ++q) in[dl + q] = amax[q];
-    xs.clear();
-    for (int j = 0; j < h1; ++j) {
-      const float* wj = W1 + (size_t)j * din;
-      const float bb = std::fabs(b1[j]) + std::fabs(wj[dl + 3] * P.agg_scale[3] * (float)N);
-      const float m = (abs_dot(wj, in, dl + 3) + bb) * kMargin;
-      if (!fits(m)) return false;
-      hb[j] = m;
-      const float t = S.t[(size_t)i * h1 + j] = pow2_to(m, 9);
-      const float cst = std::fabs(b1[j] + wj[dl + 3] * P.agg_scale[3] * (float)N);
-      const float least = (cst + abs_dot(wj + dl, amin, 3)) * t;
-      if (m == 0.f || least >= 1.f) continue;
-      if (xs.empty()) {
-        xs.resize((size_t)P.K[i] * dl);
-        for (size_t e = 0; e < xs.size(); ++e) xs[e] = std::fabs(xi[e]) * S.cx[(size_t)i * dl + e % dl];
-      }
-      float aw[MF_MAX_D_LOCAL];
-      for (int k = 0; k < dl; ++k) aw[k] = wj[k] * t / S.cx[(size_t)i * dl + k];
-      for (int o = 0; o < P.K[i]; ++o)
-        if (!(least + abs_dot(aw, xs.data() + (size_t)o * dl, dl) >= 1.f)) return false;
-    }
-    float top[2] = {0.f, 0.f};
-    for (int j = 0; j < h2; ++j) {
-      const float m = (abs_dot(W2 + (size_t)j * h1, hb, h1) + std::fabs(b2[j])) * kMargin;
-      if (!fits(m)) return false;
-      const float u = S.u[(size_t)i * h2 + j] = pow2_to(m, 14);
-      for (int r = 0; r < 2; ++r) {
-        const float v = std::fabs(W3[(size_t)r * h2 + j]) / u;
-        if (!std::isfinite(v)) return false;
-        top[r] = std::fmax(top[r], v);
-      }
-    }
-    for (int r = 0; r < 2; ++r) {
-      if (!fits(top[r]) || !std::isfinite(W3[2 * h2 + r])) return false;
-      S.v[(size_t)i * 2 + r] = pow2_to(top[r], 6);
-    }
-  }
-  return true;
-}
-
-// The fp16 variant's layout and operand images; MF_EUNSUPPORTED (nothing changed) where
-// half_ranges rules it out.
-mf_status tc_prepare_half(mf_ctx* c, const TcHost& h) {
-  const Params& P = c->P;
-  TcArgs& T = c->tc;
-  const int N = P.n_models, dl = P.d_local, h1 = P.h1, h2 = P.h2, hl = h2, din = P.d_in, sumK = c->sumK;
-  const float *w = h.w, *x = h.x;
-  HalfScales S;
-  if (!half_ranges(P, h, S)) return MF_EUNSUPPORTED;
-  T.tf = kXmHalf;
-  T.dle = dl;
-  T.k1 = 16;  // [x (8) | aggregate (3) | 1 | 0 0 0 0]
-  T.kw = 8;   // words per option: x hi pairs (4), x lo pairs (4)
-  T.h1 = h1;
-  T.h2 = h2;
-  T.hl = hl;
-  T.n3 = 16;
-  // TMEM columns: the pipelines' D (64 each), their D3 (16 each), then per pipeline
-  // H hi (32) | ones (8) | H lo (32) | A1 hi (8), A1 lo (8): 504 of 512 for three pipelines
-  T.pipes = tc_pipes(kXmHalf);
-  T.ew = 1;
-  T.ps_d = h1;
-  T.ps_d3 = T.n3;
-  T.col_d = 0;
-  T.col_d3 = T.pipes * h1;
-  T.col_h = T.col_d3 + T.pipes * T.n3;
-  T.col_ones = T.col_h + h1 / 2;
-  T.col_hlo = T.col_ones + 8;
-  T.col_a = T.col_hlo + h1 / 2;
-  T.pipe_stride = T.col_a + 16 - T.col_h;
-  for (int q = 0; q < 3; ++q) T.cagg[q] = S.cagg[q];
-  // per model: B1 [h1 x 16] hi, lo; B2 [h2 x (h1 + 16)] hi (its last K-step holds b2 hi, lo
-  // against the ones block), [h2 x h1] lo; B3 [16 x hl] hi, lo
-  const int k2 = h1 + 16;
-  const size_t b1 = (size_t)h1 * T.k1 * 2, b2 = (size_t)h2 * k2 * 2, b2lo = (size_t)h2 * h1 * 2, b3 = (size_t)T.n3 * hl * 2;
-  T.img_lo1 = (uint32_t)b1;
-  T.img_lo2 = (uint32_t)b2;
-  T.img_lo3 = (uint32_t)b3;
-  T.img_model = (uint32_t)(2 * b1 + b2 + b2lo + 2 * b3);
-  std::vector<unsigned char> img(round_up((int)(T.img_model * N), 16), 0);
-  // n columns (a multiple of 8) of row r of an image with kdim columns, hi and lo image apart
-  auto put_row = [&](size_t at, int kdim, size_t at_lo, int kdim_lo, int r, const float* v, int n) {
-    unsigned char* ph = img.data() + at + umma_off(r, 0, kdim);
-    unsigned char* pl = img.data() + at_lo + umma_off(r, 0, kdim_lo);
-    for (int k = 0; k < n; k += 8, ph += 128, pl += 128) {
-      uint16_t hi[8], lo[8];
-      split_half(v + k, 8, hi, lo);
-      std::memcpy(ph, hi, 16);
-      std::memcpy(pl, lo, 16);
-    }
-  };
-  const double s3 = P.agg_scale[3];
-  float row[MF_MAX_HIDDEN], it[MF_MAX_HIDDEN], iu[MF_MAX_HIDDEN];  // a row; 1 / t, 1 / u
-  for (int i = 0; i < N; ++i) {
-    const float* W1 = w + (size_t)i * P.per_model;
-    const float* bb1 = W1 + (size_t)h1 * din;
-    const float* W2 = bb1 + h1;
-    const float* bb2 = W2 + (size_t)h2 * h1;
-    const float* W3 = bb2 + h2;
-    const float *cx = &S.cx[(size_t)i * dl], *t = &S.t[(size_t)i * h1], *u = &S.u[(size_t)i * h2], *v = &S.v[(size_t)i * 2];
-    for (int k = 0; k < h1; ++k) it[k] = 1.f / t[k];
-    for (int k = 0; k < h2; ++k) iu[k] = 1.f / u[k];
-    T.off_b1[i] = T.img_model * i;
-    T.off_b2[i] = T.off_b1[i] + (uint32_t)(2 * b1);
-    T.off_b3[i] = T.off_b2[i] + (uint32_t)(b2 + b2lo);
-    for (int j = 0; j < h1; ++j) {
-      const float* wj = W1 + (size_t)j * din;
-      std::memset(row, 0, sizeof(float) * 16);
-      for (int k = 0; k < dl; ++k) row[k] = wj[k] * t[j] / cx[k];
-      for (int q = 0; q < 3; ++q) row[dl + q] = wj[dl + q] * t[j] / S.cagg[q];
-      // the constant-1 column: b1 plus the weight of the constant feature N * s_3
-      row[dl + 3] = (float)(((double)bb1[j] + (double)wj[dl + 3] * s3 * N) * t[j]);
-      put_row(T.off_b1[i], T.k1, T.off_b1[i] + b1, T.k1, j, row, 16);
-    }
-    for (int j = 0; j < h2; ++j) {
-      for (int k = 0; k < h1; ++k) row[k] = W2[(size_t)j * h1 + k] * u[j] * it[k];
-      put_row(T.off_b2[i], k2, T.off_b2[i] + b2, h1, j, row, h1);
-      uint16_t hi, lo;
-      row[0] = bb2[j] * u[j];
-      split_half(row, 1, &hi, &lo);
-      std::memcpy(img.data() + T.off_b2[i] + umma_off(j, h1, k2), &hi, 2);
-      std::memcpy(img.data() + T.off_b2[i] + umma_off(j, h1 + 1, k2), &lo, 2);
-    }
-    for (int r = 0; r < 2; ++r) {
-      T.back[i][r] = 1.f / v[r];
-      for (int k = 0; k < hl; ++k) row[k] = W3[(size_t)r * hl + k] * v[r] * iu[k];
-      put_row(T.off_b3[i], hl, T.off_b3[i] + b3, hl, r * (T.n3 / 2) + i, row, hl);
-    }
-  }
-  T.img_total = (uint32_t)img.size();
-  set_passes(P, T, kPassImageBudget);
-  set_pass(T, 0, nullptr);
-  std::vector<uint32_t> xw((size_t)sumK * T.kw, 0u);
-  for (int i = 0; i < N; ++i)
-    for (int r = P.off[i]; r < P.off[i] + P.K[i]; ++r) {
-      uint16_t hi[8], lo[8];  // (d_L 8)
-      for (int k = 0; k < dl; ++k) row[k] = x[(size_t)r * dl + k] * S.cx[(size_t)i * dl + k];
-      split_half(row, dl, hi, lo);
-      std::memcpy(&xw[(size_t)r * T.kw], hi, 16);
-      std::memcpy(&xw[(size_t)r * T.kw + 4], lo, 16);
-    }
-  layout_smem(P, T, 0);
-  if (T.sm_total > kSmemLimit) return MF_EUNSUPPORTED;
-  const size_t o_xw = round_up((int)img.size(), 256);
-  const size_t total = o_xw + round_up((int)(xw.size() * 4), 256);
-  MF_CUDA(cudaMalloc(&c->d_tc, total));
-  c->tc_bytes = total;
-  unsigned char* base = static_cast<unsigned char*>(c->d_tc);
-  MF_CUDA(cudaMemcpy(base, img.data(), img.size(), cudaMemcpyHostToDevice));
-  MF_CUDA(cudaMemcpy(base + o_xw, xw.data(), xw.size() * 4, cudaMemcpyHostToDevice));
-  c->stats.h2d_bytes_create += img.size() + xw.size() * 4;
-  T.img = base;
-  T.xw = reinterpret_cast<const uint32_t*>(base + o_xw);
-  for (int u = 0; u < 2; ++u) {
-    MF_CUDA(cudaFuncSetAttribute(tc_kernel(kTcRange, T, u, N), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit));
-    MF_CUDA(cudaFuncSetAttribute(tc_kernel(kTcList, T, u, N), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit));
-  }
-  return MF_OK;
-}
-
 }  // namespace
 
 mf_status tc_prepare(mf_ctx* c, bool exact, const TcHost& h) {
   const Params& P = c->P;
   TcArgs& T = c->tc;
   std::memset(&T, 0, sizeof(T));
-  if (exact) {
-    const mf_status st = tc_prepare_half(c, h);
-    if (st != MF_EUNSUPPORTED) return st;
-    std::memset(&T, 0, sizeof(T));
-    return tc_prepare_exact(c, h);
-  }
+  if (exact) return tc_prepare_exact(c, h);
   const int N = P.n_models, dl = P.d_local, h1 = P.h1, h2 = P.h2, hl = h2 > 0 ? h2 : h1;
   const int din = P.d_in;
   T.dle = dl + (dl & 1);

@@ -1,5 +1,4 @@
-// Tensor-core (tcgen05: bf16 x bf16 -> fp32, or 3-term fp16 / tf32 splits -> fp32) scorer
-// for sm_103a.  Included by the translation units that instantiate it; the host side is in
+// Tensor-core (tcgen05: bf16 x bf16 -> fp32, or 3-term tf32 split -> fp32) scorer for sm_103a.  Included by the translation units that instantiate it; the host side is in
 // k_tc.cu.
 //
 // Same computation as the exact fp32 path (arXiv 2609.02109: Eq. 1 decode, the
@@ -37,26 +36,14 @@
 // division runs in the hot loop: packed in registers in the unrolled instantiations (three
 // to seven models), else in shared memory.
 //
-// The exact fp32 variants (XM = kXmHalf, kXmTf32) run the same kernel on split operands:
-// every operand is a hi part plus a lo part (the rest), about 22 bits together, and each
-// K step issues hi.hi + hi.lo + lo.hi MMAs into the fp32 accumulator (lo.lo, about 2^-22 of
-// a product, is dropped), which keeps the scores within the fp32 path's 1e-5.
-//   kXmHalf  fp16 parts, K = 16 steps of kind::f16: twice the rate of kind::tf32 on half
-//            the bits (fp16 and tf32 both carry 11), so half the tensor time, tensor memory
-//            and weight bytes; three pipelines per SM, six models in one weight pass.  fp16's
-//            short exponent is made up for by powers of two: every feature column, hidden
-//            unit and output is scaled so that its largest possible value (from the option
-//            tables and weights) sits where hi and lo parts keep all their bits.  ReLU
-//            commutes with the scaling, so it costs nothing until the outputs, which are
-//            scaled back in the fused multiply-add that adds b3.
-//   kXmTf32  tf32 parts, K = 8 steps of kind::tf32, two pipelines: for tables and weights that
-//            the scaling cannot serve (see half_ranges).
-// 24^6 candidates, N = 6, 12->64->64->2: 31.2 ms, 367 TFLOP/s algorithmic (tf32 parts: 68.8
-// ms, 167), the error against fp64 half of theirs.  Tensor pipe 62 % busy, issue 57 %.
+// The exact fp32 variant (XM = kXmTf32) runs the same kernel on split operands: every operand
+// is a tf32 hi part plus the rest (a lo part, also read as tf32), about 22 bits together, and
+// each layer issues hi.hi, hi.lo and lo.hi MMAs (kind::tf32, K = 8) into the fp32 accumulator
+// (lo.lo, about 2^-22 of a product, is dropped), which keeps the scores within the fp32 path's
+// 1e-5.  Two pipelines per SM, three models per weight pass.
 #pragma once
 
 #include <cuda_bf16.h>
-#include <cuda_fp16.h>
 
 #include <type_traits>
 
@@ -138,11 +125,6 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
 
-// Instruction descriptor of kind::f16: fp16 A and B (K-major), fp32 D, M = 128.
-__host__ __device__ constexpr uint32_t idesc_half(int n) {
-  return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-}
-
 // Instruction descriptor of kind::tf32: tf32 A and B (K-major), fp32 D, M = 128.
 __host__ __device__ constexpr uint32_t idesc_tf32(int n) {
   return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
@@ -169,26 +151,6 @@ __device__ __forceinline__ uint32_t relu_bf16x2(uint32_t lo, uint32_t hi) {
   uint32_t d;
   asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(__uint_as_float(hi)), "f"(__uint_as_float(lo)));
   return d;
-}
-
-// (lo, hi) after ReLU as an fp16 pair, rounded toward zero, and what the rounding left of
-// each, an fp16 pair again: hi part and lo part of two activations.  A truncated hi part
-// leaves a remainder >= 0, so the ReLU of the second conversion clears the negative inputs'
-// (whose hi part is 0 and whose remainder is the input itself).
-__device__ __forceinline__ void relu_split_half2(uint32_t lo, uint32_t hi, uint32_t& h, uint32_t& l) {
-  const float a = __uint_as_float(lo), b = __uint_as_float(hi);
-  asm("cvt.rz.relu.f16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(b), "f"(a));
-  float ra, rb;
-  asm("{\n .reg .b16 x, y, m;\n mov.b32 {x, y}, %2;\n mov.b16 m, 0xBC00;\n"  // -1.0
-      " fma.rn.f32.f16 %0, x, m, %3;\n fma.rn.f32.f16 %1, y, m, %4;\n}"
-      : "=f"(ra), "=f"(rb)
-      : "r"(h), "f"(a), "f"(b));
-  asm("cvt.rn.relu.f16x2.f32 %0, %1, %2;" : "=r"(l) : "f"(rb), "f"(ra));
-}
-
-__device__ __forceinline__ uint32_t half_bits(float v) { return (uint32_t)__half_as_ushort(__float2half_rn(v)); }
-__device__ __forceinline__ float half_rest(float v, uint32_t h) {
-  return v - __half2float(__ushort_as_half((unsigned short)h));
 }
 
 __device__ __forceinline__ uint32_t bf16_bits(float v) {
@@ -251,9 +213,9 @@ __device__ __forceinline__ void tmem_st_x16(uint32_t taddr, const uint32_t (&v)[
 // ---------------------------------------------------------------------------
 enum { kTcRange = 0, kTcList = 1 };
 constexpr int kTcMaxPipes = 4;
-// Operands of the MMAs (TcArgs::tf): bf16, or the exact variants' split parts.
-enum { kXmBf16 = 0, kXmTf32 = 1, kXmHalf = 2 };
-__host__ __device__ constexpr int tc_pipes(int xm) { return xm == kXmTf32 ? 2 : xm == kXmHalf ? 3 : kTcMaxPipes; }
+// Operands of the MMAs (TcArgs::tf): bf16, or the exact variant's tf32 parts.
+enum { kXmBf16 = 0, kXmTf32 = 1 };
+__host__ __device__ constexpr int tc_pipes(int xm) { return xm == kXmTf32 ? 2 : kTcMaxPipes; }
 // Each 128-row pipeline has four epilogue warps (warp w reaches tensor-memory lanes
 // 32 (w % 4) ..) and one warp that issues its MMAs: warps [0, 4 pipes) are the epilogue
 // warps (pipeline w / 4), warps [4 pipes, 5 pipes) the issuing warps (pipeline w - 4 pipes,
@@ -262,9 +224,8 @@ __host__ __device__ constexpr int tc_pipes(int xm) { return xm == kXmTf32 ? 2 : 
 // pipeline has two epilogue warps per lane quarter (TcArgs::ew): each converts half of the
 // columns, and the work beside is split too: the first half's warps prepare inputs (digits,
 // aggregate, A1 rows), the second half's take outputs (objective, constraints, top-k).
-// 50 M candidates of eight 20->128->128->2 predictors: 15.3 ms against 16.7.  (The fp16 split
-// converts as long, but its three pipelines then leave 72 registers a thread: 22 M candidates
-// 4.08 ms against 3.84.  Four pipelines would need 1152 threads.)
+// 50 M candidates of eight 20->128->128->2 predictors: 15.3 ms against 16.7.  (Four pipelines
+// would need 1152 threads.)
 __host__ __device__ constexpr int tc_pipe_threads(int ew) { return 32 * (4 * ew + 1); }
 constexpr uint32_t kWaitLimit = 4096;  // suspended retries (~1 ms each at most)
 
@@ -428,18 +389,6 @@ __device__ __forceinline__ void mma_tf3(uint32_t d, uint32_t a_hi, uint32_t a_lo
   for (int k = 0; k < KX; ++k) mma_ts_warp_tf32(d, a_lo + 8u * k, b_hi + 16u * k, idesc, 1u);
 }
 
-// The same for fp16 parts: K-steps of 16, 8 columns of A.
-template <int KH, int KX>
-__device__ __forceinline__ void mma_half3(uint32_t d, uint32_t a_hi, uint32_t a_lo, uint64_t b_hi, uint64_t b_lo,
-                                          uint32_t idesc, uint32_t acc0) {
-#pragma unroll
-  for (int k = 0; k < KH; ++k) mma_ts_warp(d, a_hi + 8u * k, b_hi + 16u * k, idesc, k > 0 ? 1u : acc0);
-#pragma unroll
-  for (int k = 0; k < KX; ++k) mma_ts_warp(d, a_hi + 8u * k, b_lo + 16u * k, idesc, 1u);
-#pragma unroll
-  for (int k = 0; k < KX; ++k) mma_ts_warp(d, a_lo + 8u * k, b_hi + 16u * k, idesc, 1u);
-}
-
 // `steps` MMAs of K = 16 along one K extent; S > 0 unrolls a compile-time count.
 template <int S>
 __device__ __forceinline__ void mma_steps(int steps, uint32_t d_tmem, uint32_t a_tmem, uint64_t desc,
@@ -522,28 +471,6 @@ __device__ __forceinline__ void hidden_epilogue_tf(uint32_t src, uint32_t dst_hi
   }
 }
 
-// The fp16 variant's hidden epilogue: fp32 accumulators [0, W) at `src` -> ReLU (NaN kept)
-// -> fp16 hi parts at `dst_hi` and lo parts at `dst_lo`, two values per column.
-template <int W, class FL, class FS>
-__device__ __forceinline__ void hidden_epilogue_half(uint32_t src, uint32_t dst_hi, uint32_t dst_lo, FL after_load,
-                                                     FS before_store) {
-  static_assert(W > 0 && W % 32 == 0, "32-column chunks");
-  uint32_t a[W / 32][32];
-#pragma unroll
-  for (int c = 0; c < W / 32; ++c) tmem_ld_x32(src + 32 * c, a[c]);
-  tmem_wait_ld();
-  after_load();
-#pragma unroll
-  for (int c = 0; c < W / 32; ++c) {
-    uint32_t h[16], l[16];
-#pragma unroll
-    for (int j = 0; j < 16; ++j) relu_split_half2(a[c][2 * j], a[c][2 * j + 1], h[j], l[j]);
-    if (c == 0) before_store();
-    tmem_st_x16(dst_hi + 16 * c, h);
-    tmem_st_x16(dst_lo + 16 * c, l);
-  }
-}
-
 // The aggregate words of a tile's A1 rows: h (and for the tf32 variant l, the lo parts).
 struct AggW {
   uint4 h, l;
@@ -568,7 +495,7 @@ struct AggW {
 // the previous tile's last, and that tile's constraints and top-k), a stage of the next
 // tile's digits and aggregate, and the next A1 row; then D2 -> H2.  The issuing warp does
 // nothing else, so an MMA group starts as soon as its operands are stored.
-// XM: the operands (kXmBf16, kXmTf32, kXmHalf).  SB: the lists share a bar (tc_shared_bar).
+// XM: the operands (kXmBf16, kXmTf32).  SB: the lists share a bar (tc_shared_bar).
 // EW: epilogue warps per lane quarter.
 __host__ __device__ constexpr int tc_ew(int xm, int s2) { return xm == kXmBf16 && s2 == 9 ? 2 : 1; }
 
@@ -577,11 +504,9 @@ __global__ void __launch_bounds__((XM == kXmBf16 && S2 == 9 ? 2 : tc_pipes(XM)) 
 k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   static_assert(AWO < 0 || AWO == 4 || AWO == 8, "partial A1 rows are written for these layouts only");
   static_assert(NM <= 7, "packed digits hold at most seven models");
-  constexpr bool TF = XM == kXmTf32, HF = XM == kXmHalf;
+  constexpr bool TF = XM == kXmTf32;
   static_assert(!TF || (KW == 16 && S1 == 2 && S2 == 9 && S3 == 8 && N3 == 16),
-                "the exact variants run the d_L 8, 64-64 shape");
-  static_assert(!HF || (KW == 8 && AWO == 4 && S1 == 1 && S2 == 5 && S3 == 4 && N3 == 16),
-                "the exact variants run the d_L 8, 64-64 shape");
+                "the exact variant runs the d_L 8, 64-64 shape");
   constexpr int KS = TF ? 8 : 16;  // K of one MMA
   constexpr int EW = tc_ew(XM, S2);
   static_assert(EW == 1 || NM == 0, "two epilogue warps share digits through shared memory");
@@ -595,7 +520,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   __shared__ float s_shared_bar[kTcMaxPipes];
   __shared__ int s_abort;
   __shared__ unsigned long long s_count;
-  __shared__ float s_b3[MF_MAX_MODELS][HF ? 4 : 2];  // b3 (thr, lat); HF: the outputs' scales back
+  __shared__ float s_b3[MF_MAX_MODELS][2];
   const int tid = threadIdx.x;
   // compile-time K-step counts must be the layout's (else no MMA may run)
   if ((S1 > 0 && S1 != T.k1 / KS) || (S2 > 0 && S2 != T.h1 / KS + 1) || (S3 > 0 && S3 != T.hl / KS) ||
@@ -654,10 +579,6 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
                       (T.h2 > 0 ? (size_t)T.h2 * T.h1 + T.h2 : 0) + 2 * (size_t)T.hl;
     s_b3[tid][0] = b3[0];
     s_b3[tid][1] = b3[1];
-    if constexpr (HF) {
-      s_b3[tid][2] = T.back[tid][0];
-      s_b3[tid][3] = T.back[tid][1];
-    }
   }
   // option tables with ordinary loads
   const int sumK = P.off[N - 1] + P.K[N - 1];
@@ -715,7 +636,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   // and leave it waiting at the next one; the pipeline's top-k uses a third barrier
   // among its epilogue warps
   const int sig0 = 1 + 2 * pipe, barid = 1 + 2 * npipes + pipe;
-  auto idesc = [](int n) { return TF ? idesc_tf32(n) : HF ? idesc_half(n) : idesc_bf16(n); };
+  auto idesc = [](int n) { return TF ? idesc_tf32(n) : idesc_bf16(n); };
   const uint32_t id1 = idesc(T.h1), id2 = idesc(T.h2), id3 = idesc(T.n3);
   const int s1 = T.k1 / KS, s2 = T.h1 / KS + 1, s3 = T.hl / KS;
   const int m0 = MP ? T.m0 : 0, m1 = MP ? T.m1 : N;  // this pass's models
@@ -727,7 +648,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
       uint32_t z[32] = {};  // the A1 rows' unused words stay zero
       tmem_st_x32(tA + lane_off, z);
     } else {
-      uint32_t v[8] = {HF ? 0x3C003C00u : 0x3F803F80u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+      uint32_t v[8] = {0x3F803F80u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
       tmem_st_x8(tOnes + lane_off, v);
     }
   }
@@ -737,10 +658,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
 
   const uint64_t n = MODE == kTcRange ? R.len : L.n;
   // A short range or list goes to as many SMs as it has tiles, not to all pipelines of a few.
-  // (Not the exact variants' ranges, where this order costs three registers too many: spills,
-  // 22 M candidates 3.93 ms against 3.74.)
-  const uint64_t gpipe = MODE == kTcRange && XM != kXmBf16 ? (uint64_t)blockIdx.x * npipes + pipe
-                                                            : (uint64_t)pipe * gridDim.x + blockIdx.x;
+  const uint64_t gpipe = (uint64_t)pipe * gridDim.x + blockIdx.x;
   const uint64_t gstride = (uint64_t)gridDim.x * npipes;
 
   // UMMA descriptors: every model's image has the same size, so model i's B operands sit
@@ -761,19 +679,14 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   };
   auto issue_mma1 = [&](uint64_t b) {
     if constexpr (TF) mma_tf3<S1, S1>(tD, tA, tA + 16u, b, b + (T.img_lo1 >> 4), id1, 0u);
-    else if constexpr (HF) mma_half3<S1, S1>(tD, tA, tA + 8u, b, b + (T.img_lo1 >> 4), id1, 0u);
     else mma_steps<S1>(s1, tD, tA, b, id1, 0u);
   };
-  // (HF: the lo image has no bias step, so its rows are shorter: another row-group stride)
-  const uint64_t lo2 = HF ? (uint64_t)(T.img_lo2 >> 4) - ((uint64_t)(16 * 16 >> 4) << 32) : T.img_lo2 >> 4;
   auto issue_mma2 = [&](uint64_t b) {
-    if constexpr (TF) mma_tf3<S2, S2 - 1>(tD, tH1, tHlo, b, b + lo2, id2, 0u);
-    else if constexpr (HF) mma_half3<S2, S2 - 1>(tD, tH1, tHlo, b, b + lo2, id2, 0u);
+    if constexpr (TF) mma_tf3<S2, S2 - 1>(tD, tH1, tHlo, b, b + (T.img_lo2 >> 4), id2, 0u);
     else mma_steps<S2>(s2, tD, tH1, b, id2, 0u);
   };
   auto issue_mma3 = [&](uint64_t b, uint32_t acc) {
     if constexpr (TF) mma_tf3<S3, S3>(tD3, tH2, tHlo, b, b + (T.img_lo3 >> 4), id3, acc);
-    else if constexpr (HF) mma_half3<S3, S3>(tD3, tH2, tHlo, b, b + (T.img_lo3 >> 4), id3, acc);
     else mma_steps<S3>(s3, tD3, tH2, b, id3, acc);
   };
   // The epilogue warps wait on the commits' mbarriers (suspended until the phase completes).
@@ -826,19 +739,6 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
         const uint32_t al[4] = {aw.l.x, aw.l.y, aw.l.z, aw.l.w};
         tmem_st_x4(tA + 8u + lane_off, ah);
         tmem_st_x4(tA + 24u + lane_off, al);
-      }
-      return;
-    }
-    if constexpr (HF) {  // words 0-3: x hi, 4-7: aggregate hi and 1; 8-11: x lo, 12-15: aggregate lo
-      const uint4 a = src[0], b = src[1];
-      const uint32_t vh[4] = {a.x, a.y, a.z, a.w}, vl[4] = {b.x, b.y, b.z, b.w};
-      tmem_st_x4(tA + lane_off, vh);
-      tmem_st_x4(tA + 8u + lane_off, vl);
-      if (with_agg) {
-        const uint32_t ah[4] = {aw.h.x, aw.h.y, aw.h.z, aw.h.w};
-        const uint32_t al[4] = {aw.l.x, aw.l.y, aw.l.z, aw.l.w};
-        tmem_st_x4(tA + 4u + lane_off, ah);
-        tmem_st_x4(tA + 12u + lane_off, al);
       }
       return;
     }
@@ -953,12 +853,6 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
                   make_uint4(__float_as_uint(v0 - __uint_as_float(h0)), __float_as_uint(v1 - __uint_as_float(h1)),
                              __float_as_uint(v2 - __uint_as_float(h2)), 0u)};
     }
-    if constexpr (HF) {  // fp16 hi parts and 1.0; the lo parts
-      const float c0 = v0 * T.cagg[0], c1 = v1 * T.cagg[1], c2 = v2 * T.cagg[2];
-      const uint32_t h0 = half_bits(c0), h1 = half_bits(c1), h2 = half_bits(c2);
-      const uint32_t l0 = half_bits(half_rest(c0, h0)), l1 = half_bits(half_rest(c1, h1)), l2 = half_bits(half_rest(c2, h2));
-      return AggW{make_uint4(h0 | (h1 << 16), h2 | (0x3C00u << 16), 0u, 0u), make_uint4(l0 | (l1 << 16), l2, 0u, 0u)};
-    }
     const uint32_t h0 = bf16_bits(v0), h1 = bf16_bits(v1), h2 = bf16_bits(v2);
     const uint32_t l0 = bf16_bits(v0 - __uint_as_float(h0 << 16));
     const uint32_t l1 = bf16_bits(v1 - __uint_as_float(h1 << 16));
@@ -974,7 +868,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   };
   // the model-i A1 row of the current tile (aggregate words already in place when AWO >= 0)
   auto next_a1 = [&](int i, DS dg) {
-    if (TF || HF || AWO >= 0) {
+    if (TF || AWO >= 0) {
       write_a1(i, dg, false, AggW{});
     } else {  // run-time layout: the whole row, aggregate recomputed
       float A0 = 0.f, A1 = 0.f, A2 = 0.f;
@@ -1007,9 +901,8 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   // (list mode: `at` is the row's index)
   auto add_model = [&](int j, uint32_t a, uint32_t b, DS dg, uint64_t tile_f, uint64_t at) {
     tmem_wait_ld_2(a, b);
-    // (HF: the products are exact, powers of two, so this rounds once, like the sums)
-    const float thr = tc_out(P, HF ? fmaf(__uint_as_float(a), s_b3[j][HF ? 2 : 0], s_b3[j][0]) : __uint_as_float(a) + s_b3[j][0]);
-    const float lat = tc_out(P, HF ? fmaf(__uint_as_float(b), s_b3[j][HF ? 3 : 1], s_b3[j][1]) : __uint_as_float(b) + s_b3[j][1]);
+    const float thr = tc_out(P, __uint_as_float(a) + s_b3[j][0]);
+    const float lat = tc_out(P, __uint_as_float(b) + s_b3[j][1]);
     if (MODE == kTcList && L.pred) {
       // (one 8-byte store where the caller's array allows it: always, but for a bare
       // pointer that is not 8-byte aligned)
@@ -1145,22 +1038,21 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
 #pragma unroll (NM > 0 ? NM : 1)
       for (int i = m0; i < m1; ++i) {
         const bool next_l1 = i + 1 < m1 || has_next;
-        // (the descriptors are made ahead of the hand-offs, off the chain; not in HF, whose
-        // many MMAs a hand-off hide that: 13^7 14.0 ms, ahead 14.5)
+        // (the descriptors are made ahead of the hand-offs, off the chain)
         const int i1 = i + 1 < m1 ? i + 1 : m0;
-        const uint64_t d1 = HF ? 0 : desc1(i1), d2 = HF ? 0 : desc2(i), d3 = HF ? 0 : desc3(i);
+        const uint64_t d1 = desc1(i1), d2 = desc2(i), d3 = desc3(i);
         if (T.h2 > 0) {
           take();  // H1 of model i stored
-          issue_mma2(HF ? desc2(i) : d2);
+          issue_mma2(d2);
           mma_commit_warp(barA);
         }
         if (next_l1) {
           take();  // accumulators read, the next A1 row written
-          issue_mma1(HF ? desc1(i1) : d1);
+          issue_mma1(d1);
           mma_commit_warp(barA);
         }
         take();  // the last hidden layer of model i stored
-        issue_mma3(HF ? desc3(i) : d3, i > m0 ? 1u : 0u);
+        issue_mma3(d3, i > m0 ? 1u : 0u);
         mma_commit_warp(barB);
       }
     }
@@ -1254,10 +1146,6 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
           hidden_epilogue_tf<(S2 - 1) * 8>(tD + lane_off, tH1 + lane_off, tHlo + lane_off, []() {}, [&]() {
             if (l3) await_b();  // the previous model's layer 3 has read H
           });
-        } else if constexpr (HF) {
-          hidden_epilogue_half<(S2 - 1) * 16>(tD + lane_off, tH1 + lane_off, tHlo + lane_off, []() {}, [&]() {
-            if (l3) await_b();  // the previous model's layer 3 has read H
-          });
         } else {
           hidden_epilogue<(S2 > 0 ? (S2 - 1) * 16 / EW : 0)>(T.h1, tD + kColsD * half + lane_off,
                                                              tH1 + kColsD / 2 * half + lane_off, []() {}, [&]() {
@@ -1276,13 +1164,6 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
         await_a();
         if constexpr (TF) {
           hidden_epilogue_tf<S3 * 8>(
-              tD + lane_off, tH2 + lane_off, tHlo + lane_off,
-              [&]() {
-                if (next_l1) signal();  // accumulators read, next A1 written: the next layer 1
-              },
-              []() {});
-        } else if constexpr (HF) {
-          hidden_epilogue_half<S3 * 16>(
               tD + lane_off, tH2 + lane_off, tHlo + lane_off,
               [&]() {
                 if (next_l1) signal();  // accumulators read, next A1 written: the next layer 1
@@ -1351,8 +1232,8 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
 using TcFn = void (*)(const Params, const TcArgs, const RangeArgs, const TcList);
 
 // Instantiations in translation units of their own (they compile side by side): the exact
-// variants, and the bf16 kernel of the d_L 8, 64-64 shape for 3 to 7 models.
-TcFn tc_kernel_exact(int xm, int mode, bool mp, bool util);
+// variant, and the bf16 kernel of the d_L 8, 64-64 shape for 3 to 7 models.
+TcFn tc_kernel_exact(int mode, bool mp, bool util);
 TcFn tc_kernel_nm_range(int n_models, bool shared_bar);
 TcFn tc_kernel_nm_list(int n_models);
 

@@ -54,13 +54,11 @@ struct TcArgs {
   uint32_t off_b1[MF_MAX_MODELS], off_b2[MF_MAX_MODELS], off_b3[MF_MAX_MODELS];  // bytes in img
   // TMEM columns; from pipeline to pipeline D moves by ps_d, D3 by ps_d3, the rest by pipe_stride
   int32_t pipes, col_d, col_h, col_ones, col_a, col_d3, pipe_stride, ps_d, ps_d3;
-  // the exact fp32 variants (tf: 1 tf32 parts, 2 fp16 parts; 0 bf16): operands as hi and lo
-  // parts; col_hlo holds the hidden layer's lo parts, img_lo1..3 are the byte offsets of
-  // each B image's lo part after its hi part
+  // the exact fp32 variant (tf: 1; 0 bf16): operands as tf32 hi and lo parts; col_hlo holds
+  // the hidden layer's lo parts, img_lo1..3 are the byte offsets of each B image's lo part
+  // after its hi part
   int32_t tf, col_hlo;
   uint32_t img_lo1, img_lo2, img_lo3;
-  // fp16 parts: the aggregate's scales, and the factors that scale the outputs back
-  float cagg[3], back[MF_MAX_MODELS][2];
   uint32_t sm_xw, sm_dem, sm_rows, sm_topk, sm_bar, sm_total;  // shared-memory byte offsets
   uint32_t img_model;                 // bytes of one model's B1 + B2 + B3 images
   int32_t ew;                         // epilogue warps per tensor-memory lane quarter (1 or 2)

@@ -1,7 +1,6 @@
-"""The fp16 split of the exact tensor-core variant where its scaling is put to the test:
-features, weights and demands far from order one, zero columns and units, an outlier option
-(which the range rule hands to the tf32 split), every model count (one and two weight
-passes), lists too long for a full pass's weights.  1e-5 of the oracle everywhere."""
+"""The exact tensor-core variant where its operands' ranges are put to the test: features,
+weights and demands far from order one, zero columns and units, an outlier option, every
+model count (one to three weight passes), the longest lists.  1e-5 of the oracle everywhere."""
 import numpy as np
 import pytest
 
@@ -90,8 +89,8 @@ def test_model_counts_and_long_lists(mf, n, k):
         fin = np.isfinite(b["topk_score"])
         assert np.array_equal(np.isfinite(a["topk_score"]), fin)
         assert np.allclose(a["topk_score"][fin], b["topk_score"][fin], rtol=0, atol=1e-5 * max(1.0, np.abs(b["topk_score"][fin]).max(initial=0.0)))
-        # a list scores the same numbers, but for the order of the N terms' sum: long lists run
-        # in more weight passes, whose partial sums round apart (at most N ulps of N terms of
-        # order one: 8 * 8 * 2^-24)
+        # a list scores the same numbers, but for the order of the N terms' sum: models run in
+        # weight passes, whose partial sums round apart (at most N ulps of N terms of order
+        # one: 8 * 8 * 2^-24)
         sa, _ = ctx.score_batch(torch.from_numpy(a["topk_idx"][fin].astype(np.int64)).cuda())
         assert np.abs(sa.cpu().numpy() - a["topk_score"][fin]).max(initial=0.0) <= 64 * 2.0 ** -24

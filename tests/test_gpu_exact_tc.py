@@ -138,3 +138,56 @@ def test_exact_search_with_the_longest_lists(mf, oracle_mod):
     gaps = np.abs(np.diff(s_o))
     sep = (np.r_[gaps, np.inf] > 4 * RTOL["fp32"] * scale) & (np.r_[np.inf, gaps] > 4 * RTOL["fp32"] * scale)
     assert np.array_equal(np.asarray(a["topk_idx"])[fin][sep], np.asarray(b["topk_idx"])[fin][sep])
+
+
+def _dead_problem(what, scale):
+    """Four models with the first two layers `scale` times as drawn (b2 = 0) and, by `what`,
+    dead units (row and bias) in the first or the second hidden layer, or an all-zero feature
+    column or demand component under weights of order one."""
+    prob = W.make_problem([9, 8, 7, 6], 8, 64, 64, 31, 45.0, objective="soft_lat", soft_penalty=0.1)
+    per = W.param_count(8, 64, 64)
+    off = np.concatenate([[0], np.cumsum(prob["n_options"])])
+    if what == "zero_demand":
+        prob["demand"][:, 0] = 0.0
+    for i in range(4):
+        w = prob["weights"][i * per:(i + 1) * per]
+        w1, b1 = w[:768].reshape(64, 12), w[768:832]
+        w2, b2 = w[832:4928].reshape(64, 64), w[4928:4992]
+        live = w1[:, {"zero_feature": 1, "zero_demand": 8}.get(what, 0)].copy()
+        w1 *= np.float32(scale)
+        b1 *= np.float32(scale)
+        w2 *= np.float32(scale if what == "second" else 1.0)
+        b2[:] = 0.0
+        if what == "first":
+            w1[5:9] = 0.0
+            b1[5:9] = 0.0
+        elif what == "second":
+            w2[5:9] = 0.0
+        elif what == "zero_feature":
+            prob["local_feats"][off[i]:off[i + 1], 1] = 0.0
+            w1[:, 1] = live
+        elif what == "zero_demand":
+            w1[:, 8] = live
+    return prob
+
+
+@pytest.mark.parametrize("scale", [1.0, 0.3, 0.03, 0.003])
+@pytest.mark.parametrize("what", ["first", "second", "zero_feature", "zero_demand"])
+def test_dead_units_and_zero_columns(mf, oracle_mod, what, scale):
+    """Inputs that are zero for every candidate, whatever the scale of what is beside them:
+    scores, feasibility and count as the oracle's and the CUDA cores'."""
+    prob = _dead_problem(what, scale)
+    o = oracle_mod.Oracle(prob)
+    idx = np.arange(o.space_size(), dtype=np.uint64)
+    rs, rf, rp, ra = o.score_list(idx, with_pred=True)
+    with mf.Context(prob) as ctx:
+        assert ctx.stats()["scoring_path"] == PATH_EXACT
+        s, f, p = _score_all(ctx, idx)
+        a = ctx.search(64)
+    with mf.Context(prob, precision="fp32_simt") as ctx:
+        b = ctx.search(64)
+    check_scores(prob, s, f, rs, rf, rp, ra, got_pred=p)
+    assert a["count"] == b["count"] == int(rf.sum())
+    # (predictions that barely vary make near ties: the lists are compared by score)
+    scale64 = np.maximum(score_scale(prob, rs, rp)[b["topk_idx"].astype(np.int64)], 1e-30)
+    assert np.all(np.abs(a["topk_score"].astype(np.float64) - b["topk_score"]) <= 2 * RTOL["fp32"] * scale64)
