@@ -9,6 +9,7 @@
 // a table-lookup scan (k_fc_scan, ALU-bound); k_vram_count / k_vram_write build the
 // VRAM-feasible space (Lambda without its VRAM-infeasible configurations) as an
 // ascending index list.
+#include <cfloat>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -338,11 +339,13 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
       const int i = task == 0 ? last : task == 1 ? max(last - 1, 0) : task - 2 - g * N;
       const float lam = g == 0 ? 0.f : g == 1 ? 0.3f * lam1 : g == 2 ? lam1 : 3.f * lam1;
       const int off = pick(P.off, i), K = pick(P.K, i);
-      // the value a task ranks by, highest first: -V, or J - lambda V (unusable options last)
+      // the value a task ranks by, highest first: -V, or J - lambda V (unusable options last,
+      // also where lambda V overflows: a model's usable options take its first ranks, so every
+      // slot of `order` that the corner reads is written)
       auto value = [&](int o) {
         const float2 e = o < K ? tab[off + o] : make_float2(-INFINITY, INFINITY);
         if (task < 2) return -e.y;
-        return e.y < INFINITY ? __fsub_rn(e.x, __fmul_rn(lam, e.y)) : -INFINITY;
+        return e.y < INFINITY ? fmaxf(__fsub_rn(e.x, __fmul_rn(lam, e.y)), -FLT_MAX) : -INFINITY;
       };
       for (int c0 = 0; c0 < K; c0 += 32) {
         const int o = c0 + lane;

@@ -101,3 +101,24 @@ def test_special_values(mf, special):
         assert r["count"] == count
         if special != "inf_quality":
             assert np.array_equal(r["topk_idx"][:ti.size], ti) and np.array_equal(r["topk_score"][:ts.size], ts)
+
+
+@pytest.mark.parametrize("k", [5, 100])
+def test_corner_values_that_overflow(mf, k):
+    """Demands next to each other near fp32's end and utilities of order 1e34: the corner's
+    J - lambda V overflows for options that meet their floors, between others that do not."""
+    options = [12, 13]
+    prob = W.make_problem(options, 8, 32, 0, 91, 3e38)
+    prob["demand"][:, 1] = np.float32(1e38) * (1 + np.arange(25, dtype=np.float32) % 11 * np.float32(2.0 ** -23))
+    fc = W.fc_scenario(prob, 91)
+    fc["omega"] = np.full(2, 1e34, np.float32)
+    fc["tau"] = np.full(2, -5.0, np.float32)
+    with mf.Context(prob) as ctx:
+        ctx.fc_set(fc)
+        f = ctx.fc_table()[1]
+        fc["tau"] = np.array([np.sort(f[:12])[5], np.sort(f[12:])[6]], np.float32)
+        ctx.fc_set(fc)
+        count, ti, ts = brute(prob, ctx, k, 0, ctx.space_size)
+        r = ctx.fc_search(k)
+        assert count == 7 * 7 and r["count"] == count
+        assert np.array_equal(r["topk_idx"][:ti.size], ti) and np.array_equal(r["topk_score"][:ts.size], ts)
