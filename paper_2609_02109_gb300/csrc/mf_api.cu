@@ -456,7 +456,7 @@ static mf_status search_impl(mf_ctx* ctx, uint64_t lo, uint64_t hi, int32_t k, u
     launches += nl;
     score_launches += nl;
   }
-  for (uint64_t b = lo; b < hi; b += chunk) {
+  for (uint64_t b = lo; b < hi; b += a.len) {  // (a whole chunk may reach past 2^64)
     a.base = b;
     a.len = (hi - b) < chunk ? (hi - b) : chunk;
     int nl = 1;

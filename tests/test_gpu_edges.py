@@ -113,3 +113,34 @@ def test_range_at_the_top_of_a_space_beyond_2_32(mf, oracle_mod, prec):
         res = ctx.search(k, lo=lo, hi=hi)
     check_search(o, prob, res, k, (ti, ts), cnt, near_count_bound=bound, prec=prec)
     assert 0 < cnt < hi - lo
+
+
+# 2^64 - 2^28 configurations: a default launch that starts near the end would reach past 2^64
+NEAR_2_64 = [112, 192, 146, 156, 109, 95, 128, 148, 192]
+
+
+def test_last_indices_of_a_space_near_2_64(mf, oracle_mod):
+    """The last 3001 indices: scores, count and top-k as the oracle's, and the fixed-context
+    scan's and the VRAM list's as numpy's float32 sums."""
+    from test_gpu_fc_scan import brute
+    prob = W.make_problem(NEAR_2_64, 8, 32, 0, 23, 95.0)
+    o = oracle_mod.Oracle(prob)
+    n = o.space_size()
+    assert n == 2 ** 64 - 2 ** 28
+    lo, k = n - 3001, 16
+    ti, ts, cnt = o.exhaustive(k, lo=lo, hi=n)
+    _, _, pr, ag = o.score_list(np.arange(lo, n, dtype=np.uint64), with_pred=True)
+    fc = W.fc_scenario(prob, 23)
+    fc["tau"] = np.full(9, -5.0, np.float32)
+    with mf.Context(prob) as ctx:
+        res = ctx.search(k, lo=lo, hi=n)
+        ctx.fc_set(fc)
+        fres = ctx.fc_search(k, lo=lo, hi=n)
+        fcount, fi, fs = brute(prob, ctx, k, lo, n)
+        vcount, vidx = ctx.vram_feasible(lo=lo, hi=n, cap=4000)
+    check_search(o, prob, res, k, (ti, ts), cnt, near_count_bound=int(near_threshold(prob, pr, ag, "fp32").sum()))
+    assert fres["count"] == fcount and 0 < fcount < 3001
+    assert np.array_equal(fres["topk_idx"], fi) and np.array_equal(fres["topk_score"], fs)
+    got = vidx.cpu().numpy().view(np.uint64)[:vcount]
+    assert vcount == fcount and np.all(np.diff(got.astype(object)) > 0)  # (no floor binds: the same set)
+    assert np.isin(fi, got).all()
