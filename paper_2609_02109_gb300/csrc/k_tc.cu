@@ -198,9 +198,9 @@ static void set_passes(const Params& P, TcArgs& T, size_t budget) {
   }
 }
 
-// The shared-memory layout for lists of kcap entries: where two epilogue warps share a lane
-// quarter (their rows take more), with fewer models per pass if the lists would not fit next
-// to a full pass's weights.
+// The shared-memory layout for lists of kcap entries: in the shape with two epilogue warps per
+// lane quarter (48 KB of weights a model), with fewer models per pass if the lists would not
+// fit next to a full pass's weights.
 static bool layout_for(const Params& P, TcArgs& T, int kcap) {
   layout_smem(P, T, kcap);
   if (T.sm_total > kSmemLimit && T.ew == 2) {

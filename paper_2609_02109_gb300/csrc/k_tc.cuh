@@ -229,10 +229,14 @@ __host__ __device__ constexpr int tc_pipes(int xm) { return xm == kXmTf32 ? 2 : 
 __host__ __device__ constexpr int tc_pipe_threads(int ew) { return 32 * (4 * ew + 1); }
 constexpr uint32_t kWaitLimit = 4096;  // suspended retries (~1 ms each at most)
 
-// Shared memory of a pipeline's rows: byte digits of two tiles, or of three and VRAM demands.
+// Shared memory of a pipeline's rows: byte digits of two tiles; or, where two epilogue warps
+// share a lane quarter (up to 8 models), of three tiles and the VRAM demands of two.  Either
+// way 4 KB, so that both take the same tables, weights and lists.
+__host__ __device__ constexpr int tc_digit_bytes(int ew) { return (ew == 2 ? 8 : MF_MAX_MODELS) * 128; }
 __host__ __device__ constexpr int tc_row_bytes(int ew) {
-  return ew == 2 ? 3 * (MF_MAX_MODELS * 128 + 128 * 4) : 2 * MF_MAX_MODELS * 128;
+  return ew == 2 ? 3 * tc_digit_bytes(2) + 2 * 128 * 4 : 2 * tc_digit_bytes(1);
 }
+static_assert(tc_row_bytes(1) == tc_row_bytes(2), "one layout for both");
 
 struct TcList {
   const uint64_t* idx;
@@ -546,9 +550,9 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
   const uint4* xw_s = reinterpret_cast<const uint4*>(smem + T.sm_xw);
   float4* dem_s = reinterpret_cast<float4*>(smem + T.sm_dem);
   // this row's digits (option index within the model) of every model, kBufs tiles:
-  // digits[b * MF_MAX_MODELS * 128 + i * 128 + row]; EW 2: then its VRAM demand, as many tiles
+  // digits[b * tc_digit_bytes(EW) + i * 128 + row]; EW 2: then its VRAM demand, two tiles
   uint8_t* digits = reinterpret_cast<uint8_t*>(smem + T.sm_rows) + (size_t)pipe * tc_row_bytes(EW);
-  float* vrams = reinterpret_cast<float*>(digits + kBufs * MF_MAX_MODELS * 128);
+  float* vrams = reinterpret_cast<float*>(digits + kBufs * tc_digit_bytes(EW));
 
   if (tid == 0) {
     s_abort = 0;
@@ -1060,8 +1064,8 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
     // ---- the epilogue warps ----
     if (out_side) reload_bar();
     uint64_t tile = gpipe;
-    int buf = 0;
-    auto buffer = [&](int b) { return digits + b * (MF_MAX_MODELS * 128); };
+    int buf = 0, odd = 0;  // this tile's digits; its VRAM demands (EW 2)
+    auto buffer = [&](int b) { return digits + b * tc_digit_bytes(EW); };
     float vram_cur = 0.f, vram_prev = 0.f, vram_nx = 0.f;  // VRAM demand of this thread's rows
     DS dcur{}, dprev{}, dnx{};
     // list mode: the row's index in the previous, this and the next two tiles
@@ -1103,7 +1107,6 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
           if (in_side) {
             if (i + 1 < m1) next_a1(i + 1, dcur);
             stage(i);
-            if (i == st_agg && has_next) vrams[b_nx * 128 + row] = vram_nx;
             if (i + 1 >= m1 && has_next) write_a1(m0, dnx, true, aw_nx);
           } else {
             uint32_t oa, ob;
@@ -1113,7 +1116,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
             } else if (pending) {
               load_model(m1 - 1, oa, ob);
               add_model(m1 - 1, oa, ob, dprev, tile - gstride, x_prev);
-              finish_tile(tile - gstride, vrams[(buf == 0 ? kBufs - 1 : buf - 1) * 128 + row], x_prev);
+              finish_tile(tile - gstride, vrams[(odd ^ 1) * 128 + row], x_prev);
             }
             if (i == st_dig) x_nx2 = list_index(tile + 2 * gstride);
           }
@@ -1188,6 +1191,12 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
       x_nx = x_nx2;
       vram_prev = vram_cur;
       vram_cur = vram_nx;
+      if constexpr (EW == 2) {
+        // (the previous tile's were read before this tile's last hand-off; the next tile's are
+        // read after one of that tile's)
+        odd ^= 1;
+        if (in_side) vrams[odd * 128 + row] = vram_cur;
+      }
       buf = b_nx;
     }
     if (pending && out_side) {  // the last tile's last layer 3
@@ -1195,7 +1204,7 @@ k_score_tc(const Params P, const TcArgs T, const RangeArgs R, const TcList L) {
       uint32_t oa, ob;
       load_model(m1 - 1, oa, ob);
       add_model(m1 - 1, oa, ob, dprev, tile - gstride, x_prev);
-      finish_tile(tile - gstride, EW == 2 ? vrams[(buf == 0 ? kBufs - 1 : buf - 1) * 128 + row] : vram_prev, x_prev);
+      finish_tile(tile - gstride, EW == 2 ? vrams[(odd ^ 1) * 128 + row] : vram_prev, x_prev);
     }
   }
   if (MODE == kTcRange && (!MP || T.pass_last) && out_side) {  // what is still queued joins the list

@@ -129,3 +129,29 @@ def test_tc_and_fp32_paths_agree_on_large_range(mf):
     assert a["count"] == b["count"] == hi - lo
     np.testing.assert_array_equal(a["topk_idx"], b["topk_idx"])
     np.testing.assert_allclose(a["topk_score"], b["topk_score"], rtol=1e-5, atol=1e-6)
+
+
+@pytest.mark.parametrize("options,k", [([118] * 8, 8), ([20, 20], 308), ([40], 420)])
+def test_wide_shape_fills_shared_memory(mf, oracle_mod, options, k):
+    """20 -> 128 -> 128 -> 2 with the largest tables that fit beside three models' weights
+    (944 option rows), and with the longest lists that fit beside two models' and one's."""
+    prob = W.make_problem(options, 16, 128, 128, 41, 180.0, objective="soft_lat", soft_penalty=0.1, precision="bf16",
+                          sla_range=W.TIGHT_SLA)
+    o = oracle_mod.Oracle(prob)
+    n = o.space_size()
+    lo = n // 3 if n > 40000 else 0
+    hi = min(n, lo + 20001)
+    idx = np.arange(lo, hi, dtype=np.uint64)
+    r = o.score_list(idx, with_pred=True)
+    ti, ts, cnt = o.exhaustive(k, lo=lo, hi=hi)
+    with mf.Context(prob) as ctx:
+        s, f, p = _score(ctx, idx)
+        res = ctx.search(k, lo=lo, hi=hi)
+    # each head within 2e-2 of its condition scale c (which its terms can cancel below); J sums
+    # w_i thr_i - 0.1 max(0, lat_i - SLA_i), so its error is at most 2e-2 (w_i c_thr + 0.1 c_lat)
+    # summed over the models: one or two models' J can be small beside that
+    err = 2e-2 * np.maximum(np.abs(r[2]), o.pred_scale(idx))
+    assert np.all(np.abs(p - r[2]) <= err)
+    assert np.array_equal(f.astype(bool), r[1])  # (the VRAM cap does not bind)
+    assert np.all(np.abs(s - r[0])[r[1]] <= (err[..., 0] @ np.asarray(prob["obj_w"], np.float64) + 0.1 * err[..., 1].sum(axis=1))[r[1]])
+    check_search(o, prob, res, k, (ti, ts), cnt, prec="bf16")
