@@ -211,6 +211,7 @@ constexpr int kFcEndQ = kFcWarps * kFcWarpK;          // the warps' lists, merge
 constexpr int kFcLambdas = 4, kFcCornerOpts = 64;     // corner sets, options of a model in one
 constexpr int kFcCornerBits = 10;                     // configurations of a corner: 2^10
 constexpr int kFcCornerRows = 1024;                   // option rows up to which the corners are ranked
+constexpr size_t kFcScanSmem = 226 * 1024;            // dynamic shared memory a launch may take
 
 struct FcScan {
   const float2* tab;
@@ -889,6 +890,11 @@ struct FcGaArgs {
   float* out_fit;
 };
 
+// Shared memory of k_fc_ga: the table, then two generations' fitness and genes.
+constexpr size_t fc_ga_bytes(int sumK, int pop, int n) {
+  return sizeof(float2) * (size_t)sumK + 2 * (size_t)pop * (sizeof(float) + (size_t)n);
+}
+
 // (fitness, slot) as one word that orders by fitness, then by lower slot.
 __device__ __forceinline__ unsigned long long fc_rank(float f, int slot) {
   return ((unsigned long long)order_key(f) << 32) | (0xFFFFFFFFu - (uint32_t)slot);
@@ -1137,7 +1143,7 @@ mf_status fc_search_chunk(mf_ctx* c, const RangeArgs& a, int grid, cudaStream_t 
   }
   const bool wl = a.k <= kFcWarpK;  // per-warp lists
   const size_t smem = fc_scan_table_bytes(c->sumK) + fc_scan_list_bytes(a.k, wl);
-  if (smem > 226 * 1024) {
+  if (smem > kFcScanSmem) {
     set_error("fixed-context search: top-k lists do not fit shared memory; use a smaller k");
     return MF_EUNSUPPORTED;
   }
@@ -1150,7 +1156,8 @@ mf_status fc_search_chunk(mf_ctx* c, const RangeArgs& a, int grid, cudaStream_t 
   else
     fn = wl ? (n8 ? k_fc_scan<8, true, false> : k_fc_scan<MF_MAX_MODELS, true, false>)
             : (n8 ? k_fc_scan<8, false, false> : k_fc_scan<MF_MAX_MODELS, false, false>);
-  MF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // (the maximum, whatever this launch takes: another context's call may be in between)
+  MF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFcScanSmem));
   fn<<<grid, kFcThreads, smem, s>>>(P, S, a);
   MF_CUDA(cudaGetLastError());
   return MF_OK;
@@ -1310,13 +1317,15 @@ mf_status mf_fc_ga_run(mf_ctx* ctx, const mf_fc_ga_params* g, uint64_t seed, int
   A.seed = seed;
   A.out_genome = h;
   A.out_fit = (float*)(h + 16);
-  const size_t smem = sizeof(float2) * ctx->sumK + sizeof(float) * 2 * g->pop + (size_t)2 * g->pop * N;
+  const size_t smem = fc_ga_bytes(ctx->sumK, g->pop, N);
   const bool n8 = N <= 8;
   const auto fn = g->pop <= 128   ? (n8 ? k_fc_ga<1, 8> : k_fc_ga<2, 8>)
                   : g->pop <= 256 ? (n8 ? k_fc_ga<2, 4> : k_fc_ga<4, 4>)
                   : g->pop <= 512 ? (n8 ? k_fc_ga<4, 2> : k_fc_ga<8, 2>)
                                   : (n8 ? k_fc_ga<8, 1> : k_fc_ga<16, 1>);
-  MF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // (the maximum, whatever this launch takes: another context's call may be in between)
+  constexpr size_t kMost = fc_ga_bytes(MF_MAX_MODELS * MF_MAX_OPTIONS, 1024, MF_MAX_MODELS);
+  MF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMost));
   fn<<<1, 1024, smem, s>>>(ctx->P, A);
   MF_CUDA(cudaGetLastError());
   MF_CUDA(cudaStreamSynchronize(s));

@@ -322,10 +322,13 @@ mf_status merge_lists(const float* ls, const uint64_t* li, int nlists, int k, fl
                       const ResultOut& out, cudaStream_t s) {
   // tmp holds two buffers of ceil(nlists / 2) * k entries each
   const size_t half = (size_t)((nlists + 1) / 2) * k;
-  // room for 4096 survivors in short lists (k <= 256), else 16384
-  const int cap = k <= 256 ? 4096 : 16384;
+  // room for 4096 survivors in short lists (k <= 256), else 16384.  (The attribute belongs to
+  // the function, not to the launch: always the maximum, or a call of another context in
+  // another thread could lower it in between.)
+  constexpr int kCapMax = 16384;
+  const int cap = k <= 256 ? 4096 : kCapMax;
   const size_t smem = (size_t)cap * kPair;
-  MF_CUDA(cudaFuncSetAttribute(k_merge_lists, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  MF_CUDA(cudaFuncSetAttribute(k_merge_lists, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kCapMax * kPair)));
   k_merge_lists<<<1, kMergeThreads, smem, s>>>(ls, li, nlists, k, cap, tmp_s, tmp_i, tmp_s + half, tmp_i + half,
                                                out);
   MF_CUDA(cudaGetLastError());
@@ -334,15 +337,16 @@ mf_status merge_lists(const float* ls, const uint64_t* li, int nlists, int k, fl
 
 mf_status finish_shortlist(const Params& P, const uint64_t* idx, const float* pred, int n, int k,
                            const ResultOut& out, cudaStream_t s) {
+  constexpr int kMost = 8192;
   int n2 = 32;
   while (n2 < n) n2 <<= 1;
-  if (n2 > 8192) {
+  if (n2 > kMost) {
     set_error("finish_shortlist: more than 8192 entries");
     return MF_EINVAL;
   }
   const size_t smem = (size_t)n2 * kPair;
   const auto fn = P.n_models <= 8 ? k_finish<8> : k_finish<MF_MAX_MODELS>;
-  MF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  MF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMost * kPair)));  // (the maximum: see merge_lists)
   fn<<<1, 512, smem, s>>>(P, idx, pred, n, n2, k, out);
   MF_CUDA(cudaGetLastError());
   return MF_OK;
