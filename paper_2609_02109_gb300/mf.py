@@ -227,6 +227,8 @@ class Context:
     # -- calls ----------------------------------------------------------------------
     @property
     def space_size(self) -> int:
+        if not self._h:  # (closed)
+            raise MFError(MF_EINVAL, "mf_space_size", "NULL argument")
         return self._space
 
     def set_objective(self, sla=None, obj_w=None):
