@@ -121,9 +121,15 @@ def _check(status: int, where: str):
         raise MFError(status, where, _lib.mf_last_error().decode())
 
 
+# The stream's address without the Stream object that torch.cuda.current_stream builds for it; a
+# torch without this function is asked for the object.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(device) -> int:
     """torch's current stream on a device (an ordinal, or a tensor's device), as an address."""
-    return torch._C._cuda_getCurrentRawStream(device if isinstance(device, int) else device.index)
+    i = device if isinstance(device, int) else device.index
+    return torch.cuda.current_stream(i).cuda_stream if _raw_stream is None else _raw_stream(i)
 
 
 def _ptr(a) -> int:
