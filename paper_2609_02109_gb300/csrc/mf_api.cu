@@ -377,21 +377,29 @@ mf_status mf_fc_search(mf_ctx* ctx, uint64_t lo, uint64_t hi, int32_t k, uint64_
   return search_impl(ctx, lo, hi, k, chunk, out, stream, true);
 }
 
+// Candidates of a launch by default.  Each launch fills its lists and stages its tables anew (12
+// launches of 2^24 for 24^6 took the bf16 search 12.92 ms, one 12.64), but nothing else on the GPU
+// can come between: about 0.3 s of predictor work at most (at 150 TFLOP/s, what the tf32 split
+// reaches, or the CUDA cores' 30), from 2^24 candidates, as it was, to 2^31.  The table-lookup
+// scan takes 2^36, 12 ms at 24^6's rate.
+static uint64_t default_launch(const Params& P, bool tensor) {
+  const double flops = 2.0 * P.n_models * ((double)P.d_in * P.h1 + (double)P.h1 * P.h2 + 2.0 * (P.h2 > 0 ? P.h2 : P.h1));
+  const double most = (tensor ? 4.5e13 : 9e12) / flops;
+  return most >= 2147483648.0 ? 1ull << 31 : most <= 16777216.0 ? 1ull << 24 : (uint64_t)most;
+}
+
 static mf_status search_impl(mf_ctx* ctx, uint64_t lo, uint64_t hi, int32_t k, uint64_t chunk,
                              mf_result* out, void* stream, bool fc) {
   if (!ctx || !out) return einval("NULL argument");
   if (k < 1 || k > MF_MAX_TOPK) return einval("k must be in 1..1024");
   if (lo > hi || hi > ctx->P.total) return einval("need lo <= hi <= |Lambda|");
-  // by default one launch takes the range (each launch fills its lists and stages its tables
-  // anew: 12 launches for 24^6 took the bf16 search 12.92 ms, one 12.64): up to 2^31 candidates, and
-  // 2^36 of the table-lookup scan's, which are cheaper by as much
-  if (chunk == 0) chunk = fc ? 1ull << 36 : 1ull << 31;
-  else if (chunk > (1ull << 31)) chunk = 1ull << 31;
   DeviceGuard guard(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
   const bool tc = !fc && ctx->precision == MF_BF16;
   // the exact (3-term tf32) tensor-core variant, where its lists fit next to the weights
   const bool tx = !fc && !tc && ctx->tc.tf && tc_fits(ctx, k);
+  if (chunk == 0) chunk = fc ? 1ull << 36 : default_launch(ctx->P, tc || tx);
+  else if (chunk > (1ull << 31)) chunk = 1ull << 31;
   const int kcap = tc ? (k * 8 > 256 ? k * 8 : 256) : k;
   const uint64_t launch_len = hi - lo < chunk ? hi - lo : chunk;
   const int grid = fc ? fc_grid(ctx, launch_len) : (tc || tx) ? tc_grid(ctx) : f32_grid(ctx, launch_len);

@@ -243,3 +243,16 @@ def test_index_range_shards_merge_to_the_full_search(mf, world):
     assert m["count"] == full["count"] and m["best_idx"] == full["best_idx"]
     assert np.array_equal(m["topk_idx"], full["topk_idx"])
     assert np.array_equal(m["topk_score"], full["topk_score"])
+
+
+@pytest.mark.parametrize("precision,h,launches", [("fp32_simt", 256, 2), ("fp32_simt", 32, 1), ("bf16", 64, 1)])
+def test_default_launches_are_bounded(mf, precision, h, launches):
+    """65^4 candidates (more than 2^24): predictors of 256-256 units, 10 TFLOP in all, take two
+    launches on the CUDA cores, with the result of smaller ones; lighter ones take one."""
+    prob = W.make_problem([65] * 4, 8, h, 0 if h == 32 else h, 3, 45.0, precision=precision)
+    with mf.Context(prob) as ctx:
+        a = ctx.search(16)
+        assert ctx.stats()["score_launches_last"] == launches
+        b = ctx.search(16, chunk=10_000_019)
+    assert a["count"] == b["count"] and np.array_equal(a["topk_idx"], b["topk_idx"])
+    assert np.array_equal(a["topk_score"], b["topk_score"])
