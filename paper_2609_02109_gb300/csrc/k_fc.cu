@@ -872,14 +872,14 @@ k_vram_write(const Params P, const VramArgs A) {
 // and repair of an infeasible individual by rejection sampling from the uniform
 // distribution over Lambda (draws kGaRepair, j = a * N + i, at most 256 / N attempts, the
 // first feasible one kept).  The block has 1024 threads whatever the population: LPC lanes
-// breed an individual (tournament entries and genes shared out over them), and a warp's lanes
-// share the repairs of its individuals.  LPC is the most that holds the population in one
-// round (8 up to 128 individuals, 4 up to 256, 2 up to 512, else 1): the lanes cut a generation's chain,
-// but rounds of them one after another cost more than a thread per individual (population
-// 908, 11 generations, with its table: 137 us with one thread each, 224 with eight).  Bound by the latency of a generation's chain: draws, fitness
-// reads, the two tournaments, genes, their terms in model order, one block barrier.
-// Population 100, 30 generations, N = 5, some repairs: 93 us; one thread per individual, its draws
-// one after another, took 180 us.
+// breed an individual (tournament entries and genes shared out over them), and lanes share
+// the repairs (see repair).  LPC is the most that holds the population in one round (8 up to
+// 128 individuals, 4 up to 256, 2 up to 512, else 1): the lanes cut a generation's chain, but
+// rounds of them one after another cost more than a thread per individual (population 908, 11
+// generations, with its table: 137 us with one thread each, 224 with eight).  Bound by the
+// latency of a generation's chain: draws, fitness reads, the two tournaments, genes, their
+// terms in model order, one block barrier.  Population 100, 30 generations, N = 5: 66 us without
+// repairs, up to 93 with; one thread per individual, its draws one after another, took 180 us.
 // ---------------------------------------------------------------------------
 struct FcGaArgs {
   const float2* tab;
@@ -947,7 +947,6 @@ k_fc_ga(const Params P, const FcGaArgs A) {
   const int attempts = 256 / N;
   const int lane = c & 31;
   // LPC lanes per individual: lane gl of a group holds genes gl, gl + LPC, ..
-  constexpr int kGroups = 1024 / LPC;
   const int gl = lane % LPC, group = c / LPC, g0l = lane - gl;  // (g0l: the group's first lane)
   int off[NG], K[NG];
 #pragma unroll
@@ -977,35 +976,22 @@ k_fc_ga(const Params P, const FcGaArgs A) {
     if (gl == 0 && child < pop) fit[child] = ok ? J : -INFINITY;
     return ok ? J : -INFINITY;
   };
-  // Repair of the warp's infeasible children (`bad`: this lane's group has one, child `child`):
-  // the warp's lanes are shared out over them (32, 16, 8, .. lanes each), which try the child's
-  // attempts in order, so many at a time; the lowest feasible attempt of the first successful
-  // round is the sequential search's result.  The winning lane writes the child's genes and
-  // fitness over the unrepaired ones.
-  auto repair = [&](uint32_t G, bool bad, int child, uint8_t* genes, float* fit) {
-    const unsigned bal = __ballot_sync(0xffffffffu, bad && gl == 0);
-    if (!bal) return;
-    __syncwarp();
-    const int cnt = __popc(bal);
-    int gs = 32;
-    while (gs * cnt > 32) gs >>= 1;
-    const int mine = lane / gs;  // this lane works for the mine-th of them
-    unsigned rest = bal;
-    for (int j = 0; j < mine; ++j) rest &= rest - 1u;
-    const int who = __shfl_sync(0xffffffffu, child, rest ? __ffs(rest) - 1 : 0);
-    const unsigned gmask = gs == 32 ? 0xffffffffu : ((1u << gs) - 1u) << (mine * gs);
-    bool done = rest == 0u;
+  // Attempts for the infeasible child `who` (done: none) of the lane's set of gs lanes (gmask):
+  // they try the child's attempts in order, so many at a time; the lowest feasible attempt of
+  // the first successful round is the sequential search's result.  The winning lane writes the
+  // child's genes and fitness over the unrepaired ones.
+  auto attempt = [&](uint32_t G, int who, bool done, int gs, unsigned gmask, uint8_t* genes, float* fit) {
     for (int a0 = 0; a0 < attempts && __any_sync(0xffffffffu, !done); a0 += gs) {
       const int a = a0 + lane % gs;
       float Jc = -INFINITY;
-      uint64_t cand[(NG * LPC + 7) / 8] = {};
+      uint32_t cand[(NG * LPC + 3) / 4] = {};
       if (!done && a < attempts) {  // the fitness' sums, with the draws kept in registers
         float Js = 0.f, Vs = 0.f;
 #pragma unroll
         for (int i = 0; i < LPC * NG; ++i)
           if (i < N) {
             const int o = ga_unif(ga_rng(sd, G, (uint32_t)who, kGaRepair, (uint32_t)(a * N + i)), (uint32_t)P.K[i]);
-            cand[i >> 3] |= (uint64_t)o << (8 * (i & 7));
+            cand[i >> 2] |= (uint32_t)o << (8 * (i & 3));
             const float2 e = tab[P.off[i] + o];
             Js += e.x;
             Vs += e.y;
@@ -1015,13 +1001,57 @@ k_fc_ga(const Params P, const FcGaArgs A) {
       const unsigned ok = __ballot_sync(0xffffffffu, Jc != -INFINITY) & gmask;
       if (!done && ok) {
         if (lane == __ffs(ok) - 1) {
-          for (int i = 0; i < N; ++i) genes[(size_t)who * N + i] = (uint8_t)(cand[i >> 3] >> (8 * (i & 7)));
+#pragma unroll
+          for (int i = 0; i < LPC * NG; ++i)  // (unrolled: an index known at run time would put `cand` in memory)
+            if (i < N) genes[(size_t)who * N + i] = (uint8_t)(cand[i >> 2] >> (8 * (i & 3)));
           fit[who] = Jc;
         }
         done = true;
       }
     }
-    __syncwarp();
+  };
+  // Repair of the infeasible children (`bad`: this lane's group has one, child `child`): lanes
+  // are shared out over them, 32, 16, 8, .. each.  With lanes to spare for each individual the
+  // warp's lanes go to its own; with one lane each (half of a warp or more can need repair, and
+  // warps past the population have nothing else to do) the block's lanes go to all of them, at
+  // two barriers (600 individuals, N = 12, most of them infeasible, 30 generations: 530 us, by
+  // the warp 751).
+  auto repair = [&](uint32_t G, bool bad, int child, uint8_t* genes, float* fit) {
+    const unsigned bal = __ballot_sync(0xffffffffu, bad && gl == 0);
+    auto mask = [&](int gs, int mine) { return gs == 32 ? 0xffffffffu : ((1u << gs) - 1u) << (mine * gs); };
+    if constexpr (LPC > 1) {
+      if (!bal) return;
+      __syncwarp();
+      const int cnt = __popc(bal);
+      int gs = 32;
+      while (gs * cnt > 32) gs >>= 1;
+      const int mine = lane / gs;  // this lane works for the mine-th of them
+      unsigned rest = bal;
+      for (int j = 0; j < mine; ++j) rest &= rest - 1u;
+      const int who = __shfl_sync(0xffffffffu, child, rest ? __ffs(rest) - 1 : 0);
+      attempt(G, who, rest == 0u, gs, mask(gs, mine), genes, fit);
+      __syncwarp();
+    } else {
+      __shared__ uint16_t s_who[1024];
+      __shared__ int s_bad[2];  // their number: of generation G in s_bad[G & 1]
+      if (G == 0u) {
+        if (c < 2) s_bad[c] = 0;
+        __syncthreads();
+      }
+      int at = 0;
+      if (lane == 0 && bal) at = atomicAdd(&s_bad[G & 1u], __popc(bal));
+      at = __shfl_sync(0xffffffffu, at, 0) + __popc(bal & ((1u << lane) - 1u));
+      if (bad) s_who[at] = (uint16_t)child;
+      __syncthreads();
+      const int cnt = s_bad[G & 1u];
+      if (c == 0) s_bad[(G + 1u) & 1u] = 0;  // (read before the last generation's end, used after this one's)
+      if (cnt == 0) return;
+      int gs = 32;
+      while (gs * cnt > 1024) gs >>= 1;
+      const int mine = c / gs;
+      attempt(G, mine < cnt ? s_who[mine] : 0, mine >= cnt, gs, mask(gs, lane / gs), genes, fit);
+      __syncthreads();
+    }
   };
   // the fittest of the warp's individuals joins the population's (gl: one lane of a group)
   auto rank_in = [&](int child, const float* fit, unsigned long long* best) {
@@ -1030,14 +1060,20 @@ k_fc_ga(const Params P, const FcGaArgs A) {
     for (int w = LPC; w < 32; w <<= 1) r = max(r, __shfl_xor_sync(0xffffffffu, r, w));
     if (lane == 0 && r) atomicMax(best, r);
   };
-  for (int c0 = 0; c0 < pop; c0 += kGroups) {  // initial population: uniform over Lambda, repaired
-    const int child = c0 + group;
-    int gene[NG];
+  // (LPC is chosen so that every individual has a group; a warp whose individuals all lie past
+  // the population has nothing to draw)
+  const int child = group;
+  const bool breeds = (c - lane) / LPC < pop;
+  {  // initial population: uniform over Lambda, repaired
+    float J = 0.f;
+    if (breeds) {
+      int gene[NG] = {};
 #pragma unroll
-    for (int q = 0; q < NG; ++q)
-      gene[q] = ga_unif(ga_rng(sd, 0, (uint32_t)child, kGaInit, (uint32_t)(gl + LPC * q)), (uint32_t)K[q]);
-    const float J = place(child, gene, g0, fit0);
-    repair(0u, repairable && child < pop && J == -INFINITY, child, g0, fit0);
+      for (int q = 0; q < NG; ++q)
+        if (gl + LPC * q < N) gene[q] = ga_unif(ga_rng(sd, 0, (uint32_t)child, kGaInit, (uint32_t)(gl + LPC * q)), (uint32_t)K[q]);
+      J = place(child, gene, g0, fit0);
+    }
+    if (repairable) repair(0u, child < pop && J == -INFINITY, child, g0, fit0);
     rank_in(child, fit0, &s_best[0]);
   }
   __syncthreads();
@@ -1050,35 +1086,53 @@ k_fc_ga(const Params P, const FcGaArgs A) {
     // (three words in turn: the one for the generation after this is cleared now, which no
     // warp reads or writes before the barrier)
     if (c == 0) s_best[(gen + 2) % 3] = 0ull;
-    for (int c0 = 0; c0 < pop; c0 += kGroups) {
-      const int child = c0 + group;
+    float J = 0.f;
+    const bool elite = A.elitism && child == 0;  // slot 0 keeps the fittest (lowest slot among equals)
+    if (breeds) {
       const uint32_t cu = (uint32_t)child;
       // the draws that do not depend on fitness
-      bool take_b[NG], mutate[NG];
-      int mval[NG];
+      bool take_b[NG] = {}, mutate[NG] = {};
+      int mval[NG] = {};
       const bool cross = (uint32_t)(ga_rng(sd, G, cu, kGaCrossDo, 0u) >> 40) < A.cross_thr;
 #pragma unroll
       for (int q = 0; q < NG; ++q) {
         const uint32_t i = (uint32_t)(gl + LPC * q);
+        if (i >= (uint32_t)N) continue;
         take_b[q] = cross && (ga_rng(sd, G, cu, kGaCross, i) >> 63);
         mutate[q] = (uint32_t)(ga_rng(sd, G, cu, kGaMut, i) >> 40) < A.mut_thr;
         mval[q] = ga_unif(ga_rng(sd, G, cu, kGaMutVal, i), (uint32_t)K[q]);
       }
-      // the two tournaments, entries shared out over the group's lanes
-      unsigned long long win[2] = {0ull, 0ull};
-      for (int d = gl; d < 2 * A.tournament; d += LPC) {
-        const int w = d < A.tournament ? 0 : 1;
-        const int s2 = ga_unif(ga_rng(sd, G, cu, w ? kGaTourB : kGaTourA, (uint32_t)(d - w * A.tournament)), (uint32_t)pop);
-        const unsigned long long r = fc_rank(fc_[s2], s2);
-        if (w) win[1] = max(win[1], r); else win[0] = max(win[0], r);
-      }
+      // the two tournaments
+      int parent[2];
+      if constexpr (LPC == 1) {
+        // (nothing to exchange: a comparison of floats an entry takes a third less to issue than
+        // the ranks; 1024 individuals, 256 entries, 30 generations: 3.14 ms, with ranks 4.70)
+        for (int w = 0; w < 2; ++w) {
+          float best = -INFINITY;
+          int slot = 0x7fffffff;
+          for (int t = 0; t < A.tournament; ++t) {
+            const int s2 = ga_unif(ga_rng(sd, G, cu, w ? kGaTourB : kGaTourA, (uint32_t)t), (uint32_t)pop);
+            const float f = fc_[s2];
+            if (f > best || (f == best && s2 < slot)) { best = f; slot = s2; }
+          }
+          parent[w] = slot;
+        }
+      } else {  // entries shared out over the group's lanes
+        unsigned long long win[2] = {0ull, 0ull};
+        for (int d = gl; d < 2 * A.tournament; d += LPC) {
+          const int w = d < A.tournament ? 0 : 1;
+          const int s2 = ga_unif(ga_rng(sd, G, cu, w ? kGaTourB : kGaTourA, (uint32_t)(d - w * A.tournament)), (uint32_t)pop);
+          const unsigned long long r = fc_rank(fc_[s2], s2);
+          if (w) win[1] = max(win[1], r); else win[0] = max(win[0], r);
+        }
 #pragma unroll
-      for (int w = LPC / 2; w > 0; w >>= 1) {
-        win[0] = max(win[0], __shfl_xor_sync(0xffffffffu, win[0], w));
-        win[1] = max(win[1], __shfl_xor_sync(0xffffffffu, win[1], w));
+        for (int w = LPC / 2; w > 0; w >>= 1) {
+          win[0] = max(win[0], __shfl_xor_sync(0xffffffffu, win[0], w));
+          win[1] = max(win[1], __shfl_xor_sync(0xffffffffu, win[1], w));
+        }
+        parent[0] = fc_slot(win[0]);
+        parent[1] = fc_slot(win[1]);
       }
-      int parent[2] = {fc_slot(win[0]), fc_slot(win[1])};
-      const bool elite = A.elitism && child == 0;  // slot 0 keeps the fittest (lowest slot among equals)
       if (elite) parent[0] = parent[1] = fc_slot(s_best[gen % 3]);
       int gene[NG];
 #pragma unroll
@@ -1087,10 +1141,10 @@ k_fc_ga(const Params P, const FcGaArgs A) {
         gene[q] = i < N ? gc[(size_t)(take_b[q] ? parent[1] : parent[0]) * N + i] : 0;
         if (mutate[q] && !elite && i < N) gene[q] = mval[q];
       }
-      const float J = place(child, gene, gn, fn);
-      repair(G, repairable && child < pop && !elite && J == -INFINITY, child, gn, fn);
-      rank_in(child, fn, &s_best[(gen + 1) % 3]);
+      J = place(child, gene, gn, fn);
     }
+    if (repairable) repair(G, child < pop && !elite && J == -INFINITY, child, gn, fn);
+    rank_in(child, fn, &s_best[(gen + 1) % 3]);
     __syncthreads();
     uint8_t* tg = gc; gc = gn; gn = tg;
     float* tf = fc_; fc_ = fn; fn = tf;

@@ -82,9 +82,9 @@ def _run(prob, ctx, p, seed):
     return f[b], g[b]
 
 
-@pytest.mark.parametrize("pop", [2, 100, 128, 129, 256, 257, 512, 513, 1024])
+@pytest.mark.parametrize("pop", [2, 100, 128, 129, 256, 257, 512, 513, 600, 1024])
 @pytest.mark.parametrize("options,cap", [([12, 9, 9, 9, 9], 55.0), ([12, 9, 9, 9, 9], 25.0), ([7, 10, 7], 30.0),
-                                         ([3] * 16, 160.0), ([30], 8.0)])
+                                         ([3] * 16, 160.0), ([30], 8.0), ([10] * 12, 118.0)])
 def test_every_population(mf, pop, options, cap):
     prob = W.make_problem(options, 8, 64, 64, 5, cap)
     fc = W.fc_scenario(prob, 9)
