@@ -716,30 +716,35 @@ __device__ __forceinline__ unsigned vram_row_count(const float* vl, float V, flo
   return c;
 }
 
-// Counts of the segments: a thread takes one setting of models 0 .. N - 3 at a time (segments
-// are whole such settings) and runs over the options of models N - 2 and N - 1.
-template <int NMAX>
+// Counts of the segments.  PAIR: a thread takes one setting of models 0 .. N - 3 at a time
+// (segments cut them) and runs over the options of models N - 2 and N - 1, whose settings it
+// decodes once; else one setting of models 0 .. N - 2.
+template <int NMAX, bool PAIR>
 __global__ void __launch_bounds__(kVramThreads, 2)
 k_vram_count(const Params P, const VramArgs A) {
   extern __shared__ __align__(16) float vr[];  // [sumK] VRAM of each option
   __shared__ unsigned long long s_sum;
-  const int N = P.n_models, K = pick(P.K, N - 1), KA = N >= 2 ? pick(P.K, N - 2) : 1;
+  const int N = P.n_models, K = pick(P.K, N - 1), KA = PAIR ? pick(P.K, N - 2) : 1;
   const int sumK = pick(P.off, N - 1) + K;
   const int tid = threadIdx.x;
   if (tid == 0) s_sum = 0ull;
   for (int e = tid; e < sumK; e += kVramThreads) vr[e] = P.dem[e].y;
   __syncthreads();
   const float* vl = vr + (sumK - K);
-  const float* va = vl - KA;
   const float cap = P.vram_cap;
-  // units of this segment (in settings of N - 2 models), and its first and last setting
+  // this segment's first and last setting
   const uint64_t s0 = A.first + (uint64_t)blockIdx.x * A.seg;
   const uint64_t s1 = s0 + A.seg < A.first + A.n ? s0 + A.seg : A.first + A.n;
-  const uint64_t u0 = s0 / KA, u1 = (s1 + KA - 1) / KA;
   unsigned long long mine = 0;
-  for (uint64_t u = u0 + tid; u < u1; u += kVramThreads) {
-    float V2 = 0.f;
-    {
+  auto count = [&](uint64_t s, float V) {
+    const uint64_t i0 = s * (uint64_t)K;
+    const int o0 = i0 < A.lo ? (int)(A.lo - i0) : 0, o1 = A.hi - i0 < (uint64_t)K ? (int)(A.hi - i0) : K;
+    mine += vram_row_count(vl, V, cap, o0, o1);
+  };
+  if constexpr (PAIR) {
+    const float* va = vl - KA;
+    const uint64_t u1 = (s1 + KA - 1) / KA;
+    for (uint64_t u = s0 / KA + tid; u < u1; u += kVramThreads) {
       int row[NMAX];
       uint64_t p = u;
 #pragma unroll
@@ -756,16 +761,22 @@ k_vram_count(const Params P, const VramArgs A) {
           }
           row[i] = P.off[i] + (int)d;
         }
+      float V2 = 0.f;
 #pragma unroll
       for (int i = 0; i < NMAX; ++i)
         if (i < N - 2) V2 += vr[row[i]];
+      for (int a = 0; a < KA; ++a) {
+        const uint64_t s = u * KA + a;
+        if (s >= s0 && s < s1) count(s, V2 + va[a]);
+      }
     }
-    for (int a = 0; a < KA; ++a) {
-      const uint64_t s = u * KA + a;  // the setting of N - 1 models
-      if (s < s0 || s >= s1) continue;
-      const uint64_t i0 = s * (uint64_t)K;
-      const int o0 = i0 < A.lo ? (int)(A.lo - i0) : 0, o1 = A.hi - i0 < (uint64_t)K ? (int)(A.hi - i0) : K;
-      mine += vram_row_count(vl, N >= 2 ? V2 + va[a] : V2, cap, o0, o1);
+  } else {
+    VramRows<NMAX> rows;
+    uint64_t s = s0 + tid;
+    if (s < s1) rows.start(P, s);
+    for (; s < s1; s += kVramThreads) {
+      count(s, rows.sum(P, vr));
+      rows.advance(P, A.step);
     }
   }
 #pragma unroll
@@ -845,16 +856,24 @@ k_vram_write(const Params P, const VramArgs A) {
         for (unsigned e = lane; e < room; e += 32) out[e] = w0 + list[e];
         __syncwarp();
       } else {
-        for (int u = 0; u < 32; ++u) {
+        // (the settings that list anything; four rows of 32 options in flight)
+        for (unsigned rest = __ballot_sync(0xffffffffu, c > 0); rest; rest &= rest - 1u) {
+          const int u = __ffs(rest) - 1;
           const float Vu = __shfl_sync(0xffffffffu, V, u);
           const int a0 = __shfl_sync(0xffffffffu, o0, u), a1 = __shfl_sync(0xffffffffu, o1, u);
-          for (int c0 = 0; c0 < K; c0 += 32) {
-            const int o = c0 + lane;
-            const bool ok = o >= a0 && o < a1 && Vu + vl[o] <= cap;
-            const unsigned m = __ballot_sync(0xffffffffu, ok);
-            const uint64_t to = pos + __popc(m & ((1u << lane) - 1u));
-            if (ok && to < A.cap) A.out[to] = w0 + (uint64_t)u * K + o;
-            pos += __popc(m);
+          for (int c0 = 0; c0 < K; c0 += 128) {
+            unsigned m[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const int o = c0 + 32 * j + lane;
+              m[j] = __ballot_sync(0xffffffffu, o >= a0 && o < a1 && Vu + vl[o] <= cap);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const uint64_t to = pos + __popc(m[j] & ((1u << lane) - 1u));
+              if (((m[j] >> lane) & 1u) && to < A.cap) A.out[to] = w0 + (uint64_t)u * K + (c0 + 32 * j + lane);
+              pos += __popc(m[j]);
+            }
           }
         }
       }
@@ -1314,6 +1333,9 @@ mf_status mf_vram_feasible(mf_ctx* ctx, uint64_t lo, uint64_t hi, uint64_t* d_ou
   const uint64_t steps = (A.n + kVramThreads - 1) / kVramThreads;
   const uint64_t most = 4ull * ctx->num_sms;
   A.seg = (steps + most - 1) / most * kVramThreads;
+  // (fewer steps than SMs: shorter ones, in warps, so that every SM takes part)
+  const uint64_t sms = (uint64_t)ctx->num_sms;
+  if (steps < sms) A.seg = ((A.n + sms - 1) / sms + 31) / 32 * 32;
   const unsigned grid = (unsigned)((A.n + A.seg - 1) / A.seg);
   mf_status st = ensure_scratch(ctx, sizeof(unsigned long long) * grid);
   if (st != MF_OK) return st;
@@ -1329,7 +1351,14 @@ mf_status mf_vram_feasible(mf_ctx* ctx, uint64_t lo, uint64_t hi, uint64_t* d_ou
   A.cap = cap;
   A.total = (unsigned long long*)ctx->h_stage;
   const size_t smem = sizeof(float) * (size_t)ctx->sumK;
-  (N <= 8 ? k_vram_count<8> : k_vram_count<MF_MAX_MODELS>)<<<grid, kVramThreads, smem, s>>>(ctx->P, A);
+  // Settings of N - 2 models where a segment holds one for a quarter of its threads: with 43 units
+  // (24^5) the call takes 71 us by them and 57 by settings of N - 1, with one or two (255^2, 255^3)
+  // 581 and 593 against 58 and 65; with 128 (40^3 x 8 x 16) 56 and 55; with 331 (48 M
+  // configurations) 110 and 117, with 554 (24^6) 199 and 221.
+  const bool pair = N >= 2 && A.seg >= (uint64_t)ctx->P.K[N - 2] * (kVramThreads / 4);
+  const auto count_fn = pair ? (N <= 8 ? k_vram_count<8, true> : k_vram_count<MF_MAX_MODELS, true>)
+                             : (N <= 8 ? k_vram_count<8, false> : k_vram_count<MF_MAX_MODELS, false>);
+  count_fn<<<grid, kVramThreads, smem, s>>>(ctx->P, A);
   MF_CUDA(cudaGetLastError());
   (N <= 8 ? k_vram_write<8> : k_vram_write<MF_MAX_MODELS>)<<<grid, kVramThreads, smem, s>>>(ctx->P, A);
   MF_CUDA(cudaGetLastError());

@@ -21,6 +21,9 @@ def mf():
     ([9], 10.0), ([255], 10.0), ([40, 1], 9.0), ([61, 47, 2], 30.0), ([31, 29, 3], 32.0), ([13, 17, 19, 31], 40.0),
     ([13, 17, 19, 32], 44.0), ([13, 17, 19, 33], 44.0), ([5, 6, 70], 33.0), ([40, 255], 20.0), ([2] * 14, 147.0),
     ([70, 70, 70], 4.0), ([70, 70, 70], 1000.0),
+    # either side of the line between the counting kernels, segments of one and two steps
+    ([13, 17, 4, 31], 40.0), ([13, 17, 5, 31], 40.0), ([40, 40, 40, 8, 3], 50.0), ([40, 40, 40, 9, 3], 50.0),
+    ([255, 255, 3], 30.0), ([3, 140, 129], 30.0),
 ])
 @pytest.mark.parametrize("special", [None, "nonfinite"])
 def test_list_is_the_brute_force(mf, options, cap, special):
