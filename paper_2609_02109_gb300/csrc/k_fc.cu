@@ -179,8 +179,9 @@ k_fc_local(const Params P, const FcLayout L, const FcInputs I, const FcConst C) 
 //     whether all or none of the K_{N-2} K_{N-1} configurations fit, and where some do, the
 //     boundary moves one way as model N - 2's demand grows: two pointers count them in
 //     K_{N-2} + K_{N-1} steps;
-//   - the sums with the largest terms bound every J below from above, and where that bound
-//     does not reach the list's k-th entry no candidate is looked at.
+//   - the sums with the largest terms bound every J below from above, and where a candidate of
+//     that score with the setting's first index would not enter the list none is looked at
+//     (so equal scores, which enter by index, are not looked at over and over).
 // The counts and the top-k are exactly those of the sums taken one by one.  This needs
 // finite demands and a finite cap (REG); other tables are scanned one candidate at a time.
 //
@@ -478,9 +479,13 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
     if (*(volatile int*)wt.qn > 32) topk_merge_sorted(wt, lane, 32, [] __device__() { __syncwarp(); });
     else if (*(volatile int*)wt.qn > 0) topk_merge(wt, lane, 32, [] __device__() { __syncwarp(); });
   };
+  // entries queued before a warp merges: room for a row of 32 less, but as soon as its list can
+  // be filled the first time (equal scores, which the corners' bar admits, then stop coming)
+  int limit = min(R.k, kFcWarpQ - 31);
   auto raise_bar = [&]() {  // the list's k-th entry where it is the better bar (none while not full)
     const float ks = wt.ls[R.k - 1];
     const uint64_t ki = wt.li[R.k - 1];
+    if (ki != kEmptyIdx) limit = kFcWarpQ - 31;
     if (ki != kEmptyIdx && precedes(ks, ki, thr_s, thr_i)) { thr_s = ks; thr_i = ki; }
   };
   for (;;) {  // rounds; WL needs one only
@@ -500,7 +505,7 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
             look = count_there = true;  // looked at one by one
           } else if (big) {
             const bool none = !((pV2 + spa.vmin) + sb.vmin <= cap);
-            look = !none && (pJ2 + spa.jmax) + sb.jmax >= thr_s;
+            look = !none && precedes((pJ2 + spa.jmax) + sb.jmax, t0, thr_s, thr_i);
             count_there = false;
             if ((pV2 + spa.vmax) + sb.vmax <= cap) {
               my_count += (unsigned)(spa.n * sb.n);
@@ -523,7 +528,7 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
               if (pV2 + sv[mid] <= cap) lo = mid + 1; else hi = mid;
             }
             my_count += (unsigned)lo;
-            look = lo > 0 && pJ2 + sb.jmax >= thr_s;
+            look = lo > 0 && precedes(pJ2 + sb.jmax, t0, thr_s, thr_i);
             count_there = false;
           }
         }
@@ -536,6 +541,7 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
         const float bJ = __shfl_sync(0xffffffffu, pJ2, src), bV = __shfl_sync(0xffffffffu, pV2, src);
         const bool cnt = __shfl_sync(0xffffffffu, count_there ? 1 : 0, src) != 0;
         const uint64_t t0 = (u0 + __shfl_sync(0xffffffffu, my, src)) * unit;
+        const bool later = t0 > thr_i;  // (all of the unit comes after the bar's entry)
         for (; at_a < na; at_a += 32) {
           // this lane's option of model N - 2, and the options of the row worth a look
           float aJ = bJ, aV = bV;
@@ -546,7 +552,8 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
             aV += e.y;
           }
           if (!open) {
-            todo = __ballot_sync(0xffffffffu, have && (!REG || cnt || (aV + sb.vmin <= cap && aJ + sb.jmax >= thr_s)));
+            const float top = aJ + sb.jmax;
+            todo = __ballot_sync(0xffffffffu, have && (!REG || cnt || (aV + sb.vmin <= cap && (later ? top > thr_s : top >= thr_s))));
             open = true;
           }
           for (; todo; todo &= todo - 1u) {
@@ -556,7 +563,7 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
             for (; at_b < klast; at_b += 32) {
               // room for this row of 32 (in a CTA's queue: for a row of every warp)
               if (WL) {
-                if (*(volatile int*)wt.qn > kFcWarpQ - 32) {
+                if (*(volatile int*)wt.qn >= limit) {
                   merge_warp();
                   raise_bar();
                 }
@@ -617,10 +624,21 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
     if (!more) break;
     raise_bar();
   }
-  if (WL) {  // the warps' lists join the CTA's
+  if (WL) {  // the warps' lists join the CTA's: no entry after the foremost of their k-th ones
+    __shared__ float s_ks[kFcWarps];
+    __shared__ uint64_t s_ki[kFcWarps];
+    if (lane == 0) {
+      s_ks[warp] = wt.ls[R.k - 1];
+      s_ki[warp] = wt.li[R.k - 1];
+    }
     __syncthreads();
+    float ks = -INFINITY;
+    uint64_t ki = kEmptyIdx;
+#pragma unroll 4
+    for (int w = 0; w < kFcWarps; ++w)
+      if (precedes(s_ks[w], s_ki[w], ks, ki)) { ks = s_ks[w]; ki = s_ki[w]; }
     for (int e = lane; e < R.k; e += 32)
-      if (wt.li[e] != kEmptyIdx) {
+      if (wt.li[e] != kEmptyIdx && !precedes(ks, ki, wt.ls[e], wt.li[e])) {
         const int pos = atomicAdd(tk.qn, 1);
         tk.qs[pos] = wt.ls[e];
         tk.qi[pos] = wt.li[e];
