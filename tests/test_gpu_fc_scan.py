@@ -122,3 +122,26 @@ def test_corner_values_that_overflow(mf, k):
         r = ctx.fc_search(k)
         assert count == 7 * 7 and r["count"] == count
         assert np.array_equal(r["topk_idx"][:ti.size], ti) and np.array_equal(r["topk_score"][:ts.size], ts)
+
+
+@pytest.mark.parametrize("k", [1, 32, 64, 65, 300])
+@pytest.mark.parametrize("levels", ["one", "few"])
+@pytest.mark.parametrize("cap", [500.0, 52.0])
+def test_equal_scores(mf, k, levels, cap):
+    """Utilities of one value, or of a reload cost paid or not: by index among equals, where
+    whole settings of the leading models only tie with the bar."""
+    options = [24, 23, 22, 21, 5]
+    prob = W.make_problem(options, 8, 32, 0, 93, cap)
+    fc = W.fc_scenario(prob, 93)
+    fc["tau"] = np.full(5, -5.0, np.float32)
+    fc["omega"] = np.zeros(5, np.float32)
+    fc["prev_variant"] = np.zeros(5, np.int32)
+    fc["beta"], fc["alpha"] = 0.0, 0.0 if levels == "one" else 1.0 / 60.0
+    with mf.Context(prob) as ctx:
+        ctx.fc_set(fc)
+        total = ctx.space_size
+        for lo, hi in ((0, total), (total // 3, total - 7)):
+            count, ti, ts = brute(prob, ctx, k, lo, hi)
+            r = ctx.fc_search(k, lo=lo, hi=hi)
+            assert r["count"] == count
+            assert np.array_equal(r["topk_idx"], ti) and np.array_equal(r["topk_score"], ts)
