@@ -317,7 +317,9 @@ k_score_f32(const Params P, const RangeArgs R, const ListArgs L) {
 // weights in shared memory with one round of wide loads, where reading each row from L2 as
 // it is needed cost a dependent round trip per input of layer 1 and per batch of layer 2
 // (256 candidates x 6 models of 12->64->64->2: 6.6 us staged, 18.8 from L2; 20->128->128->2
-// x 8: 19 and 104).
+// x 8: 19 and 104).  Weights too large to stage are read in batches with nothing conditional
+// between them (100 candidates x 3 models of 12->256->256->2, with the call: 51 us; under a
+// condition each, 107 and 265).
 // ---------------------------------------------------------------------------
 template <int U1, int U2, bool ST>
 __global__ void __launch_bounds__(kWideWarps * 32)
@@ -384,16 +386,35 @@ k_wide_f32(const Params P, const uint64_t* __restrict__ idx, const int32_t* __re
     const float* W1T = w;
     const float* b1 = W1T + (size_t)din * h1;
     float hv1[U1];
+    if constexpr (ST) {
 #pragma unroll
-    for (int u = 0; u < U1; ++u) {
-      const int j = lane + 32 * u;
-      float s = j < h1 ? ldw(b1 + j) : 0.f;
+      for (int u = 0; u < U1; ++u) {
+        const int j = lane + 32 * u;
+        float s = j < h1 ? ldw(b1 + j) : 0.f;
+#pragma unroll 4
+        for (int k = 0; k < din; ++k) {
+          const float zk = __shfl_sync(0xffffffffu, zown, k);
+          if (j < h1) s = fmaf(ldw(W1T + (size_t)k * h1 + j), zk, s);
+        }
+        hv1[u] = j < h1 ? relu(s) : 0.f;
+      }
+    } else {
+      // All units of an input at once, a round trip per four inputs.  Lanes past the last unit
+      // read it again (their sums are dropped): no condition stands between the loads.
+      int at[U1];
+#pragma unroll
+      for (int u = 0; u < U1; ++u) {
+        at[u] = min(lane + 32 * u, h1 - 1);
+        hv1[u] = ldw(b1 + at[u]);
+      }
 #pragma unroll 4
       for (int k = 0; k < din; ++k) {
         const float zk = __shfl_sync(0xffffffffu, zown, k);
-        if (j < h1) s = fmaf(ldw(W1T + (size_t)k * h1 + j), zk, s);
+#pragma unroll
+        for (int u = 0; u < U1; ++u) hv1[u] = fmaf(ldw(W1T + (size_t)k * h1 + at[u]), zk, hv1[u]);
       }
-      hv1[u] = j < h1 ? relu(s) : 0.f;
+#pragma unroll
+      for (int u = 0; u < U1; ++u) hv1[u] = lane + 32 * u < h1 ? relu(hv1[u]) : 0.f;
     }
     const float* p = b1 + h1;
     float t = 0.f, l = 0.f;
@@ -407,17 +428,51 @@ k_wide_f32(const Params P, const uint64_t* __restrict__ idx, const int32_t* __re
         const int j = lane + 32 * u2;
         acc2[u2] = j < h2 ? ldw(b2 + j) : 0.f;
       }
+      if constexpr (ST) {
 #pragma unroll
-      for (int u = 0; u < U1; ++u) {
+        for (int u = 0; u < U1; ++u) {
 #pragma unroll
-        for (int kk = 0; kk < 32; ++kk) {
-          const int k = 32 * u + kk;
-          if (k < h1) {
-            const float hk = __shfl_sync(0xffffffffu, hv1[u], kk);
+          for (int kk = 0; kk < 32; ++kk) {
+            const int k = 32 * u + kk;
+            if (k < h1) {
+              const float hk = __shfl_sync(0xffffffffu, hv1[u], kk);
 #pragma unroll
-            for (int u2 = 0; u2 < U2; ++u2) {
-              const int j = lane + 32 * u2;
-              if (j < h2) acc2[u2] = fmaf(ldw(W2T + (size_t)k * h2 + j), hk, acc2[u2]);
+              for (int u2 = 0; u2 < U2; ++u2) {
+                const int j = lane + 32 * u2;
+                if (j < h2) acc2[u2] = fmaf(ldw(W2T + (size_t)k * h2 + j), hk, acc2[u2]);
+              }
+            }
+          }
+        }
+      } else {  // G rows' weights are read before the first is used
+        constexpr int G = 8;
+        int at[U2];
+#pragma unroll
+        for (int u2 = 0; u2 < U2; ++u2) at[u2] = min(lane + 32 * u2, h2 - 1);
+#pragma unroll
+        for (int u = 0; u < U1; ++u) {
+#pragma unroll 1
+          for (int kk = 0; kk < 32 && 32 * u + kk < h1; kk += G) {
+            const float* rows = W2T + (size_t)(32 * u + kk) * h2;
+            if (32 * u + kk + G <= h1) {
+              float wv[G][U2];
+#pragma unroll
+              for (int g = 0; g < G; ++g)
+#pragma unroll
+                for (int u2 = 0; u2 < U2; ++u2) wv[g][u2] = ldw(rows + (size_t)g * h2 + at[u2]);
+#pragma unroll
+              for (int g = 0; g < G; ++g) {
+                const float hk = __shfl_sync(0xffffffffu, hv1[u], kk + g);
+#pragma unroll
+                for (int u2 = 0; u2 < U2; ++u2) acc2[u2] = fmaf(wv[g][u2], hk, acc2[u2]);
+              }
+            } else {
+#pragma unroll 1
+              for (int g = 0; 32 * u + kk + g < h1; ++g) {
+                const float hk = __shfl_sync(0xffffffffu, hv1[u], kk + g);
+#pragma unroll
+                for (int u2 = 0; u2 < U2; ++u2) acc2[u2] = fmaf(ldw(rows + (size_t)g * h2 + at[u2]), hk, acc2[u2]);
+              }
             }
           }
         }

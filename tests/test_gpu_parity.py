@@ -256,3 +256,19 @@ def test_default_launches_are_bounded(mf, precision, h, launches):
         b = ctx.search(16, chunk=10_000_019)
     assert a["count"] == b["count"] and np.array_equal(a["topk_idx"], b["topk_idx"])
     assert np.array_equal(a["topk_score"], b["topk_score"])
+
+
+@pytest.mark.parametrize("d_local,h1,h2", [(8, 256, 256), (8, 203, 197), (3, 129, 255), (8, 255, 100), (28, 160, 161), (5, 150, 151)])
+def test_small_lists_of_wide_predictors(mf, oracle_mod, d_local, h1, h2):
+    """Weights too large to stage in shared memory (above 96 KB a model): widths that are no
+    multiple of the 8 rows or 32 units that are read together, and that differ."""
+    assert 4 * W.param_count(d_local, h1, h2) > 96 * 1024
+    prob = W.make_problem([5, 6, 4], d_local, h1, h2, 6, 30.0, sla_range=W.TIGHT_SLA)
+    o = oracle_mod.Oracle(prob)
+    idx = np.random.default_rng(2).integers(0, 120, 333).astype(np.uint64)
+    r = o.score_list(idx, with_pred=True)
+    with mf.Context(prob) as ctx:
+        import torch
+        out = ctx.score_batch(torch.from_numpy(idx.astype(np.int64)).cuda(), with_pred=True)
+        s, f, p = (t.cpu().numpy() for t in out)
+    check_scores(prob, s, f, *r, got_pred=p)
