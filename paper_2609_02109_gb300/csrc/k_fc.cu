@@ -182,8 +182,9 @@ k_fc_local(const Params P, const FcLayout L, const FcInputs I, const FcConst C) 
 //   - the sums with the largest terms bound every J below from above, and where a candidate of
 //     that score with the setting's first index would not enter the list none is looked at
 //     (so equal scores, which enter by index, are not looked at over and over).
-// The counts and the top-k are exactly those of the sums taken one by one.  This needs
-// finite demands and a finite cap (REG); other tables are scanned one candidate at a time.
+// The counts and the top-k are exactly those of the sums taken one by one.  This needs sums
+// that do not turn to NaN (REG): no demand of -inf, and +inf only under a finite cap, where such
+// options fit nowhere.  Other tables are scanned one candidate at a time.
 //
 // The bar starts high: J is a sum of per-model terms, so the best configurations sit where
 // every model has one of its best options.  Every CTA first scores a corner of the space, the
@@ -234,7 +235,7 @@ __host__ __device__ inline size_t fc_scan_table_bytes(int sumK) {
   return (((size_t)sumK * sizeof(float2) + 15) & ~(size_t)15) + 2 * 256 * sizeof(float);
 }
 
-// The extremes of a model's usable options (finite VRAM in the CTA's table).
+// The extremes of a model's usable options (their VRAM in the CTA's table is not NaN).
 struct FcSpan {
   float jmax, jmin, vmin, vmax;
   int n;
@@ -276,11 +277,12 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
   } else {
     wt = tk;
   }
-  // an option below its floor (utility -inf, or NaN) carries VRAM +inf here, so one
-  // compare against the cap decides feasibility
+  // an option below its floor (utility -inf, or NaN) carries VRAM NaN here, so one compare
+  // against the cap decides feasibility, whatever the cap; REG: so does an option whose demand
+  // no cap allows
   for (int e = tid; e < sumK; e += blockDim.x) {
     float2 v = S.tab[e];
-    if (!(v.x > -INFINITY)) v.y = INFINITY;
+    if (!(v.x > -INFINITY) || (REG && !(v.y < INFINITY))) v.y = NAN;
     tab[e] = v;
   }
   const size_t gl = (size_t)blockIdx.x * R.k;
@@ -346,7 +348,7 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
       // slot of `order` that the corner reads is written)
       auto value = [&](int o) {
         const float2 e = o < K ? tab[off + o] : make_float2(-INFINITY, INFINITY);
-        if (task < 2) return -e.y;
+        if (task < 2) return e.y < INFINITY ? -e.y : -INFINITY;
         return e.y < INFINITY ? fmaxf(__fsub_rn(e.x, __fmul_rn(lam, e.y)), -FLT_MAX) : -INFINITY;
       };
       for (int c0 = 0; c0 < K; c0 += 32) {
@@ -1208,7 +1210,7 @@ mf_status fc_search_chunk(mf_ctx* c, const RangeArgs& a, int grid, cudaStream_t 
   const int N = P.n_models;
   FcScan S{};
   S.tab = L.tab;
-  const bool reg = c->finite_vram && std::isfinite(P.vram_cap);
+  const bool reg = !c->vram_minus_inf && (!c->vram_plus_inf || P.vram_cap < INFINITY);
   if (reg && c->sumK <= kFcCornerRows && a.k <= (1 << kFcCornerBits)) {
     // one bit of the corner for each model in turn, while it has options for it
     int left = kFcCornerBits;

@@ -187,8 +187,10 @@ mf_status mf_create(const mf_problem* p, mf_ctx** out) {
 
   // host-side images
   std::vector<float> dem4((size_t)sumK * 4, 0.f);
-  c->finite_vram = true;
-  for (int r = 0; r < sumK; ++r) c->finite_vram = c->finite_vram && std::isfinite(p->demand[(size_t)r * 3 + 1]);
+  for (int r = 0; r < sumK; ++r) {
+    c->vram_plus_inf = c->vram_plus_inf || p->demand[(size_t)r * 3 + 1] == INFINITY;
+    c->vram_minus_inf = c->vram_minus_inf || p->demand[(size_t)r * 3 + 1] == -INFINITY;
+  }
   for (int r = 0; r < sumK; ++r)
     for (int j = 0; j < 3; ++j) dem4[(size_t)r * 4 + j] = p->demand[(size_t)r * 3 + j];
   std::vector<float> w32((size_t)N * per_pad, 0.f), wT((size_t)N * per_pad, 0.f);

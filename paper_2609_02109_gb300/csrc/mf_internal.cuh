@@ -385,7 +385,7 @@ struct mf_ctx {
   // fixed-context mode: the per-option table of the last mf_fc_set
   void* d_fc = nullptr;           // see mf::FcLayout
   int fc_ready = 0;
-  bool finite_vram = false;       // every option's VRAM demand is finite
+  bool vram_plus_inf = false, vram_minus_inf = false;  // an option's VRAM demand is infinite
   float4* d_util = nullptr;       // [sumK] utility table of mf_set_utility
   int32_t base_objective = 0;     // the problem's own objective
   size_t tc_bytes = 0;

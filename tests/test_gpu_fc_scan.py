@@ -74,13 +74,14 @@ def test_scan_is_the_brute_force(mf, options, cap, tau, k):
             assert (r["topk_idx"][n:] == np.uint64(mf.EMPTY)).all()
 
 
-@pytest.mark.parametrize("special", ["cap_on_a_sum", "equal_terms", "inf_demand", "nan_demand", "inf_quality"])
+@pytest.mark.parametrize("special", ["cap_on_a_sum", "equal_terms", "inf_demand", "nan_demand", "inf_quality",
+                                     "plus_inf_demand", "inf_cap", "inf_cap_and_demand", "minus_inf_cap", "large_demands"])
 def test_special_values(mf, special):
     options = [11, 12, 13]
     prob = W.make_problem(options, 8, 32, 0, 77, 30.0)
     dem = prob["demand"]
     fc = W.fc_scenario(prob, 77)
-    fc["tau"] = np.full(3, -5.0, np.float32)
+    fc["tau"] = np.full(3, 0.1 if "inf_cap" in special else -5.0, np.float32)  # (0.1: some options below)
     if special == "cap_on_a_sum":  # the bound is inclusive
         prob["vram_cap"] = float((dem[3, 1] + dem[11 + 5, 1]) + dem[23 + 7, 1])
     elif special == "equal_terms":
@@ -89,14 +90,24 @@ def test_special_values(mf, special):
         dem[:, 1] = 4.0
     elif special == "inf_demand":
         dem[[2, 15, 30], 1] = [np.inf, -np.inf, np.inf]
+    elif special == "plus_inf_demand":
+        dem[[2, 15, 30], 1] = np.inf
+    elif special.startswith("inf_cap") or special == "minus_inf_cap":
+        prob["vram_cap"] = -np.inf if special == "minus_inf_cap" else np.inf
+        if special == "inf_cap_and_demand":
+            dem[[2, 15, 30], 1] = np.inf
+    elif special == "large_demands":  # sums beyond fp32's range, of either sign
+        dem[:, 1] *= np.float32(1e37)
+        dem[11:17, 1] *= -1
     elif special == "nan_demand":
         dem[[0, 20], 1] = np.nan
     else:
         fc["quality"][[4, 17]] = np.inf
     with mf.Context(prob) as ctx:
         ctx.fc_set(fc)
-        with np.errstate(invalid="ignore"):
+        with np.errstate(invalid="ignore", over="ignore"):
             count, ti, ts = brute(prob, ctx, 40, 0, ctx.space_size)
+        assert "inf_cap" not in special or not ctx.fc_table()[3].all()
         r = ctx.fc_search(40)
         assert r["count"] == count
         if special != "inf_quality":
