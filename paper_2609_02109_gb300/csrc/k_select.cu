@@ -13,6 +13,67 @@ constexpr int kMergeMaxLists = 32 * kMergeLane;
 static_assert(kMergeMaxLists == kMaxTops, "one bound for both");
 constexpr size_t kPair = sizeof(uint64_t) + sizeof(float);
 
+// Entries of a sorted row of 32 ahead of (s, id), where scores tie with s: by index too.  Out of
+// line (ties are rare and the kernels' instructions are read once a launch).  (One after
+// another, the ties of 18 lists of 32 equal scores took 45 us.)
+__device__ __noinline__ int row_rank(const float* rs, const uint64_t* ri, float s, uint64_t id) {
+  int lo = 0;
+#pragma unroll
+  for (int step = 16; step > 0; step >>= 1) lo += precedes(rs[lo + step - 1], ri[lo + step - 1], s, id) ? step : 0;
+  return lo + (precedes(rs[lo], ri[lo], s, id) ? 1 : 0);
+}
+
+// The part of a warp's bound (see k_merge_lists) that ties need: of the lists whose entry at
+// position p has the score key v, the last index that is wanted so that `need` lists come up to
+// (v, that index).  `tied`: room for kMergeMaxLists indices.  Out of line, as above.
+__device__ __noinline__ uint64_t tied_index(const float* in_s, const uint64_t* in_i, int nlists, int k, int p, uint32_t v,
+                                            int need, uint64_t* tied) {
+  const int lane = threadIdx.x & 31;
+  int above = 0;
+  uint32_t hi = 0u;
+  for (int l = lane; l < kMergeMaxLists; l += 32) {
+    const uint32_t key = l < nlists ? order_key(in_s[(size_t)l * k + p]) : 0u;
+    const uint64_t id = key == v ? in_i[(size_t)l * k + p] : kEmptyIdx;
+    above += key > v ? 1 : 0;
+    tied[l] = id;
+    if (id != kEmptyIdx) hi |= (uint32_t)(id >> 32);
+  }
+  const int want = need - __reduce_add_sync(0xffffffffu, above);
+  hi = __reduce_or_sync(0xffffffffu, hi);
+  uint64_t x = 0ull;  // the largest bound with fewer than `want` indices below it
+  for (int b = hi ? 63 - __clz(hi) : 31; b >= 0; --b) {
+    const uint64_t t = x | (1ull << b);
+    int c = 0;
+#pragma unroll 4
+    for (int j = 0; j < kMergeLane; ++j) c += tied[lane + 32 * j] < t ? 1 : 0;
+    if (__reduce_add_sync(0xffffffffu, c) < want) x = t;
+  }
+  return x;
+}
+
+// The gather of k_merge_lists where the bar cuts equal scores by index: the entries of the
+// lists `which` up to (bar, the least of the lanes' bound_i).  Out of line, as above.
+__device__ __noinline__ void gather_cut(const float* in_s, const uint64_t* in_i, int k, const int* which, int n, uint32_t bar,
+                                        uint64_t bound_i, int cap, float* ss, uint64_t* si, int* count) {
+  const int lane = threadIdx.x & 31;
+  for (int w = 16; w > 0; w >>= 1) bound_i = min(bound_i, __shfl_xor_sync(0xffffffffu, bound_i, w));
+  for (int q = threadIdx.x >> 5; q < n; q += blockDim.x >> 5) {
+    const size_t l = (size_t)which[q] * k;
+    unsigned m = 0xffffffffu;  // the lanes whose entry stays: a prefix (the lists are sorted)
+    for (int pos = lane; m == 0xffffffffu; pos += 32) {
+      const float sc = pos < k ? in_s[l + pos] : -INFINITY;
+      const uint64_t ix = pos < k ? in_i[l + pos] : kEmptyIdx;
+      const uint32_t key = order_key(sc);
+      const bool keep = ix != kEmptyIdx && (key > bar || (key == bar && ix <= bound_i));
+      m = __ballot_sync(0xffffffffu, keep);
+      int at = 0;
+      if (lane == 0 && m) at = atomicAdd(count, __popc(m));
+      at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+      if (keep && at < cap) { ss[at] = sc; si[at] = ix; }
+    }
+  }
+}
+
 // Sorts n distinct entries (ss, si) of shared memory best first and writes the first k
 // to the output, empty slots after them.  Up to one entry per thread: each warp sorts its
 // 32 in registers (shuffles), then an entry's position is its place in its own row of 32
@@ -51,14 +112,7 @@ __device__ void sort_out(float* ss, uint64_t* si, int n, int k, const ResultOut&
         for (int step = 16; step > 0; step >>= 1) lo += rs[lo + step - 1] > s ? step : 0;
         lo += rs[lo] > s ? 1 : 0;
         if (r == row) continue;
-        if (lo < 32 && rs[lo] == s) {  // ties, by index (one after another, 18 lists of 32 equal scores took 45 us)
-          const uint64_t* ri = si + 32 * r;
-          lo = 0;
-#pragma unroll
-          for (int step = 16; step > 0; step >>= 1)
-            lo += precedes(rs[lo + step - 1], ri[lo + step - 1], s, id) ? step : 0;
-          lo += precedes(rs[lo], ri[lo], s, id) ? 1 : 0;
-        }
+        if (lo < 32 && rs[lo] == s) lo = row_rank(rs, si + 32 * r, s, id);
         rank += lo;
       }
     }
@@ -163,24 +217,31 @@ __device__ __noinline__ void merge_tree(const float* in_s, const uint64_t* in_i,
 // position p bounds the k-th best entry from below.  Warp j takes the bound of position
 // p = 4^j - 1 (bisection over the score keys, each lane holding up to kMergeLane lists),
 // and the largest bound is the bar: at most k / 4^j lists then hold more than 4^j - 1
-// entries above it, so one to two k entries remain, and 4 k (log4(k) + 1) at most, ties
-// with the bar aside.  They are gathered into shared memory (`cap` entries) and sorted there.  Where
-// ties leave more than that, and above kMergeMaxLists lists, a merge tree through global
-// memory takes over.
+// entries above it, so one to two k entries remain, and 4 k (log4(k) + 1) at most.  Where more
+// than T lists reach the bound, some only tie with it: a bisection over the tied entries'
+// indices then tells which T come first, so that entries equal to the bar in score are cut by
+// index.  What remains is gathered into shared memory (`cap` entries) and sorted there.  Where
+// that is more than the room, and above kMergeMaxLists lists, a merge tree through global memory
+// takes over.
 //
 // Bound by latency (a few dependent L2 reads and block barriers).  608 lists of 256
-// entries: 14 us, where the tree alone took 380-560; 304 lists of 32: 9 (tree: 35).
+// entries: 14 us, where the tree alone took 380-560; 304 lists of 32: 9 (tree: 35).  608 lists of
+// 800 equal scores, with the re-scoring that follows: 94 us (by the tree 2.15 ms).
 __global__ void __launch_bounds__(kMergeThreads)
 k_merge_lists(const float* __restrict__ in_s, const uint64_t* __restrict__ in_i, int nlists, int k, int cap,
               float* a_s, uint64_t* a_i, float* b_s, uint64_t* b_i, const ResultOut out) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ uint32_t s_bar[32];
+  __shared__ uint32_t s_bar[32];      // a warp's bound: score key, and the last index among equals
+  __shared__ uint64_t s_bar_i[32];
   __shared__ int s_lists[kMergeMaxLists];
   __shared__ int s_nlist, s_n;
   uint64_t* si = reinterpret_cast<uint64_t*>(smem);
   float* ss = reinterpret_cast<float*>(si + cap);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid < 32) s_bar[tid] = 0u;
+  if (tid < 32) {
+    s_bar[tid] = 0u;
+    s_bar_i[tid] = kEmptyIdx;
+  }
   if (tid == 0) {
     s_nlist = 0;
     s_n = 0;
@@ -200,6 +261,7 @@ k_merge_lists(const float* __restrict__ in_s, const uint64_t* __restrict__ in_i,
         key[j] = l < nlists ? order_key(in_s[(size_t)l * k + p]) : 0u;
       }
       uint32_t v = 0u;
+      bool exact = false;  // `need` lists reach v, no more
       for (int b = 31; b >= 0; --b) {
         const uint32_t t = v | (1u << b);
         int c[4] = {0, 0, 0, 0};  // (short chains of dependent adds)
@@ -207,20 +269,31 @@ k_merge_lists(const float* __restrict__ in_s, const uint64_t* __restrict__ in_i,
         for (int j = 0; j < kMergeLane; ++j) c[j & 3] += key[j] >= t ? 1 : 0;
         const int reach = __reduce_add_sync(0xffffffffu, (c[0] + c[1]) + (c[2] + c[3]));
         if (reach >= need) v = t;
-        if (reach == need) break;  // (lower bits would only tighten the bar past ties)
+        exact = reach == need;
+        if (exact) break;  // (lower bits would only tighten the bar past ties)
       }
-      if (lane == 0) s_bar[warp] = v;
+      // (the gather's room is not in use yet)
+      const uint64_t x = exact || v <= kKeyMinusInf
+                             ? kEmptyIdx
+                             : tied_index(in_s, in_i, nlists, k, p, v, need, si + (size_t)warp * kMergeMaxLists);
+      if (lane == 0) {
+        s_bar[warp] = v;
+        s_bar_i[warp] = x;
+      }
     }
     __syncthreads();
     const uint32_t bar = __reduce_max_sync(0xffffffffu, s_bar[lane]);
+    const uint64_t bound_i = s_bar[lane] == bar ? s_bar_i[lane] : kEmptyIdx;
+    const bool cut = __any_sync(0xffffffffu, bound_i != kEmptyIdx);  // equal scores by index
     // the lists whose best entry reaches the bar, then their entries that do
     for (int l = tid; l < nlists; l += kMergeThreads)
       if (order_key(in_s[(size_t)l * k]) >= bar)
         s_lists[atomicAdd(&s_nlist, 1)] = l;
     __syncthreads();
     const int nl = s_nlist;
+    if (cut) gather_cut(in_s, in_i, k, s_lists, nl, bar, bound_i, cap, ss, si, &s_n);
     constexpr int kBatch = 8;  // lists a warp has in flight
-    for (int q0 = warp; q0 < nl; q0 += (kMergeThreads / 32) * kBatch) {
+    for (int q0 = warp; q0 < nl && !cut; q0 += (kMergeThreads / 32) * kBatch) {
       float v[kBatch];
       uint64_t id[kBatch];
 #pragma unroll

@@ -1,7 +1,6 @@
-"""The merge of the per-CTA lists where it can go wrong: scores that all tie (more entries
-reach the bar than the merge gathers, so the tree takes over), scores with many ties (exact
-integers, against the oracle), list lengths around the 32-entry rows, and a range that
-leaves most lists empty."""
+"""The merge of the per-CTA lists where it can go wrong: scores that all tie (the bar cuts them
+by index, also beyond 2^32), scores with many ties (exact integers, against the oracle), list
+lengths around the 32-entry rows, and a range that leaves most lists empty."""
 import numpy as np
 import pytest
 
@@ -47,3 +46,30 @@ def test_many_ties_match_the_oracle(mf, oracle_mod, k):
         r = ctx.search(k)
     assert r["count"] == cnt
     assert np.array_equal(r["topk_idx"], ti) and np.array_equal(r["topk_score"].astype(np.float64), ts)
+
+
+@pytest.mark.parametrize("k", [1, 5, 100, 1024])
+@pytest.mark.parametrize("levels", [1, 3])
+def test_ties_at_indices_beyond_2_32(mf, k, levels):
+    """The last 300001 indices of 255^5: one score, or three that the last model's option
+    chooses, spread over all lists."""
+    prob = W.make_problem([255] * 5, 8, 32, 0, 34, 1e6, precision="fp32_simt")
+    prob["obj_w"] = np.zeros(5, np.float32)
+    prob["sla"] = np.full(5, 100.0, np.float32)
+    prob["weights"][:] = 0.0
+    if levels == 3:  # throughput of the last model = its first feature: 2, 1 or 0
+        prob["obj_w"][4] = 1.0
+        per = W.param_count(8, 32, 0)
+        prob["local_feats"][4 * 255:, 0] = np.arange(255) % 3
+        w = prob["weights"][4 * per:]
+        w[0] = 1.0                 # W1[0, 0]
+        w[32 * 12 + 32] = 1.0      # W3[0, 0]
+    n = 255 ** 5
+    lo = n - 300001
+    idx = np.arange(lo, n, dtype=np.uint64)
+    J = (idx % np.uint64(255) % np.uint64(3)).astype(np.float32) if levels == 3 else np.zeros(idx.size, np.float32)
+    order = np.lexsort((idx, -J))[:k]
+    with mf.Context(prob) as ctx:
+        r = ctx.search(k, lo=lo, hi=n)
+    assert r["count"] == 300001
+    assert np.array_equal(r["topk_idx"], idx[order]) and np.array_equal(r["topk_score"], J[order])
