@@ -179,9 +179,10 @@ k_fc_local(const Params P, const FcLayout L, const FcInputs I, const FcConst C) 
 //     whether all or none of the K_{N-2} K_{N-1} configurations fit, and where some do, the
 //     boundary moves one way as model N - 2's demand grows: two pointers count them in
 //     K_{N-2} + K_{N-1} steps;
-//   - the sums with the largest terms bound every J below from above, and where a candidate of
-//     that score with the setting's first index would not enter the list none is looked at
-//     (so equal scores, which enter by index, are not looked at over and over).
+//   - the sums with the largest terms bound every J below from above, and where that bound
+//     does not reach the list's k-th entry no candidate is looked at; where it only equals it,
+//     none of a setting that comes after that entry (so equal scores, which enter by index,
+//     are not looked at over and over).
 // The counts and the top-k are exactly those of the sums taken one by one.  This needs sums
 // that do not turn to NaN (REG): no demand of -inf, and +inf only under a finite cap, where such
 // options fit nowhere.  Other tables are scanned one candidate at a time.
@@ -446,7 +447,10 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
   const uint64_t end = R.base + R.len, u0 = R.base / unit;
   const uint64_t nu = R.len == 0 ? 0 : (end - 1) / unit - u0 + 1;  // units of the range
   const uint64_t nthreads = (uint64_t)gridDim.x * blockDim.x;
-  uint64_t my = (uint64_t)blockIdx.x * blockDim.x + tid;           // this lane's unit, from u0
+  // this lane's unit, from u0 (where most are looked at they go round the warps, which look at
+  // their units one after another)
+  uint64_t my = !S.corner && nu < nthreads ? (uint64_t)lane * (nthreads / 32) + (uint64_t)warp * gridDim.x + blockIdx.x
+                                           : (uint64_t)blockIdx.x * blockDim.x + tid;
   int row[NMAX];  // option rows of models 0 .. lead - 1
   {
     uint64_t v = my < nu ? u0 + my : 0;
@@ -481,13 +485,9 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
     if (*(volatile int*)wt.qn > 32) topk_merge_sorted(wt, lane, 32, [] __device__() { __syncwarp(); });
     else if (*(volatile int*)wt.qn > 0) topk_merge(wt, lane, 32, [] __device__() { __syncwarp(); });
   };
-  // entries queued before a warp merges: room for a row of 32 less, but as soon as its list can
-  // be filled the first time (equal scores, which the corners' bar admits, then stop coming)
-  int limit = min(R.k, kFcWarpQ - 31);
   auto raise_bar = [&]() {  // the list's k-th entry where it is the better bar (none while not full)
     const float ks = wt.ls[R.k - 1];
     const uint64_t ki = wt.li[R.k - 1];
-    if (ki != kEmptyIdx) limit = kFcWarpQ - 31;
     if (ki != kEmptyIdx && precedes(ks, ki, thr_s, thr_i)) { thr_s = ks; thr_i = ki; }
   };
   for (;;) {  // rounds; WL needs one only
@@ -507,7 +507,7 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
             look = count_there = true;  // looked at one by one
           } else if (big) {
             const bool none = !((pV2 + spa.vmin) + sb.vmin <= cap);
-            look = !none && precedes((pJ2 + spa.jmax) + sb.jmax, t0, thr_s, thr_i);
+            look = !none && (pJ2 + spa.jmax) + sb.jmax >= thr_s;
             count_there = false;
             if ((pV2 + spa.vmax) + sb.vmax <= cap) {
               my_count += (unsigned)(spa.n * sb.n);
@@ -530,7 +530,7 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
               if (pV2 + sv[mid] <= cap) lo = mid + 1; else hi = mid;
             }
             my_count += (unsigned)lo;
-            look = lo > 0 && precedes(pJ2 + sb.jmax, t0, thr_s, thr_i);
+            look = lo > 0 && pJ2 + sb.jmax >= thr_s;
             count_there = false;
           }
         }
@@ -565,7 +565,7 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
             for (; at_b < klast; at_b += 32) {
               // room for this row of 32 (in a CTA's queue: for a row of every warp)
               if (WL) {
-                if (*(volatile int*)wt.qn >= limit) {
+                if (*(volatile int*)wt.qn > kFcWarpQ - 32) {
                   merge_warp();
                   raise_bar();
                 }
@@ -626,21 +626,10 @@ k_fc_scan(const Params P, const FcScan S, const RangeArgs R) {
     if (!more) break;
     raise_bar();
   }
-  if (WL) {  // the warps' lists join the CTA's: no entry after the foremost of their k-th ones
-    __shared__ float s_ks[kFcWarps];
-    __shared__ uint64_t s_ki[kFcWarps];
-    if (lane == 0) {
-      s_ks[warp] = wt.ls[R.k - 1];
-      s_ki[warp] = wt.li[R.k - 1];
-    }
+  if (WL) {  // the warps' lists join the CTA's
     __syncthreads();
-    float ks = -INFINITY;
-    uint64_t ki = kEmptyIdx;
-#pragma unroll 4
-    for (int w = 0; w < kFcWarps; ++w)
-      if (precedes(s_ks[w], s_ki[w], ks, ki)) { ks = s_ks[w]; ki = s_ki[w]; }
     for (int e = lane; e < R.k; e += 32)
-      if (wt.li[e] != kEmptyIdx && !precedes(ks, ki, wt.ls[e], wt.li[e])) {
+      if (wt.li[e] != kEmptyIdx) {
         const int pos = atomicAdd(tk.qn, 1);
         tk.qs[pos] = wt.ls[e];
         tk.qi[pos] = wt.li[e];
@@ -1195,11 +1184,19 @@ k_fc_ga(const Params P, const FcGaArgs A) {
   }
 }
 
-// One CTA per SM, fewer where the range has fewer settings of the leading N - 1 models
-// than they have threads (a short list of lists to merge).
-int fc_grid(const mf_ctx* c, uint64_t len) {
+// Whether the corners are worth their ranking: where the range's share of their configurations
+// can hold k.
+static bool fc_corner(const mf_ctx* c, uint64_t len, int k) {
+  return c->sumK <= kFcCornerRows && (double)len * (1 << kFcCornerBits) >= (double)k * (double)c->P.total;
+}
+
+// One CTA per SM, fewer where the range has fewer settings of the leading N - 1 models than
+// they have threads (a short list of lists to merge), or, without a bar from the corners, four
+// settings a warp, since it looks at most of them.
+int fc_grid(const mf_ctx* c, uint64_t len, int k) {
   const uint64_t units = len / (uint64_t)c->P.K[c->P.n_models - 1] + 2;
-  const uint64_t ctas = (units + kFcThreads - 1) / kFcThreads;
+  const uint64_t per = fc_corner(c, len, k) ? kFcThreads : 4 * kFcWarps;
+  const uint64_t ctas = (units + per - 1) / per;
   return (int)(ctas < (uint64_t)c->num_sms ? ctas : (uint64_t)c->num_sms);
 }
 
@@ -1211,7 +1208,7 @@ mf_status fc_search_chunk(mf_ctx* c, const RangeArgs& a, int grid, cudaStream_t 
   FcScan S{};
   S.tab = L.tab;
   const bool reg = !c->vram_minus_inf && (!c->vram_plus_inf || P.vram_cap < INFINITY);
-  if (reg && c->sumK <= kFcCornerRows && a.k <= (1 << kFcCornerBits)) {
+  if (reg && fc_corner(c, a.len, a.k)) {
     // one bit of the corner for each model in turn, while it has options for it
     int left = kFcCornerBits;
     for (bool grew = true; grew && left > 0;) {

@@ -404,7 +404,7 @@ static mf_status search_impl(mf_ctx* ctx, uint64_t lo, uint64_t hi, int32_t k, u
   else if (chunk > (1ull << 31)) chunk = 1ull << 31;
   const int kcap = tc ? (k * 8 > 256 ? k * 8 : 256) : k;
   const uint64_t launch_len = hi - lo < chunk ? hi - lo : chunk;
-  const int grid = fc ? fc_grid(ctx, launch_len) : (tc || tx) ? tc_grid(ctx) : f32_grid(ctx, launch_len);
+  const int grid = fc ? fc_grid(ctx, launch_len, k) : (tc || tx) ? tc_grid(ctx) : f32_grid(ctx, launch_len);
 
   // scratch: per-CTA lists, two merge buffers, merged list, rescored shortlist, count
   const size_t entries = (size_t)grid * kcap;

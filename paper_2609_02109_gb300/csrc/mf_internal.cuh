@@ -472,7 +472,7 @@ mf_status f32_prepare(mf_ctx* c);
 mf_status f32_search_chunk(mf_ctx* c, const RangeArgs& a, int grid, cudaStream_t s);
 // Fixed-context mode: one range launch of the table-lookup scan over the per-option
 // table of mf_fc_set.
-int fc_grid(const mf_ctx* c, uint64_t len);
+int fc_grid(const mf_ctx* c, uint64_t len, int k);
 mf_status fc_search_chunk(mf_ctx* c, const RangeArgs& a, int grid, cudaStream_t s);
 mf_status f32_search_chunk_params(const Params& P, int grid, const RangeArgs& a, cudaStream_t s);
 mf_status f32_score_list(mf_ctx* c, const uint64_t* idx, const int32_t* genes, uint64_t n,
