@@ -33,8 +33,6 @@ struct ListArgs {
   float* pred;             // [n][N][2] or null
 };
 
-__host__ __device__ constexpr int round4(int v) { return (v + 3) & ~3; }
-
 // ---------------------------------------------------------------------------
 // One model's predictor on one candidate, compile-time shape.
 // w: the model's packed weights (16-byte aligned), z: the d_in inputs.
@@ -584,8 +582,6 @@ size_t topk_bytes(int k) {
 }
 
 }  // namespace
-
-bool f32_supported(const Params& P) { return P.d_local <= MF_MAX_D_LOCAL; }
 
 size_t f32_smem_bytes(const Params& P, int k, bool& resident) {
   const size_t wbytes = (size_t)P.n_models * P.per_model * sizeof(float);

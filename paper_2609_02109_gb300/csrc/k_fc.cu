@@ -204,8 +204,9 @@ k_fc_local(const Params P, const FcLayout L, const FcInputs I, const FcConst C) 
 // otherwise one list and queue per CTA, whose warps meet for a merge when it fills up.
 //
 // Bound by latency (shared-memory chains of the counts; the prologue's ranking and corner).
-// 24^6, VRAM binding, k = 32: one launch of 36 us, where the scan of every candidate took 12
-// launches of 75-125 us, each of which also filled its lists from nothing.
+// 24^6, VRAM binding: one launch of 23 us at k = 1, 27 at k = 32, 35 at k = 100; everything fits:
+// 15.  The scan of every candidate took 12 launches of 75-125 us, each of which also filled its
+// lists from nothing.
 // ---------------------------------------------------------------------------
 constexpr int kFcThreads = 512;
 constexpr int kFcWarpK = 64, kFcWarps = kFcThreads / 32;

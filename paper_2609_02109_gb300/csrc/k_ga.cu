@@ -98,13 +98,6 @@ mf_status ga_step(mf_ctx* c, const mf_ga_params* g, uint64_t seed, int32_t gen,
   return MF_OK;
 }
 
-mf_status ga_best(mf_ctx* c, const int32_t* pop, const float* fit, int P, int32_t* out_genome,
-                  float* out_fit, cudaStream_t s) {
-  k_ga_best<<<1, 1024, 0, s>>>(P, c->P.n_models, pop, fit, out_genome, out_fit);
-  MF_CUDA(cudaGetLastError());
-  return MF_OK;
-}
-
 }  // namespace mf
 
 namespace mf {

@@ -101,18 +101,6 @@ __device__ __forceinline__ void named_bar(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
-// OR of `pred` over the threads of a named barrier (also a barrier).
-__device__ __forceinline__ bool named_bar_or(int id, int nthreads, bool pred) {
-  uint32_t r;
-  asm volatile(
-      "{\n .reg .pred pi, po;\n setp.ne.u32 pi, %1, 0;\n bar.red.or.pred po, %2, %3, pi;\n"
-      " selp.u32 %0, 1, 0, po;\n}"
-      : "=r"(r)
-      : "r"((uint32_t)pred), "r"(id), "r"(nthreads)
-      : "memory");
-  return r != 0;
-}
-
 // UMMA shared-memory descriptor: K-major, no swizzle.  lbo = byte distance of
 // core matrices adjacent in K, sbo = byte distance of adjacent 8-row groups.
 __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
@@ -128,22 +116,6 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int n) {
 // Instruction descriptor of kind::tf32: tf32 A and B (K-major), fp32 D, M = 128.
 __host__ __device__ constexpr uint32_t idesc_tf32(int n) {
   return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-}
-
-// D[tmem] (+)= A[tmem] . B[smem]^T, one 128 x n x 16 MMA.
-__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   smem_u32(bar))
-               : "memory");
 }
 
 // ReLU then round to bf16, two values per register: `lo` in the low half.
@@ -168,12 +140,6 @@ __device__ __forceinline__ uint32_t tmem_ld_x1(uint32_t taddr) {
   uint32_t r;
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr));
   return r;
-}
-
-__device__ __forceinline__ void tmem_ld_x16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-               : "r"(taddr));
 }
 
 __device__ __forceinline__ void tmem_ld_x32(uint32_t taddr, uint32_t (&r)[32]) {
@@ -251,9 +217,8 @@ struct NamedSync128 {
   __device__ void operator()() const { named_bar(id, 128); }
 };
 
-// (a queue of 128 into a list of 256: 3 k cycles sorted, 15 k by counting)
 // The pipeline's top-k merge, out of line: it runs rarely and its registers stay off
-// the hot loop.
+// the hot loop.  (A queue of 128 into a list of 256: 3 k cycles sorted, 15 k by counting.)
 static __device__ __noinline__ void tc_topk_merge(const CtaTopK& tk, int row, int barid) {
   if (*tk.qn <= 24) topk_merge(tk, row, 128, NamedSync128{barid});
   else topk_merge_sorted(tk, row, 128, NamedSync128{barid});
@@ -349,9 +314,9 @@ __device__ __forceinline__ float tc_out(const Params& P, float v) {
   return P.out_act == MF_ACT_SIGMOID ? tc_sigmoid(v) : v;
 }
 
-// MMA issue by a whole warp: every lane executes the instruction stream (so the
-// operands stay warp-uniform) and one elected lane issues.  The same lane is elected
-// for the MMAs and for the commit that tracks them.
+// D[tmem] (+)= A[tmem] . B[smem]^T, one 128 x n x 16 MMA, issued by a whole warp: every lane
+// executes the instruction stream (so the operands stay warp-uniform) and one elected lane
+// issues.  The same lane is elected for the MMAs and for the commit that tracks them.
 __device__ __forceinline__ void mma_ts_warp(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
                                             uint32_t accumulate) {
   asm volatile(

@@ -465,7 +465,6 @@ __device__ __forceinline__ unsigned long long device_ns() {
 __device__ __forceinline__ void stamp_start(const RangeArgs& R) {
   if (R.first && R.start && blockIdx.x == 0 && threadIdx.x == 0) *R.start = device_ns();
 }
-bool f32_supported(const Params& P);
 size_t f32_smem_bytes(const Params& P, int k, bool& resident);
 int f32_grid(const mf_ctx* c, uint64_t len);
 mf_status f32_prepare(mf_ctx* c);
@@ -522,13 +521,11 @@ mf_status tc_score_list(mf_ctx* c, const uint64_t* idx, uint64_t n, float* score
 mf_status ga_init(mf_ctx* c, const mf_ga_params* g, uint64_t seed, int32_t* pop, cudaStream_t s);
 mf_status ga_step(mf_ctx* c, const mf_ga_params* g, uint64_t seed, int32_t gen,
                   const int32_t* pop, const float* fit, int32_t* next, cudaStream_t s);
-mf_status ga_best(mf_ctx* c, const int32_t* pop, const float* fit, int P, int32_t* out_genome,
-                  float* out_fit, cudaStream_t s);
 // Whole GA decision as one CUDA graph launch on `s`; the result lands in c->d_ga_out
 // and the pinned staging buffer is sized for it.
 mf_status ga_run_graph(mf_ctx* c, const mf_ga_params* g, uint64_t seed, cudaStream_t s);
-// Whole GA decision in one cooperative kernel; MF_EUNSUPPORTED (nothing launched) when
-// the shape or the device does not allow it.
+// Whole GA decision in one cooperative kernel, whose result lands in the pinned staging
+// buffer; MF_EUNSUPPORTED (nothing launched) when the shape or the device does not allow it.
 mf_status ga_run_persistent(mf_ctx* c, const mf_ga_params* g, uint64_t seed, cudaStream_t s);
 
 }  // namespace mf
