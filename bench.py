@@ -46,8 +46,10 @@ L2_FLUSH_BYTES = 256 << 20
 
 # DRAM bytes (read + write) of one scoring launch from the ncu capture of the scoring
 # kernel on this workload, valid only while the kernel's sources are the ones that were
-# captured (sha256 prefix of k_tc.cuh + mf_internal.cuh).
-NCU_TRAFFIC = {"bf16": ("69358510742953d4", 225280), "fp32": ("69358510742953d4", 265216)}
+# captured (sha256 prefix of k_tc.cuh + mf_internal.cuh).  fp32: a first-pass launch of
+# the exact variant (models 0-2), which writes the 16-byte partial record of each of its
+# 2^24 candidates for the second pass (which reads them back).
+NCU_TRAFFIC = {"bf16": ("33faf51dda2c6380", 235776), "fp32": ("33faf51dda2c6380", 206913536)}
 
 
 def _traffic(prec):
