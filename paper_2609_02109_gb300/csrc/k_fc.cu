@@ -210,7 +210,9 @@ k_fc_local(const Params P, const FcLayout L, const FcInputs I, const FcConst C) 
 // ---------------------------------------------------------------------------
 constexpr int kFcThreads = 512;
 constexpr int kFcWarpK = 64, kFcWarps = kFcThreads / 32;
-constexpr int kFcCtaQ = 4096, kFcWarpQ = 256;         // a CTA's and a warp's queue
+// A CTA's and a warp's queue.  (128 for a warp: with 256, warps that queue equal scores sorted
+// twice as many before the list's bar stopped them: 3^14 of one score 194 us, 171 with 128.)
+constexpr int kFcCtaQ = 4096, kFcWarpQ = 128;
 constexpr int kFcEndQ = kFcWarps * kFcWarpK;          // the warps' lists, merged at the end (a power of two)
 constexpr int kFcLambdas = 4, kFcCornerOpts = 64;     // corner sets, options of a model in one
 constexpr int kFcCornerBits = 10;                     // configurations of a corner: 2^10
